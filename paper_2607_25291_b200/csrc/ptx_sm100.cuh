@@ -88,9 +88,28 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
   const bool ok = mbar_wait(bar, parity, abort_flag, budget);
   return unanimous ? (__all_sync(0xffffffffu, ok) != 0) : ok;
 }
+// A bounded wait (all lanes, one answer) that never suspends beyond its budget: mbarrier.try_wait may be suspended until the phase
+// completes and then report success, however short the budget is.
+__device__ __forceinline__ bool mbar_poll_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget) {
+  const long long t0 = clock64();
+  bool ok;
+  while (!(ok = mbar_test_wait(bar, parity)) && !*abort_flag && clock64() - t0 <= budget) __nanosleep(32);
+  return __all_sync(0xffffffffu, ok) != 0;
+}
 // named barrier among `nthreads` threads of the CTA (ids 1..15; 0 is __syncthreads)
 __device__ __forceinline__ void bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
+// the same barrier; true for every thread iff `pred` is true for any
+__device__ __forceinline__ bool bar_red_or(int id, int nthreads, bool pred) {
+  uint32_t any;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %3, 0;\n\tbar.red.or.pred q, %1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(any)
+      : "r"(id), "r"(nthreads), "r"((uint32_t)pred)
+      : "memory");
+  return any != 0;
 }
 
 // ---------------------------------------------------------------- TMA
@@ -332,6 +351,21 @@ __device__ __forceinline__ void mma_ss_x8(uint32_t d_tmem, uint64_t adesc0, uint
       "add.s64 a, %1, %10;\n\tadd.s64 b, %2, %10;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p1;\n\t"
       "}" ::"r"(d_tmem),
       "l"(adesc0), "l"(bdesc0), "r"(idesc), "n"(S1), "n"(S2), "n"(S3), "n"(S4), "n"(S5), "n"(S6), "n"(S7)
+      : "memory");
+}
+// Four MMAs over K = 64, both operands in shared memory: A advances by A1.., B by B1.. (16-byte units).
+template <int A1, int A2, int A3, int B1, int B2, int B3>
+__device__ __forceinline__ void mma_ss_x4(uint32_t d_tmem, uint64_t adesc0, uint64_t bdesc0, uint32_t idesc, bool accumulate_first) {
+  uint32_t acc = accumulate_first ? 1u : 0u;
+  asm volatile(
+      "{\n\t.reg .pred p0, p1;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 p0, %4, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p0;\n\t"
+      "add.s64 a, %1, %5;\n\tadd.s64 b, %2, %8;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p1;\n\t"
+      "add.s64 a, %1, %6;\n\tadd.s64 b, %2, %9;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p1;\n\t"
+      "add.s64 a, %1, %7;\n\tadd.s64 b, %2, %10;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p1;\n\t"
+      "}" ::"r"(d_tmem),
+      "l"(adesc0), "l"(bdesc0), "r"(idesc), "r"(acc), "n"(A1), "n"(A2), "n"(A3), "n"(B1), "n"(B2), "n"(B3)
       : "memory");
 }
 // The mbarrier receives one arrival when every MMA issued so far by this thread has finished.

@@ -416,6 +416,29 @@ def test_osk_4k_workload(cfg1, impl):
     print("4k", stats)
 
 
+@pytest.mark.parametrize("length", [1, 2, 3, 4, 7])
+@pytest.mark.parametrize("tb,skip_scale", [(1.0, -1.0), (0.999, 100.0), (0.999, 900.0), (0.13, 500.0), (0.3, -1.0)])
+def test_osk_short_walks_with_growing_maxima(small, length, tb, skip_scale):
+    """Walks of one to seven blocks (tile slots change roles with every decision; the cap ends walks at one, two or three
+    computed blocks), keys scaled so that the running maximum moves by less and by more than the factor above which O is
+    rescaled, blocks listed by ascending maximum in half of the lists.  Bars as everywhere: P and the output are bf16."""
+    q, k, v = small["dev"]
+    qf, kf, vf = small["f64"]
+    rng = np.random.Generator(np.random.Philox(key=[length, 5]))
+    hq, nqb = 4, 8
+    factors = np.repeat(rng.permutation(2.0 ** np.arange(-4, 4)), 128)          # powers of two: exact in bf16
+    k2 = (k.float() * torch.from_numpy(factors).float().cuda()[None, None, :, None]).to(torch.bfloat16)
+    kf2 = kf * factors[None, :, None]
+    order = np.full((1, hq, nqb, nqb), -1, np.int32)
+    for h in range(hq):
+        for i in range(nqb):
+            ids = rng.choice(nqb, size=length, replace=False)
+            order[0, h, i, :length] = ids if h % 2 else ids[np.argsort(factors[ids * 128])]
+    count = np.full((1, hq, nqb), length, np.int32)
+    bufs = run_osk(q, k2, v, torch.from_numpy(order).cuda(), torch.from_numpy(count).cuda(), tb, skip_scale, causal=False)
+    check_osk_against_oracle(qf, kf2, vf, order[0], count[0], bufs, tb, skip_scale, range(hq), range(nqb), causal=False)
+
+
 @pytest.mark.parametrize("impl", OSK_IMPLS)
 def test_osk_noncausal(small, impl):
     q, k, v = small["dev"]
