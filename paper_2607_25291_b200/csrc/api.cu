@@ -21,15 +21,47 @@ static int cuda_fail(cudaError_t e, const char* what) {
   return COSA_ERR_CUDA;
 }
 
+// Facts about a device that do not change while the process lives, asked once per device.
 int32_t* device_status_word() {
-  void* ptr = nullptr;
-  if (cudaGetSymbolAddress(&ptr, g_status_word) != cudaSuccess) return nullptr;
-  return static_cast<int32_t*>(ptr);
+  static std::atomic<int32_t*> known[kMaxDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+  int32_t* word = known[dev].load(std::memory_order_relaxed);
+  if (!word) {
+    void* ptr = nullptr;
+    if (cudaGetSymbolAddress(&ptr, g_status_word) != cudaSuccess) return nullptr;
+    word = static_cast<int32_t*>(ptr);
+    known[dev].store(word, std::memory_order_relaxed);
+  }
+  return word;
+}
+int device_sm_count() {
+  static std::atomic<int> known[kMaxDevices];
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+  sms = known[dev].load(std::memory_order_relaxed);
+  if (sms <= 0) {
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 0;
+    known[dev].store(sms, std::memory_order_relaxed);
+  }
+  return sms;
+}
+cudaError_t raise_smem_limit(const void* kernel, SmemLimit* state, size_t bytes) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (state->bytes[dev].load(std::memory_order_acquire) >= (int)bytes) return cudaSuccess;
+  static std::mutex mu;      // two threads must not lower each other's limit
+  std::lock_guard<std::mutex> lock(mu);
+  if (state->bytes[dev].load(std::memory_order_acquire) >= (int)bytes) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) state->bytes[dev].store((int)bytes, std::memory_order_release);
+  return e;
 }
 
 // ---- the library's own per-device scratch (used when options.workspace is NULL) ----
 namespace {
-constexpr int kMaxDevices = 64;
 struct OwnScratch { void* ptr = nullptr; size_t bytes = 0; };
 OwnScratch g_scratch[kMaxDevices];
 std::mutex g_scratch_mu;
@@ -121,7 +153,7 @@ cosa_options resolve_options(const cosa_options* opt) {
 }  // namespace
 
 // scratch the kernels of one call need (beyond inputs and outputs)
-struct KapScratch { size_t scores, jstar, ambmask, hard, redo_list, k2max, q2max, slot_taken, maxima, kstage, total; int slots; bool gather; };
+struct KapScratch { size_t scores, jstar, ambmask, hard, redo_list, k2max, k2part, q2max, slot_taken, maxima, kstage, total; int slots; bool gather; };
 static KapScratch kap_scratch_layout(const cosa_shape* s, const cosa_options& o) {
   KapScratch L{};
   const int stride = o.stride > 0 ? o.stride : 8;
@@ -142,6 +174,7 @@ static KapScratch kap_scratch_layout(const cosa_shape* s, const cosa_options& o)
   L.hard = off; off += align_up(heads * nqb, 256);
   L.redo_list = off; off += align_up((1 + heads * nqb) * 4, 256);
   L.k2max = off; off += 256;
+  L.k2part = off; off += align_up(kNormParts * 4, 256);
   L.q2max = off; off += align_up(heads * nqb * 4, 256);
   // the screen's parked block maxima: one area per CTA that can be resident on the current device
   L.slots = kap_screen_slots();
@@ -260,7 +293,8 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
   sp.hard = reinterpret_cast<uint8_t*>(ws + L.hard);
   sp.redo_list = reinterpret_cast<int32_t*>(ws + L.redo_list);
   sp.slot_taken = reinterpret_cast<int32_t*>(ws + L.slot_taken);
-  sp.k2max = reinterpret_cast<const float*>(ws + L.k2max);
+  sp.k2max = reinterpret_cast<float*>(ws + L.k2max);
+  sp.k2part = reinterpret_cast<float*>(ws + L.k2part);
   sp.q2max = reinterpret_cast<float*>(ws + L.q2max);
   sp.maxima = reinterpret_cast<float*>(ws + L.maxima);
   sp.slots = L.slots;
@@ -280,7 +314,7 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
   }
   sp.pg = p.pg;
   sp.qs = p.qs; sp.ks = p.ks;
-  cudaError_t e = launch_kap_norms(sp.k, sp.pg, sp.ks, p.batch, p.hkv, p.n, s, reinterpret_cast<float*>(ws + L.k2max), st);
+  cudaError_t e = launch_kap_norms(&sp, st);
   if (e != cudaSuccess) return cuda_fail(e, "kap norms launch");
   e = launch_kap_screen(sp, st);
   if (e != cudaSuccess) return cuda_fail(e, "kap screen launch");

@@ -5,6 +5,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+#include <utility>
+
 #include "cosa.h"
 
 namespace cosa {
@@ -103,8 +106,10 @@ struct KapScreenParams {
   uint8_t* hard;         // [B,Hq,nQB]      1 = three blocks too close on some row: whole query block goes to double precision
   int32_t* redo_list;    // [1 + B*Hq*nQB]  [0] = number of entries, then flat (b*Hq+h)*nQB+i of query blocks to redo
   float* maxima;         // [slots][key tiles][128 rows x 128/R blocks]  per-row block maxima of the CTA that holds the slot
-  int32_t* slot_taken;   // [slots]  0 = free; zeroed before every launch
-  const float* k2max;    // [1]  largest squared norm of a sampled key row of the call (kap_norms_kernel)
+  int32_t* slot_taken;   // [slots]  0 = free; zeroed by kap_norms_kernel
+  float* k2part;         // [kNormParts]  largest squared norms of sampled key rows of the call, one per CTA of kap_norms_kernel
+  int k2parts;           // ... how many
+  float* k2max;          // [1]  their maximum, left by the screen for the sort stage
   float* q2max;          // [B,Hq,nQB]  largest squared norm of the sampled query rows of every (head, query block)
   int slots;             // CTAs that can be resident at once
   int batch, hq, hkv, n, nqb;
@@ -205,13 +210,43 @@ __host__ __device__ inline float screen_error_bound(float q2max, float k2max, fl
 
 // device status word (one per device), set by kernels whose bounded waits give up
 int32_t* device_status_word();
+// SM count of the current device, 0 if it cannot be read
+int device_sm_count();
+
+// The kernels of a call follow one another closely and the small ones last a few microseconds, as long as a launch takes.
+// launch_chained lets a kernel's launch overlap the kernel before it in the stream (programmatic dependent launch); the kernel
+// calls chain_begin() before it touches global memory: it waits until everything before it in the stream has finished
+// and its writes are visible, then lets the next launch begin.  (Two memsets and four launches one after the other to
+// launches that overlap, norms folded in: 31 blocks of 32 heads 96 -> 75 us a pass.)
+__device__ __forceinline__ void chain_begin() {
+#if defined(__CUDA_ARCH__)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+template <typename... Params, typename... Args>
+cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+// Raises a kernel's dynamic shared memory limit on the current device, once (`state`: one per kernel, zero-initialised: the
+// limit set so far per device)
+constexpr int kMaxDevices = 64;
+struct SmemLimit { std::atomic<int> bytes[kMaxDevices]; };
+cudaError_t raise_smem_limit(const void* kernel, SmemLimit* state, size_t bytes);
 
 // redo_list == nullptr: every (head, query block); else only the listed ones (count in [0])
 cudaError_t launch_kap_exact(const KapParams& p, const int32_t* redo_list, cudaStream_t st);
 bool kap_screen_supported(int rows, int group, int stride, const KvPaging& pg);
 cudaError_t launch_kap_screen(const KapScreenParams& p, cudaStream_t st);
-cudaError_t launch_kap_norms(const __nv_bfloat16* k, const KvPaging& pg, const Strides& ks, int batch, int hkv, int n, int stride,
-                             float* k2max, cudaStream_t st);
+constexpr int kNormParts = 296;   // CTAs of kap_norms_kernel at most
+// writes sp->k2part and sp->k2parts, clears sp->slot_taken
+cudaError_t launch_kap_norms(KapScreenParams* sp, cudaStream_t st);
 // CTAs of the screen kernel that can be resident at once on the current device (0 on failure), and the bytes of
 // block-maxima scratch each of them needs
 int kap_screen_slots();

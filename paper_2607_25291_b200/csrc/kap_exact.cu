@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(kThreads) kap_exact_kernel(KapParams p, int kb
 // 1-d grid: the CTAs share out the entries of a redo list (usually empty)
 __global__ void __launch_bounds__(kThreads) kap_exact_list_kernel(KapParams p, const int32_t* redo_list, int kb_per_iter,
                                                                  int sort_cap, const int32_t* status) {
+  chain_begin();
   if (*reinterpret_cast<const volatile int32_t*>(status) != 0) return;   // an earlier kernel of the call gave up: the list is not to be trusted
   const int n = redo_list[0];
   for (int e = blockIdx.x; e < n; e += gridDim.x) {
@@ -233,12 +234,13 @@ size_t kap_exact_smem_bytes(int rows, int nqb, int qtiles) {
 cudaError_t launch_kap_exact(const KapParams& p, const int32_t* redo_list, cudaStream_t st) {
   size_t smem = kap_exact_smem_bytes(p.rows, p.nqb, p.qtiles);
   if (redo_list) {
-    cudaError_t e = cudaFuncSetAttribute(kap_exact_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemLimit limit;
+    cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kap_exact_list_kernel), &limit, smem);
     if (e != cudaSuccess) return e;
     const int32_t* status = device_status_word();
     if (!status) return cudaErrorInvalidSymbol;
-    kap_exact_list_kernel<<<148, kThreads, smem, st>>>(p, redo_list, kb_per_iter_for(p.rows), next_pow2(p.nqb), status);
-    return cudaGetLastError();
+    return launch_chained(kap_exact_list_kernel, dim3(148), kThreads, smem, st, p, redo_list, kb_per_iter_for(p.rows), next_pow2(p.nqb),
+                          status);
   }
   cudaError_t e = cudaFuncSetAttribute(kap_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

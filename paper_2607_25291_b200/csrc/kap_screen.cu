@@ -70,6 +70,15 @@ __device__ __forceinline__ void screen_timeout(ScreenCtl* c, int32_t* status) {
 }
 
 // kStrict: every multi-lane wait answers per warp (see mbar_wait_warp)
+// (a whole warp) the largest squared norm of a sampled key row of the call
+__device__ __forceinline__ float largest_key_norm(const KapScreenParams& p, int lane) {
+  float k2 = 0.f;
+  for (int t = lane; t < p.k2parts; t += 32) k2 = fmaxf(k2, p.k2part[t]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) k2 = fmaxf(k2, __shfl_xor_sync(0xffffffffu, k2, o));
+  return k2;
+}
+
 template <int R, bool kStrict>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
@@ -78,6 +87,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - raw);
+  chain_begin();
   const uint32_t a_sm = base;
   const uint32_t k_sm = base + kRowTiles * kTileBytes;
   ScreenCtl* ctl = reinterpret_cast<ScreenCtl*>(smem + (size_t)kTileBytes * (kRowTiles + kStages));
@@ -100,13 +110,21 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const int n_tiles = (n_keys + 127) / 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  if (blockIdx.x == 0 && threadIdx.x == 0) p.redo_list[0] = 0;   // the sort stage (a later launch) appends to it
+  if (blockIdx.x == 0 && warp == 0) {
+    const float k2 = largest_key_norm(p, lane);
+    if (lane == 0) {
+      *p.k2max = k2;          // for the sort stage (a later launch) ...
+      p.redo_list[0] = 0;     // ... which appends to this list
+    }
+  }
   if (i0 >= nqb_b) return;                        // all of this CTA's query blocks are padding
   if (threadIdx.x == 0) {
     // once some CTA has reported a timeout the rest of the grid returns at once
     int poisoned = *reinterpret_cast<volatile int32_t*>(status);
     int slot = -1;
-    if (poisoned == 0) {
+    if (poisoned == 0 && (int)gridDim.x <= p.slots) {
+      slot = (int)blockIdx.x;               // an area for every CTA: nothing to search for
+    } else if (poisoned == 0) {
       // a scratch area no resident CTA holds: there are as many as CTAs can be resident, so one is free; the
       // search starts at this SM's number and normally ends at once
       unsigned smid;
@@ -248,6 +266,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     // each half tile; the swizzle permutes 16-byte chunks inside a row, which a sum of squares does not notice; the
     // chunk order is rotated by the lane so that the rows of a warp hit different banks)
     float q2 = 0.f;
+    const float k2 = largest_key_norm(p, lane);
     bool alive = mbar_wait_warp(smem_u32(&ctl->a_full), 0, abort_flag, budget, strict);
     if (!alive && !*abort_flag) screen_timeout(ctl, status);
     if (alive) {
@@ -334,7 +353,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       // the row's best block, and whether the runner-up is too close to call
       // (the threshold grows with the magnitude of the row and of the call's keys, which is what the rounding error of a
       // logit follows)
-      const float tau_row = fmaxf(p.tau_row, 2.f * screen_error_bound(q2, *p.k2max, p.scale));
+      const float tau_row = fmaxf(p.tau_row, 2.f * screen_error_bound(q2, k2, p.scale));
       const bool amb = row_ok && (top1 - top2) * p.scale <= tau_row;
       const bool amb3 = row_ok && (top1 - top3) * p.scale <= tau_row;
       const unsigned any_amb = __ballot_sync(0xffffffffu, amb), any_amb3 = __ballot_sync(0xffffffffu, amb3);
@@ -461,6 +480,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     for (size_t off = (size_t)threadIdx.x * 128; off < bytes; off += (size_t)kThreads * 128)
       asm volatile("discard.global.L2 [%0], 128;" ::"l"(area + off) : "memory");
   }
+  if ((int)gridDim.x <= p.slots) return;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -482,11 +502,7 @@ int kap_screen_grid(int batch, int hq, int hkv, int nqb, int stride) {
 }
 
 int kap_screen_slots() {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-    return 0;
-  return sms * kCtasPerSm;
+  return device_sm_count() * kCtasPerSm;
 }
 
 size_t kap_screen_slot_bytes(int n, int stride) {
@@ -498,8 +514,6 @@ cudaError_t launch_kap_screen(const KapScreenParams& p_in, cudaStream_t st) {
   KapScreenParams p = p_in;
   const int R = 128 / p.stride;
   if (!p.maxima || !p.slot_taken || p.slots <= 0) return cudaErrorInvalidValue;
-  cudaError_t e0 = cudaMemsetAsync(p.slot_taken, 0, (size_t)p.slots * sizeof(int32_t), st);
-  if (e0 != cudaSuccess) return e0;
   const uint64_t ns = (uint64_t)p.n / p.stride;
   CUtensorMap qm, km;
   // every `stride`-th row of q and k: the row stride of the maps is `stride` rows of the tensor (of the page pool)
@@ -521,16 +535,16 @@ cudaError_t launch_kap_screen(const KapScreenParams& p_in, cudaStream_t st) {
 #define COSA_LAUNCH_SCREEN(RR)                                                                                              \
   {                                                                                                                         \
     auto kernel = wait_budget_is_short(p.wait_budget) ? kap_screen_kernel<RR, true> : kap_screen_kernel<RR, false>;         \
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScreenSmem);                        \
+    static SmemLimit limits[2];                                                                                             \
+    e = raise_smem_limit(reinterpret_cast<const void*>(kernel), &limits[wait_budget_is_short(p.wait_budget)], kScreenSmem); \
     if (e != cudaSuccess) return e;                                                                                         \
-    kernel<<<grid, kThreads, kScreenSmem, st>>>(qm, km, p, status);                                                         \
+    return launch_chained(kernel, dim3(grid), kThreads, kScreenSmem, st, qm, km, p, status);                                \
   }
   if (R == 8) { COSA_LAUNCH_SCREEN(8) }
   else if (R == 16) { COSA_LAUNCH_SCREEN(16) }
   else if (R == 32) { COSA_LAUNCH_SCREEN(32) }
-  else return cudaErrorInvalidValue;
+  return cudaErrorInvalidValue;
 #undef COSA_LAUNCH_SCREEN
-  return cudaGetLastError();
 }
 
 }  // namespace cosa

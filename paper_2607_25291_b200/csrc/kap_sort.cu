@@ -393,6 +393,7 @@ __global__ void __launch_bounds__(kThreads, 6) kap_sort_kernel(KapParams p, KapS
   __shared__ int j1[kMaxRows], j2[kMaxRows];
   __shared__ int n_tied, tail_end;
 
+  chain_begin();
   const int R = p.rows;                       // sampled rows per 128-row tile
   const int T = p.qtiles;                     // row tiles that share this ranking
   const int RT = R * T;
@@ -725,13 +726,13 @@ cudaError_t launch_kap_sort(const KapParams& p, const KapScreenParams& sp, float
   const int cap = next_pow2(p.nqb);
   const int tie_bytes = (cap + 15) / 16 * 16;
   size_t smem = (size_t)cap * 8 + tie_bytes + (size_t)p.rows * p.qtiles * kPad * 8;
-  cudaError_t e = cudaFuncSetAttribute(kap_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static SmemLimit limit;
+  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kap_sort_kernel), &limit, smem);
   if (e != cudaSuccess) return e;
   dim3 grid(p.nqb / p.qtiles, p.hq, p.batch);
   const int32_t* status = device_status_word();
   if (!status) return cudaErrorInvalidSymbol;
-  kap_sort_kernel<<<grid, kThreads, smem, st>>>(p, sp, tau_score, cap, tie_bytes, status);
-  return cudaGetLastError();
+  return launch_chained(kap_sort_kernel, grid, kThreads, smem, st, p, sp, tau_score, cap, tie_bytes, status);
 }
 
 }  // namespace cosa

@@ -122,6 +122,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
   const int i = p.nqb - 1 - (wk % per_kv) / G;
   const int h = g * G + (wk % per_kv) % G;
   const size_t row = (size_t)(b * p.hq + h) * p.nqb + i;
+  chain_begin();
   const int nqb_b = item_blocks(p.pg, b, p.nqb);   // the item's own length in blocks; query blocks past it are padding
   const int J = p.causal ? i + 1 : max(nqb_b, 1);
   const int32_t* list = p.order + row * p.order_stride;   // unused when kMask
@@ -546,7 +547,8 @@ cudaError_t launch_osk_tc(const OskParams& p_in, cudaStream_t st) {
                     : (small_pages ? osk_tc_kernel<M, false, true> : osk_tc_kernel<M, false, false>);
   };
   auto kernel = p.mask ? pick(std::true_type{}) : pick(std::false_type{});
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+  static SmemLimit limits[8];
+  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kernel), &limits[(p.mask ? 4 : 0) + (p.stage2 ? 2 : 0) + (small_pages ? 1 : 0)], kSmemBytes);
   if (e != cudaSuccess) return e;
   if (p.decisions) {
     size_t words = (size_t)p.batch * p.hq * p.nqb * ((p.order_stride + 31) / 32);
@@ -555,12 +557,9 @@ cudaError_t launch_osk_tc(const OskParams& p_in, cudaStream_t st) {
   }
   int32_t* status = device_status_word();
   if (!status) return cudaErrorInvalidSymbol;
-  int dev = 0, n_sm = 0;
-  p.wave = 1 << 30;   // (no prefetch if the SM count cannot be read)
-  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n_sm > 0)
-    p.wave = kCtasPerSm * n_sm;
-  kernel<<<p.batch * p.hq * p.nqb, kThreads, kSmemBytes, st>>>(qm, km, vm, om, p, status);
-  return cudaGetLastError();
+  const int n_sm = device_sm_count();
+  p.wave = n_sm > 0 ? kCtasPerSm * n_sm : 1 << 30;   // (no prefetch if the SM count cannot be read)
+  return launch_chained(kernel, dim3(p.batch * p.hq * p.nqb), kThreads, kSmemBytes, st, qm, km, vm, om, p, status);
 }
 
 }  // namespace cosa

@@ -953,6 +953,34 @@ def test_reserved_scratch_makes_plain_calls_allocation_free(cfg1):
     assert cosa.cosa_device_status() == 0
 
 
+@pytest.mark.parametrize("passes", [2, 5])
+def test_passes_that_nothing_waits_between_equal_passes_on_their_own(small, cfg1, passes):
+    """The kernels of a call begin while the kernel before them is still running (and wait for it before they touch memory):
+    passes over two inputs in turn, on shared scratch and outputs, give the bits that each gives on its own."""
+    def run(case, order, count, bufs):
+        q, k, v = case["dev"]
+        w = case["w"]
+        cosa.cosa_kap_select(q, k, w.kap_budget, order, count, opt=cosa.default_options(stride=8))
+        cosa.cosa_osk_attention(q, k, v, order, count, 0.5, bufs["out"], bufs["lse"], bufs["visited"],
+                                opt=cosa.default_options(skip_scale=w.n * 0.8))
+
+    state, alone = [], []
+    for case in (small, cfg1):
+        w = case["w"]
+        state.append((*alloc_lists(w.hq, w.n // 128), alloc_outputs(case["dev"][0], w.n // 128)))
+        run(case, *state[-1])
+        assert cosa.cosa_device_status() == 0
+        order, count, bufs = state[-1]
+        alone.append([t.clone() for t in (order, count, bufs["out"], bufs["lse"], bufs["visited"])])
+    for _ in range(passes):
+        for case, st in zip((small, cfg1), state):
+            run(case, *st)
+    assert cosa.cosa_device_status() == 0
+    for (order, count, bufs), want in zip(state, alone):
+        for got, ref in zip((order, count, bufs["out"], bufs["lse"], bufs["visited"]), want):
+            assert torch.equal(got, ref)
+
+
 def test_osk_is_deterministic(cfg1):
     w = cfg1["w"]
     q, k, v = cfg1["dev"]
