@@ -119,17 +119,24 @@ def _check(status: int, where: str):
         raise CosaError(status, where)
 
 
+# The current stream's handle without building a torch.cuda.Stream around it (0.3 us a call instead of 3.3: for a short
+# prompt the enqueue is what the GPU waits for).  Where this torch has no such function, the long way.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream_ptr(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device())
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream)
 
 
 def make_shape(q: torch.Tensor, k: torch.Tensor, causal: bool = True, block: int = 128) -> CosaShape:
     """q [B,Hq,N,d], k [B,Hkv,N,d] (3-d tensors are taken as B = 1)."""
-    qs = tuple(q.shape) if q.dim() == 4 else (1, *q.shape)
-    ks = tuple(k.shape) if k.dim() == 4 else (1, *k.shape)
-    return CosaShape(qs[0], qs[1], ks[1], qs[2], qs[3], block, block, 1 if causal else 0)
+    b, hq, n, d = q.shape if q.dim() == 4 else (1, *q.shape)
+    return CosaShape(b, hq, k.shape[-3], n, d, block, block, 1 if causal else 0)
 
 
 def default_options(**kw) -> CosaOptions:
@@ -155,28 +162,34 @@ def _dev_ptr(t: torch.Tensor, dtype, name: str) -> int:
     return t.data_ptr()
 
 
+_BF16, _I32, _F32 = torch.bfloat16, torch.int32, torch.float32
+_DENSE = (ctypes.c_int64 * 3)(0, 0, 0)
+
+
 def _strided_ptr(t: torch.Tensor, name: str):
     """Pointer and (batch, head, token) element strides of a [B,H,N,d] bf16 CUDA tensor or view whose rows are contiguous;
-    strides (0, 0, 0) stand for the dense layout."""
+    _DENSE stands for the dense layout."""
     if t.dim() == 3:
         t = t[None]                                         # [H,N,d]: one batch item
-    if not t.is_cuda or t.dtype != torch.bfloat16 or t.dim() != 4 or t.stride(3) != 1:
+    if not t.is_cuda or t.dtype != _BF16 or t.dim() != 4 or t.stride(3) != 1:
         raise ValueError(f"{name}: expected a [B,H,N,d] CUDA bfloat16 tensor with contiguous rows")
-    return t.data_ptr(), ((0, 0, 0) if t.is_contiguous() else tuple(int(x) for x in t.stride()[:3]))
+    return t.data_ptr(), (_DENSE if t.is_contiguous() else (ctypes.c_int64 * 3)(*t.stride()[:3]))
 
 
 def _set_strides(opt, q=None, k=None, v=None, out=None):
     """Writes the layouts of the call's tensors into the options (creating them when a tensor needs strides)."""
-    given = {"q_strides": q, "kv_strides": k, "out_strides": out}
-    if v is not None and k is not None and v != k:
+    if v is not None and v is not k and tuple(v) != tuple(k):
         raise ValueError("k and v must share one layout")
     if opt is None:
-        if all(s is None or s == (0, 0, 0) for s in given.values()):
+        if (q is None or q is _DENSE) and (k is None or k is _DENSE) and (out is None or out is _DENSE):
             return None
         opt = default_options()
-    for field, strides in given.items():
-        if strides is not None:
-            setattr(opt, field, (ctypes.c_int64 * 3)(*strides))
+    if q is not None:
+        opt.q_strides = q
+    if k is not None:
+        opt.kv_strides = k
+    if out is not None:
+        opt.out_strides = out
     return opt
 
 
@@ -196,25 +209,25 @@ def cosa_kap_select(q, k, budget: float, out_order, out_count, causal=True, stre
                     block_q: int = 128):
     """Stage 1: fills out_order [B,Hq,nQB,order_stride] / out_count [B,Hq,nQB] (int32); block_q = 256 makes one ranking
     per 256-row query block (the lists stay per 128-row tile, see cosa.h)."""
-    lib = _load()
+    lib = _lib or _load()
     shape = make_shape(q, k, causal)
-    shape.block_q = block_q
-    (qp, qstr), (kp, kstr) = _strided_ptr(q, "q"), _strided_ptr(k, "k") if k.dim() == 4 and not _is_pool(opt) else (_dev_ptr(k, torch.bfloat16, "k"), None)
+    if block_q != 128:
+        shape.block_q = block_q
+    qp, qstr = _strided_ptr(q, "q")
+    kp, kstr = _strided_ptr(k, "k") if k.dim() == 4 and not _is_pool(opt) else (_dev_ptr(k, _BF16, "k"), None)
     had_opt = opt is not None
     opt = _set_strides(opt, q=qstr, k=kstr)
     if opt is not None and not had_opt:
         opt.order_stride = out_order.shape[-1]
-    args = (qp, kp, byref(shape), c_float(budget),
-            _dev_ptr(out_order, torch.int32, "out_order"), _dev_ptr(out_count, torch.int32, "out_count"),
-            _stream_ptr(stream))
+    op, cp = _dev_ptr(out_order, _I32, "out_order"), _dev_ptr(out_count, _I32, "out_count")
     if opt is None:
         if out_order.shape[-1] != shape.n // 128:
             raise ValueError("without options the order tensor must have pitch nQB")
-        _check(lib.cosa_kap_select(*args), "cosa_kap_select")
+        _check(lib.cosa_kap_select(qp, kp, byref(shape), budget, op, cp, _stream_ptr(stream)), "cosa_kap_select")
     else:
         if opt.order_stride == 0:
             opt.order_stride = out_order.shape[-1]
-        _check(lib.cosa_kap_select_ex(*args, byref(opt)), "cosa_kap_select_ex")
+        _check(lib.cosa_kap_select_ex(qp, kp, byref(shape), budget, op, cp, _stream_ptr(stream), byref(opt)), "cosa_kap_select_ex")
 
 
 def cosa_kap_select_static_max_bytes() -> int:
@@ -239,30 +252,28 @@ def cosa_kap_select_static(q, k, budget: float, out_order, out_count, causal=Tru
 def cosa_osk_attention(q, k, v, order, count, tightened_budget: float, out, out_lse=None, out_visited=None,
                        causal=True, stream=None, opt: CosaOptions | None = None):
     """Stage 2: fills out [B,Hq,N,d] bf16, out_lse [B,Hq,N] f32, out_visited [B,Hq,nQB] int32."""
-    lib = _load()
+    lib = _lib or _load()
     shape = make_shape(q, k, causal)
     (qp, qstr), (op, ostr) = _strided_ptr(q, "q"), _strided_ptr(out, "out")
     if _is_pool(opt):
-        (kp, kstr), (vp, vstr) = (_dev_ptr(k, torch.bfloat16, "k"), None), (_dev_ptr(v, torch.bfloat16, "v"), None)
+        (kp, kstr), (vp, vstr) = (_dev_ptr(k, _BF16, "k"), None), (_dev_ptr(v, _BF16, "v"), None)
     else:
         (kp, kstr), (vp, vstr) = _strided_ptr(k, "k"), _strided_ptr(v, "v")
     had_opt = opt is not None
     opt = _set_strides(opt, q=qstr, k=kstr, v=vstr, out=ostr)
     if opt is not None and not had_opt and order is not None:
         opt.order_stride = order.shape[-1]
-    args = (qp, kp, vp,
-            byref(shape), _dev_ptr(order, torch.int32, "order"), _dev_ptr(count, torch.int32, "count"),
-            c_float(tightened_budget), op,
-            _dev_ptr(out_lse, torch.float32, "out_lse"), _dev_ptr(out_visited, torch.int32, "out_visited"),
-            _stream_ptr(stream))
+    lists = (_dev_ptr(order, _I32, "order"), _dev_ptr(count, _I32, "count"))
+    outs = (op, _dev_ptr(out_lse, _F32, "out_lse"), _dev_ptr(out_visited, _I32, "out_visited"), _stream_ptr(stream))
     if opt is None:
         if order.shape[-1] != shape.n // 128:
             raise ValueError("without options the order tensor must have pitch nQB")
-        _check(lib.cosa_osk_attention(*args), "cosa_osk_attention")
+        _check(lib.cosa_osk_attention(qp, kp, vp, byref(shape), *lists, tightened_budget, *outs), "cosa_osk_attention")
     else:
         if opt.order_stride == 0 and order is not None:
             opt.order_stride = order.shape[-1]
-        _check(lib.cosa_osk_attention_ex(*args, byref(opt)), "cosa_osk_attention_ex")
+        _check(lib.cosa_osk_attention_ex(qp, kp, vp, byref(shape), *lists, tightened_budget, *outs, byref(opt)),
+               "cosa_osk_attention_ex")
 
 
 def cosa_validate_order(order, count, shape: CosaShape, status_word: torch.Tensor, stream=None):
