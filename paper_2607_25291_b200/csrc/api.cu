@@ -153,7 +153,7 @@ cosa_options resolve_options(const cosa_options* opt) {
 }  // namespace
 
 // scratch the kernels of one call need (beyond inputs and outputs)
-struct KapScratch { size_t scores, jstar, ambmask, hard, redo_list, k2max, k2part, q2max, slot_taken, maxima, kstage, total; int slots; bool gather; };
+struct KapScratch { size_t scores, jstar, ambmask, hard, redo_list, k2part, qk2max, slot_taken, maxima, kstage, total; int slots; bool gather; };
 static KapScratch kap_scratch_layout(const cosa_shape* s, const cosa_options& o) {
   KapScratch L{};
   const int stride = o.stride > 0 ? o.stride : 8;
@@ -173,9 +173,8 @@ static KapScratch kap_scratch_layout(const cosa_shape* s, const cosa_options& o)
   L.ambmask = off; off += align_up(heads * nqb * 4, 256);
   L.hard = off; off += align_up(heads * nqb, 256);
   L.redo_list = off; off += align_up((1 + heads * nqb) * 4, 256);
-  L.k2max = off; off += 256;
   L.k2part = off; off += align_up(kNormParts * 4, 256);
-  L.q2max = off; off += align_up(heads * nqb * 4, 256);
+  L.qk2max = off; off += align_up(heads * nqb * 4, 256);
   // the screen's parked block maxima: one area per CTA that can be resident on the current device
   L.slots = kap_screen_slots();
   if (L.slots <= 0) L.slots = 160;   // no usable device (a size query only): the count of the largest sm_100a part, rounded up
@@ -293,9 +292,8 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
   sp.hard = reinterpret_cast<uint8_t*>(ws + L.hard);
   sp.redo_list = reinterpret_cast<int32_t*>(ws + L.redo_list);
   sp.slot_taken = reinterpret_cast<int32_t*>(ws + L.slot_taken);
-  sp.k2max = reinterpret_cast<float*>(ws + L.k2max);
   sp.k2part = reinterpret_cast<float*>(ws + L.k2part);
-  sp.q2max = reinterpret_cast<float*>(ws + L.q2max);
+  sp.qk2max = reinterpret_cast<float*>(ws + L.qk2max);
   sp.maxima = reinterpret_cast<float*>(ws + L.maxima);
   sp.slots = L.slots;
   sp.batch = p.batch; sp.hq = p.hq; sp.hkv = p.hkv; sp.n = p.n; sp.nqb = nqb;
@@ -314,7 +312,7 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
   }
   sp.pg = p.pg;
   sp.qs = p.qs; sp.ks = p.ks;
-  cudaError_t e = launch_kap_norms(&sp, st);
+  cudaError_t e = kap_screen_is_short(p.n, s) ? cudaSuccess : launch_kap_norms(&sp, st);
   if (e != cudaSuccess) return cuda_fail(e, "kap norms launch");
   e = launch_kap_screen(sp, st);
   if (e != cudaSuccess) return cuda_fail(e, "kap screen launch");

@@ -109,8 +109,8 @@ struct KapScreenParams {
   int32_t* slot_taken;   // [slots]  0 = free; zeroed by kap_norms_kernel
   float* k2part;         // [kNormParts]  largest squared norms of sampled key rows of the call, one per CTA of kap_norms_kernel
   int k2parts;           // ... how many
-  float* k2max;          // [1]  their maximum, left by the screen for the sort stage
-  float* q2max;          // [B,Hq,nQB]  largest squared norm of the sampled query rows of every (head, query block)
+  float* qk2max;         // [B,Hq,nQB]  largest squared norm of the sampled query rows of every (head, query block), times the largest of
+                         // the sampled key rows (of the call, or in a short call of the keys the block's CTA multiplied)
   int slots;             // CTAs that can be resident at once
   int batch, hq, hkv, n, nqb;
   int causal;
@@ -119,6 +119,7 @@ struct KapScreenParams {
   float tau_row;         // two block maxima of a row closer than this (scaled logits) are "too close to call"
   Strides qs, ks;        // strides of q and of k (dense k; pools are contiguous)
   TileOrder qo, ko;      // coordinate order of the tensor maps over the sampled rows of q and of k (set by the launcher)
+  int q_box_heads;       // query heads one box of the map over q takes (set by the launcher)
   long long wait_budget; // clock cycles a device-side wait may take before the kernel gives up
   KvPaging pg;
 };
@@ -199,13 +200,13 @@ inline long long budget_to_fx(float budget) {
 }
 
 // What the float32 screen may be off by: bound used for the error of a difference of two scaled logits of one sampled
-// row -- and so, relatively, of a block score, a sum of exponentials of such differences -- given the largest squared
-// norms of the sampled rows involved.  Products of two bf16 numbers are exact in float32; what is lost is lost in adding
+// row -- and so, relatively, of a block score, a sum of exponentials of such differences -- given the product of the largest
+// squared norms of the sampled query and key rows involved.  Products of two bf16 numbers are exact in float32; what is lost is lost in adding
 // 128 of them, in proportion to their size, which |q| |k| bounds.  The factor (8 x 2^-24) is calibrated: the largest
 // error seen on the measured workloads, all lists of all heads, is 3.4 times smaller (asserted by the tests at the
 // sizes the benchmark runs).
-__host__ __device__ inline float screen_error_bound(float q2max, float k2max, float scale) {
-  return 4.76837158203125e-7f * sqrtf(q2max * k2max) * scale;
+__host__ __device__ inline float screen_error_bound(float qk2max, float scale) {
+  return 4.76837158203125e-7f * sqrtf(qk2max) * scale;
 }
 
 // device status word (one per device), set by kernels whose bounded waits give up
@@ -242,6 +243,8 @@ cudaError_t raise_smem_limit(const void* kernel, SmemLimit* state, size_t bytes)
 
 // redo_list == nullptr: every (head, query block); else only the listed ones (count in [0])
 cudaError_t launch_kap_exact(const KapParams& p, const int32_t* redo_list, cudaStream_t st);
+// the whole call's key tiles fit the screen's stages: it needs no scratch areas and no norms kernel
+bool kap_screen_is_short(int n, int stride);
 bool kap_screen_supported(int rows, int group, int stride, const KvPaging& pg);
 cudaError_t launch_kap_screen(const KapScreenParams& p, cudaStream_t st);
 constexpr int kNormParts = 296;   // CTAs of kap_norms_kernel at most

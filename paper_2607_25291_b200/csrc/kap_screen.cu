@@ -17,6 +17,11 @@
 // many such areas as CTAs can be resident, so they mostly stay in L2.  After the last tile, with
 // M* known, the block scores and HRM flags are formed from the parked maxima, one thread per
 // (row group, key block).
+// Short calls (kShort: all key tiles of the call fit the key stages, n <= 4096 at stride 8) park nothing: a thread keeps its
+// block maxima in registers and, when every product is done, lays them into the key stages, from where the scores are
+// formed; the norms of the sampled keys are taken from the stages as well, which saves the norms kernel's launch.  At 4K
+// tokens the time of this kernel is a chain of latencies: the whole of Stage 1 takes 25.9 us instead of 29.4 at 31 blocks of
+// 32 heads, 19.5 instead of 23 at 1K tokens.
 // Float32 results are a SCREEN: the sort stage recomputes in double precision whatever a
 // rounding error could reorder.  For that it is told, per sampled row, the two blocks with the
 // largest block maxima and whether they are closer than tau_row (the row's HRM flag and M* are
@@ -60,6 +65,7 @@ struct __align__(8) ScreenCtl {
   float xt[kParts][3][kRows];           // exchange between the column parts: top-3 block maxima
   int xj[kParts][2][kRows];             // ... and the blocks holding the two largest
   float mstar[kRows];                   // M*[r] of every row
+  float k2w[kEpiThreads / 32];          // (kShort) largest squared key norm each epilogue warp saw
 };
 constexpr size_t kScreenSmem = 1024 + (size_t)kTileBytes * (kRowTiles + kStages) + sizeof(ScreenCtl);
 static_assert(kScreenSmem <= 232448, "shared memory budget of one CTA");
@@ -69,7 +75,6 @@ __device__ __forceinline__ void screen_timeout(ScreenCtl* c, int32_t* status) {
   atomicMin(status, (int32_t)COSA_ERR_DEVICE_TIMEOUT);
 }
 
-// kStrict: every multi-lane wait answers per warp (see mbar_wait_warp)
 // (a whole warp) the largest squared norm of a sampled key row of the call
 __device__ __forceinline__ float largest_key_norm(const KapScreenParams& p, int lane) {
   float k2 = 0.f;
@@ -79,7 +84,8 @@ __device__ __forceinline__ float largest_key_norm(const KapScreenParams& p, int 
   return k2;
 }
 
-template <int R, bool kStrict>
+// kStrict: every multi-lane wait answers per warp (see mbar_wait_warp).  kShort: see above
+template <int R, bool kStrict, bool kShort>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                   KapScreenParams p, int32_t* status) {
@@ -87,6 +93,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - raw);
+  if (threadIdx.x == 0) { prefetch_tensormap(&q_map); prefetch_tensormap(&k_map); }
   chain_begin();
   const uint32_t a_sm = base;
   const uint32_t k_sm = base + kRowTiles * kTileBytes;
@@ -110,19 +117,15 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const int n_tiles = (n_keys + 127) / 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  if (blockIdx.x == 0 && warp == 0) {
-    const float k2 = largest_key_norm(p, lane);
-    if (lane == 0) {
-      *p.k2max = k2;          // for the sort stage (a later launch) ...
-      p.redo_list[0] = 0;     // ... which appends to this list
-    }
-  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) p.redo_list[0] = 0;   // the sort stage (a later launch) appends to it
   if (i0 >= nqb_b) return;                        // all of this CTA's query blocks are padding
   if (threadIdx.x == 0) {
     // once some CTA has reported a timeout the rest of the grid returns at once
     int poisoned = *reinterpret_cast<volatile int32_t*>(status);
     int slot = -1;
-    if (poisoned == 0 && (int)gridDim.x <= p.slots) {
+    if (kShort) {
+      slot = 0;                             // (none needed)
+    } else if (poisoned == 0 && (int)gridDim.x <= p.slots) {
       slot = (int)blockIdx.x;               // an area for every CTA: nothing to search for
     } else if (poisoned == 0) {
       // a scratch area no resident CTA holds: there are as many as CTAs can be resident, so one is free; the
@@ -152,7 +155,6 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     ctl->t_issued = 0; ctl->t_done = 0; ctl->c_fetched = 0; ctl->c_done = 0;
     mbar_fence_init();
     fence_proxy_async_smem();
-    prefetch_tensormap(&q_map); prefetch_tensormap(&k_map);
   }
   if (warp == 0) { tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols); tmem_relinquish(); }
   tc_fence_before();
@@ -165,15 +167,19 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
 
   if (warp == 0) {
     int t_issued = 0;   // (lane 0) key tiles requested so far
+    // A tiles: strided boxes of R sampled rows of q_box_heads query heads of the group (all of them, if the layout has rows
+    // inside heads) per query block, a box pair per lane (one lane issuing 32 boxes in turn: 2 us)
+    if (lane == 0) mbar_expect_tx(smem_u32(&ctl->a_full), kRowTiles * kTileBytes);
+    __syncwarp();
+    static_assert(kGroups <= 32, "a lane per box pair");
+    const int a_grp = lane * p.q_box_heads;
+    if (a_grp < kGroups) {
+      const int i = i0 + a_grp / G, h = g * G + a_grp % G;
+      const uint32_t dst = a_sm + (a_grp * R / 128) * kTileBytes + (a_grp * R % 128) * 128;   // (rows past the head's last are zero-filled)
+      tma_load_tile(dst, &q_map, 0, i * R, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->a_full));
+      tma_load_tile(dst + kHalfBytes, &q_map, 64, i * R, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->a_full));
+    }
     if (lane == 0) {
-      // A tiles: one strided box of R sampled rows per (query block, query head of the group)
-      mbar_expect_tx(smem_u32(&ctl->a_full), kRowTiles * kTileBytes);
-      for (int grp = 0; grp < kGroups; ++grp) {
-        const int i = i0 + grp / G, h = g * G + grp % G;
-        const uint32_t dst = a_sm + (grp * R / 128) * kTileBytes + (grp * R % 128) * 128;   // (rows past the head's last are zero-filled)
-        tma_load_tile(dst, &q_map, 0, i * R, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->a_full));
-        tma_load_tile(dst + kHalfBytes, &q_map, 64, i * R, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->a_full));
-      }
       if (!p.pg.table) {
         for (int t = 0; t < n_tiles; ++t) {
           const int st = t % kStages;
@@ -265,8 +271,8 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     // squared norm of this thread's sampled query row, from the A tile in shared memory (a row is 2 x 128 bytes, one in
     // each half tile; the swizzle permutes 16-byte chunks inside a row, which a sum of squares does not notice; the
     // chunk order is rotated by the lane so that the rows of a warp hit different banks)
-    float q2 = 0.f;
-    const float k2 = largest_key_norm(p, lane);
+    float q2 = 0.f, g2 = 0.f;
+    float k2 = kShort ? 0.f : largest_key_norm(p, lane);
     bool alive = mbar_wait_warp(smem_u32(&ctl->a_full), 0, abort_flag, budget, strict);
     if (!alive && !*abort_flag) screen_timeout(ctl, status);
     if (alive) {
@@ -281,15 +287,17 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
           q2 = fmaf(lo, lo, fmaf(hi, hi, q2));
         }
       }
-      float g2 = q2;                                     // the group's rows are R consecutive lanes
+      g2 = q2;                                           // the group's rows are R consecutive lanes
 #pragma unroll
       for (int o = 1; o < R; o <<= 1) g2 = fmaxf(g2, __shfl_xor_sync(0xffffffffu, g2, o));
-      if (part == 0 && r == 0 && row_ok) p.q2max[(size_t)(b * p.hq + h) * p.nqb + i] = g2;
     }
-    for (int t = 0; t < n_tiles && alive; ++t) {
+    // one key tile: this row's block maxima, and the three largest so far
+    auto take_tile = [&](int t, float (&mb)[BPC]) {
       const int sb = t % kSteps, st = t % kStages;
-      alive = mbar_wait_warp(smem_u32(&ctl->k_empty[st]), (t / kStages) & 1, abort_flag, budget, strict);   // this tile's MMAs finished
-      if (!alive) { if (!*abort_flag) screen_timeout(ctl, status); break; }
+      if (!mbar_wait_warp(smem_u32(&ctl->k_empty[st]), (t / kStages) & 1, abort_flag, budget, strict)) {   // this tile's MMAs finished
+        if (!*abort_flag) screen_timeout(ctl, status);
+        return false;
+      }
       tc_fence_after();
       uint32_t v[kPartCols / 32][32];
 #pragma unroll
@@ -298,7 +306,6 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       tmem_wait_ld();
       tc_fence_before();
       mbar_arrive(smem_u32(&ctl->s_empty[sb]));
-      float mb[BPC];
 #pragma unroll
       for (int bb = 0; bb < BPC; ++bb) {
         const int c0 = bb * R;                              // first column of the block within the part
@@ -317,9 +324,11 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         }
         mb[bb] = fmaxf(m0, m1);
       }
-      float* dst = mine + (size_t)t * kTileFloats;
+      if (!kShort) {
+        float* dst = mine + (size_t)t * kTileFloats;
 #pragma unroll
-      for (int bb = 0; bb < BPC; ++bb) st_l2_hint(dst + bb * R, mb[bb], keep);
+        for (int bb = 0; bb < BPC; ++bb) st_l2_hint(dst + bb * R, mb[bb], keep);
+      }
 #pragma unroll
       for (int bb = 0; bb < BPC; ++bb) {
         const float m = mb[bb];
@@ -328,6 +337,40 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         else if (m > top2) { top3 = top2; top2 = m; jstar2 = jb; }
         else if (m > top3) top3 = m;
       }
+      return true;
+    };
+    float mb_all[kShort ? kStages : 1][BPC];
+    if (kShort) {
+      // (a stage is never filled twice: its key tile stays until the maxima take its place)
+#pragma unroll
+      for (int t = 0; t < kStages; ++t) {
+        if (t < n_tiles && alive) {
+          alive = take_tile(t, mb_all[t]) && mbar_wait_warp(smem_u32(&ctl->k_full[t]), 0, abort_flag, budget, strict);
+          // squared norms of the tile's sampled keys: four threads a row, the chunks of odd rows in another order (other banks)
+          const int et = threadIdx.x - 64, krow = et >> 2;
+          const unsigned char* src = smem + (size_t)kTileBytes * (kRowTiles + t) + krow * 128;
+          float s2 = 0.f;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int c = ((et & 3) + 4 * u) ^ ((krow & 1) << 2);
+            const uint4 wv = *reinterpret_cast<const uint4*>(src + (c >> 3) * kHalfBytes + (c & 7) * 16);
+            const unsigned ws4[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float lo = __uint_as_float(ws4[e] << 16), hi = __uint_as_float(ws4[e] & 0xffff0000u);
+              s2 = fmaf(lo, lo, fmaf(hi, hi, s2));
+            }
+          }
+          s2 += __shfl_xor_sync(0xffffffffu, s2, 1);
+          s2 += __shfl_xor_sync(0xffffffffu, s2, 2);
+          if (s2 == s2 && t * 128 + krow < ns_b) k2 = fmaxf(k2, s2);   // (a NaN row is left to the later stages; padding is no key)
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) k2 = fmaxf(k2, __shfl_xor_sync(0xffffffffu, k2, o));
+      if (lane == 0) ctl->k2w[ew] = k2;
+    } else {
+      for (int t = 0; t < n_tiles && alive; ++t) alive = take_tile(t, mb_all[0]);
     }
     if (alive) {
       // all tiles seen: merge the column parts' top-3 block maxima of every row
@@ -353,7 +396,12 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       // the row's best block, and whether the runner-up is too close to call
       // (the threshold grows with the magnitude of the row and of the call's keys, which is what the rounding error of a
       // logit follows)
-      const float tau_row = fmaxf(p.tau_row, 2.f * screen_error_bound(q2, k2, p.scale));
+      if (kShort) {
+#pragma unroll
+        for (int e = 0; e < kEpiThreads / 32; ++e) k2 = fmaxf(k2, ctl->k2w[e]);
+      }
+      if (part == 0 && r == 0 && row_ok) p.qk2max[(size_t)(b * p.hq + h) * p.nqb + i] = g2 * k2;
+      const float tau_row = fmaxf(p.tau_row, 2.f * screen_error_bound(q2 * k2, p.scale));
       const bool amb = row_ok && (top1 - top2) * p.scale <= tau_row;
       const bool amb3 = row_ok && (top1 - top3) * p.scale <= tau_row;
       const unsigned any_amb = __ballot_sync(0xffffffffu, amb), any_amb3 = __ballot_sync(0xffffffffu, amb3);
@@ -367,6 +415,16 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
           if (r == 0) {
             p.ambmask[(size_t)(b * p.hq + h) * p.nqb + i] = (any_amb & grp_mask) >> shift;
             p.hard[(size_t)(b * p.hq + h) * p.nqb + i] = (any_amb3 & grp_mask) ? 1 : 0;
+          }
+        }
+      }
+      if (kShort) {                 // every product is done and every key read: the stages take the maxima
+#pragma unroll
+        for (int t = 0; t < kStages; ++t) {
+          if (t < n_tiles) {
+            float* dst = reinterpret_cast<float*>(smem + (size_t)kTileBytes * (kRowTiles + t)) + ((size_t)grp * BPT + part * BPC) * R + r;
+#pragma unroll
+            for (int bb = 0; bb < BPC; ++bb) dst[bb * R] = mb_all[t][bb];
           }
         }
       }
@@ -396,7 +454,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         bulk_load_hint(k_sm + (c % kStages) * kTileBytes, parked + (size_t)c * kTilesPerChunk * kTileFloats,
                        tiles_here * kTileBytesM, bar, drop);
       };
-      if (et == 0) {
+      if (!kShort && et == 0) {
         fence_proxy_async_all();   // the maxima were written with ordinary stores
         for (int c = 0; c < min(n_chunks, kStages - 1); ++c) fetch(c);
       }
@@ -418,8 +476,34 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         for (int q = 0; q < 4; ++q) ms[v4 * 4 + q] = ctl->mstar[og * R + src + q];
       }
       float* srow = p.scores + ((size_t)(b * p.hq + oh) * p.nqb + min(oi, p.nqb - 1)) * p.nqb;
+      // the score of tile tl's outputs that are this thread's, from the maxima at `maxima`
+      auto score = [&](int tile, const float* maxima) {
+        const int j = tile * BPT + blk;
+        if (oi < nqb_b && j < J) {
+          const float4* src = reinterpret_cast<const float4*>(maxima + ((size_t)og * BPT + blk) * R);
+          float e0 = 0.f, e1 = 0.f;
+          bool fl = false;
+#pragma unroll
+          for (int v4 = 0; v4 < kVecs; ++v4) {
+            const float4 x = src[(v4 + rot) % kVecs];
+            e0 += ex2_approx((x.x - ms[v4 * 4]) * scale2);       // exp(M[r,j] - M*[r]); 0 for invisible blocks
+            e1 += ex2_approx((x.y - ms[v4 * 4 + 1]) * scale2);
+            e0 += ex2_approx((x.z - ms[v4 * 4 + 2]) * scale2);
+            e1 += ex2_approx((x.w - ms[v4 * 4 + 3]) * scale2);
+            fl = fl || x.x == ms[v4 * 4] || x.y == ms[v4 * 4 + 1] || x.z == ms[v4 * 4 + 2] || x.w == ms[v4 * 4 + 3];
+          }
+          const float e = e0 + e1;
+          srow[j] = fl ? -e : e;                                 // sign bit carries the HRM flag
+        }
+      };
+      if (kShort) {
+        for (int o = et; o < n_tiles * kOutsPerTile; o += kEpiThreads) {
+          const int tl = o / kOutsPerTile;
+          score(tl, reinterpret_cast<const float*>(smem + (size_t)kTileBytes * (kRowTiles + tl)));
+        }
+      }
       int c_done = 0;
-      for (int c = 0; c < n_chunks && alive; ++c) {
+      for (int c = 0; !kShort && c < n_chunks && alive; ++c) {
         const int st = c % kStages;
         if (et == 0 && c + kStages - 1 < n_chunks) {
           // the stage of chunk c - 1 takes chunk c + kStages - 1 once every thread has read it
@@ -435,23 +519,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         const float* stage = reinterpret_cast<const float*>(smem + (size_t)kTileBytes * (kRowTiles + st));
         for (int o = et; o < tiles_here * kOutsPerTile; o += kEpiThreads) {
           const int tl = o / kOutsPerTile;
-          const int j = (c * kTilesPerChunk + tl) * BPT + blk;
-          if (oi < nqb_b && j < J) {
-            const float4* src = reinterpret_cast<const float4*>(stage + (size_t)tl * kTileFloats + ((size_t)og * BPT + blk) * R);
-            float e0 = 0.f, e1 = 0.f;
-            bool fl = false;
-#pragma unroll
-            for (int v4 = 0; v4 < kVecs; ++v4) {
-              const float4 x = src[(v4 + rot) % kVecs];
-              e0 += ex2_approx((x.x - ms[v4 * 4]) * scale2);       // exp(M[r,j] - M*[r]); 0 for invisible blocks
-              e1 += ex2_approx((x.y - ms[v4 * 4 + 1]) * scale2);
-              e0 += ex2_approx((x.z - ms[v4 * 4 + 2]) * scale2);
-              e1 += ex2_approx((x.w - ms[v4 * 4 + 3]) * scale2);
-              fl = fl || x.x == ms[v4 * 4] || x.y == ms[v4 * 4 + 1] || x.z == ms[v4 * 4 + 2] || x.w == ms[v4 * 4 + 3];
-            }
-            const float e = e0 + e1;
-            srow[j] = fl ? -e : e;                                 // sign bit carries the HRM flag
-          }
+          score(c * kTilesPerChunk + tl, stage + (size_t)tl * kTileFloats);
         }
         mbar_arrive(smem_u32(&ctl->m_empty[st]));
         c_done = c + 1;
@@ -473,6 +541,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   }
   __syncwarp();
   if (warp == 0) tmem_dealloc(tmem, kTmemCols);
+  if (kShort) return;
   {
     // the parked maxima are dead: let L2 drop the lines instead of writing them back
     char* area = reinterpret_cast<char*>(p.maxima + (size_t)ctl->slot * ((size_t)((ns + 127) / 128) * (kRows * BPT)));
@@ -505,6 +574,8 @@ int kap_screen_slots() {
   return device_sm_count() * kCtasPerSm;
 }
 
+bool kap_screen_is_short(int n, int stride) { return n / stride <= 128 * kStages; }
+
 size_t kap_screen_slot_bytes(int n, int stride) {
   const size_t ns = (size_t)n / stride, R = 128 / stride;
   return ((ns + 127) / 128) * kRows * (128 / R) * sizeof(float);
@@ -513,13 +584,21 @@ size_t kap_screen_slot_bytes(int n, int stride) {
 cudaError_t launch_kap_screen(const KapScreenParams& p_in, cudaStream_t st) {
   KapScreenParams p = p_in;
   const int R = 128 / p.stride;
-  if (!p.maxima || !p.slot_taken || p.slots <= 0) return cudaErrorInvalidValue;
+  const bool is_short = kap_screen_is_short(p.n, p.stride);
+  if (!is_short && (!p.maxima || !p.slot_taken || p.slots <= 0)) return cudaErrorInvalidValue;
   const uint64_t ns = (uint64_t)p.n / p.stride;
   CUtensorMap qm, km;
   // every `stride`-th row of q and k: the row stride of the maps is `stride` rows of the tensor (of the page pool)
   const int k_box = p.pg.table ? ((p.pg.page_size / p.stride) < 128 ? p.pg.page_size / p.stride : 128) : 128;
   const Strides qs = {p.qs.b, p.qs.h, p.qs.t * p.stride};
-  bool ok = make_tile_map(&qm, &p.qo, p.q, ns, (uint64_t)p.hq, (uint64_t)p.batch, qs, R);
+  // the heads of a group in one box, if rows lie inside heads (so that the box lays them out head by head) and 128 rows hold it
+  const int group = p.hq / p.hkv;
+  p.q_box_heads = group * R <= 128 ? group : 128 / R;
+  bool ok = make_tile_map(&qm, &p.qo, p.q, ns, (uint64_t)p.hq, (uint64_t)p.batch, qs, R, p.q_box_heads);
+  if (ok && p.qo.row > p.qo.head) {
+    p.q_box_heads = 1;
+    ok = make_tile_map(&qm, &p.qo, p.q, ns, (uint64_t)p.hq, (uint64_t)p.batch, qs, R);
+  }
   if (p.pg.table) {
     const Strides pool = dense_strides(p.hkv, p.pg.page_size);
     ok = ok && make_tile_map(&km, &p.ko, p.k, (uint64_t)(p.pg.page_size / p.stride), (uint64_t)p.hkv, (uint64_t)p.pg.num_pages,
@@ -534,9 +613,11 @@ cudaError_t launch_kap_screen(const KapScreenParams& p_in, cudaStream_t st) {
   cudaError_t e;
 #define COSA_LAUNCH_SCREEN(RR)                                                                                              \
   {                                                                                                                         \
-    auto kernel = wait_budget_is_short(p.wait_budget) ? kap_screen_kernel<RR, true> : kap_screen_kernel<RR, false>;         \
-    static SmemLimit limits[2];                                                                                             \
-    e = raise_smem_limit(reinterpret_cast<const void*>(kernel), &limits[wait_budget_is_short(p.wait_budget)], kScreenSmem); \
+    const bool strict = wait_budget_is_short(p.wait_budget);                                                                \
+    auto kernel = is_short ? (strict ? kap_screen_kernel<RR, true, true> : kap_screen_kernel<RR, false, true>)              \
+                           : (strict ? kap_screen_kernel<RR, true, false> : kap_screen_kernel<RR, false, false>);           \
+    static SmemLimit limits[4];                                                                                             \
+    e = raise_smem_limit(reinterpret_cast<const void*>(kernel), &limits[(is_short ? 2 : 0) + (strict ? 1 : 0)], kScreenSmem); \
     if (e != cudaSuccess) return e;                                                                                         \
     return launch_chained(kernel, dim3(grid), kThreads, kScreenSmem, st, qm, km, p, status);                                \
   }

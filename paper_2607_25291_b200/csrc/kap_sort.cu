@@ -415,13 +415,12 @@ __global__ void __launch_bounds__(kThreads, 6) kap_sort_kernel(KapParams p, KapS
   }
   // a screen kernel that gave up has left the scratch half written: nothing of it may be used for addressing
   const int poisoned = *reinterpret_cast<const volatile int32_t*>(status);   // (tested together with `hard` below)
-  const float k2 = *sp.k2max;
   unsigned hard = 0u;                         // (tested only after the scores have been requested: one round trip, not two)
-  float q2 = 0.f;                             // largest squared norm among the block's sampled query rows
+  float qk2 = 0.f;                            // largest product of squared norms of the block's sampled query rows and of its keys
   unsigned long long amb = 0ULL;              // bit r: sampled row r of the block was too close to call
   for (int t = 0; t < T; ++t) {
     hard |= sp.hard[row_lo + t];
-    q2 = fmaxf(q2, sp.q2max[row_lo + t]);
+    qk2 = fmaxf(qk2, sp.qk2max[row_lo + t]);
     amb |= (unsigned long long)sp.ambmask[row_lo + t] << (t * R);
   }
   const __nv_bfloat16* qh = p.q + elem_off(p.qs, b, h, 0);
@@ -469,7 +468,7 @@ __global__ void __launch_bounds__(kThreads, 6) kap_sort_kernel(KapParams p, KapS
   }
   if (poisoned != 0) return;
   // near ties: never closer than twice what the screen may be off by on rows of this magnitude
-  tau_score = fmaxf(tau_score, 2.f * screen_error_bound(q2, k2, sp.scale));
+  tau_score = fmaxf(tau_score, 2.f * screen_error_bound(qk2, sp.scale));
   if (hard) {  // left to the double-precision kernel
     if (tid == 0) sp.redo_list[1 + atomicAdd(sp.redo_list, 1)] = (int)row_lo;
     return;

@@ -31,9 +31,9 @@ inline EncodeTiledFn encode_tiled_fn() {
 
 // `s` in elements; `rows`, `heads`, `outer` the extents.  The map lists the three dimensions by ascending stride (a
 // token-major tensor has its head stride below its row stride) and *order says where each went; boxes are box_rows
-// rows of one head of one outer index.  False if the strides cannot be mapped (not multiples of 16 bytes, or equal).
+// rows of box_heads heads of one outer index.  False if the strides cannot be mapped (not multiples of 16 bytes, or equal).
 inline bool make_tile_map(CUtensorMap* map, TileOrder* order, const void* basep, uint64_t rows, uint64_t heads, uint64_t outer,
-                          const Strides& s, int box_rows = kBlock) {
+                          const Strides& s, int box_rows = kBlock, int box_heads = 1) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return false;
   struct Dim { long long stride; uint64_t extent; int what; } d[3] = {{s.t, rows, 0}, {s.h, heads, 1}, {s.b, outer, 2}};
@@ -58,6 +58,7 @@ inline bool make_tile_map(CUtensorMap* map, TileOrder* order, const void* basep,
     strides[a] = (cuuint64_t)d[a].stride * 2;
     slot[d[a].what] = a;
     if (d[a].what == 0) box[a + 1] = (cuuint32_t)box_rows;
+    if (d[a].what == 1) box[a + 1] = (cuuint32_t)box_heads;
   }
   order->row = slot[0]; order->head = slot[1]; order->outer = slot[2];
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(basep), dims, strides, box, estr,

@@ -352,6 +352,19 @@ def test_kap_inputs_of_large_magnitude(factor, outlier_factor):
         assert np.array_equal(_np(order), ref_order), impl
 
 
+@pytest.mark.parametrize("n,stride", [(4096, 8), (4224, 8), (2048, 4), (2176, 4), (8192, 16), (8320, 16), (3968, 8), (128, 8)])
+def test_kap_lists_around_the_longest_short_call(n, stride):
+    """Calls whose key tiles all fit the screen's stages (512 sampled keys) take another route through the screen: lists on
+    both sides of that length, against the oracle."""
+    w = tiny(seed=n + stride, hq=2, hkv=1, n=n, needles=3)
+    qb, kb, vb, _ = w.make()
+    q, k = to_dev(qb), to_dev(kb)
+    qf, kf, _ = widen(qb, kb, vb)
+    order, count = run_kap(q, k, 0.3, stride)
+    ref_order, ref_count = O.kap_select(qf, kf, s=stride, budget=0.3, order_stride=order.shape[-1])
+    assert np.array_equal(_np(count), ref_count) and np.array_equal(_np(order), ref_order)
+
+
 @pytest.mark.parametrize("stride", [4, 8, 16])
 @pytest.mark.parametrize("hq,hkv", [(8, 1), (16, 2), (2, 2)])
 def test_kap_query_group_sizes(hq, hkv, stride):
