@@ -89,10 +89,10 @@ typedef struct {
                               different streams must each bring a workspace of their own          */
   size_t  workspace_bytes;
   int32_t impl;            /* 0 = fastest available; 1 = plain CUDA-core check kernels; 2 and 3 = as 0,
-                              but the sort stage of cosa_kap_select takes the route it otherwise
-                              keeps for the lists its fastest route cannot settle: 2 = the head of
-                              the order selected by radix, 3 = the whole order sorted (same lists,
-                              slower; for tests and comparisons); 4 = as 0, but cosa_osk_attention
+                              but the sort stage of cosa_kap_select works the way it otherwise does only for
+                              the lists that need it: 2 = every key compared with every other, 3 = the whole
+                              order sorted, not its head alone (same lists, slower; for tests and
+                              comparisons); 4 = as 0, but cosa_osk_attention
                               runs the kernel that walks two work items per CTA, each with a softmax
                               group, an S and an O accumulator of its own (the arrangement a 256-row
                               query block with one vote per 128-row tile takes; measured slower than

@@ -352,6 +352,34 @@ def test_kap_inputs_of_large_magnitude(factor, outlier_factor):
         assert np.array_equal(_np(order), ref_order), impl
 
 
+@pytest.mark.parametrize("budget,top_p", [(0.05, 0.0), (0.6, 0.0), (1.0, 0.9)])
+@pytest.mark.parametrize("blocks,stride", [(128, 8), (129, 8), (257, 16), (1100, 16)])
+def test_kap_order_where_the_sort_changes_its_way(blocks, stride, budget, top_p):
+    """128 candidates are compared all with all, more are dealt into buckets (a thread keeps the places of up to 1024, the
+    rest is dealt again); the head alone, the whole order, and all keys in one bucket: the same lists as the oracle's."""
+    n = blocks * 128
+    w = tiny(seed=blocks, hq=1, hkv=1, n=n, needles=8)
+    qb, kb, vb, _ = w.make()
+    q, k = to_dev(qb), to_dev(kb)
+    qf, kf, _ = widen(qb, kb, vb)
+    some = sorted({0, 1, 63, 64, 126, 127, blocks - 3, blocks - 2, blocks - 1} | ({1023, 1024, 1030} if blocks > 1030 else set()))
+    if top_p:                          # counts are decided on float32 scores there: the kept ids are a prefix of the order
+        ref_order, ref_count = O.kap_select(qf, kf, s=stride, budget=1.0, order_stride=blocks, query_blocks=some)
+    else:
+        ref_order, ref_count = O.kap_select(qf, kf, s=stride, budget=budget, order_stride=blocks, query_blocks=some)
+    first = None
+    for impl in (0, 2, 3):
+        order, count = run_kap(q, k, budget, stride, order_stride=blocks, impl=impl, top_p=top_p)
+        if first is None:
+            first = (order, count)
+        assert torch.equal(order, first[0]) and torch.equal(count, first[1]), impl
+    o, c = _np(first[0])[0], _np(first[1])[0]
+    for i in some:
+        kept = int(c[i])
+        assert kept >= 1 and (top_p or kept == ref_count[0, i])
+        assert np.array_equal(o[i, :kept], ref_order[0, i, :kept]) and (o[i, kept:] == -1).all()
+
+
 @pytest.mark.parametrize("n,stride", [(4096, 8), (4224, 8), (2048, 4), (2176, 4), (8192, 16), (8320, 16), (3968, 8), (128, 8)])
 def test_kap_lists_around_the_longest_short_call(n, stride):
     """Calls whose key tiles all fit the screen's stages (512 sampled keys) take another route through the screen: lists on
