@@ -153,7 +153,7 @@ cosa_options resolve_options(const cosa_options* opt) {
 }  // namespace
 
 // scratch the kernels of one call need (beyond inputs and outputs)
-struct KapScratch { size_t scores, jstar, ambmask, hard, redo_list, k2part, qk2max, slot_taken, maxima, kstage, total; int slots; bool gather; };
+struct KapScratch { size_t scores, jstar, ambmask, hard, redo_list, tied_list, k2part, qk2max, slot_taken, maxima, kstage, total; int slots; bool gather; };
 static KapScratch kap_scratch_layout(const cosa_shape* s, const cosa_options& o) {
   KapScratch L{};
   const int stride = o.stride > 0 ? o.stride : 8;
@@ -173,6 +173,7 @@ static KapScratch kap_scratch_layout(const cosa_shape* s, const cosa_options& o)
   L.ambmask = off; off += align_up(heads * nqb * 4, 256);
   L.hard = off; off += align_up(heads * nqb, 256);
   L.redo_list = off; off += align_up((1 + heads * nqb) * 4, 256);
+  L.tied_list = off; off += align_up((1 + heads * nqb) * 4, 256);
   L.k2part = off; off += align_up(kNormParts * 4, 256);
   L.qk2max = off; off += align_up(heads * nqb * 4, 256);
   // the screen's parked block maxima: one area per CTA that can be resident on the current device
@@ -269,7 +270,7 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const KapScratch L = kap_scratch_layout(shape, o);
   if (L.total == 0) {   // double precision throughout
-    cudaError_t e = launch_kap_exact(p, nullptr, st);
+    cudaError_t e = launch_kap_exact(p, st);
     if (e != cudaSuccess) return cuda_fail(e, "kap launch");
     return COSA_OK;
   }
@@ -291,6 +292,7 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
   sp.ambmask = reinterpret_cast<uint32_t*>(ws + L.ambmask);
   sp.hard = reinterpret_cast<uint8_t*>(ws + L.hard);
   sp.redo_list = reinterpret_cast<int32_t*>(ws + L.redo_list);
+  sp.tied_list = reinterpret_cast<int32_t*>(ws + L.tied_list);
   sp.slot_taken = reinterpret_cast<int32_t*>(ws + L.slot_taken);
   sp.k2part = reinterpret_cast<float*>(ws + L.k2part);
   sp.qk2max = reinterpret_cast<float*>(ws + L.qk2max);
@@ -320,7 +322,7 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
   // largest error on the measured workloads; larger for inputs of larger magnitude (see screen_error_bound)
   e = launch_kap_sort(p, sp, 3.0517578125e-5f, st);
   if (e != cudaSuccess) return cuda_fail(e, "kap sort launch");
-  e = launch_kap_exact(p, sp.redo_list, st);
+  e = launch_kap_fixup(p, sp, st);
   if (e != cudaSuccess) return cuda_fail(e, "kap recount launch");
   return COSA_OK;
 }

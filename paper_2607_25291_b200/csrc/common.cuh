@@ -105,6 +105,8 @@ struct KapScreenParams {
   uint32_t* ambmask;     // [B,Hq,nQB]      bit r: sampled row r's two best blocks are too close to call in float32
   uint8_t* hard;         // [B,Hq,nQB]      1 = three blocks too close on some row: whole query block goes to double precision
   int32_t* redo_list;    // [1 + B*Hq*nQB]  [0] = number of entries, then flat (b*Hq+h)*nQB+i of query blocks to redo
+  int32_t* tied_list;    // [1 + B*Hq*nQB]  the same for lists with near ties; their rows of `scores` then hold the chained entries (see
+                         // kap_recount.cuh)
   float* maxima;         // [slots][key tiles][128 rows x 128/R blocks]  per-row block maxima of the CTA that holds the slot
   int32_t* slot_taken;   // [slots]  0 = free; zeroed by kap_norms_kernel
   float* k2part;         // [kNormParts]  largest squared norms of sampled key rows of the call, one per CTA of kap_norms_kernel
@@ -241,8 +243,10 @@ constexpr int kMaxDevices = 64;
 struct SmemLimit { std::atomic<int> bytes[kMaxDevices]; };
 cudaError_t raise_smem_limit(const void* kernel, SmemLimit* state, size_t bytes);
 
-// redo_list == nullptr: every (head, query block); else only the listed ones (count in [0])
-cudaError_t launch_kap_exact(const KapParams& p, const int32_t* redo_list, cudaStream_t st);
+// every (head, query block) in double precision
+cudaError_t launch_kap_exact(const KapParams& p, cudaStream_t st);
+// works off sp.tied_list (near ties recounted) and sp.redo_list (whole lists redone)
+cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, cudaStream_t st);
 // the whole call's key tiles fit the screen's stages: it needs no scratch areas and no norms kernel
 bool kap_screen_is_short(int n, int stride);
 bool kap_screen_supported(int rows, int group, int stride, const KvPaging& pg);

@@ -4,7 +4,10 @@
 //   s_j = sum_r exp(M[r,j] - M*[r]),  h_j = any_r [M[r,j] == M*[r]]
 //   order = sort by (h desc, s desc, j asc);  keep K_i = budget_count(candidates), or the Top-p prefix.
 // Products of two bf16 values are exact in double, so scores carry ~1e-16 relative error.
+#include <algorithm>
+
 #include "common.cuh"
+#include "kap_recount.cuh"
 
 namespace cosa {
 namespace {
@@ -26,17 +29,26 @@ __global__ void __launch_bounds__(kThreads) kap_exact_kernel(KapParams p, int kb
   kap_exact_item(p, blockIdx.z, blockIdx.y, (p.nqb / p.qtiles - 1 - (int)blockIdx.x) * p.qtiles, kb_per_iter, sort_cap);
 }
 
-// 1-d grid: the CTAs share out the entries of a redo list (usually empty)
-__global__ void __launch_bounds__(kThreads) kap_exact_list_kernel(KapParams p, const int32_t* redo_list, int kb_per_iter,
-                                                                 int sort_cap, const int32_t* status) {
+// 1-d grid: the CTAs share out what the sort stage left.  kTied: lists with near ties to recount; kRedo: lists to do over (normally none).
+// In one launch where the second's shared memory leaves room for several CTAs on an SM, in two otherwise.
+template <bool kTied, bool kRedo>
+__global__ void __launch_bounds__(kThreads, kRedo ? 2 : 4) kap_fixup_kernel(KapParams p, KapScreenParams sp, int kb_per_iter, int sort_cap,
+                                                                          const int32_t* status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   chain_begin();
-  if (*reinterpret_cast<const volatile int32_t*>(status) != 0) return;   // an earlier kernel of the call gave up: the list is not to be trusted
-  const int n = redo_list[0];
-  for (int e = blockIdx.x; e < n; e += gridDim.x) {
-    const int flat = redo_list[1 + e];
-    const int i = flat % p.nqb, bh = flat / p.nqb;
-    kap_exact_item(p, bh / p.hq, bh % p.hq, i, kb_per_iter, sort_cap);   // i: first row tile of the block
-    __syncthreads();
+  if (*reinterpret_cast<const volatile int32_t*>(status) != 0) return;   // an earlier kernel of the call gave up: the lists are not to be trusted
+  if (kTied) {
+    const int n = sp.tied_list[0];
+    for (int e = blockIdx.x; e < n; e += gridDim.x) kap_recount_item(p, sp, sp.tied_list[1 + e], smem_raw);
+  }
+  if (kRedo) {
+    const int n = sp.redo_list[0];
+    for (int e = blockIdx.x; e < n; e += gridDim.x) {
+      const int flat = sp.redo_list[1 + e];
+      const int i = flat % p.nqb, bh = flat / p.nqb;
+      kap_exact_item(p, bh / p.hq, bh % p.hq, i, kb_per_iter, sort_cap);   // i: first row tile of the block
+      __syncthreads();
+    }
   }
 }
 
@@ -231,22 +243,33 @@ size_t kap_exact_smem_bytes(int rows, int nqb, int qtiles) {
   return doubles * 8 + (size_t)sort_cap * 12 + (size_t)((nqb | 1) + 15) / 16 * 16;
 }
 
-cudaError_t launch_kap_exact(const KapParams& p, const int32_t* redo_list, cudaStream_t st) {
-  size_t smem = kap_exact_smem_bytes(p.rows, p.nqb, p.qtiles);
-  if (redo_list) {
-    static SmemLimit limit;
-    cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kap_exact_list_kernel), &limit, smem);
-    if (e != cudaSuccess) return e;
-    const int32_t* status = device_status_word();
-    if (!status) return cudaErrorInvalidSymbol;
-    return launch_chained(kap_exact_list_kernel, dim3(148), kThreads, smem, st, p, redo_list, kb_per_iter_for(p.rows), next_pow2(p.nqb),
-                          status);
-  }
-  cudaError_t e = cudaFuncSetAttribute(kap_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t launch_kap_exact(const KapParams& p, cudaStream_t st) {
+  const size_t smem = kap_exact_smem_bytes(p.rows, p.nqb, p.qtiles);
+  static SmemLimit limit;
+  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kap_exact_kernel), &limit, smem);
   if (e != cudaSuccess) return e;
   dim3 grid(p.nqb / p.qtiles, p.hq, p.batch);
   kap_exact_kernel<<<grid, kThreads, smem, st>>>(p, kb_per_iter_for(p.rows), next_pow2(p.nqb));
   return cudaGetLastError();
+}
+
+cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, cudaStream_t st) {
+  static_assert(kThreads == kRecountThreads, "one kernel does both");
+  const int32_t* status = device_status_word();
+  if (!status) return cudaErrorInvalidSymbol;
+  const int lists = p.batch * p.hq * (p.nqb / p.qtiles), sms = 148;
+  const int kb = kb_per_iter_for(p.rows), cap = next_pow2(p.nqb);
+  const size_t redo = kap_exact_smem_bytes(p.rows, p.nqb, p.qtiles), tied = kap_recount_smem_bytes(p.rows, p.qtiles, p.nqb);
+  static SmemLimit limits[3];
+  auto launch = [&](auto kernel, SmemLimit* limit, size_t smem, int ctas) {
+    cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kernel), limit, smem);
+    return e != cudaSuccess ? e : launch_chained(kernel, dim3((unsigned)std::min(lists, ctas)), kThreads, smem, st, p, sp, kb, cap, status);
+  };
+  // (a launch costs as much as either does on a short call; at 64K tokens the second alone would leave one CTA per SM)
+  const size_t both = std::max(redo, tied);
+  if (both <= 56 * 1024) return launch(kap_fixup_kernel<true, true>, &limits[0], both, 2 * sms);
+  const cudaError_t e = launch(kap_fixup_kernel<true, false>, &limits[1], tied, 4 * sms);
+  return e != cudaSuccess ? e : launch(kap_fixup_kernel<false, true>, &limits[2], redo, sms);
 }
 
 }  // namespace cosa

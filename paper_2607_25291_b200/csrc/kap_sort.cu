@@ -3,7 +3,9 @@
 // on the float32 screen, with a double-precision recount of every decision a rounding error
 // could change.
 //
-// One CTA per (query head, query block).
+// One CTA of four warps per (query head, query block): its time is a chain of short steps, and what counts is how many lists an SM
+// has in work: ten, where eight warps a list and the recount's register needs allowed six (this kernel and the recount: 372 ->
+// 193 + 75 us at 128K tokens, 338 -> 99 + 118 at 64K and 50 %, 66 -> 48 + 13 at 32K).
 //  1. Rows whose two largest block maxima the screen could not tell apart (ambmask) are settled
 //     first: both blocks are re-evaluated with double-precision FMAs on the exact bf16 inputs,
 //     which fixes the row's M* and which block(s) earn the HRM flag from that row (Eq. 12).
@@ -13,99 +15,65 @@
 //     small budget only the buckets of the order's head (the kept prefix plus a margin for step 3) are.
 //  3. Two sorted neighbours with the same flag whose scores differ by less than tau_score
 //     (relative) are a "near tie"; a maximal chain of near ties that starts inside the kept
-//     prefix (or straddles its end) is recounted: M[r,j] of each of its blocks and M*[r] are
-//     recomputed in double precision (same operation order as the double-precision kernel) and
-//     the chain is re-sorted by the double-precision score, ties by ascending block id.
+//     prefix (or straddles its end) is left to be recounted in double precision (kap_recount.cuh): its entries go to the
+//     list's row of scores, which is not needed any more.
 // Everything outside such chains is ordered as exact arithmetic would order it provided the
 // screen's error stays below tau_score / 2, which the tests check.  Query blocks the screen
-// marked "hard", or with more chained entries than fit, go to the double-precision kernel.
+// marked "hard", or with more chained entries than fit their row, go to the double-precision kernel.
 #include <math.h>
 
 #include "common.cuh"
+#include "kap_recount.cuh"
 
 namespace cosa {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kMaxTied = 96;      // chained entries one list may have before it is left to the double-precision kernel
+constexpr int kThreads = 128;
 constexpr int kMaxRows = 64;   // sampled rows of one (possibly two-tile) query block
 constexpr int kHeadCap = 256;     // entries of the order's head that are sorted on their own
 constexpr int kAllPairs = 128;    // keys up to which every key is compared with every other
 constexpr int kSamples = 64;      // sample keys, of which every second splits: 33 buckets
 constexpr int kSplit = 32;
-constexpr int kPerThread = 4;     // keys a thread keeps the place of
-constexpr int kPad = kHeadDim + 1;
-constexpr int kSetChunk = 8;      // blocks recounted together in the near-tie stage
+constexpr int kPerThread = 8;     // keys a thread keeps the place of
+constexpr int kPad = kHeadDim + 4;   // row pitch in floats
 constexpr int kTieMargin = 32;    // ... of which this many lie beyond the kept prefix
 
-struct Tied { int pos; unsigned id; double s; };
-
-__device__ __forceinline__ double bf16_lo(unsigned w) { return (double)__uint_as_float(w << 16); }
-__device__ __forceinline__ double bf16_hi(unsigned w) { return (double)__uint_as_float(w & 0xffff0000u); }
-
-// A quarter of a dot product of 128 elements in double precision against kRowsPer query rows (widened to double, kPad apart):
-// the 16-byte chunks quarter, quarter + 4, ... of the key row, all four requested before any is used.  (One thread per dot
-// took its key row 32 bytes at a time, eight round trips to L2 one after the other.)
-template <int kRowsPer>
-__device__ __forceinline__ void dot_quarter_f64(const double* q0, const uint4* key, int quarter, double (&acc)[kRowsPer]) {
-  uint4 w[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) w[u] = key[u * 4 + quarter];
-#pragma unroll
-  for (int rr = 0; rr < kRowsPer; ++rr) acc[rr] = 0.0;
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const unsigned kw[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
-    const double* q = q0 + (u * 4 + quarter) * 8;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const double lo = bf16_lo(kw[e]), hi = bf16_hi(kw[e]);
-#pragma unroll
-      for (int rr = 0; rr < kRowsPer; ++rr) acc[rr] = fma(q[rr * kPad + 2 * e], lo, acc[rr]);
-#pragma unroll
-      for (int rr = 0; rr < kRowsPer; ++rr) acc[rr] = fma(q[rr * kPad + 2 * e + 1], hi, acc[rr]);
-    }
-  }
-#pragma unroll
-  for (int rr = 0; rr < kRowsPer; ++rr) {          // (q0 + q1) + (q2 + q3): the same in every lane
-    acc[rr] += __shfl_xor_sync(0xffffffffu, acc[rr], 1);
-    acc[rr] += __shfl_xor_sync(0xffffffffu, acc[rr], 2);
-  }
-}
-
-// Block maxima in double precision, straight from the bf16 keys; Qs holds the query block's sampled rows widened to double, kPad
-// apart.  out[set][r] = max over the visible sampled keys c of (Q~[r] . K~[block * R + c]) * scale, -inf when row r sees nothing
-// of the block that block_of(set, first row of the group) names (negative: no block, the entries are left alone).  A warp takes
-// kRowsPer rows against one block, four lanes a key, eight keys at a time.  kRowsPer = 1: a block of its own per row; 4: one block
-// per set, every key element widened once for four rows (widening float to double runs at a quarter of the FP64 FMA
-// rate on this GPU; with eight rows the accumulators spill under this kernel's register limit).  All threads of the CTA call it.
-template <int kRowsPer, typename BlockOf>
-__device__ void f64_block_maxima(const KapParams& p, const double* Qs, int b, int g, int row0, int rows, int R, int n_sets,
+// Block maxima in double precision, straight from the bf16 keys; Qs holds the query block's sampled rows as floats, kPad apart.
+// out[set][r] = max over the visible sampled keys c of block_of(set, r) of (Q~[r] . K~[c]) * scale, -inf when row r sees
+// nothing of the block; entries whose block is negative are left alone.  A warp takes one row against one block: four
+// lanes a key, eight keys at a time; (q0 + q1) + (q2 + q3) is the same in every lane.  All threads of the CTA call it.
+template <typename BlockOf>
+__device__ void f64_block_maxima(const KapParams& p, const float* Qs, int b, int g, int row0, int rows, int R, int n_sets,
                                  BlockOf block_of, double (*out)[kMaxRows], int tid) {
-  const int lane = tid & 31, groups = rows / kRowsPer;
-  for (int item = tid >> 5; item < n_sets * groups; item += kThreads / 32) {
-    const int set = item / groups, r0 = (item % groups) * kRowsPer;
-    const int j = block_of(set, r0);
+  const int lane = tid & 31, quarter = lane & 3;
+  for (int item = tid >> 5; item < n_sets * rows; item += kThreads / 32) {
+    const int set = item / rows, r = item % rows;
+    const int j = block_of(set, r);
     if (j < 0) continue;                           // (the whole warp)
-    double best[kRowsPer];
-#pragma unroll
-    for (int rr = 0; rr < kRowsPer; ++rr) best[rr] = -INFINITY;
+    double best = -INFINITY;
 #pragma unroll 1
     for (int c0 = 0; c0 < R; c0 += 8) {
       const int kc = j * R + c0 + (lane >> 2);     // sampled key index
-      double z[kRowsPer];
-      dot_quarter_f64<kRowsPer>(Qs + (size_t)r0 * kPad, reinterpret_cast<const uint4*>(p.k + kv_off(p.pg, p.ks, b, p.hkv, g, kc * p.stride)),
-                                lane & 3, z);
+      const uint4* key = reinterpret_cast<const uint4*>(p.k + kv_off(p.pg, p.ks, b, p.hkv, g, kc * p.stride));
+      double acc = 0.0;
+#pragma unroll 2
+      for (int u = 0; u < 4; ++u) {
+        const uint4 w = key[u * 4 + quarter];
+        const unsigned kw[4] = {w.x, w.y, w.z, w.w};
+        const float* q = Qs + r * kPad + (u * 4 + quarter) * 8;
 #pragma unroll
-      for (int rr = 0; rr < kRowsPer; ++rr)
-        if (!p.causal || kc <= row0 + r0 + rr) best[rr] = fmax(best[rr], z[rr] * p.scale);
+        for (int e = 0; e < 4; ++e) {
+          acc = fma((double)q[2 * e], bf16_lo(kw[e]), acc);
+          acc = fma((double)q[2 * e + 1], bf16_hi(kw[e]), acc);
+        }
+      }
+      acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+      acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+      if (!p.causal || kc <= row0 + r) best = fmax(best, acc * p.scale);
     }
 #pragma unroll
-    for (int rr = 0; rr < kRowsPer; ++rr) {
-#pragma unroll
-      for (int o = 4; o < 32; o <<= 1) best[rr] = fmax(best[rr], __shfl_xor_sync(0xffffffffu, best[rr], o));
-      if (lane == 0) out[set][r0 + rr] = best[rr];
-    }
+    for (int o = 4; o < 32; o <<= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
+    if (lane == 0) out[set][r] = best;
   }
   __syncthreads();
 }
@@ -138,7 +106,7 @@ __device__ int sort_head_desc(unsigned long long* a, int n, int want, unsigned l
                               unsigned char* bucket, SortShared* sh, bool one_bucket, int tid, unsigned long long** out) {
   *out = a;
   if (n <= kAllPairs && !one_bucket) {
-    int shift = 5;                                 // 2^shift threads per key
+    int shift = 5;                                 // 2^shift threads per key (one for 65 to 128 keys)
     while ((n << shift) > kThreads) --shift;
     const int k = tid >> shift, part = tid & ((1 << shift) - 1);
     const unsigned long long key = k < n ? a[k] : 0ULL;
@@ -151,7 +119,7 @@ __device__ int sort_head_desc(unsigned long long* a, int n, int want, unsigned l
     __syncthreads();
     return n;
   }
-  // 64 samples, one from each stretch of n / 64 keys, ranked by four threads each
+  // 64 samples, one from each stretch of n / 64 keys, ranked by two threads each
   if (tid < kSamples) {
     const int lo = (int)((long long)tid * n / kSamples), len = max(1, n / kSamples);
     sh->samp[tid] = a[lo + (tid * 5) % len];
@@ -161,16 +129,16 @@ __device__ int sort_head_desc(unsigned long long* a, int n, int want, unsigned l
   if (one_bucket) {
     if (tid < kSplit) sh->split[tid] = ~0u;
   } else {
-    const unsigned long long mine = sh->samp[tid >> 2];
+    static_assert(kThreads == 2 * kSamples, "two threads per sample");
+    const unsigned long long mine = sh->samp[tid >> 1];
     int rank = 0;
 #pragma unroll 8
-    for (int u = 0; u < kSamples / 4; ++u) rank += (sh->samp[u * 4 + (tid & 3)] > mine) ? 1 : 0;
+    for (int u = 0; u < kSamples / 2; ++u) rank += (sh->samp[u * 2 + (tid & 1)] > mine) ? 1 : 0;
     rank += __shfl_xor_sync(0xffffffffu, rank, 1);
-    rank += __shfl_xor_sync(0xffffffffu, rank, 2);
-    if ((tid & 3) == 0 && (rank & 1)) sh->split[rank >> 1] = (unsigned)(mine >> 32);
+    if ((tid & 1) == 0 && (rank & 1)) sh->split[rank >> 1] = (unsigned)(mine >> 32);
   }
   __syncthreads();
-  // every key to its bucket's count; a thread keeps bucket and place of its first four keys (all there are up to 1024)
+  // every key to its bucket's count; a thread keeps bucket and place of its first eight keys (all there are up to 1024)
   unsigned place[kPerThread];
 #pragma unroll
   for (int q = 0; q < kPerThread; ++q) {
@@ -237,16 +205,15 @@ __device__ int sort_head_desc(unsigned long long* a, int n, int want, unsigned l
   return len;
 }
 
-__global__ void __launch_bounds__(kThreads, 6) kap_sort_kernel(KapParams p, KapScreenParams sp, float tau_score, int sort_cap,
+__global__ void __launch_bounds__(kThreads, 10) kap_sort_kernel(KapParams p, KapScreenParams sp, float tau_score, int sort_cap,
                                                             int tie_bytes, const int32_t* status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem_raw);  // [sort_cap]
   unsigned char* tie = reinterpret_cast<unsigned char*>(keys + sort_cap);        // [tie_bytes]
-  double* Qs = reinterpret_cast<double*>(tie + tie_bytes);                       // [R * tiles][kPad], filled on demand; the sort's
+  float* Qs = reinterpret_cast<float*>(tie + tie_bytes);                         // [R * tiles][kPad], filled on demand; the sort's
   unsigned long long* tmp = reinterpret_cast<unsigned long long*>(Qs);           // [sort_cap] scratch keys take the same place
-  __shared__ Tied tied[kMaxTied];
   __shared__ double Mstar[kMaxRows];
-  __shared__ double Mset[kSetChunk][kMaxRows];
+  __shared__ double Mset[2][kMaxRows];
   __shared__ int j1[kMaxRows], j2[kMaxRows];
   __shared__ int n_tied, tail_end;
   __shared__ SortShared sort_sh;
@@ -288,17 +255,17 @@ __global__ void __launch_bounds__(kThreads, 6) kap_sort_kernel(KapParams p, KapS
   // scores of the block = sum over its row tiles (the sum of Eq. 11 splits over the rows), flags = OR; a tile has
   // no score for key blocks wholly after it
   if (T == 1) {
-    // four scores per thread requested before any is used: the loads of a list are one round trip, not four
+    // eight scores per thread requested before any is used: the loads of a list are one round trip, not four
     const float* srow = sp.scores + row_lo * p.nqb;
-    for (int j0 = 0; j0 < J; j0 += 4 * kThreads) {
-      float v[4];
+    for (int j0 = 0; j0 < J; j0 += 8 * kThreads) {
+      float v[8];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < 8; ++u) {
         const int j = j0 + u * kThreads + tid;
         v[u] = j < J ? srow[j] : 0.f;
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < 8; ++u) {
         const int j = j0 + u * kThreads + tid;
         if (j < J) {
           const unsigned flag = (v[u] < 0.f) ? 0x80000000u : 0u;
@@ -328,36 +295,27 @@ __global__ void __launch_bounds__(kThreads, 6) kap_sort_kernel(KapParams p, KapS
   }
   if (tid == 0) { n_tied = 0; tail_end = 0; }
   if (tid < RT) { j1[tid] = js.x; j2[tid] = js.y; }
-  bool have_mstar = false, have_q = false;
-  auto load_q = [&]() {   // the block's sampled query rows, widened once
-    if (!have_q) {
-      for (int e = tid; e < RT * (kHeadDim / 8); e += kThreads) {
-        const int r = e / (kHeadDim / 8), c8 = e % (kHeadDim / 8);
-        const uint4 w = reinterpret_cast<const uint4*>(qh + ((size_t)(i_lo * R + r) * p.stride) * p.qs.t)[c8];
-        const unsigned ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          Qs[r * kPad + c8 * 8 + 2 * u] = bf16_lo(ws[u]);
-          Qs[r * kPad + c8 * 8 + 2 * u + 1] = bf16_hi(ws[u]);
-        }
-      }
-      __syncthreads();
-      have_q = true;
-    }
-  };
   __syncthreads();
 
   if (amb) {
     // ---- 1. settle the rows the screen could not call: set 0 = every row's best block, set 1 = the runner-up of
     // the rows in question
     if (tid < RT) Mset[1][tid] = -INFINITY;
-    load_q();
+    for (int e = tid; e < RT * (kHeadDim / 8); e += kThreads) {
+      const int r = e / (kHeadDim / 8), c8 = e % (kHeadDim / 8);
+      const uint4 w = reinterpret_cast<const uint4*>(qh + ((size_t)(i_lo * R + r) * p.stride) * p.qs.t)[c8];
+      const unsigned ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        Qs[r * kPad + c8 * 8 + 2 * u] = __uint_as_float(ws[u] << 16);
+        Qs[r * kPad + c8 * 8 + 2 * u + 1] = __uint_as_float(ws[u] & 0xffff0000u);
+      }
+    }
     __syncthreads();
-    f64_block_maxima<1>(p, Qs, b, g, i_lo * R, RT, R, 2,
+    f64_block_maxima(p, Qs, b, g, i_lo * R, RT, R, 2,
                      [&](int set, int r) { return set == 0 ? j1[r] : (((amb >> r) & 1ULL) ? j2[r] : -1); }, Mset, tid);
     double* Msecond = Mset[1];
     if (tid < RT) Mstar[tid] = Mset[0][tid];
-    have_mstar = true;
     __syncthreads();
     if (tid == 0) {
       for (int r = 0; r < RT; ++r) {
@@ -376,8 +334,6 @@ __global__ void __launch_bounds__(kThreads, 6) kap_sort_kernel(KapParams p, KapS
           keys[j] = (keys[j] & 0x7fffffffffffffffULL) | (flag ? 0x8000000000000000ULL : 0ULL);
         }
       }
-      for (int r = 0; r < RT; ++r)
-        if ((amb >> r) & 1ULL) Mstar[r] = fmax(Mstar[r], Msecond[r]);
     }
     __syncthreads();
   }
@@ -399,7 +355,6 @@ __global__ void __launch_bounds__(kThreads, 6) kap_sort_kernel(KapParams p, KapS
   const int want = p.sort_mode == 2 || p.top_p > 0.0 ? J : min(J, K + kTieMargin);
   unsigned long long* srt;          // the sorted order: srt[0 .. L)
   int L = sort_head_desc(keys, J, want, head, tmp, tie, &sort_sh, p.sort_mode == 1, tid, &srt);
-  have_q = false;                   // (its place was the sort's)
   if (p.top_p > 0.0) {
       // Top-p retention: the shortest prefix of the order whose scores reach top_p of the total.  Every thread
       // owns a run of consecutive sorted entries; sums are double precision in a fixed order (deterministic).
@@ -447,7 +402,6 @@ __global__ void __launch_bounds__(kThreads, 6) kap_sort_kernel(KapParams p, KapS
   // (none that begins inside the kept prefix: the usual case, and nothing more to do)
   bool any = false;
   for (int t = tid; t < K && t + 1 < L; t += kThreads) any = any || near_tie(t);
-  int nt = 0;
   if (__syncthreads_or(any)) {
     for (;;) {
       for (int t = tid; t < L; t += kThreads) tie[t] = t + 1 < L && near_tie(t) ? 1 : 0;
@@ -462,75 +416,27 @@ __global__ void __launch_bounds__(kThreads, 6) kap_sort_kernel(KapParams p, KapS
       if (!need_full) break;
       L = sort_head_desc(keys, J, J, head, tmp, tie, &sort_sh, p.sort_mode == 1, tid, &srt);
     }
+    // entries: position and "tied with the next", id
+    int* row_words = reinterpret_cast<int*>(sp.scores + row_lo * p.nqb);
+    const int fit = min(kRecountMax, (p.nqb * T - 2) / 2);
     for (int t = tid; t < tail_end; t += kThreads) {
       if ((t > 0 && tie[t - 1]) || tie[t]) {
         const int slot = atomicAdd(&n_tied, 1);
-        if (slot < kMaxTied) { tied[slot].pos = t; tied[slot].id = 0xffffffffu - (unsigned)(srt[t] & 0xffffffffu); }
+        if (slot < fit) {
+          row_words[2 + 2 * slot] = 2 * t + tie[t];
+          row_words[3 + 2 * slot] = (int)(0xffffffffu - (unsigned)(srt[t] & 0xffffffffu));
+        }
       }
     }
     __syncthreads();
-    nt = n_tied;
-    if (nt > kMaxTied) {  // pathological: too many near ties
+    const int nt = n_tied;
+    if (nt > fit) {   // pathological: too many near ties
       if (tid == 0) sp.redo_list[1 + atomicAdd(sp.redo_list, 1)] = (int)row_lo;
       return;
     }
-    if (nt > 0) {
-      // Double-precision scores of the chained entries: M*[r] from every row's best block (unless the ambiguous rows
-      // above already needed it), then the entries a few at a time: block maxima of the entry's block for all rows,
-      // one thread per (entry, row) takes the exponential and one per entry adds the rows in order.
-      load_q();
-      if (!have_mstar) {
-        f64_block_maxima<1>(p, Qs, b, g, i_lo * R, RT, R, 1, [&](int, int r) { return j1[r]; }, Mset, tid);
-        if (tid < RT) Mstar[tid] = Mset[0][tid];
-        __syncthreads();
-      }
-      for (int base = 0; base < nt; base += kSetChunk) {
-        const int n_sets = min(kSetChunk, nt - base);
-        f64_block_maxima<4>(p, Qs, b, g, i_lo * R, RT, R, n_sets,
-                            [&](int set, int) { return (int)tied[base + set].id; }, Mset, tid);
-        for (int e = tid; e < n_sets * RT; e += kThreads) {
-          const int sl = e / RT, r = e % RT;
-          Mset[sl][r] = exp(Mset[sl][r] - Mstar[r]);   // exp(-inf) = 0: the row sees nothing of the block
-        }
-        __syncthreads();
-        if (tid < n_sets) {
-          double sum = 0.0;
-          for (int r = 0; r < RT; ++r) sum += Mset[tid][r];
-          tied[base + tid].s = sum;
-        }
-        __syncthreads();
-      }
-      have_mstar = true;
-      if (tid == 0) {
-        // order the chained entries by position, then re-sort every chain by (score desc, id asc)
-        for (int a = 1; a < nt; ++a) {
-          Tied x = tied[a];
-          int c = a - 1;
-          while (c >= 0 && tied[c].pos > x.pos) { tied[c + 1] = tied[c]; --c; }
-          tied[c + 1] = x;
-        }
-        int a = 0;
-        while (a < nt) {
-          int e = a;
-          while (e + 1 < nt && tied[e + 1].pos == tied[e].pos + 1 && tie[tied[e].pos]) ++e;
-          const int first_pos = tied[a].pos;
-          for (int x = a + 1; x <= e; ++x) {  // insertion sort of one chain; the positions stay
-            const unsigned idx = tied[x].id;
-            const double sx = tied[x].s;
-            int c = x - 1;
-            while (c >= a && (tied[c].s < sx || (tied[c].s == sx && tied[c].id > idx))) {
-              tied[c + 1].id = tied[c].id; tied[c + 1].s = tied[c].s; --c;
-            }
-            tied[c + 1].id = idx; tied[c + 1].s = sx;
-          }
-          for (int x = a; x <= e; ++x) {
-            const int pos = first_pos + (x - a);
-            srt[pos] = (srt[pos] & 0xffffffff00000000ULL) | (unsigned long long)(0xffffffffu - tied[x].id);
-          }
-          a = e + 1;
-        }
-      }
-      __syncthreads();
+    if (tid == 0 && nt > 0) {
+      row_words[0] = nt; row_words[1] = K;
+      sp.tied_list[1 + atomicAdd(sp.tied_list, 1)] = (int)row_lo;
     }
   }
   // the last row tile of the block takes the kept entries as they are; an earlier tile leaves out the key blocks that
@@ -561,7 +467,7 @@ cudaError_t launch_kap_sort(const KapParams& p, const KapScreenParams& sp, float
   if (p.rows * p.qtiles > kMaxRows || p.nqb % p.qtiles != 0 || p.qtiles < 1 || p.qtiles > 2) return cudaErrorInvalidValue;
   const int cap = (p.nqb + 1) & ~1;            // keys, 16-byte pieces
   const int tie_bytes = (cap + 15) / 16 * 16;
-  const size_t q_bytes = (size_t)p.rows * p.qtiles * kPad * 8, tmp_bytes = (size_t)cap * 8;
+  const size_t q_bytes = (size_t)p.rows * p.qtiles * kPad * 4, tmp_bytes = (size_t)cap * 8;
   const size_t smem = (size_t)cap * 8 + tie_bytes + (q_bytes > tmp_bytes ? q_bytes : tmp_bytes);
   static SmemLimit limit;
   cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kap_sort_kernel), &limit, smem);

@@ -268,6 +268,28 @@ def test_kap_duplicate_key_blocks_tie_break(small):
         assert np.array_equal(_np(count), ref_count) and np.array_equal(_np(order), ref_order)
 
 
+@pytest.mark.parametrize("block_q", [128, 256])
+@pytest.mark.parametrize("stride", [4, 8, 16])
+@pytest.mark.parametrize("budget", [0.1, 0.3, 0.5, 0.9])
+def test_kap_chains_of_equal_scores(cfg1, budget, stride, block_q):
+    """Groups of two to twenty identical key blocks: chains of ties at the head, in the middle and across the end of the kept
+    prefix, in more than one chunk of the recount, with rows too close to call among them, 8 to 32 sampled rows per tile and
+    one or two tiles per ranking; exact ties go by ascending id, so the lists are the oracle's."""
+    q, k, _ = cfg1["dev"]
+    qf, kf, _ = cfg1["f64"]
+    k2, kf2 = k.clone(), kf.copy()
+    for src, dsts in ((0, (4,)), (5, (6, 9, 30)), (7, tuple(range(10, 29)))):
+        for dst in dsts:
+            k2[0, :, dst * 128:(dst + 1) * 128] = k2[0, :, src * 128:(src + 1) * 128]
+            kf2[:, dst * 128:(dst + 1) * 128] = kf2[:, src * 128:(src + 1) * 128]
+    order, count = alloc_lists(4, 32)
+    cosa.cosa_kap_select(q, k2, budget, order, count, opt=cosa.default_options(stride=stride), block_q=block_q)
+    assert cosa.cosa_device_status() == 0
+    select = O.kap_select_wide if block_q == 256 else O.kap_select
+    ref_order, ref_count = select(qf, kf2, s=stride, budget=budget, order_stride=32)
+    assert np.array_equal(_np(count), ref_count) and np.array_equal(_np(order), ref_order)
+
+
 @pytest.mark.parametrize("impl", IMPLS)
 def test_kap_lists_bit_exact_4k(cfg1, impl):
     w = cfg1["w"]
