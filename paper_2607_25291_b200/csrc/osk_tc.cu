@@ -27,7 +27,7 @@
 // controller warp, the arrangement before: 8.05, 1.22 and 1.95).  Measured and not used: P over S in tensor memory (7.7 / 1.09 /
 // 2.08), two threads per row (8.2 / 1.15 / 2.12).
 // Every wait is bounded; a wait that runs out sets the device status word and the CTA winds down without writing
-// results: load and issue warps leave, the row threads leave together at their next vote.
+// results: load and issue warps leave, the row threads, whom no wait holds any more, run to the end of their list.
 #include <math.h>
 
 #include <type_traits>
@@ -66,8 +66,6 @@ struct __align__(8) Control {
   uint32_t tmem_base;
   int poisoned;
   volatile int abort_flag;
-  volatile int grp_bad[2];         // by position parity: a row thread gave up waiting (two words, so that a fast warp's mark
-                                   // at position k+1 is not taken for one at k)
   volatile int req[4];             // tiles requested so far: K by parity, V by half (read when a walk was given up)
   volatile uint32_t dec[2];
 };
@@ -182,7 +180,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       }
       mbar_init(smem_u32(&ctl->s_full), 1); mbar_init(smem_u32(&ctl->s_read), kBlock);
       mbar_init(smem_u32(&ctl->fin), 1);
-      ctl->abort_flag = 0; ctl->grp_bad[0] = 0; ctl->grp_bad[1] = 0;
+      ctl->abort_flag = 0;
       for (int q = 0; q < 4; ++q) ctl->req[q] = 0;
       mbar_fence_init();
       fence_proxy_async_smem();
@@ -358,23 +356,22 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         }
       };
       uint32_t s[kBlock];                       // this row's raw logits, then probabilities
-      // rows only ask whether a position's block is the diagonal one, which an ascending mask walk meets last, if at all; the
-      // list entry is requested a turn ahead
+      // rows only ask whether a position's block is the diagonal one, which an ascending mask walk meets last, if at all: a warp
+      // looks at 32 list entries at a time
       const bool mask_diag = kMask && ((walk.mask[i >> 5] >> (i & 31)) & 1u);
-      int j_ahead = kMask ? 0 : list[0];
+      uint32_t diag_bits = 0;
       for (;; ++kk) {
-        const int j = kMask ? ((kk == cnt - 1 && mask_diag) ? i : -1) : j_ahead;
-        if (!kMask && kk + 1 < cnt) j_ahead = list[kk + 1];
+        if (!kMask && p.causal && (kk & 31) == 0) diag_bits = __ballot_sync(0xffffffffu, kk + lane < cnt && list[kk + lane] == i);
+        const bool diag = kMask ? p.causal && mask_diag && kk == cnt - 1 : ((diag_bits >> (kk & 31)) & 1u) != 0;
         wait(&ctl->s_full, kk);
-        if (kStage2) __syncwarp();
-        else if (__any_sync(0xffffffffu, bad)) break;
+        __syncwarp();
         tc_fence_after();
 #pragma unroll
         for (int c = 0; c < 4; ++c) tmem_ld32(tmem_s + lane_addr + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
         tmem_wait_ld();
         tc_fence_before();
         mbar_arrive(smem_u32(&ctl->s_read));
-        if (p.causal && j == i) {                   // token-level causal mask on the diagonal block
+        if (diag) {                   // token-level causal mask on the diagonal block
 #pragma unroll
           for (int c = 0; c < kBlock; ++c) if (c > r) s[c] = 0xff800000u;  // -inf
         }
@@ -389,10 +386,9 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         const float m_new = fmaxf(m, m_loc);
         bool last = kk == cnt - 1;
         if (kStage2) {
-          // Eq. (5): skip iff max over the 128 rows of (m_loc - m) < ln(Delta/N), m including this block.  A thread that gave
-          // up votes for computing, so that a skip is always everybody's, and the group leaves together
-          if (bad) ctl->grp_bad[kk & 1] = 1;
-          const bool compute = bar_red_or(1, kBlock, !(thr_on && (m_loc - m_new) < theta2) || bad);
+          // Eq. (5): skip iff max over the 128 rows of (m_loc - m) < ln(Delta/N), m including this block.  (Rows of a walk that was given
+          // up vote on as long as their list lasts: nothing holds them any more)
+          const bool compute = bar_red_or(1, kBlock, !(thr_on && (m_loc - m_new) < theta2));
           last = last || n + (compute ? 1 : 0) == cap;
           if (r == 0) {
             ctl->dec[kk & 1] = (compute ? kDecComputed : 0u) | (last ? kDecEnd : 0u);
@@ -404,7 +400,6 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
             if (last) break;
             continue;
           }
-          if (ctl->grp_bad[kk & 1]) break;
         }
         m = m_new;
         // ---- the exponentials refer to m_ref, an earlier running maximum, until the maximum has moved by more than 2^8:
