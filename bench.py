@@ -446,7 +446,7 @@ def main():
                            "causal_block_pairs": pairs, "input_generation_s": round(t_gen, 1)},
                 "latency_ms": {"kap": kap_ms, "osk": osk_ms, "kap_plus_osk": ms_per_step},
                 "latency_ms_as_a_burst": ({"kap": burst_run["kap_ms"], "osk": burst_run["osk_ms"], "how": burst_run["how"]} if burst_run else None),
-                "e2e": e2e, "gpu_launches": 4 * args.steps, "clocks": clocks, "roofline": roofline,
+                "e2e": e2e, "gpu_launches": 6 * args.steps, "clocks": clocks, "roofline": roofline,
                 "roofline_osk": roof_osk, "roofline_kap": roof_kap, "cpu_baseline": cpu, "comparators": extras,
                 "wall_s_timed_region": t_wall}
         print(json.dumps(line), flush=True)

@@ -522,15 +522,17 @@ int cosa_prefill_host(const void* q_host, const void* k_host, const void* v_host
 
   // One chunk per (batch item, KV head): its query heads, lists and outputs are contiguous slices of every tensor,
   // so the chunks run as independent calls.  Copies to the device go on a second stream and copies back on a third,
-  // so that the transfers of the other chunks overlap a chunk's kernels; `stream` waits for the last copy back.
+  // so that the transfers of the other chunks overlap a chunk's kernels; `stream` waits for the last copy back.  The link
+  // to the device is what bounds the call; after the last byte has arrived, the last chunk's kernels and copy back
+  // remain.  The last chunk is therefore taken query head by query head (16K tokens, 32 / 8 heads: 4.55 -> 4.49 ms).
   const int G = shape->hq / shape->hkv, chunks = shape->batch * shape->hkv;
-  const size_t nqb = shape->n / kBlock;
-  const size_t q_chunk = L.q_bytes / chunks, kv_chunk = L.kv_bytes / chunks, lse_chunk = L.lse_bytes / chunks;
-  const size_t order_chunk = L.order_bytes / chunks, cnt_chunk = L.cnt_bytes / chunks;
+  const size_t kv_chunk = L.kv_bytes / chunks;
+  const size_t heads = (size_t)shape->batch * shape->hq;
+  const size_t q_head = L.q_bytes / heads, lse_head = L.lse_bytes / heads, order_head = L.order_bytes / heads, cnt_head = L.cnt_bytes / heads;
   cudaStream_t up = nullptr, down = nullptr;
   if (!copy_streams(&up, &down)) return cuda_fail(cudaGetLastError(), "copy streams");
   cosa_shape sub = *shape;
-  sub.batch = 1; sub.hq = G; sub.hkv = 1;
+  sub.batch = 1; sub.hkv = 1;
   cudaEvent_t ev = nullptr;
   auto order_after = [&](cudaStream_t later, cudaStream_t earlier) -> bool {   // later waits for what earlier holds now
     if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) return false;
@@ -541,34 +543,39 @@ int cosa_prefill_host(const void* q_host, const void* k_host, const void* v_host
   };
   if (!order_after(up, st)) return cuda_fail(e, "stream order");   // the workspace may still be in use on `stream`
   if (!order_after(down, st)) return cuda_fail(e, "stream order");
-  (void)nqb;
   for (int c = 0; c < chunks; ++c) {
-    const char* qh = static_cast<const char*>(q_host) + c * q_chunk;
     const char* kh = static_cast<const char*>(k_host) + c * kv_chunk;
     const char* vh = static_cast<const char*>(v_host) + c * kv_chunk;
-    char* qd = ws + L.q + c * q_chunk; char* kd = ws + L.k + c * kv_chunk; char* vd = ws + L.v + c * kv_chunk;
-    char* od = ws + L.out + c * q_chunk;
-    if ((e = cudaMemcpyAsync(kd, kh, kv_chunk, cudaMemcpyHostToDevice, up)) != cudaSuccess) return cuda_fail(e, "H2D k");
-    if ((e = cudaMemcpyAsync(qd, qh, q_chunk, cudaMemcpyHostToDevice, up)) != cudaSuccess) return cuda_fail(e, "H2D q");
-    if ((e = cudaMemcpyAsync(vd, vh, kv_chunk, cudaMemcpyHostToDevice, up)) != cudaSuccess) return cuda_fail(e, "H2D v");
-    if (!order_after(st, up)) return cuda_fail(e, "stream order");
-    int32_t* order_d = reinterpret_cast<int32_t*>(ws + L.order + c * order_chunk);
-    int32_t* count_d = reinterpret_cast<int32_t*>(ws + L.count + c * cnt_chunk);
-    int32_t* visited_d = reinterpret_cast<int32_t*>(ws + L.visited + c * cnt_chunk);
-    float* lse_d = reinterpret_cast<float*>(ws + L.lse + c * lse_chunk);
+    char* kd = ws + L.k + c * kv_chunk; char* vd = ws + L.v + c * kv_chunk;
     cosa_options oc = o;
     if (o.seq_lens) oc.seq_lens = o.seq_lens + c / shape->hkv;   // the slice's batch item (lengths live on the device: padding is copied too)
-    rc = cosa_kap_select_ex(qd, kd, &sub, budget, order_d, count_d, stream, &oc);
-    if (rc != COSA_OK) return rc;
-    rc = cosa_osk_attention_ex(qd, kd, vd, &sub, order_d, count_d, tightened_budget, od, lse_d, visited_d, stream, &oc);
-    if (rc != COSA_OK) return rc;
-    if (!order_after(down, st)) return cuda_fail(e, "stream order");
-    if ((e = cudaMemcpyAsync(static_cast<char*>(out_host) + c * q_chunk, od, q_chunk, cudaMemcpyDeviceToHost, down)) != cudaSuccess)
-      return cuda_fail(e, "D2H out");
-    if (out_lse_host && (e = cudaMemcpyAsync(reinterpret_cast<char*>(out_lse_host) + c * lse_chunk, lse_d, lse_chunk,
-                                             cudaMemcpyDeviceToHost, down)) != cudaSuccess) return cuda_fail(e, "D2H lse");
-    if (out_visited_host && (e = cudaMemcpyAsync(reinterpret_cast<char*>(out_visited_host) + c * cnt_chunk, visited_d, cnt_chunk,
-                                                 cudaMemcpyDeviceToHost, down)) != cudaSuccess) return cuda_fail(e, "D2H visited");
+    if ((e = cudaMemcpyAsync(kd, kh, kv_chunk, cudaMemcpyHostToDevice, up)) != cudaSuccess) return cuda_fail(e, "H2D k");
+    const int step = c == chunks - 1 ? 1 : G;
+    sub.hq = step;
+    for (int h0 = 0; h0 < G; h0 += step) {
+      const size_t h = (size_t)c * G + h0;                       // the slice's first query head
+      const size_t q_bytes = step * q_head;
+      char* qd = ws + L.q + h * q_head; char* od = ws + L.out + h * q_head;
+      if ((e = cudaMemcpyAsync(qd, static_cast<const char*>(q_host) + h * q_head, q_bytes, cudaMemcpyHostToDevice, up)) != cudaSuccess)
+        return cuda_fail(e, "H2D q");
+      if (h0 == 0 && (e = cudaMemcpyAsync(vd, vh, kv_chunk, cudaMemcpyHostToDevice, up)) != cudaSuccess) return cuda_fail(e, "H2D v");
+      if (!order_after(st, up)) return cuda_fail(e, "stream order");
+      int32_t* order_d = reinterpret_cast<int32_t*>(ws + L.order + h * order_head);
+      int32_t* count_d = reinterpret_cast<int32_t*>(ws + L.count + h * cnt_head);
+      int32_t* visited_d = reinterpret_cast<int32_t*>(ws + L.visited + h * cnt_head);
+      float* lse_d = reinterpret_cast<float*>(ws + L.lse + h * lse_head);
+      rc = cosa_kap_select_ex(qd, kd, &sub, budget, order_d, count_d, stream, &oc);
+      if (rc != COSA_OK) return rc;
+      rc = cosa_osk_attention_ex(qd, kd, vd, &sub, order_d, count_d, tightened_budget, od, lse_d, visited_d, stream, &oc);
+      if (rc != COSA_OK) return rc;
+      if (!order_after(down, st)) return cuda_fail(e, "stream order");
+      if ((e = cudaMemcpyAsync(static_cast<char*>(out_host) + h * q_head, od, q_bytes, cudaMemcpyDeviceToHost, down)) != cudaSuccess)
+        return cuda_fail(e, "D2H out");
+      if (out_lse_host && (e = cudaMemcpyAsync(reinterpret_cast<char*>(out_lse_host) + h * lse_head, lse_d, step * lse_head,
+                                               cudaMemcpyDeviceToHost, down)) != cudaSuccess) return cuda_fail(e, "D2H lse");
+      if (out_visited_host && (e = cudaMemcpyAsync(reinterpret_cast<char*>(out_visited_host) + h * cnt_head, visited_d, step * cnt_head,
+                                                   cudaMemcpyDeviceToHost, down)) != cudaSuccess) return cuda_fail(e, "D2H visited");
+    }
   }
   if (!order_after(st, down)) return cuda_fail(e, "stream order");   // outputs are valid once `stream` is synchronised
   return COSA_OK;
