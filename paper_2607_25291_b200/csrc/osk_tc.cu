@@ -1,12 +1,11 @@
 // OSK on the sm_100a tensor cores (Sec. 4.3; Algorithm A steps 7-21; skip rule Eq. 5).
 //
-// One CTA per (query head, query block), two CTAs per SM.  The walk of one work item is a chain of dependent steps --
-// K tile -> S = Q K_j^T -> row maxima -> tile vote -> (exponentials -> O += P V_j) -> next block -- whose start (list
-// entries, Q and K tiles) and end (last product, epilogue) leave the SM idle altogether; two independent walks fill each
-// other's gaps, and the SM starts the next one the moment either ends.  An SM's resources are therefore halved: 256 columns
-// of tensor memory, 113 KB of shared memory and 32 K registers per CTA, eight warps:
+// Two CTAs per SM, each walking one work item -- a (query head, query block) -- after another.  The walk of a work item is a
+// chain of dependent steps -- K tile -> S = Q K_j^T -> row maxima -> tile vote -> (exponentials -> O += P V_j) -> next block
+// -- and two independent walks fill each other's gaps.  An SM's resources are therefore halved: 256 columns of tensor memory,
+// 113 KB of shared memory and 32 K registers per CTA, eight warps:
 //   warps 0..3   one thread per query row: S row to registers, row maximum, vote, exponentials, P, epilogue
-//   warp 4       K and V tiles ("physical jumping": only listed blocks are ever fetched)
+//   warp 4       work items; Q, K and V tiles ("physical jumping": only listed blocks are ever fetched)
 //   warp 5       issues the products
 //   warps 6, 7   idle (they give their registers to the first four)
 // The running row maxima live in the threads' registers, the tile vote of Eq. (5) is one barrier with an OR over the 128
@@ -21,11 +20,19 @@
 // Tiles: two slots X and Y.  When block k is decided, X holds K(k+1) and Y is free or holds the last V tile.  Skipped: K(k+2)
 // goes to Y, and the slots change roles.  Computed: V(k) goes to Y, each 64-key half as soon as the product on the half before
 // it has released it, and K(k+2) to X when Q K^T of k+1 is done.
+// Work items: the grid has one CTA per item, but a CTA that nears the end of its walk takes over one that has not been started
+// (clusterlaunchcontrol): the next walk's list, Q and K tiles are fetched during the last product, and its first S is there when
+// the rows have written the output.  With a CTA an item, start and end of a walk kept a CTA 11,000 cycles busy (barriers, tensor
+// memory, list, first tiles, output, next CTA), three computed blocks' worth.  Asked too early, the last items are dealt out badly:
+// at a walk's start, all blocks of 16K (walks of 1 to 128 blocks) take 3 % longer than when four positions are left.  What
+// runs once an item is cold in the instruction cache and costs by its size: code is shared rather than unrolled or inlined
+// twice wherever a walk passes once (26 KB more: 20 % slower than a CTA an item).
 // What bounds it: tensor pipe and exponentials both want about 1,024 cycles of an SM per computed block (512 per skipped one);
-// a computed position takes a CTA 4,000 cycles, a skipped one 1,220.  32 query heads, single launches: 7.2 ms at 128K tokens and
-// 4 % computed, 1.00 at 32K and 8 %, 1.84 for all blocks of 16K (one CTA of twelve warps per SM with two softmax groups and a
-// controller warp, the arrangement before: 8.05, 1.22 and 1.95).  Measured and not used: P over S in tensor memory (7.7 / 1.09 /
-// 2.08), two threads per row (8.2 / 1.15 / 2.12).
+// a computed position takes a CTA 4,000 cycles, a skipped one 1,220.  Single launches, a CTA an item -> now: 128K tokens and 4 %
+// computed 7.15 -> 7.07 ms, 32K and 8 % 1.02 -> 0.97, all blocks of 16K 1.85 -> 1.83, walks of 3.4 blocks (2 x 7,808 tokens)
+// 0.210 -> 0.186, 16,384 items of 4.2 blocks 1.03 -> 0.92 (32 query heads everywhere; one CTA of twelve warps per SM with two
+// softmax groups and a controller warp, the arrangement before both: 8.05, 1.22 and 1.95 on the first three).  Measured and not
+// used: P over S in tensor memory (7.9 / 1.11 / 2.26), two threads per row (8.2 / 1.15 / 2.12), tiles prefetched into L2 (+2 to 5 %).
 // Every wait is bounded; a wait that runs out sets the device status word and the CTA winds down without writing
 // results: load and issue warps leave, the row threads, whom no wait holds any more, run to the end of their list.
 #include <math.h>
@@ -49,34 +56,45 @@ constexpr int kThreads = 256;
 constexpr int kCtasPerSm = 2;
 constexpr int kTmemCols = 256;
 constexpr int kLoadWarp = 4, kMmaWarp = 5;
+constexpr int kAskAhead = 4;                       // positions (or two computed blocks) before a walk's end at which more work is asked for
 constexpr float kRescaleAbove = 8.f;               // (base 2) see the exponentials
 constexpr uint32_t kDecComputed = 1, kDecEnd = 2;
+constexpr int kTimedOut = 1, kPoisoned = 2;
 
-struct __align__(8) Control {
-  unsigned long long q_full;       // the Q tile has landed
+struct Item {                      // a work item as the load warp hands it to the others
+  int b, h, i;                     // batch item (< 0: there are no more), query head, query block
+  int cnt, cap;                    // listed blocks, computed blocks at which Stage 2 ends the walk
+  int q;                           // which Q tile it is
+  float theta2;                    // ln(Delta / N) in base 2
+};
+
+struct __align__(16) Control {
+  unsigned long long grant[2];     // the grid's answer to a request for another work item (16 bytes)
+  unsigned long long grant_bar;    // it has come
+  unsigned long long item_bar[2];  // the t-th work item (by parity of t) is in item[]
+  unsigned long long empty_done;   // rows and issuing thread are done with an item that has no blocks
+  unsigned long long q_full;       // the item's Q tile has landed
   unsigned long long k_full[2];    // K(k) has landed (by parity of k)
   unsigned long long v_full[2];    // by half: the n-th V tile's half has landed
   unsigned long long s_full;       // Q K^T of the position has finished
+  unsigned long long s_first;      // the same for the first position of a walk (a waiter may come when the second has finished, too)
   unsigned long long s_read;       // every row has taken its S to registers
   unsigned long long dec_bar[2];   // the decision of a position (by parity) is in dec[]
   unsigned long long p_full[2];    // by half: the n-th P's half is in shared memory
   unsigned long long pv_done[2];   // by half: the n-th product with that half has finished (one barrier each: a waiter may be
                                    // a whole block late, and one parity bit cannot tell two phases apart)
-  unsigned long long fin;          // every product of the walk has finished
+  unsigned long long fin;          // every product has finished
   uint32_t tmem_base;
-  int poisoned;
-  volatile int abort_flag;
-  volatile int req[4];             // tiles requested so far: K by parity, V by half (read when a walk was given up)
+  volatile int abort_flag;         // kTimedOut, kPoisoned
+  volatile int req[6];             // requested by the time the load warp left: K tiles by parity, V tiles by half, Q tiles, work items
+  volatile int diag[2];            // K(k) (by parity of k) is the diagonal block
   volatile uint32_t dec[2];
+  volatile Item item[2];
 };
 
 constexpr size_t kSmemBytes = (size_t)kTileBytes * 3 + kHalfBytes + sizeof(Control);
 static_assert(kSmemBytes + 1024 <= 233472 / 2, "shared memory budget of one of two CTAs");
 
-__device__ __forceinline__ void report_timeout(Control* c, int32_t* status) {
-  c->abort_flag = 1;
-  atomicMin(status, (int32_t)COSA_ERR_DEVICE_TIMEOUT);
-}
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   __nv_bfloat162 t = __floats2bfloat162_rn(a, b);
@@ -95,8 +113,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 template <bool kMask, bool kStage2, bool kSmallPages>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
-              const __grid_constant__ CUtensorMap v_map, const __grid_constant__ CUtensorMap o_map, OskParams p,
-              int32_t* status) {
+              const __grid_constant__ CUtensorMap v_map, OskParams p, int32_t* status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];   // swizzled tiles need 1024-byte alignment
   unsigned char* smem = smem_raw;
   const uint32_t base = smem_u32(smem_raw);
@@ -109,44 +126,37 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
   const uint32_t p_sm = base + 3 * kTileBytes;      // 64 keys of P
   Control* ctl = reinterpret_cast<Control*>(smem + (size_t)kTileBytes * 3 + kHalfBytes);
 
-  // work item: KV head major, then query blocks from the longest list down, the group's query
-  // heads innermost, so that CTAs resident together read the same K/V pages
-  const int G = p.hq / p.hkv;
-  const int per_kv = G * p.nqb;
-  const int w = blockIdx.x;
-  const int b = w / (p.hkv * per_kv);
-  const int wk = w % (p.hkv * per_kv);
-  const int g = wk / per_kv;
-  const int i = p.nqb - 1 - (wk % per_kv) / G;
-  const int h = g * G + (wk % per_kv) % G;
-  const size_t row = (size_t)(b * p.hq + h) * p.nqb + i;
-  chain_begin();
-  const int nqb_b = item_blocks(p.pg, b, p.nqb);   // the item's own length in blocks; query blocks past it are padding
-  const int J = p.causal ? i + 1 : max(nqb_b, 1);
-  const int32_t* list = p.order + row * p.order_stride;   // unused when kMask
-  BlockWalk walk;                         // (kMask only) every thread that needs block ids walks on its own
-  if (kMask) walk.init(p, row, J);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int G = p.hq / p.hkv;
+  chain_begin();
 
-  // the load warp's first list entries, requested before anything waits
-  int id0 = 0, id1 = 0;
-  int poisoned_early = 0;
-  if (warp == kLoadWarp) {
-    if (!kMask) {
-      id0 = list[0];
-      id1 = p.order_stride > 1 ? list[1] : 0;
-    }
-    poisoned_early = *reinterpret_cast<volatile int32_t*>(status);
-  }
-  const int cnt = i >= nqb_b ? 0 : (kMask ? min(walk.kept(), p.order_stride) : max(0, min(p.count[row], p.order_stride)));
-  const int cap = p.stage2 ? min(cnt, budget_count_fx(p.cap_fx, J)) : cnt;
+  // work items: KV head major, then query blocks from the longest list down, the group's query heads innermost, so that CTAs
+  // resident together read the same K/V pages
+  int b = 0, g = 0, h = 0, i = 0;          // (load warp) the item
+  auto decode = [&](int w) {
+    const int per_kv = G * p.nqb, bg = w / per_kv, wk = w - bg * per_kv, back = wk / G;
+    b = bg / p.hkv;
+    g = bg - b * p.hkv;
+    i = p.nqb - 1 - back;
+    h = g * G + wk - back * G;
+  };
+  // its count, its first two list entries and the status word, one in each of the first lanes
+  auto look_up = [&]() {
+    const size_t row = (size_t)(b * p.hq + h) * p.nqb + i;
+    int v = 0;
+    if (lane == 3) v = *reinterpret_cast<volatile int32_t*>(status);   // once some CTA has reported a timeout no further work is begun
+    else if (!kMask && lane == 0) v = p.count[row];
+    else if (!kMask && lane < 3 && lane <= p.order_stride) v = p.order[row * p.order_stride + lane - 1];
+    return v;
+  };
+  int head = 0;
+  if (warp == kLoadWarp) { decode(blockIdx.x); head = look_up(); }
 
   // (whole load warp) rows [first, first + rows) of key block j of K or V to dst, box after box: `box` bytes from one 64-column half
   // of d to the other.  Lane 0 arms the barrier; with small pages every lane then fetches one page's part
-  auto fetch = [&](const CUtensorMap* map, int q, unsigned long long* bar_ptr, int j, int first, int rows, uint32_t dst, uint32_t box) {
+  auto fetch = [&](const CUtensorMap* map, unsigned long long* bar_ptr, int j, int first, int rows, uint32_t dst, uint32_t box) {
     const uint32_t bar = smem_u32(bar_ptr);
     if (lane == 0) {
-      ctl->req[q] = ctl->req[q] + 1;
       mbar_expect_tx(bar, 2 * box);
       if (!kSmallPages) {                 // a page holds whole key blocks
         const KvCoord c = kv_coord(p.pg, b, g, j * kBlock + first);
@@ -164,41 +174,41 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       }
     }
   };
-  auto fetch_k = [&](int k, int j, int slot) { fetch(&k_map, k & 1, &ctl->k_full[k & 1], j, 0, kBlock, x_sm + slot * kTileBytes, kHalfBytes); };
+  auto fetch_k = [&](int k, int j, int slot) {
+    if (lane == 0) ctl->diag[k & 1] = p.causal && j == i;
+    fetch(&k_map, &ctl->k_full[k & 1], j, 0, kBlock, x_sm + slot * kTileBytes, kHalfBytes);
+  };
   auto fetch_v = [&](int half, int j, int slot) {
-    fetch(&v_map, 2 + half, &ctl->v_full[half], j, half * kHalfKeys, kHalfKeys, x_sm + slot * kTileBytes + half * kHalfBytes, kQuarterBytes);
+    fetch(&v_map, &ctl->v_full[half], j, half * kHalfKeys, kHalfKeys, x_sm + slot * kTileBytes + half * kHalfBytes, kQuarterBytes);
+  };
+  auto fetch_q = [&]() {                  // (one lane)
+    mbar_expect_tx(smem_u32(&ctl->q_full), kTileBytes);
+    tma_load_tile(q_sm, &q_map, 0, i * kBlock, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->q_full));
+    tma_load_tile(q_sm + kHalfBytes, &q_map, 64, i * kBlock, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->q_full));
   };
   auto clamp_id = [&](int j) { return min(max(j, 0), p.nqb - 1); };
 
   if (warp == kLoadWarp) {
     if (lane == 0) {
+      mbar_init(smem_u32(&ctl->grant_bar), 1); mbar_init(smem_u32(&ctl->empty_done), 2);
       mbar_init(smem_u32(&ctl->q_full), 1);
       for (int s = 0; s < 2; ++s) {
+        mbar_init(smem_u32(&ctl->item_bar[s]), 1);
         mbar_init(smem_u32(&ctl->k_full[s]), 1); mbar_init(smem_u32(&ctl->v_full[s]), 1);
         mbar_init(smem_u32(&ctl->dec_bar[s]), 1); mbar_init(smem_u32(&ctl->p_full[s]), kBlock);
         mbar_init(smem_u32(&ctl->pv_done[s]), 1);
       }
-      mbar_init(smem_u32(&ctl->s_full), 1); mbar_init(smem_u32(&ctl->s_read), kBlock);
+      mbar_init(smem_u32(&ctl->s_full), 1); mbar_init(smem_u32(&ctl->s_first), 1); mbar_init(smem_u32(&ctl->s_read), kBlock);
       mbar_init(smem_u32(&ctl->fin), 1);
       ctl->abort_flag = 0;
-      for (int q = 0; q < 4; ++q) ctl->req[q] = 0;
+      for (int q = 0; q < 6; ++q) ctl->req[q] = 0;
       mbar_fence_init();
       fence_proxy_async_smem();
-      // Q at once: its address needs nothing from global memory, while the list entries, the count and the status word
-      // requested above are still on their way
-      mbar_expect_tx(smem_u32(&ctl->q_full), kTileBytes);
-      tma_load_tile(q_sm, &q_map, 0, i * kBlock, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->q_full));
-      tma_load_tile(q_sm + kHalfBytes, &q_map, 64, i * kBlock, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->q_full));
-      ctl->poisoned = poisoned_early;    // once some CTA has reported a timeout the rest of the grid returns at once
+      // the first Q at once: its address needs nothing from global memory, while the list entries, the count and the status
+      // word requested above are still on their way
+      fetch_q();
     }
     __syncwarp();
-    poisoned_early = __shfl_sync(0xffffffffu, poisoned_early, 0);
-    if (poisoned_early == 0 && cnt > 0) {      // the first tiles, before the rest of the CTA has finished setting up
-      if (kMask) { id0 = walk.at(0); id1 = cnt > 1 ? walk.at(1) : 0; }
-      id0 = clamp_id(id0); id1 = clamp_id(id1);
-      fetch_k(0, id0, 0);
-      if (cap > 1) fetch_k(1, id1, 1);         // (the first block is always computed: with a cap of 1 the walk ends there)
-    }
   } else if (warp == kMmaWarp) {
     tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols);
     tmem_relinquish();
@@ -206,103 +216,184 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (ctl->poisoned != 0) {
-    if (warp == kMmaWarp) tmem_dealloc(ctl->tmem_base, kTmemCols);
-    if (threadIdx.x == 0) (void)mbar_wait_noabort(smem_u32(&ctl->q_full), 0);   // no copy may be in flight when the CTA retires
-    return;
-  }
   const uint32_t tmem_s = ctl->tmem_base, tmem_o = tmem_s + 128u;
   volatile int* abort_flag = &ctl->abort_flag;
   const long long budget = p.wait_budget;
-  const int n_pos = cap > 1 ? cnt : min(cnt, 1);   // positions the walk can reach
 
   if (warp >= kLoadWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     if (warp == kLoadWarp) {
-      // ---------------------------------------------------------------- K and V tiles
+      // ---------------------------------------------------------------- work items, tiles
+      // Counters run on from walk to walk, as the barriers' phases do: tiles K(k), positions decided, blocks computed before
+      // this walk.  All roles count alike.
       // (one answer per warp: all lanes fetch together)
       auto wait = [&](unsigned long long* bar, int phase) { return mbar_wait_warp(smem_u32(bar), phase & 1, abort_flag, budget, true); };
-      bool alive = n_pos > 0;
-      int j0 = id0, j1 = id1, j2 = 0;          // key blocks of positions k, k + 1 and, requested a turn ahead, k + 2
-      if (!kMask && n_pos > 2) j2 = list[2];
+      // Further items come from the grid itself, in launch order, as long as CTAs of it are waiting for an SM.  (A grid that fits
+      // on the chip asks for none: a CTA might take what an SM is about to start)
+      const bool ask = (int)gridDim.x > p.wave;
+      BlockWalk walk;                          // (kMask only)
+      int n_q = 1, n_k = 0, n_v = 0, n_grant = 0;   // requested (Q: the first above)
+      int n_walk = 0, n_empty = 0;             // items with and without blocks
       int y = 0;                               // slot that takes the next V tile (or K tile after a skipped block)
-      int n = 0;                               // computed blocks before position k
-      bool v_in_y = false;                     // slot y holds, or held last, the V tile of block n - 1
-      for (int k = 0; alive && k < n_pos; ++k) {
-        if (kMask && k + 2 < n_pos) j2 = walk.at(k + 2);
-        uint32_t d = kDecComputed | (k == cnt - 1 ? kDecEnd : 0u);
-        if (k == 0) {
-          // (never satisfied on the spot: a wait budget of a few cycles always runs out here)
-          alive = mbar_poll_warp(smem_u32(kStage2 ? &ctl->dec_bar[0] : &ctl->s_full), 0, abort_flag, budget);
-        } else if (kStage2) {
-          alive = wait(&ctl->dec_bar[k & 1], k >> 1);
+      bool v_in_y = false;                     // slot y holds, or held last, the V tile of the last computed block
+      int k_base = 0, pos_base = 0, n_base = 0;
+      int b_known = -1, nqb_b = 0;             // batch item of the lengths below
+      float theta2 = 0.f;
+      bool alive = true, more = true;
+      for (int t = 0; alive; ++t) {
+        const int raw_cnt = __shfl_sync(0xffffffffu, head, 0);
+        // key blocks of positions k, k + 1 and k + 2 (the last one requested a turn ahead), k starting at -2
+        int j0 = 0, j1 = 0, j2 = __shfl_sync(0xffffffffu, head, 1), j3 = __shfl_sync(0xffffffffu, head, 2);
+        if (__shfl_sync(0xffffffffu, head, 3) != 0) {
+          more = false;
+          if (t == 0) *abort_flag = kPoisoned; // (Q has been requested for nothing)
         }
-        if (kStage2 && alive) d = ctl->dec[k & 1];
-        if (alive && (d & kDecComputed)) {
-          for (int half = 0; half < 2 && alive; ++half) {
-            if (v_in_y) alive = wait(&ctl->pv_done[half], n - 1);
-            if (alive) fetch_v(half, clamp_id(j0), y);
+        int cnt = 0, cap = 0, n_pos = 0;
+        if (more) {
+          if (b != b_known) {
+            b_known = b;
+            nqb_b = item_blocks(p.pg, b, p.nqb);   // the item's own length in blocks; query blocks past it are padding
+            theta2 = (p.use_threshold ? item_theta(p.pg, b, p.theta, p.skip_scale, nqb_b) : 0.f) * 1.4426950408889634f;
           }
-          if (!(d & kDecEnd) && k + 2 < n_pos && alive) {
-            alive = wait(&ctl->s_full, k + 1);
-            if (alive) fetch_k(k + 2, clamp_id(j2), y ^ 1);
+          const int J = p.causal ? i + 1 : max(nqb_b, 1);
+          if (kMask) walk.init(p, (size_t)(b * p.hq + h) * p.nqb + i, J);
+          cnt = i >= nqb_b ? 0 : (kMask ? min(walk.kept(), p.order_stride) : max(0, min(raw_cnt, p.order_stride)));
+          cap = p.stage2 ? min(cnt, budget_count_fx(p.cap_fx, J)) : cnt;
+          n_pos = cap > 1 ? cnt : min(cnt, 1);  // positions the walk can reach (the first block is always computed: with a cap of 1 the walk ends there)
+          if (kMask && cnt > 0) { j2 = walk.at(0); j3 = cnt > 1 ? walk.at(1) : 0; }
+          if (n_pos > 0 && t > 0) {             // Q's tile and slot y are free when the last Q K^T of the walk before has finished
+            if (k_base > 0) alive = wait(&ctl->s_full, k_base - 1);
+            if (!alive) break;
+            if (lane == 0) fetch_q();
+            ++n_q;
           }
-          v_in_y = true;
-          ++n;
-        } else if (alive && !(d & kDecEnd)) {
-          if (k + 2 < n_pos) {
-            if (v_in_y) alive = wait(&ctl->pv_done[1], n - 1);
-            if (alive) fetch_k(k + 2, clamp_id(j2), y);
+        }
+        if (lane == 0) {
+          volatile Item* it = &ctl->item[t & 1];
+          it->b = more ? b : -1; it->h = h; it->i = i; it->cnt = cnt; it->cap = cap; it->q = n_q - 1; it->theta2 = theta2;
+          mbar_arrive(smem_u32(&ctl->item_bar[t & 1]));
+        }
+        if (!more) break;
+        bool asked = !ask;
+        auto request = [&]() {
+          asked = true;
+          ++n_grant;
+          if (lane == 0) {
+            fence_proxy_async_smem();
+            mbar_expect_tx(smem_u32(&ctl->grant_bar), 16);
+            request_work(smem_u32(ctl->grant), smem_u32(&ctl->grant_bar));
           }
+        };
+        if (n_pos == 0) {
+          if (t == 0) alive = wait(&ctl->q_full, 0);          // (requested before the count was known)
+          if (alive) alive = wait(&ctl->empty_done, n_empty++);
+        } else {
+          const int32_t* list = p.order + ((size_t)(b * p.hq + h) * p.nqb + i) * p.order_stride;   // unused when kMask
+          // Turn k fetches V(k) and K(k + 2); turns -2 and -1: the first two K tiles, K(1) to the slot of the last V tile of the walk
+          // before
+          int k = -2, n = 0;                    // n: computed blocks before position k
+          const bool v_before = v_in_y;
           v_in_y = false;
-          y ^= 1;
+          while (true) {
+            uint32_t d = 0;
+            if (k >= 0) {
+              d = kDecComputed | (k == cnt - 1 ? kDecEnd : 0u);
+              if (k == 0 && t == 0) {
+                // (never satisfied on the spot: a wait budget of a few cycles always runs out here)
+                alive = mbar_poll_warp(smem_u32(kStage2 ? &ctl->dec_bar[0] : &ctl->s_first), 0, abort_flag, budget);
+              } else if (kStage2) {
+                alive = wait(&ctl->dec_bar[(pos_base + k) & 1], (pos_base + k) >> 1);
+              } else if (k == 0) {
+                alive = wait(&ctl->s_first, n_walk);
+              }
+              if (kStage2) d = ctl->dec[(pos_base + k) & 1];
+              if (d & kDecComputed) {
+#pragma unroll 1
+                for (int half = 0; half < 2 && alive; ++half) {
+                  if (v_in_y) alive = wait(&ctl->pv_done[half], n_base + n - 1);
+                  if (alive) { fetch_v(half, clamp_id(j0), y); ++n_v; }
+                }
+              }
+            }
+            const bool computed = (d & kDecComputed) != 0;
+            if (alive && !(d & kDecEnd) && k + 2 < n_pos) {
+              if (computed) alive = wait(&ctl->s_full, k_base + k + 1);
+              else if (k == -1 ? v_before : v_in_y) alive = wait(&ctl->pv_done[1], n_base + n - 1);
+              if (alive) { fetch_k(k_base + k + 2, clamp_id(j2), computed || k == -1 ? y ^ 1 : y); ++n_k; }
+            }
+            if (!alive) break;
+            if (!asked && (k + kAskAhead >= n_pos || n + 2 >= cap)) request();
+            if (computed) { v_in_y = true; ++n; }
+            if (d & kDecEnd) break;
+            if (k >= 0 && !computed) { v_in_y = false; y ^= 1; }
+            j0 = j1; j1 = j2; j2 = j3;
+            if (k + 4 < n_pos) j3 = kMask ? walk.at(k + 4) : list[k + 4];
+            ++k;
+          }
+          k_base += min(k + 2, n_pos); pos_base += k + 1; n_base += n;
+          ++n_walk;
+          y ^= 1;                               // (v_in_y: of the slot that is y ^ 1 from here on)
         }
-        if (!alive) { if (lane == 0 && !*abort_flag) report_timeout(ctl, status); break; }
-        if (d & kDecEnd) break;
-        j0 = j1; j1 = j2;
-        if (!kMask && k + 3 < n_pos) j2 = list[k + 3];
+        if (alive) {
+          more = false;
+          if (ask) {
+            if (!asked) request();
+            alive = wait(&ctl->grant_bar, n_grant - 1);
+            const int w2 = granted_work(smem_u32(ctl->grant));
+            more = alive && w2 >= 0;
+            head = 0;
+            if (more) { decode(w2); head = look_up(); }
+          }
+        }
+      }
+      if (lane == 0) {
+        if (!alive && !*abort_flag) *abort_flag = kTimedOut;
+        ctl->req[0] = (n_k + 1) / 2; ctl->req[1] = n_k / 2; ctl->req[2] = (n_v + 1) / 2; ctl->req[3] = n_v / 2; ctl->req[4] = n_q; ctl->req[5] = n_grant;
       }
     } else if (warp == kMmaWarp && lane == 0) {
-      // The count and the head of the list of the work item one wave of CTAs further on: the tiles streamed since KAP
-      // wrote them have pushed these lines out of L2, and that CTA's first loads would wait for HBM
-      if (!kMask && w + (int)p.wave < (int)gridDim.x) {
-        const int w2 = w + (int)p.wave;
-        const int b2 = w2 / (p.hkv * per_kv), wk2 = w2 % (p.hkv * per_kv);
-        const int g2 = wk2 / per_kv, i2 = p.nqb - 1 - (wk2 % per_kv) / G, h2 = g2 * G + (wk2 % per_kv) % G;
-        const size_t row2 = (size_t)(b2 * p.hq + h2) * p.nqb + i2;
-        prefetch_l2(p.order + row2 * p.order_stride);
-        prefetch_l2(p.count + row2);
-      }
       // ---------------------------------------------------------------- products
-      if (n_pos > 0) {
-        auto wait = [&](unsigned long long* bar, int phase) { return mbar_wait(smem_u32(bar), phase & 1, abort_flag, budget); };
-        const uint32_t idesc_qk = idesc_bf16(kBlock, kBlock, 0, 0);    // Q [M x K], K_j [N x K], both K-major
-        const uint32_t idesc_pv = idesc_bf16(kBlock, kHeadDim, 0, 1);  // P [M x K] K-major, V_j [K x N] N-major
-        const uint64_t qdesc = smem_desc_sw128(q_sm, 16, 1024), kdesc0 = smem_desc_sw128(x_sm, 16, 1024);
-        const uint64_t pdesc = smem_desc_sw128(p_sm, 16, 1024), vdesc0 = smem_desc_sw128(x_sm, kQuarterBytes, 1024);
-        auto issue_qk = [&](int k, int slot) {      // S = Q K^T of position k
-          if (!wait(&ctl->k_full[k & 1], k >> 1)) return false;
-          tc_fence_after();
-          mma_ss_x8<2, 4, 6, kHalfBytes / 16, kHalfBytes / 16 + 2, kHalfBytes / 16 + 4, kHalfBytes / 16 + 6>(
-              tmem_s, qdesc, kdesc0 + (uint64_t)(slot * (kTileBytes / 16)), idesc_qk);
-          mma_commit(smem_u32(&ctl->s_full));
-          return true;
-        };
-        bool alive = wait(&ctl->q_full, 0) && issue_qk(0, 0);
-        int y = 0, n = 0;                           // as in the load warp
-        for (int k = 0; alive && k < n_pos; ++k) {
-          alive = wait(&ctl->s_read, k);
-          if (alive && k + 1 < n_pos) alive = issue_qk(k + 1, y ^ 1);
+      auto wait = [&](unsigned long long* bar, int phase) { return mbar_wait(smem_u32(bar), phase & 1, abort_flag, budget); };
+      const uint32_t idesc_qk = idesc_bf16(kBlock, kBlock, 0, 0);    // Q [M x K], K_j [N x K], both K-major
+      const uint32_t idesc_pv = idesc_bf16(kBlock, kHeadDim, 0, 1);  // P [M x K] K-major, V_j [K x N] N-major
+      const uint64_t qdesc = smem_desc_sw128(q_sm, 16, 1024), kdesc0 = smem_desc_sw128(x_sm, 16, 1024);
+      const uint64_t pdesc = smem_desc_sw128(p_sm, 16, 1024), vdesc0 = smem_desc_sw128(x_sm, kQuarterBytes, 1024);
+      auto issue_qk = [&](int k, int slot) {      // S = Q K^T with the k-th K tile
+        if (!wait(&ctl->k_full[k & 1], k >> 1)) return false;
+        tc_fence_after();
+        mma_ss_x8<2, 4, 6, kHalfBytes / 16, kHalfBytes / 16 + 2, kHalfBytes / 16 + 4, kHalfBytes / 16 + 6>(
+            tmem_s, qdesc, kdesc0 + (uint64_t)(slot * (kTileBytes / 16)), idesc_qk);
+        mma_commit(smem_u32(&ctl->s_full));
+        return true;
+      };
+      int y = 0, k_base = 0, pos_base = 0, n_base = 0;   // as in the load warp
+      bool alive = true;
+      for (int t = 0;; ++t) {
+        alive = wait(&ctl->item_bar[t & 1], t >> 1);
+        if (!alive) break;
+        volatile Item* it = &ctl->item[t & 1];
+        const int cnt = it->cnt, n_pos = it->cap > 1 ? cnt : min(cnt, 1);
+        if (it->b < 0) break;
+        if (n_pos == 0) { mbar_arrive(smem_u32(&ctl->empty_done)); continue; }
+        alive = wait(&ctl->q_full, it->q);
+        int k = -1, n = 0;
+        while (alive) {
+          if (k >= 0) alive = wait(&ctl->s_read, pos_base + k);
+          if (alive && k + 1 < n_pos) alive = issue_qk(k_base + k + 1, k < 0 ? y : y ^ 1);
+          if (k < 0) {
+            if (!kStage2 && alive) mma_commit(smem_u32(&ctl->s_first));
+            ++k;
+            continue;
+          }
           uint32_t d = kDecComputed | (k == cnt - 1 ? kDecEnd : 0u);
           if (kStage2 && alive) {
-            alive = wait(&ctl->dec_bar[k & 1], k >> 1);
-            d = ctl->dec[k & 1];
+            alive = wait(&ctl->dec_bar[(pos_base + k) & 1], (pos_base + k) >> 1);
+            d = ctl->dec[(pos_base + k) & 1];
           }
           if (!alive) break;
           if (d & kDecComputed) {
 #pragma unroll 1
             for (int half = 0; half < 2 && alive; ++half) {
-              alive = wait(&ctl->v_full[half], n) && wait(&ctl->p_full[half], n);
+              alive = wait(&ctl->v_full[half], n_base + n) && wait(&ctl->p_full[half], n_base + n);
               if (!alive) break;
               tc_fence_after();
               // 16 keys per MMA: 32 bytes of a P row, 2 KiB (two 8-key groups) of the V half
@@ -311,63 +402,71 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
               mma_commit(smem_u32(&ctl->pv_done[half]));
             }
             ++n;
-          } else {
+          } else if (!(d & kDecEnd)) {
             y ^= 1;
           }
           if (d & kDecEnd) break;
+          ++k;
         }
-        if (!alive && !*abort_flag) report_timeout(ctl, status);
-        mma_commit(smem_u32(&ctl->fin));            // also after a walk that was given up: tensor memory is released behind it
+        if (!alive) break;
+        k_base += min(k + 2, n_pos); pos_base += k + 1; n_base += n;
+        y ^= 1;
       }
+      if (!alive && !*abort_flag) *abort_flag = kTimedOut;
+      mma_commit(smem_u32(&ctl->fin));                // also after a walk that was given up: tensor memory is released behind it
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
+    // ------------------------------------------------------------------ one thread per query row
     const int r = threadIdx.x;                // query row inside the tile
-    const size_t lse_at = (size_t)(b * p.hq + h) * p.n + i * kBlock + r;
-    if (cnt == 0) {
-      // an empty list (not produced by KAP except for padding): zero output, nothing visited
-      uint4 z = make_uint4(0, 0, 0, 0);
-      uint4* dst = reinterpret_cast<uint4*>(p.out + elem_off(p.os, b, h, i * kBlock + r));
-      for (int c = 0; c < kHeadDim / 8; ++c) dst[c] = z;
-      if (p.lse) p.lse[lse_at] = -INFINITY;
-      if (r == 0) {
-        if (p.visited) p.visited[row] = 0;
-        if (p.scored) p.scored[row] = 0;
-        (void)mbar_wait_noabort(smem_u32(&ctl->q_full), 0);   // the Q tile was requested all the same
+    const uint32_t lane_addr = (uint32_t)(warp * 32) << 16;
+    const float scale2 = p.scale * 1.4426950408889634f;   // work in base 2: exp(x) = exp2(x * log2 e)
+    const int dec_words = (p.order_stride + 31) / 32;
+    bool bad = false;                         // a wait of this thread ran out
+    auto wait = [&](unsigned long long* bar, int phase) {
+      if (!mbar_wait(smem_u32(bar), phase & 1, abort_flag, budget)) {
+        bad = true;
+        if (!*abort_flag) *abort_flag = kTimedOut;
       }
-    } else {
-      // -------------------------------------------------------------- one thread per query row
-      const uint32_t lane_addr = (uint32_t)(warp * 32) << 16;
-      const float kLog2e = 1.4426950408889634f;
-      const float scale2 = p.scale * kLog2e;    // work in base 2: exp(x) = exp2(x * log2 e)
-      const float theta2 = (p.use_threshold ? item_theta(p.pg, b, p.theta, p.skip_scale, nqb_b) : 0.f) * kLog2e;
+    };
+    int k_base = 0, pos_base = 0, n_base = 0; // as in the load warp
+    for (int t = 0;; ++t) {
+      wait(&ctl->item_bar[t & 1], t >> 1);
+      if (bar_red_or(1, kBlock, bad || *abort_flag)) break;
+      volatile Item* it = &ctl->item[t & 1];
+      const int b = it->b, h = it->h, i = it->i, cnt = it->cnt, cap = it->cap;
+      const float theta2 = it->theta2;
+      if (b < 0) break;
+      const size_t row = (size_t)(b * p.hq + h) * p.nqb + i;
+      const size_t lse_at = (size_t)(b * p.hq + h) * p.n + i * kBlock + r;
+      if (cnt == 0) {
+        // an empty list (not produced by KAP except for padding): zero output, nothing visited
+        uint4 z = make_uint4(0, 0, 0, 0);
+        uint4* dst = reinterpret_cast<uint4*>(p.out + elem_off(p.os, b, h, i * kBlock + r));
+#pragma unroll 1
+        for (int c = 0; c < kHeadDim / 8; ++c) dst[c] = z;
+        if (p.lse) p.lse[lse_at] = -INFINITY;
+        if (r == 0) {
+          if (p.visited) p.visited[row] = 0;
+          if (p.scored) p.scored[row] = 0;
+          mbar_arrive(smem_u32(&ctl->empty_done));
+        }
+        continue;
+      }
       // a batch item no longer than Delta would have ln(Delta/N) >= 0 and lose even its first block: the test is off for it
       const bool thr_on = p.use_threshold && theta2 < 0.f;
       float m = -INFINITY, m_ref = -INFINITY;   // running row maximum (base 2); the one the exponentials refer to
       float l = 0.f;                            // row sum
       int n = 0, kk = 0;                        // computed blocks, list position
       uint32_t dec_word = 0;
-      const int dec_words = (p.order_stride + 31) / 32;
-      bool bad = false;                         // a wait of this thread ran out
-      auto wait = [&](unsigned long long* bar, int phase) {
-        if (!mbar_wait(smem_u32(bar), phase & 1, abort_flag, budget)) {
-          bad = true;
-          if (!*abort_flag) report_timeout(ctl, status);
-        }
-      };
       uint32_t s[kBlock];                       // this row's raw logits, then probabilities
-      // rows only ask whether a position's block is the diagonal one, which an ascending mask walk meets last, if at all: a warp
-      // looks at 32 list entries at a time
-      const bool mask_diag = kMask && ((walk.mask[i >> 5] >> (i & 31)) & 1u);
-      uint32_t diag_bits = 0;
       for (;; ++kk) {
-        if (!kMask && p.causal && (kk & 31) == 0) diag_bits = __ballot_sync(0xffffffffu, kk + lane < cnt && list[kk + lane] == i);
-        const bool diag = kMask ? p.causal && mask_diag && kk == cnt - 1 : ((diag_bits >> (kk & 31)) & 1u) != 0;
-        wait(&ctl->s_full, kk);
+        wait(&ctl->s_full, k_base + kk);
         __syncwarp();
         tc_fence_after();
 #pragma unroll
         for (int c = 0; c < 4; ++c) tmem_ld32(tmem_s + lane_addr + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
+        const bool diag = ctl->diag[(k_base + kk) & 1] != 0;
         tmem_wait_ld();
         tc_fence_before();
         mbar_arrive(smem_u32(&ctl->s_read));
@@ -391,8 +490,8 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
           const bool compute = bar_red_or(1, kBlock, !(thr_on && (m_loc - m_new) < theta2));
           last = last || n + (compute ? 1 : 0) == cap;
           if (r == 0) {
-            ctl->dec[kk & 1] = (compute ? kDecComputed : 0u) | (last ? kDecEnd : 0u);
-            mbar_arrive(smem_u32(&ctl->dec_bar[kk & 1]));
+            ctl->dec[(pos_base + kk) & 1] = (compute ? kDecComputed : 0u) | (last ? kDecEnd : 0u);
+            mbar_arrive(smem_u32(&ctl->dec_bar[(pos_base + kk) & 1]));
             if (compute) dec_word |= 1u << (kk & 31);
             if (p.decisions && ((kk & 31) == 31 || last)) { p.decisions[row * dec_words + (kk >> 5)] = dec_word; dec_word = 0; }
           }
@@ -410,7 +509,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
           m_ref = m;
         }
         if (n > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {   // O = diag(alpha) O
-          wait(&ctl->pv_done[1], n - 1);
+          wait(&ctl->pv_done[1], n_base + n - 1);
           __syncwarp();
           tc_fence_after();
 #pragma unroll 1
@@ -433,9 +532,9 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         for (int half = 0; half < 2; ++half) {
           // the buffer's last reader: the second half of the block before, the first half of this one (asked now, needed
           // after the exponentials)
-          const int last_n = n - 1 + half;
+          const int last_n = n_base + n - 1 + half;
           unsigned long long* last_reader = &ctl->pv_done[half ^ 1];
-          const bool is_free = last_n < 0 || mbar_test_wait(smem_u32(last_reader), last_n & 1);
+          const bool is_free = n + half == 0 || mbar_test_wait(smem_u32(last_reader), last_n & 1);
 #pragma unroll
           for (int c = half * kHalfKeys; c < (half + 1) * kHalfKeys; c += 4) {
             float e0, e1, e2, e3;
@@ -465,65 +564,79 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         ++n;
         if (last) break;
       }
-      // ---- epilogue: the last product, then O / l as bf16 through shared memory (Q's tile is done with)
-      wait(&ctl->fin, 0);
-      __syncwarp();
-      if (!bar_red_or(1, kBlock, bad || *abort_flag)) {
-        tc_fence_after();
-        const float inv = l > 0.f ? 1.f / l : 0.f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) tmem_ld32(tmem_o + lane_addr + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
+      // ---- epilogue: the last product, then O / l as bf16.  The next walk's Q and K tiles are on their way meanwhile; the rows
+      // of a warp go out through the warp's own rows of P, 64 columns at a time, so that a store covers whole 128-byte lines
+      // and no warp waits for another
+      n_base += n;
+      wait(&ctl->pv_done[1], n_base - 1);
+      const int n_pos = cap > 1 ? cnt : 1, n_issued = min(kk + 2, n_pos);   // (Q K^T of a position that was not reached: done, too)
+      k_base += n_issued; pos_base += kk + 1;
+      if (bar_red_or(1, kBlock, bad || *abort_flag)) break;
+      tc_fence_after();
+      const float inv = l > 0.f ? 1.f / l : 0.f;
+      unsigned char* stage = smem + 3 * kTileBytes + warp * 4096;
+      __nv_bfloat16* out = p.out + elem_off(p.os, b, h, i * kBlock + warp * 32 + (lane >> 3)) + (lane & 7) * 8;
+      const long long out_step = elem_off(p.os, b, h, 4) - elem_off(p.os, b, h, 0);
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {
+        uint32_t o[64];
+        tmem_ld32(tmem_o + lane_addr + half * 64, *reinterpret_cast<uint32_t(*)[32]>(&o[0]));
+        tmem_ld32(tmem_o + lane_addr + half * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&o[32]));
         tmem_wait_ld();
-        unsigned char* stage = smem + r * 128;
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
+        for (int c = 0; c < 8; ++c) {
+          const uint32_t* e = &o[c * 8];
           uint4 pk;
-          pk.x = pack_bf16(__uint_as_float(s[8 * c + 0]) * inv, __uint_as_float(s[8 * c + 1]) * inv);
-          pk.y = pack_bf16(__uint_as_float(s[8 * c + 2]) * inv, __uint_as_float(s[8 * c + 3]) * inv);
-          pk.z = pack_bf16(__uint_as_float(s[8 * c + 4]) * inv, __uint_as_float(s[8 * c + 5]) * inv);
-          pk.w = pack_bf16(__uint_as_float(s[8 * c + 6]) * inv, __uint_as_float(s[8 * c + 7]) * inv);
-          *reinterpret_cast<uint4*>(stage + (c >> 3) * kHalfBytes + (((c & 7) ^ (r & 7)) << 4)) = pk;
+          pk.x = pack_bf16(__uint_as_float(e[0]) * inv, __uint_as_float(e[1]) * inv);
+          pk.y = pack_bf16(__uint_as_float(e[2]) * inv, __uint_as_float(e[3]) * inv);
+          pk.z = pack_bf16(__uint_as_float(e[4]) * inv, __uint_as_float(e[5]) * inv);
+          pk.w = pack_bf16(__uint_as_float(e[6]) * inv, __uint_as_float(e[7]) * inv);
+          *reinterpret_cast<uint4*>(stage + lane * 128 + ((c ^ (lane & 7)) << 4)) = pk;
         }
-        fence_proxy_async_smem();
-        bar_sync(1, kBlock);
-        if (r == 0) {
-          tma_store_tile(&o_map, 0, i * kBlock, h, b, p.oo.row, p.oo.head, p.oo.outer, q_sm);
-          tma_store_tile(&o_map, 64, i * kBlock, h, b, p.oo.row, p.oo.head, p.oo.outer, q_sm + kHalfBytes);
+        __syncwarp();
+#pragma unroll 4
+        for (int c = 0; c < 8; ++c) {         // four rows, eight lanes a row
+          const int rr = c * 4 + (lane >> 3);
+          *reinterpret_cast<uint4*>(out + c * out_step + half * 64) =
+              *reinterpret_cast<const uint4*>(stage + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
         }
-        if (p.lse) p.lse[lse_at] = (m_ref + log2f(l)) * 0.6931471805599453f;
-        if (r == 32) {
-          if (p.visited) p.visited[row] = n;
-          if (p.scored) p.scored[row] = kk + 1;
-          if (!kStage2 && p.decisions)
-            for (int wd = 0; wd * 32 < cnt; ++wd) p.decisions[row * dec_words + wd] = cnt - wd * 32 >= 32 ? 0xffffffffu : ((1u << (cnt - wd * 32)) - 1u);
-        }
-        if (r == 0) tma_store_commit_and_wait_read();
+        __syncwarp();
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (p.lse) p.lse[lse_at] = (m_ref + log2f(l)) * 0.6931471805599453f;
+      if (r == 32) {
+        if (p.visited) p.visited[row] = n;
+        if (p.scored) p.scored[row] = kk + 1;
+        if (!kStage2 && p.decisions)
+          for (int wd = 0; wd * 32 < cnt; ++wd) p.decisions[row * dec_words + wd] = cnt - wd * 32 >= 32 ? 0xffffffffu : ((1u << (cnt - wd * 32)) - 1u);
       }
     }
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && cnt > 0 && *abort_flag) {
+  if (*abort_flag) {
     // A walk that was given up: products and copies in flight finish on their own and must have done so before the CTA
     // retires.  (Otherwise everything fetched has been waited for: Q K^T of the position after the last takes its tile, too.)
-    (void)mbar_wait_noabort(smem_u32(&ctl->fin), 0);
-    (void)mbar_wait_noabort(smem_u32(&ctl->q_full), 0);
-    for (int q = 0; q < 4; ++q) {
-      const int c = ctl->req[q];
-      if (c > 0) (void)mbar_wait_noabort(smem_u32(q < 2 ? &ctl->k_full[q] : &ctl->v_full[q - 2]), (c - 1) & 1);
+    if (threadIdx.x == 0) {
+      if (*abort_flag == kTimedOut) atomicMin(status, (int32_t)COSA_ERR_DEVICE_TIMEOUT);
+#pragma unroll 1
+      for (int q = 0; q < 6; ++q) {
+        unsigned long long* bar = q < 2 ? &ctl->k_full[q] : (q < 4 ? &ctl->v_full[q - 2] : (q == 4 ? &ctl->q_full : &ctl->grant_bar));
+        const int c = ctl->req[q];
+        if (c > 0) (void)mbar_wait_noabort(smem_u32(bar), (c - 1) & 1);
+      }
+      (void)mbar_wait_noabort(smem_u32(&ctl->fin), 0);
     }
+    __syncthreads();
   }
-  if (warp == kMmaWarp) {
-    if (cnt > 0 && *abort_flag) (void)mbar_wait_noabort(smem_u32(&ctl->fin), 0);   // before tensor memory goes
-    __syncwarp();
-    tmem_dealloc(tmem_s, kTmemCols);
-  }
+  if (warp == kMmaWarp) tmem_dealloc(tmem_s, kTmemCols);
 }
 
 }  // namespace
 
 cudaError_t launch_osk_tc(const OskParams& p_in, cudaStream_t st) {
-  CUtensorMap qm, km, vm, om;
+  CUtensorMap qm, km, vm;
   OskParams p = p_in;
   TileOrder vo;
   // K and V: the dense tensors, or page pools whose pages hold whole key blocks
@@ -532,8 +645,7 @@ cudaError_t launch_osk_tc(const OskParams& p_in, cudaStream_t st) {
   const int v_box = k_box < kHalfKeys ? k_box : kHalfKeys;
   if (!make_tile_map(&qm, &p.qo, p.q, (uint64_t)p.n, (uint64_t)p.hq, (uint64_t)p.batch, p.qs) ||
       !make_kv_map(&km, &p.ko, p.k, p.pg, p.ks, p.batch, p.hkv, p.n, k_box) ||
-      !make_kv_map(&vm, &vo, p.v, p.pg, p.ks, p.batch, p.hkv, p.n, v_box) ||
-      !make_tile_map(&om, &p.oo, p.out, (uint64_t)p.n, (uint64_t)p.hq, (uint64_t)p.batch, p.os))
+      !make_kv_map(&vm, &vo, p.v, p.pg, p.ks, p.batch, p.hkv, p.n, v_box))
     return cudaErrorInvalidValue;
   const bool small_pages = p.pg.table && p.pg.page_size < kBlock;
   auto pick = [&](auto mask_c) {
@@ -553,8 +665,8 @@ cudaError_t launch_osk_tc(const OskParams& p_in, cudaStream_t st) {
   int32_t* status = device_status_word();
   if (!status) return cudaErrorInvalidSymbol;
   const int n_sm = device_sm_count();
-  p.wave = n_sm > 0 ? kCtasPerSm * n_sm : 1 << 30;   // (no prefetch if the SM count cannot be read)
-  return launch_chained(kernel, dim3(p.batch * p.hq * p.nqb), kThreads, kSmemBytes, st, qm, km, vm, om, p, status);
+  p.wave = n_sm > 0 ? kCtasPerSm * n_sm : 1 << 30;   // (a CTA an item if the SM count cannot be read)
+  return launch_chained(kernel, dim3(p.batch * p.hq * p.nqb), kThreads, kSmemBytes, st, qm, km, vm, p, status);
 }
 
 }  // namespace cosa

@@ -67,12 +67,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // The same without the abort flag: for copies and products already in flight, which complete on their own and must have
 // done so before the CTA retires (its shared and tensor memory go to the next CTA)
 __device__ __forceinline__ bool mbar_wait_noabort(uint32_t bar, uint32_t parity, long long budget = (1LL << 31)) {
-  if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
-  while (true) {
-    if (mbar_try_wait(bar, parity)) return true;
+  while (!mbar_try_wait(bar, parity))
     if (clock64() - t0 > budget) return false;
-  }
+  return true;
 }
 // For code all 32 lanes of a warp run together: the same bounded wait, with one answer for the whole warp when
 // `unanimous` is set.  Lanes poll on their own (the cheapest way to wait), so they can see the budget run out at
@@ -166,7 +164,6 @@ __device__ __forceinline__ void tma_store_commit_and_wait_read() {
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
   asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
-__device__ __forceinline__ void prefetch_l2(const void* ptr) { asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr)); }
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
@@ -218,6 +215,28 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
       "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
       "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
+}
+
+// ---------------------------------------------------------------- work from the grid
+// Asks for the index of a CTA of this grid that has not been started, which then never will be: the caller does its work.
+// The 16-byte answer (16-byte aligned) completes 16 bytes on the mbarrier.  Not to be asked again after a refusal.
+__device__ __forceinline__ void request_work(uint32_t answer, uint32_t bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer), "r"(bar)
+               : "memory");
+}
+// blockIdx.x of that CTA, -1 if there was none
+__device__ __forceinline__ int granted_work(uint32_t answer) {
+  int x;
+  asm volatile(
+      "{\n\t.reg .b128 a;\n\t.reg .pred p;\n\t"
+      "ld.shared.b128 a, [%1];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n\t"
+      "mov.b32 %0, -1;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, a;\n\t}"
+      : "=r"(x)
+      : "r"(answer)
+      : "memory");
+  return x;
 }
 
 // ---------------------------------------------------------------- MMA

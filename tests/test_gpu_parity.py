@@ -502,6 +502,51 @@ def test_osk_short_walks_with_growing_maxima(small, length, tb, skip_scale):
     check_osk_against_oracle(qf, kf2, vf, order[0], count[0], bufs, tb, skip_scale, range(hq), range(nqb), causal=False)
 
 
+@pytest.mark.parametrize("walk", ["dense", "mask", "page16"])
+@pytest.mark.parametrize("tb,skip_scale", [(1.0, -1.0), (0.999, 300.0), (0.3, -1.0), (0.15, 500.0)])
+def test_osk_ctas_that_take_over_further_work_items(tb, skip_scale, walk):
+    """More work items than CTAs fit on the chip: a CTA walks several, of 0 to 8 blocks, in any succession (also first or last ones
+    without blocks, and padding).  Bit-equal to one call per batch item, whose 64 work items get a CTA each."""
+    batch, hq, hkv, n = 16, 8, 2, 1024
+    nqb = n // 128
+    g = torch.Generator(device="cuda").manual_seed(11)
+    q, k, v = (torch.randn(batch, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv, hkv))
+    order = torch.argsort(torch.rand(batch, hq, nqb, nqb, device="cuda", generator=g), dim=-1).to(torch.int32)
+    length = torch.randint(0, nqb + 1, (batch, hq, nqb), device="cuda", generator=g, dtype=torch.int32)
+    lens = torch.full((batch,), n, dtype=torch.int32, device="cuda")
+    lens[::5] = 640
+    extra = lambda b: {}
+    if walk == "mask":
+        bits = torch.randint(0, 256, (batch, hq, nqb, 1), device="cuda", generator=g, dtype=torch.int32)
+        extra = lambda b: {"logical_mask": bits[b].contiguous(), "order_stride": nqb}
+    if walk == "page16":
+        table = torch.randperm(batch * n // 16, device="cuda", generator=g).to(torch.int32).view(batch, n // 16)
+        pools = []
+        for x in (k, v):
+            pool = torch.empty(batch * n // 16, hkv, 16, 128, dtype=torch.bfloat16, device="cuda")
+            pool[table.view(-1).long()] = x.view(batch, hkv, n // 16, 16, 128).transpose(1, 2).reshape(-1, hkv, 16, 128)
+            pools.append(pool)
+        k, v = pools
+        extra = lambda b: {"kv_page_table": table[b].contiguous(), "kv_page_size": 16, "kv_num_pages": batch * n // 16,
+                           "kv_pages_in_place": 1}
+
+    def call(b):
+        out = torch.full_like(q[b], 3.0)
+        lse = torch.full((*q[b].shape[:3],), 3.0, device="cuda")
+        vis = torch.full((*length[b].shape,), -7, dtype=torch.int32, device="cuda")
+        opt = cosa.default_options(skip_scale=skip_scale, seq_lens=lens[b].contiguous(), **extra(b))
+        kv = (k, v) if walk == "page16" else (k[b].contiguous(), v[b].contiguous())
+        cosa.cosa_osk_attention(q[b].contiguous(), *kv, order[b].contiguous(), length[b].contiguous(), tb, out, lse, vis, causal=False,
+                                opt=opt)
+        assert cosa.cosa_device_status() == 0
+        return out, lse, vis
+
+    whole = call(slice(None))
+    for b in range(batch):
+        for x, y in zip(whole, call(slice(b, b + 1))):
+            assert torch.equal(x[b:b + 1], y)
+
+
 @pytest.mark.parametrize("impl", OSK_IMPLS)
 def test_osk_noncausal(small, impl):
     q, k, v = small["dev"]
