@@ -57,7 +57,6 @@ constexpr int kCtasPerSm = 2;
 constexpr int kTmemCols = 256;
 constexpr int kLoadWarp = 4, kMmaWarp = 5;
 constexpr int kAskAhead = 4;                       // positions (or two computed blocks) before a walk's end at which more work is asked for
-constexpr float kRescaleAbove = 8.f;               // (base 2) see the exponentials
 constexpr uint32_t kDecComputed = 1, kDecEnd = 2;
 constexpr int kTimedOut = 1, kPoisoned = 2;
 
@@ -455,7 +454,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       }
       // a batch item no longer than Delta would have ln(Delta/N) >= 0 and lose even its first block: the test is off for it
       const bool thr_on = p.use_threshold && theta2 < 0.f;
-      float m = -INFINITY, m_ref = -INFINITY;   // running row maximum (base 2); the one the exponentials refer to
+      float m = -INFINITY;                      // running row maximum (base 2)
       float l = 0.f;                            // row sum
       int n = 0, kk = 0;                        // computed blocks, list position
       uint32_t dec_word = 0;
@@ -500,32 +499,15 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
             continue;
           }
         }
+        const float alpha = ex2_approx(m - m_new);  // (the first block: m = -inf)
         m = m_new;
-        // ---- the exponentials refer to m_ref, an earlier running maximum, until the maximum has moved by more than 2^8:
-        // O and l then need no rescaling for the small steps (P may reach 2^8: its relative precision is the same)
-        float alpha = 1.f;
-        if (m - m_ref > kRescaleAbove) {            // (the first block: m_ref = -inf)
-          alpha = ex2_approx(m_ref - m);
-          m_ref = m;
-        }
-        if (n > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {   // O = diag(alpha) O
-          wait(&ctl->pv_done[1], n_base + n - 1);
-          __syncwarp();
-          tc_fence_after();
-#pragma unroll 1
-          for (int c = 0; c < 4; ++c) {
-            uint32_t o[32];
-            tmem_ld32(tmem_o + lane_addr + c * 32, o);
-            tmem_wait_ld();
-#pragma unroll
-            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-            tmem_st32(tmem_o + lane_addr + c * 32, o);
-          }
-          tmem_wait_st();
-        }
-        // ---- P = exp(S - m), row sums (two elements per FMA and per add: the packed float32 forms), 64 keys at a time
+        const bool moved = n > 0 && __any_sync(0xffffffffu, alpha != 1.f);
+        // ---- P = exp(S - m), row sums (two elements per FMA and per add: the packed float32 forms), 64 keys at a time.
+        // m is the maximum up to this block, so that an element that raises it weighs exactly 1 in bf16, and O is rescaled
+        // whenever it moves.  (Left until it has moved by 2^8, a pass is 2 % faster, but the largest weights are rounded: error
+        // against double precision over all blocks of 16K tokens 2.115e-3 instead of 2.016e-3, largest 6.6e-3 instead of 4.3e-3)
         l *= alpha;
-        const unsigned long long sc2 = pack_f32x2(scale2, scale2), nm2 = pack_f32x2(-m_ref, -m_ref);
+        const unsigned long long sc2 = pack_f32x2(scale2, scale2), nm2 = pack_f32x2(-m, -m);
         unsigned long long acc01 = pack_f32x2(0.f, 0.f), acc23 = acc01;
         unsigned char* prow = smem + 3 * kTileBytes + r * 128;
 #pragma unroll
@@ -546,6 +528,20 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
             s[c / 2] = pack_bf16(e0, e1); s[c / 2 + 1] = pack_bf16(e2, e3);
           }
           if (!is_free) wait(last_reader, last_n);
+          if (half == 0 && moved) {                 // O = diag(alpha) O: the last product on it is the buffer's last reader
+            __syncwarp();
+            tc_fence_after();
+#pragma unroll 1
+            for (int c = 0; c < 4; ++c) {
+              uint32_t o[32];
+              tmem_ld32(tmem_o + lane_addr + c * 32, o);
+              tmem_wait_ld();
+#pragma unroll
+              for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+              tmem_st32(tmem_o + lane_addr + c * 32, o);
+            }
+            tmem_wait_st();
+          }
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
             const uint32_t* e = &s[half * 32 + c * 4];
@@ -604,7 +600,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       }
       tc_fence_before();
       __syncwarp();
-      if (p.lse) p.lse[lse_at] = (m_ref + log2f(l)) * 0.6931471805599453f;
+      if (p.lse) p.lse[lse_at] = (m + log2f(l)) * 0.6931471805599453f;
       if (r == 32) {
         if (p.visited) p.visited[row] = n;
         if (p.scored) p.scored[row] = kk + 1;

@@ -483,7 +483,7 @@ def test_osk_4k_workload(cfg1, impl):
 @pytest.mark.parametrize("tb,skip_scale", [(1.0, -1.0), (0.999, 100.0), (0.999, 900.0), (0.13, 500.0), (0.3, -1.0)])
 def test_osk_short_walks_with_growing_maxima(small, length, tb, skip_scale):
     """Walks of one to seven blocks (tile slots change roles with every decision; the cap ends walks at one, two or three
-    computed blocks), keys scaled so that the running maximum moves by less and by more than the factor above which O is
+    computed blocks), keys scaled so that the running maximum moves by small and by large steps, O being
     rescaled, blocks listed by ascending maximum in half of the lists.  Bars as everywhere: P and the output are bf16."""
     q, k, v = small["dev"]
     qf, kf, vf = small["f64"]
@@ -500,6 +500,41 @@ def test_osk_short_walks_with_growing_maxima(small, length, tb, skip_scale):
     count = np.full((1, hq, nqb), length, np.int32)
     bufs = run_osk(q, k2, v, torch.from_numpy(order).cuda(), torch.from_numpy(count).cuda(), tb, skip_scale, causal=False)
     check_osk_against_oracle(qf, kf2, vf, order[0], count[0], bufs, tb, skip_scale, range(hq), range(nqb), causal=False)
+
+
+@pytest.mark.parametrize("impl", [0, 4])
+@pytest.mark.parametrize("tb", [1.0, 0.999])
+@pytest.mark.parametrize("sharpness", [2.0, 4.0, 8.0])
+def test_osk_weight_of_a_rows_maximum_is_exact(sharpness, tb, impl):
+    """An element that raises its row's running maximum has the weight exp(0) = 1, exact in bf16, whatever the step: only
+    the other weights and the output are rounded to bf16.  Error per element, in units of 2^-8 (half a bf16 ulp at most):
+    |out| from the output, sum of w |v| over the elements that were no new maximum when their block came; 2^-14 of
+    sum w |v| covers float32 (logits below 2^6 with 128 added products, exponentials of two ulp)."""
+    n, nkb = 1024, 8
+    rng = np.random.Generator(np.random.Philox(key=[int(sharpness), 77]))
+    q = torch.from_numpy(rng.standard_normal((1, 1, n, 128)) * sharpness).to(torch.bfloat16)
+    k, v = (torch.from_numpy(rng.standard_normal((1, 1, n, 128))).to(torch.bfloat16) for _ in range(2))
+    order = torch.from_numpy(np.stack([rng.permutation(nkb) for _ in range(nkb)]).astype(np.int32))[None, None]
+    count = torch.full((1, 1, nkb), nkb, dtype=torch.int32)
+    bufs = run_osk(q.cuda(), k.cuda(), v.cuda(), order.cuda(), count.cuda(), tb, -1.0, impl=impl, causal=False)
+    qf, kf, vf = (x[0, 0].double().numpy() for x in (q, k, v))
+    out = bufs["out"][0, 0].double().cpu().numpy()
+    z = qf @ kf.T / math.sqrt(128)
+    w = np.exp(z - z.max(1, keepdims=True))
+    w /= w.sum(1, keepdims=True)
+    rest = w.copy()
+    for i in range(nkb):
+        rows = np.arange(i * 128, (i + 1) * 128)
+        top = np.full(128, -np.inf)
+        for j in order[0, 0, i].tolist():
+            zb = z[rows, j * 128:(j + 1) * 128]
+            new = zb.max(1) > top
+            rest[rows[new], j * 128 + zb.argmax(1)[new]] = 0.0
+            top = np.maximum(top, zb.max(1))
+    ref = w @ vf
+    bound = 2.0 ** -8 * (np.abs(ref) + rest @ np.abs(vf)) + 2.0 ** -14 * (w @ np.abs(vf))
+    over = np.abs(out - ref) > bound
+    assert not over.any(), (int(over.sum()), float((np.abs(out - ref) / bound).max()))
 
 
 @pytest.mark.parametrize("walk", ["dense", "mask", "page16"])
