@@ -524,7 +524,9 @@ int cosa_prefill_host(const void* q_host, const void* k_host, const void* v_host
   // so the chunks run as independent calls.  Copies to the device go on a second stream and copies back on a third,
   // so that the transfers of the other chunks overlap a chunk's kernels; `stream` waits for the last copy back.  The link
   // to the device is what bounds the call; after the last byte has arrived, the last chunk's kernels and copy back
-  // remain.  The last chunk is therefore taken query head by query head (16K tokens, 32 / 8 heads: 4.55 -> 4.49 ms).
+  // remain.  The last chunk is therefore taken query head by query head (16K tokens, 32 / 8 heads: 4.55 -> 4.49 ms), unless the
+  // scratch does not hold what one head asks for: where the screen takes single heads but not the shape's groups, the
+  // layout has none, and every chunk goes in one piece through the double-precision route.
   const int G = shape->hq / shape->hkv, chunks = shape->batch * shape->hkv;
   const size_t kv_chunk = L.kv_bytes / chunks;
   const size_t heads = (size_t)shape->batch * shape->hq;
@@ -532,7 +534,8 @@ int cosa_prefill_host(const void* q_host, const void* k_host, const void* v_host
   cudaStream_t up = nullptr, down = nullptr;
   if (!copy_streams(&up, &down)) return cuda_fail(cudaGetLastError(), "copy streams");
   cosa_shape sub = *shape;
-  sub.batch = 1; sub.hkv = 1;
+  sub.batch = 1; sub.hkv = 1; sub.hq = 1;
+  const bool by_head = kap_scratch_bytes(&sub, o) <= o.workspace_bytes;
   cudaEvent_t ev = nullptr;
   auto order_after = [&](cudaStream_t later, cudaStream_t earlier) -> bool {   // later waits for what earlier holds now
     if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) return false;
@@ -550,7 +553,7 @@ int cosa_prefill_host(const void* q_host, const void* k_host, const void* v_host
     cosa_options oc = o;
     if (o.seq_lens) oc.seq_lens = o.seq_lens + c / shape->hkv;   // the slice's batch item (lengths live on the device: padding is copied too)
     if ((e = cudaMemcpyAsync(kd, kh, kv_chunk, cudaMemcpyHostToDevice, up)) != cudaSuccess) return cuda_fail(e, "H2D k");
-    const int step = c == chunks - 1 ? 1 : G;
+    const int step = by_head && c == chunks - 1 ? 1 : G;
     sub.hq = step;
     for (int h0 = 0; h0 < G; h0 += step) {
       const size_t h = (size_t)c * G + h0;                       // the slice's first query head

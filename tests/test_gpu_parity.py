@@ -1202,3 +1202,25 @@ def test_host_call_with_different_lengths():
     assert torch.equal(vis_h, vis.cpu()) and torch.equal(out_h, out.cpu())
     assert torch.equal(lse_h[0, :, :lens[0]], lse.cpu()[0, :, :lens[0]]) and torch.equal(lse_h[1], lse.cpu()[1])
     assert bool((out_h[0, :, lens[0]:] == 0).all()) and bool((vis_h[0, :, lens[0] // 128:] == 0).all())
+
+
+@pytest.mark.parametrize("hq,hkv,stride", [(3, 1, 8), (28, 4, 8), (24, 8, 8), (32, 1, 8), (16, 1, 4), (16, 1, 8), (12, 2, 16)])
+def test_host_call_takes_every_group_size(hq, hkv, stride):
+    """Groups of query heads that the tensor-core screen takes and groups that it does not (their lists come from the
+    double-precision kernel, without scratch): the host call gives the device calls' results."""
+    n = 1024
+    g = torch.Generator(device="cuda").manual_seed(hq * 100 + stride)
+    q, k, v = (torch.randn(1, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv, hkv))
+    order, count = run_kap(q, k, 0.5, stride)
+    ref = run_osk(q, k, v, order, count, 0.3, 200.0)
+    shape = cosa.make_shape(q, k, True)
+    opt = cosa.default_options(stride=stride, skip_scale=200.0)
+    ws = torch.empty(cosa.cosa_host_call_workspace_bytes(shape, opt), dtype=torch.uint8, device="cuda")
+    out_h = torch.empty(q.shape, dtype=torch.bfloat16).pin_memory()
+    lse_h = torch.empty(ref["lse"].shape, dtype=torch.float32).pin_memory()
+    vis_h = torch.empty(ref["visited"].shape, dtype=torch.int32).pin_memory()
+    qh, kh, vh = (t.cpu().pin_memory() for t in (q, k, v))
+    cosa.cosa_prefill_host(qh, kh, vh, shape, 0.5, 0.3, out_h, lse_h, vis_h, ws, opt=opt)
+    assert cosa.cosa_device_status() == 0
+    assert torch.equal(out_h, ref["out"].cpu()) and torch.equal(lse_h, ref["lse"].cpu())
+    assert torch.equal(vis_h, ref["visited"].cpu())
