@@ -544,6 +544,15 @@ int cosa_prefill_host(const void* q_host, const void* k_host, const void* v_host
     cudaEventDestroy(ev);   // released once the recorded work has completed
     return e == cudaSuccess;
   };
+  // An error return, too, leaves `stream` behind the copies that still read and write the caller's buffers.
+  struct Join {
+    decltype(order_after)& after;
+    cudaStream_t st, up, down;
+    bool wanted = true;
+    ~Join() {
+      if (wanted) { after(st, up); after(st, down); }
+    }
+  } join{order_after, st, up, down};
   if (!order_after(up, st)) return cuda_fail(e, "stream order");   // the workspace may still be in use on `stream`
   if (!order_after(down, st)) return cuda_fail(e, "stream order");
   for (int c = 0; c < chunks; ++c) {
@@ -581,6 +590,7 @@ int cosa_prefill_host(const void* q_host, const void* k_host, const void* v_host
     }
   }
   if (!order_after(st, down)) return cuda_fail(e, "stream order");   // outputs are valid once `stream` is synchronised
+  join.wanted = false;
   return COSA_OK;
 }
 

@@ -1224,3 +1224,25 @@ def test_host_call_takes_every_group_size(hq, hkv, stride):
     assert cosa.cosa_device_status() == 0
     assert torch.equal(out_h, ref["out"].cpu()) and torch.equal(lse_h, ref["lse"].cpu())
     assert torch.equal(vis_h, ref["visited"].cpu())
+
+
+def test_host_call_that_fails_leaves_its_stream_behind_its_copies():
+    """An error found after copies have been enqueued (a budget that the first stage refuses): what the caller's stream does
+    next comes after those copies, so that synchronising it makes the host buffers safe to free."""
+    n = 65536
+    gen = torch.Generator().manual_seed(3)
+    qh, kh, vh = (torch.randint(-2 ** 14, 2 ** 14, (1, 1, n, 128), generator=gen, dtype=torch.int16).view(torch.bfloat16).pin_memory()
+                  for _ in range(3))
+    out_h = torch.zeros(1, 1, n, 128, dtype=torch.bfloat16).pin_memory()
+    shape = cosa.CosaShape(1, 1, 1, n, 128, 128, 128, 1)
+    ws = torch.zeros(cosa.cosa_host_call_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    one = n * 128 * 2
+    seen = torch.empty(3 * one, dtype=torch.uint8, device="cuda").copy_(ws[:3 * one])   # (and the copy is warm)
+    torch.cuda.synchronize()
+    with pytest.raises(cosa.CosaError) as e:
+        cosa.cosa_prefill_host(qh, kh, vh, shape, 0.0, 0.3, out_h, None, None, ws)
+    seen.copy_(ws[:3 * one])                        # q, k and v are the workspace's first areas
+    torch.cuda.synchronize()
+    assert e.value.status == -1
+    want = torch.cat([t.view(torch.int16).view(-1) for t in (qh, kh, vh)]).view(torch.uint8)
+    assert torch.equal(seen.cpu(), want)
