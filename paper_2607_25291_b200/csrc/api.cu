@@ -467,6 +467,7 @@ bool copy_streams(cudaStream_t* up, cudaStream_t* down) {
   *up = streams[dev][0]; *down = streams[dev][1];
   return true;
 }
+constexpr size_t kSplitBytes = 3u << 19;   // queries of one head from which on the host call splits its last chunk
 struct HostCallLayout {
   size_t q, k, v, out, lse, order, count, visited, scratch, total;
   size_t q_bytes, kv_bytes, lse_bytes, order_bytes, cnt_bytes;
@@ -524,9 +525,12 @@ int cosa_prefill_host(const void* q_host, const void* k_host, const void* v_host
   // so the chunks run as independent calls.  Copies to the device go on a second stream and copies back on a third,
   // so that the transfers of the other chunks overlap a chunk's kernels; `stream` waits for the last copy back.  The link
   // to the device is what bounds the call; after the last byte has arrived, the last chunk's kernels and copy back
-  // remain.  The last chunk is therefore taken query head by query head (16K tokens, 32 / 8 heads: 4.55 -> 4.49 ms), unless the
-  // scratch does not hold what one head asks for: where the screen takes single heads but not the shape's groups, the
-  // layout has none, and every chunk goes in one piece through the double-precision route.
+  // remain.  The last chunk of a long call is therefore taken query head by query head.  Every further head costs the host some
+  // 25 us of enqueueing, which its transfers have to last for: measured whole -> by head, 16 / 1 heads: 1K tokens 236 -> 458 us,
+  // 4K 733 -> 781, 6K 1,074 -> 1,040, 16K 2,811 -> 2,256; 4 / 1: 114 -> 161, 268 -> 265, 376 -> 351, 886 -> 733; 32 / 8: 539 -> 571,
+  // 1,394 -> 1,406, 1,921 -> 1,935, 4,552 -> 4,489.  The line: 1.5 MiB of queries a head.  Never where the scratch does not hold
+  // what one head asks for: if the screen takes single heads but not the shape's groups, the layout has none, and every
+  // chunk goes in one piece through the double-precision route.
   const int G = shape->hq / shape->hkv, chunks = shape->batch * shape->hkv;
   const size_t kv_chunk = L.kv_bytes / chunks;
   const size_t heads = (size_t)shape->batch * shape->hq;
@@ -535,7 +539,7 @@ int cosa_prefill_host(const void* q_host, const void* k_host, const void* v_host
   if (!copy_streams(&up, &down)) return cuda_fail(cudaGetLastError(), "copy streams");
   cosa_shape sub = *shape;
   sub.batch = 1; sub.hkv = 1; sub.hq = 1;
-  const bool by_head = kap_scratch_bytes(&sub, o) <= o.workspace_bytes;
+  const bool by_head = q_head >= kSplitBytes && kap_scratch_bytes(&sub, o) <= o.workspace_bytes;
   cudaEvent_t ev = nullptr;
   auto order_after = [&](cudaStream_t later, cudaStream_t earlier) -> bool {   // later waits for what earlier holds now
     if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) return false;

@@ -1246,3 +1246,25 @@ def test_host_call_that_fails_leaves_its_stream_behind_its_copies():
     assert e.value.status == -1
     want = torch.cat([t.view(torch.int16).view(-1) for t in (qh, kh, vh)]).view(torch.uint8)
     assert torch.equal(seen.cpu(), want)
+
+
+@pytest.mark.parametrize("n", [6016, 6144])
+@pytest.mark.parametrize("hq,hkv", [(4, 1), (4, 2), (2, 2), (3, 1)])
+def test_host_call_on_both_sides_of_the_split(n, hq, hkv):
+    """The last (batch item, KV head) slice goes query head by query head from 1.5 MiB of queries a head up."""
+    g = torch.Generator(device="cuda").manual_seed(n + hq)
+    q, k, v = (torch.randn(2, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv, hkv))
+    nqb = n // 128
+    order = torch.empty(2, hq, nqb, nqb, dtype=torch.int32, device="cuda")
+    count, vis = (torch.empty(2, hq, nqb, dtype=torch.int32, device="cuda") for _ in range(2))
+    out, lse = torch.empty_like(q), torch.empty(2, hq, n, dtype=torch.float32, device="cuda")
+    opt = cosa.default_options(skip_scale=3000.0)
+    cosa.cosa_kap_select(q, k, 0.2, order, count, opt=opt)
+    cosa.cosa_osk_attention(q, k, v, order, count, 0.1, out, lse, vis, opt=opt)
+    shape = cosa.make_shape(q, k, True)
+    ws = torch.empty(cosa.cosa_host_call_workspace_bytes(shape, opt), dtype=torch.uint8, device="cuda")
+    qh, kh, vh = (t.cpu().pin_memory() for t in (q, k, v))
+    out_h, lse_h, vis_h = (torch.empty(t.shape, dtype=t.dtype).pin_memory() for t in (out, lse, vis))
+    cosa.cosa_prefill_host(qh, kh, vh, shape, 0.2, 0.1, out_h, lse_h, vis_h, ws, opt=opt)
+    assert cosa.cosa_device_status() == 0
+    assert torch.equal(vis_h, vis.cpu()) and torch.equal(out_h, out.cpu()) and torch.equal(lse_h, lse.cpu())
