@@ -153,7 +153,7 @@ cosa_options resolve_options(const cosa_options* opt) {
 }  // namespace
 
 // scratch the kernels of one call need (beyond inputs and outputs)
-struct KapScratch { size_t scores, jstar, ambmask, hard, redo_list, tied_list, k2part, qk2max, slot_taken, maxima, kstage, total; int slots; bool gather; };
+struct KapScratch { size_t scores, jstar, ambmask, hard, todo, qk2max, slot_taken, maxima, kstage, total; int slots; bool gather; };
 static KapScratch kap_scratch_layout(const cosa_shape* s, const cosa_options& o) {
   KapScratch L{};
   const int stride = o.stride > 0 ? o.stride : 8;
@@ -172,9 +172,7 @@ static KapScratch kap_scratch_layout(const cosa_shape* s, const cosa_options& o)
   L.jstar = off; off += align_up(heads * (s->n / stride) * 8, 256);
   L.ambmask = off; off += align_up(heads * nqb * 4, 256);
   L.hard = off; off += align_up(heads * nqb, 256);
-  L.redo_list = off; off += align_up((1 + heads * nqb) * 4, 256);
-  L.tied_list = off; off += align_up((1 + heads * nqb) * 4, 256);
-  L.k2part = off; off += align_up(kNormParts * 4, 256);
+  L.todo = off; off += align_up((2 + heads * nqb) * 4, 256);
   L.qk2max = off; off += align_up(heads * nqb * 4, 256);
   // the screen's parked block maxima: one area per CTA that can be resident on the current device
   L.slots = kap_screen_slots();
@@ -291,10 +289,9 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
   sp.jstar = reinterpret_cast<int32_t*>(ws + L.jstar);
   sp.ambmask = reinterpret_cast<uint32_t*>(ws + L.ambmask);
   sp.hard = reinterpret_cast<uint8_t*>(ws + L.hard);
-  sp.redo_list = reinterpret_cast<int32_t*>(ws + L.redo_list);
-  sp.tied_list = reinterpret_cast<int32_t*>(ws + L.tied_list);
+  sp.todo = reinterpret_cast<int32_t*>(ws + L.todo);
   sp.slot_taken = reinterpret_cast<int32_t*>(ws + L.slot_taken);
-  sp.k2part = reinterpret_cast<float*>(ws + L.k2part);
+  sp.k2part = reinterpret_cast<float*>(sp.todo + 2);
   sp.qk2max = reinterpret_cast<float*>(ws + L.qk2max);
   sp.maxima = reinterpret_cast<float*>(ws + L.maxima);
   sp.slots = L.slots;

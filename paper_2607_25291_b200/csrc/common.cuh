@@ -104,12 +104,13 @@ struct KapScreenParams {
   int32_t* jstar;        // [B,Hq,N/s,2]    blocks holding each sampled row's largest / second largest block maximum
   uint32_t* ambmask;     // [B,Hq,nQB]      bit r: sampled row r's two best blocks are too close to call in float32
   uint8_t* hard;         // [B,Hq,nQB]      1 = three blocks too close on some row: whole query block goes to double precision
-  int32_t* redo_list;    // [1 + B*Hq*nQB]  [0] = number of entries, then flat (b*Hq+h)*nQB+i of query blocks to redo
-  int32_t* tied_list;    // [1 + B*Hq*nQB]  the same for lists with near ties; their rows of `scores` then hold the chained entries (see
-                         // kap_recount.cuh)
+  int32_t* todo;         // [2 + B*Hq*nQB]  what the sort stage leaves to the next: [0] = lists to redo, [1] = lists with near ties (their rows of
+                         // `scores` then hold the chained entries, see kap_recount.cuh); behind them, as flat (b*Hq+h)*nQB+i, the
+                         // former from the front, the latter from the end: no list is both
   float* maxima;         // [slots][key tiles][128 rows x 128/R blocks]  per-row block maxima of the CTA that holds the slot
   int32_t* slot_taken;   // [slots]  0 = free; zeroed by kap_norms_kernel
-  float* k2part;         // [kNormParts]  largest squared norms of sampled key rows of the call, one per CTA of kap_norms_kernel
+  float* k2part;         // largest squared norms of sampled key rows of the call, one per CTA of kap_norms_kernel; they lie where the
+                         // entries of `todo` come when the screen has read them (128 sampled keys make a part, so there are fewer)
   int k2parts;           // ... how many
   float* qk2max;         // [B,Hq,nQB]  largest squared norm of the sampled query rows of every (head, query block), times the largest of
                          // the sampled key rows (of the call, or in a short call of the keys the block's CTA multiplied)
@@ -245,7 +246,7 @@ cudaError_t raise_smem_limit(const void* kernel, SmemLimit* state, size_t bytes)
 
 // every (head, query block) in double precision
 cudaError_t launch_kap_exact(const KapParams& p, cudaStream_t st);
-// works off sp.tied_list (near ties recounted) and sp.redo_list (whole lists redone)
+// works off sp.todo: near ties recounted, whole lists redone
 cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, cudaStream_t st);
 // the whole call's key tiles fit the screen's stages: it needs no scratch areas and no norms kernel
 bool kap_screen_is_short(int n, int stride);

@@ -38,13 +38,13 @@ __global__ void __launch_bounds__(kThreads, kRedo ? 2 : 4) kap_fixup_kernel(KapP
   chain_begin();
   if (*reinterpret_cast<const volatile int32_t*>(status) != 0) return;   // an earlier kernel of the call gave up: the lists are not to be trusted
   if (kTied) {
-    const int n = sp.tied_list[0];
-    for (int e = blockIdx.x; e < n; e += gridDim.x) kap_recount_item(p, sp, sp.tied_list[1 + e], smem_raw);
+    const int n = sp.todo[1], last = 1 + p.batch * p.hq * p.nqb;
+    for (int e = blockIdx.x; e < n; e += gridDim.x) kap_recount_item(p, sp, sp.todo[last - e], smem_raw);
   }
   if (kRedo) {
-    const int n = sp.redo_list[0];
+    const int n = sp.todo[0];
     for (int e = blockIdx.x; e < n; e += gridDim.x) {
-      const int flat = sp.redo_list[1 + e];
+      const int flat = sp.todo[2 + e];
       const int i = flat % p.nqb, bh = flat / p.nqb;
       kap_exact_item(p, bh / p.hq, bh % p.hq, i, kb_per_iter, sort_cap);   // i: first row tile of the block
       __syncthreads();

@@ -117,7 +117,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const int n_tiles = (n_keys + 127) / 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  if (blockIdx.x == 0 && threadIdx.x == 0) { p.redo_list[0] = 0; p.tied_list[0] = 0; }   // the sort stage (a later launch) appends to them
+  if (blockIdx.x == 0 && threadIdx.x == 0) { p.todo[0] = 0; p.todo[1] = 0; }   // the sort stage (a later launch) counts there
   if (i0 >= nqb_b) return;                        // all of this CTA's query blocks are padding
   if (threadIdx.x == 0) {
     // once some CTA has reported a timeout the rest of the grid returns at once

@@ -62,3 +62,14 @@ def test_argument_checks_need_no_gpu(lib):
     opt = B.default_options(stride=3)
     assert L.cosa_kap_select_ex(one, one, ctypes.byref(shape), 0.5, one, one, None, ctypes.byref(opt)) == B.COSA_ERR_UNSUPPORTED
     assert B.cosa_host_call_workspace_bytes(shape) > 4 * 4096 * 128 * 2
+
+
+@pytest.mark.parametrize("batch,hq,hkv,stride,blocks,want", [
+    (1, 32, 8, 16, 55, 4193792), (1, 32, 4, 16, 55, 4193792), (4, 8, 2, 16, 55, 4193792), (1, 32, 8, 8, 32, 2373376), (1, 1, 1, 8, 17, 54272)])
+def test_calls_that_the_built_in_scratch_serves_stay_within_it(lib, batch, hq, hkv, stride, blocks, want):
+    """Stage 1 without allocation serves what fits its 4 MiB; callers sized their calls by this need, which may shrink only.
+    (Fewer screen CTAs than any device has SMs: the figures do not depend on the device.)"""
+    from paper_2607_25291_b200 import binding as B
+    shape = B.CosaShape(batch, hq, hkv, blocks * 128, 128, 128, 128, 1)
+    need = B.cosa_workspace_bytes(0, shape, B.default_options(stride=stride))
+    assert 0 < need <= want <= B.cosa_kap_select_static_max_bytes()

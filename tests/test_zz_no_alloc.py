@@ -109,3 +109,16 @@ print("ok", before - mid)
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
     assert res.returncode == 0 and "ok" in res.stdout, res.stdout + res.stderr
+
+
+@pytest.mark.parametrize("hq,hkv,n,stride", [(32, 8, 55 * 128, 16), (4, 1, 24 * 128, 4), (1, 1, 128, 8)])
+def test_static_scratch_up_to_its_limit_and_down_to_one_block(hq, hkv, n, stride):
+    """The largest call the array serves (4,193,792 bytes or less of 4,194,304), a long call at stride 4 and a single block."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q, k = (torch.randn(1, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv))
+    opt = cosa.default_options(stride=stride)
+    (order, count), (ref_order, ref_count) = alloc_lists(hq, n // 128), alloc_lists(hq, n // 128)
+    cosa.cosa_kap_select_static(q, k, 0.3, order, count, opt=opt)
+    cosa.cosa_kap_select(q, k, 0.3, ref_order, ref_count, opt=opt)
+    assert cosa.cosa_device_status() == 0
+    assert torch.equal(order, ref_order) and torch.equal(count, ref_count) and int(count.min()) >= 1
