@@ -257,7 +257,7 @@ cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, cuda
   static_assert(kThreads == kRecountThreads, "one kernel does both");
   const int32_t* status = device_status_word();
   if (!status) return cudaErrorInvalidSymbol;
-  const int lists = p.batch * p.hq * (p.nqb / p.qtiles), sms = 148;
+  const int lists = p.batch * p.hq * (p.nqb / p.qtiles), sms = std::max(1, device_sm_count());
   const int kb = kb_per_iter_for(p.rows), cap = next_pow2(p.nqb);
   const size_t redo = kap_exact_smem_bytes(p.rows, p.nqb, p.qtiles), tied = kap_recount_smem_bytes(p.rows, p.qtiles, p.nqb);
   static SmemLimit limits[3];
@@ -269,7 +269,11 @@ cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, cuda
   const size_t both = std::max(redo, tied);
   if (both <= 56 * 1024) return launch(kap_fixup_kernel<true, true>, &limits[0], both, 2 * sms);
   const cudaError_t e = launch(kap_fixup_kernel<true, false>, &limits[1], tied, 4 * sms);
-  return e != cudaSuccess ? e : launch(kap_fixup_kernel<false, true>, &limits[2], redo, sms);
+  // As many CTAs as fit the chip (227 KB of shared memory, 3 x 256 threads of registers on an SM): the launch overlaps the recount,
+  // whose CTAs still hold SMs, and one CTA per SM was placed two and three to an SM, where they share the FP64 unit and the
+  // others idle (200 blocks of 8 heads, all keys the same: 8,223 us with one per SM, 4,942 when the launch came later)
+  const int fit = (int)std::min<size_t>(3, 227 * 1024 / (redo + 1024));
+  return e != cudaSuccess ? e : launch(kap_fixup_kernel<false, true>, &limits[2], redo, std::max(1, fit) * sms);
 }
 
 }  // namespace cosa

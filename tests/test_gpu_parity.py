@@ -290,6 +290,24 @@ def test_kap_chains_of_equal_scores(cfg1, budget, stride, block_q):
     assert np.array_equal(_np(count), ref_count) and np.array_equal(_np(order), ref_order)
 
 
+@pytest.mark.parametrize("blocks,stride,block_q", [(144, 8, 128), (150, 8, 256), (300, 8, 128), (600, 16, 128), (100, 4, 128)])
+def test_kap_lists_to_redo_beside_lists_to_recount(blocks, stride, block_q):
+    """Lists that are done over (rows with three best blocks alike) and lists with near ties, at lengths where each kind has a
+    launch of its own with one, two or three CTAs per SM: what the double-precision kernel gives for all of them."""
+    g = torch.Generator(device="cuda").manual_seed(blocks)
+    q, k = (torch.randn(1, heads, blocks * 128, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (4, 2))
+    kb = k.view(1, 2, blocks, 128, 128)
+    kb[:, 0, 5::7] = kb[:, 0, 5:6]                   # many alike: mostly lists to do over
+    kb[:, 1, 40] = kb[:, 1, 9]                       # one pair: lists to recount
+    lists = []
+    for impl in (0, 1):
+        order, count = alloc_lists(4, blocks)
+        cosa.cosa_kap_select(q, k, 0.3, order, count, opt=cosa.default_options(stride=stride, impl=impl), block_q=block_q)
+        assert cosa.cosa_device_status() == 0
+        lists.append((order, count))
+    assert torch.equal(lists[0][0], lists[1][0]) and torch.equal(lists[0][1], lists[1][1])
+
+
 @pytest.mark.parametrize("impl", IMPLS)
 def test_kap_lists_bit_exact_4k(cfg1, impl):
     w = cfg1["w"]
