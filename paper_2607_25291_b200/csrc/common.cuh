@@ -219,14 +219,24 @@ int device_sm_count();
 
 // The kernels of a call follow one another closely and the small ones last a few microseconds, as long as a launch takes.
 // launch_chained lets a kernel's launch overlap the kernel before it in the stream (programmatic dependent launch); the kernel
-// calls chain_begin() before it touches global memory: it waits until everything before it in the stream has finished
-// and its writes are visible, then lets the next launch begin.  (Two memsets and four launches one after the other to
+// calls chain_wait() before it touches global memory: it waits until everything before it in the stream has finished
+// and its writes are visible; chain_next() lets the next launch begin.  A kernel that uses tensor memory calls chain_next()
+// when it has its share: the next kernel in the stream may be anyone's, and one that allocates tensor memory before its own
+// wait would otherwise take, for as long as it waits for this kernel, what a CTA of this kernel still waits for.  (Two memsets and four launches one after the other to
 // launches that overlap, norms folded in: 31 blocks of 32 heads 96 -> 75 us a pass.)
-__device__ __forceinline__ void chain_begin() {
+__device__ __forceinline__ void chain_wait() {
 #if defined(__CUDA_ARCH__)
   asm volatile("griddepcontrol.wait;" ::: "memory");
+#endif
+}
+__device__ __forceinline__ void chain_next() {
+#if defined(__CUDA_ARCH__)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #endif
+}
+__device__ __forceinline__ void chain_begin() {
+  chain_wait();
+  chain_next();
 }
 template <typename... Params, typename... Args>
 cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args&&... args) {

@@ -94,7 +94,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - raw);
   if (threadIdx.x == 0) { prefetch_tensormap(&q_map); prefetch_tensormap(&k_map); }
-  chain_begin();
+  chain_wait();
   const uint32_t a_sm = base;
   const uint32_t k_sm = base + kRowTiles * kTileBytes;
   ScreenCtl* ctl = reinterpret_cast<ScreenCtl*>(smem + (size_t)kTileBytes * (kRowTiles + kStages));
@@ -160,6 +160,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  chain_next();                            // (tensor memory is allocated)
   const uint32_t tmem = ctl->tmem_base;
   volatile int* abort_flag = &ctl->abort_flag;
   const long long budget = p.wait_budget;

@@ -127,7 +127,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = p.hq / p.hkv;
-  chain_begin();
+  chain_wait();
 
   // work items: KV head major, then query blocks from the longest list down, the group's query heads innermost, so that CTAs
   // resident together read the same K/V pages
@@ -215,6 +215,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  chain_next();                            // (tensor memory is allocated)
   const uint32_t tmem_s = ctl->tmem_base, tmem_o = tmem_s + 128u;
   volatile int* abort_flag = &ctl->abort_flag;
   const long long budget = p.wait_budget;

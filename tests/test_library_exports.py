@@ -73,3 +73,18 @@ def test_calls_that_the_built_in_scratch_serves_stay_within_it(lib, batch, hq, h
     shape = B.CosaShape(batch, hq, hkv, blocks * 128, 128, 128, 128, 1)
     need = B.cosa_workspace_bytes(0, shape, B.default_options(stride=stride))
     assert 0 < need <= want <= B.cosa_kap_select_static_max_bytes()
+
+
+def test_chained_kernels_let_the_next_launch_begin_after_their_tensor_memory_allocation():
+    """A kernel launched behind one of these, by anyone, may allocate tensor memory before it waits for its predecessor:
+    that must not happen before every CTA of the predecessor has its own share, or both wait for good."""
+    csrc = os.path.join(ROOT, "paper_2607_25291_b200", "csrc")
+    chained = 0
+    for name in sorted(os.listdir(csrc)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        if name.endswith(".cu") and "launch_chained(" in text:
+            assert text.count("chain_wait();") + text.count("chain_begin();") == 1, name
+            if "tmem_alloc(" in text:
+                chained += 1
+                assert text.index("chain_wait();") < text.index("tmem_alloc(") < text.index("chain_next();"), name
+    assert chained == 2
