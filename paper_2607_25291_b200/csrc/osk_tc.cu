@@ -493,7 +493,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
             ctl->dec[(pos_base + kk) & 1] = (compute ? kDecComputed : 0u) | (last ? kDecEnd : 0u);
             mbar_arrive(smem_u32(&ctl->dec_bar[(pos_base + kk) & 1]));
             if (compute) dec_word |= 1u << (kk & 31);
-            if (p.decisions && ((kk & 31) == 31 || last)) { p.decisions[row * dec_words + (kk >> 5)] = dec_word; dec_word = 0; }
+            if (p.decisions && ((kk & 31) == 31 || last) && !*abort_flag) { p.decisions[row * dec_words + (kk >> 5)] = dec_word; dec_word = 0; }
           }
           if (!compute) {                           // skipped: nothing is added to l or O, and no maximum has moved
             if (last) break;

@@ -91,3 +91,31 @@ def test_status_word_set_by_hand_makes_both_stages_return_at_once(cfg1):
     assert int((count == -7).sum()) == count.numel() and int((order == -7).sum()) == order.numel()
     assert int((bufs["visited"] == -7).sum()) == bufs["visited"].numel()
     assert bool((bufs["out"] == 3.0).all())
+
+
+def test_osk_writes_no_decisions_of_a_walk_that_was_given_up(cfg1):
+    """Budgets at which waits run out at every stage of a walk: the decisions of a work item (its 32 positions are one word,
+    written when the walk reaches its end) are those of an undisturbed call or not written at all."""
+    w, (q, k, v) = cfg1["w"], cfg1["dev"]
+    nqb = w.n // 128
+    order = torch.arange(nqb, dtype=torch.int32, device="cuda").expand(1, w.hq, nqb, nqb).contiguous()
+    count = torch.full((1, w.hq, nqb), nqb, dtype=torch.int32, device="cuda")
+
+    def words_and_visited(**kw):
+        bufs = alloc_outputs(q, nqb)
+        bufs["visited"].fill_(-7)
+        cosa.cosa_osk_attention(q, k, v, order, count, 0.999, bufs["out"], bufs["lse"], bufs["visited"], causal=False,
+                                opt=cosa.default_options(skip_scale=w.skip_scale, out_decisions=bufs["decisions"], **kw))
+        assert cosa.cosa_device_status() in (0, TIMEOUT)
+        return bufs["decisions"][0, :, :, 0], bufs["visited"][0]
+
+    want, want_visited = words_and_visited()
+    assert int((want == -1).sum()) < want.numel() // 2     # (most walks skip something)
+    given_up = 0
+    for cycles in range(200, 6200, 100):
+        words, visited = words_and_visited(wait_cycles=cycles)
+        done = visited != -7
+        assert torch.equal(words[done], want[done]) and torch.equal(visited[done], want_visited[done]), cycles
+        assert bool(((words == 0) | (words == want)).all()), cycles
+        given_up += int((~done).sum())
+    assert given_up > 0
