@@ -80,18 +80,25 @@ __device__ void f64_block_maxima(const KapParams& p, const float* Qs, int b, int
 
 struct SortShared {
   unsigned long long samp[kSamples];
-  unsigned split[kSplit];                               // upper words (flag and score) of the splitters, descending: one bank each
+  unsigned split[kSplit], split_id[kSplit];             // upper (flag and score) and lower words of the splitters, descending: one bank each
   int start[kSplit + 2], cursor[kSplit + 1];            // by bucket: first position; keys so far
   int head_len;
 };
 
-// The bucket of a key: how many of the (descending) splitters lie above its upper word.
-__device__ __forceinline__ int bucket_of(const unsigned* split, unsigned hi) {
+// The bucket of a key: how many of the (descending) splitters lie above it.  The upper words decide, unless splitters share
+// theirs (alike): many keys have one score then, as blocks whose exponentials all underflow to 0, and are parted by id.  In one
+// bucket they would be compared all with all (Stage 1 of 2048 blocks of 4 heads, stride 16, Top-p, nine scores in ten 0: 2,311 us;
+// parted 810, with the sorting network of before 1,088).
+__device__ __forceinline__ int bucket_of(const SortShared* sh, unsigned long long key, bool alike) {
+  const unsigned hi = (unsigned)(key >> 32);
   int b = 0;
 #pragma unroll
   for (int step = kSplit / 2; step > 0; step >>= 1)
-    if (split[b + step - 1] > hi) b += step;
-  return b + (split[b] > hi ? 1 : 0);
+    if (sh->split[b + step - 1] > hi) b += step;
+  b += sh->split[b] > hi ? 1 : 0;
+  if (alike)
+    while (b < kSplit && sh->split[b] == hi && sh->split_id[b] > (unsigned)key) ++b;
+  return b;
 }
 
 // Sorts the distinct keys a[0 .. n) descending, at least the first `want` of them.  If the sorted head is shorter than n and
@@ -135,21 +142,23 @@ __device__ int sort_head_desc(unsigned long long* a, int n, int want, unsigned l
 #pragma unroll 8
     for (int u = 0; u < kSamples / 2; ++u) rank += (sh->samp[u * 2 + (tid & 1)] > mine) ? 1 : 0;
     rank += __shfl_xor_sync(0xffffffffu, rank, 1);
-    if ((tid & 1) == 0 && (rank & 1)) sh->split[rank >> 1] = (unsigned)(mine >> 32);
+    if ((tid & 1) == 0 && (rank & 1)) { sh->split[rank >> 1] = (unsigned)(mine >> 32); sh->split_id[rank >> 1] = (unsigned)mine; }
   }
   __syncthreads();
+  const int lane = tid & 31;
+  const bool alike = !one_bucket && __any_sync(0xffffffffu, lane < kSplit - 1 && sh->split[lane] == sh->split[min(lane + 1, kSplit - 1)]);
   // every key to its bucket's count; a thread keeps bucket and place of its first eight keys (all there are up to 1024)
   unsigned place[kPerThread];
 #pragma unroll
   for (int q = 0; q < kPerThread; ++q) {
     const int t = tid + q * kThreads;
     if (t < n) {
-      const int b = bucket_of(sh->split, (unsigned)(a[t] >> 32));
+      const int b = bucket_of(sh, a[t], alike);
       place[q] = ((unsigned)b << 16) | (unsigned)atomicAdd(&sh->cursor[b], 1);
     }
   }
   if (n > kPerThread * kThreads) __syncthreads();     // (those come first in their buckets)
-  for (int t = tid + kPerThread * kThreads; t < n; t += kThreads) atomicAdd(&sh->cursor[bucket_of(sh->split, (unsigned)(a[t] >> 32))], 1);
+  for (int t = tid + kPerThread * kThreads; t < n; t += kThreads) atomicAdd(&sh->cursor[bucket_of(sh, a[t], alike)], 1);
   const int first_n = min(n, kPerThread * kThreads);
   __syncthreads();
   if (tid < 32) {                                  // where every bucket begins, and how many buckets the head takes
@@ -183,7 +192,7 @@ __device__ int sort_head_desc(unsigned long long* a, int n, int want, unsigned l
     // more than 1024 keys: the rest finds its places again, from the ends of the buckets down (uniform over the CTA)
     for (int t = tid + first_n; t < n; t += kThreads) {
       const unsigned long long key = a[t];
-      const int b = bucket_of(sh->split, (unsigned)(key >> 32));
+      const int b = bucket_of(sh, key, alike);
       const int at = sh->start[b] + atomicSub(&sh->cursor[b], 1) - 1;
       if (sh->start[b] < len) {
         tmp[at] = key;

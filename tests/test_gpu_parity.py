@@ -420,6 +420,23 @@ def test_kap_order_where_the_sort_changes_its_way(blocks, stride, budget, top_p)
         assert np.array_equal(o[i, :kept], ref_order[0, i, :kept]) and (o[i, kept:] == -1).all()
 
 
+@pytest.mark.parametrize("blocks,stride,scale", [(129, 8, 40.0), (257, 8, 20.0), (520, 16, 20.0), (1100, 16, 40.0)])
+def test_kap_order_where_many_scores_are_alike(blocks, stride, scale):
+    """Logits so far apart that the exponentials of most blocks underflow to 0 in float32: equal scores share a splitter's
+    score and are dealt into buckets by id.  The whole order is sorted (Top-p); the kept ids are the same with one
+    bucket for all keys and a prefix of the order that the double-precision kernel gives."""
+    g = torch.Generator(device="cuda").manual_seed(blocks)
+    q, k = ((torch.randn(1, 1, blocks * 128, 128, device="cuda", generator=g) * scale).to(torch.bfloat16) for _ in range(2))
+    order, count, kw = run_kap(q, k, 1.0, stride, order_stride=blocks, top_p=0.95, scores=True)
+    assert int((kw["kap_scores"][0, 0, -1] == 0).sum()) > blocks // 4
+    for impl in (2, 3):
+        order2, count2 = run_kap(q, k, 1.0, stride, order_stride=blocks, impl=impl, top_p=0.95)
+        assert torch.equal(order, order2) and torch.equal(count, count2), impl
+    exact, _ = run_kap(q, k, 1.0, stride, order_stride=blocks, impl=1)
+    kept = torch.arange(blocks, device="cuda") < count[..., None]
+    assert int(count.min()) >= 1 and torch.equal(torch.where(kept, order, -1), torch.where(kept, exact, -1))
+
+
 @pytest.mark.parametrize("n,stride", [(4096, 8), (4224, 8), (2048, 4), (2176, 4), (8192, 16), (8320, 16), (3968, 8), (128, 8)])
 def test_kap_lists_around_the_longest_short_call(n, stride):
     """Calls whose key tiles all fit the screen's stages (512 sampled keys) take another route through the screen: lists on
