@@ -105,7 +105,7 @@ __device__ __forceinline__ int bucket_of(const SortShared* sh, unsigned long lon
 // fits kHeadCap it goes to head[] and a stays as it is; otherwise everything is sorted, in place.  Returns the length of the
 // sorted part and sets *out to it.  tmp: n keys; bucket: n bytes.  one_bucket: as if no splitter were of any use (for
 // tests).  All threads of the CTA call it.
-// What counts is latency and shared-memory traffic: six lists are in work on an SM, each a chain of short steps between
+// What counts is latency and shared-memory traffic: ten lists are in work on an SM (six when this was measured), each a chain of short steps between
 // barriers.  A bitonic network (21 to 55 dependent rounds, one to eight warps) took 6.4 k cycles for 61 keys and 21 k for
 // 512, a selection by pivots followed by a rank sort of the head 10.4 k for 1024; this takes 1.2, 7.8 and 6.6 k (Stage 1
 // at 128K tokens 1540 -> 1425 us, at 64K and 50 % 724 -> 645, at 32K 207 -> 177, 61 blocks 85.5 -> 69.7).

@@ -26,7 +26,7 @@
 // memory, list, first tiles, output, next CTA), three computed blocks' worth.  Asked too early, the last items are dealt out badly:
 // at a walk's start, all blocks of 16K (walks of 1 to 128 blocks) take 3 % longer than when four positions are left.  What
 // runs once an item is cold in the instruction cache and costs by its size: code is shared rather than unrolled or inlined
-// twice wherever a walk passes once (26 KB more: 20 % slower than a CTA an item).
+// twice wherever a walk passes once (a form of 88 KB instead of 61: 236 us instead of 209 on walks of 3.4 blocks).
 // What bounds it: tensor pipe and exponentials both want about 1,024 cycles of an SM per computed block (512 per skipped one);
 // a computed position takes a CTA 4,000 cycles, a skipped one 1,220.  Single launches, a CTA an item -> now: 128K tokens and 4 %
 // computed 7.15 -> 7.07 ms, 32K and 8 % 1.02 -> 0.97, all blocks of 16K 1.85 -> 1.83, walks of 3.4 blocks (2 x 7,808 tokens)
@@ -299,7 +299,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
             if (k >= 0) {
               d = kDecComputed | (k == cnt - 1 ? kDecEnd : 0u);
               if (k == 0 && t == 0) {
-                // (never satisfied on the spot: a wait budget of a few cycles always runs out here)
+                // (polled: a budget of a few cycles must run out here, see cosa_options.wait_cycles, and the wait is long)
                 alive = mbar_poll_warp(smem_u32(kStage2 ? &ctl->dec_bar[0] : &ctl->s_first), 0, abort_flag, budget);
               } else if (kStage2) {
                 alive = wait(&ctl->dec_bar[(pos_base + k) & 1], (pos_base + k) >> 1);

@@ -76,10 +76,9 @@ __device__ __forceinline__ bool mbar_wait_noabort(uint32_t bar, uint32_t parity,
 // `unanimous` is set.  Lanes poll on their own (the cheapest way to wait), so they can see the budget run out at
 // different moments, and what follows -- tcgen05.ld/st, __syncwarp -- must be executed by all lanes or by none.  With
 // the regular budget (about a second) the lanes of a warp, which start their waits within a few cycles of each other,
-// cannot disagree unless the barrier completes in the very cycles in which a second of waiting ends; the vote costs 2 %
-// of the OSK kernel (and a run-time switch more: the kernel is sensitive to its code size), so the kernels exist in
-// two instantiations and the one with the votes is launched when the caller has set a short budget
-// (wait_budget_is_short), where lanes disagreeing is the expected case.
+// cannot disagree unless the barrier completes in the very cycles in which a second of waiting ends.  The OSK's load warp always
+// votes; the screen, in which sixteen warps wait for every tile, has an instantiation with the votes, launched when the
+// caller has set a short budget (wait_budget_is_short), where lanes disagreeing is the expected case.
 __host__ __device__ inline bool wait_budget_is_short(long long budget) { return budget < (1LL << 24); }
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget,
                                                bool unanimous) {
@@ -235,28 +234,6 @@ __device__ __forceinline__ uint64_t l2_policy_evict_first() {
 }
 __device__ __forceinline__ void st_l2_hint(float* ptr, float a, uint64_t pol) {
   asm volatile("st.global.L1::no_allocate.L2::cache_hint.f32 [%0], %1, %2;" ::"l"(ptr), "f"(a), "l"(pol) : "memory");
-}
-__device__ __forceinline__ void st_l2_hint(float2* ptr, float2 a, uint64_t pol) {
-  asm volatile("st.global.L1::no_allocate.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;" ::"l"(ptr), "f"(a.x), "f"(a.y), "l"(pol)
-               : "memory");
-}
-__device__ __forceinline__ void st_l2_hint(float4* ptr, float4 a, uint64_t pol) {
-  asm volatile("st.global.L1::no_allocate.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(ptr), "f"(a.x), "f"(a.y),
-               "f"(a.z), "f"(a.w), "l"(pol)
-               : "memory");
-}
-__device__ __forceinline__ float4 ld_l2_hint(const float4* ptr, uint64_t pol) {
-  float4 a;
-  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
-               : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w)
-               : "l"(ptr), "l"(pol)
-               : "memory");
-  return a;
-}
-__device__ __forceinline__ float ld_l2_hint(const float* ptr, uint64_t pol) {
-  float a;
-  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(a) : "l"(ptr), "l"(pol) : "memory");
-  return a;
 }
 // packed pairs of float32 (sm_100: one instruction works on both halves of a 64-bit register)
 __device__ __forceinline__ unsigned long long pack_f32x2(float a, float b) {

@@ -27,7 +27,7 @@ def _draw_heads(rng):
 
 
 def test_random_kap_routes_agree():
-    """Screen + pivot selection, radix selection, full sort and the fp64 kernel write the same lists (bit-exact)."""
+    """Screen + buckets at the head, all keys in one bucket, full sort and the fp64 kernel write the same lists (bit-exact)."""
     rng = np.random.default_rng(20260725)
     for _ in range(24):
         hq, hkv = _draw_heads(rng)

@@ -43,7 +43,7 @@ def test_kap_wait_budget_of_one_cycle_reports_a_timeout_and_the_next_call_is_cle
     assert torch.equal(order, ref_order) and torch.equal(count, ref_count)
 
 
-@pytest.mark.parametrize("impl", [0, 4, 5])     # one work item per CTA, two work items per CTA, the two row tiles of a 256-row block per CTA
+@pytest.mark.parametrize("impl", [0, 4, 5])     # one work item at a time, two side by side, the two row tiles of a 256-row block per CTA
 def test_osk_wait_budget_of_one_cycle_reports_a_timeout_and_the_next_call_is_clean(cfg1, impl):
     w, (q, k, v) = cfg1["w"], cfg1["dev"]
     nqb = w.n // 128
