@@ -89,4 +89,6 @@ def test_launches_per_step_are_what_a_profiler_counts(n, stride, page_size, in_p
         step()
         torch.cuda.synchronize()
     names = [e.name for e in prof.events() if "cosa" in e.name and e.device_type == torch.autograd.DeviceType.CUDA]
+    if not any(e.device_type == torch.autograd.DeviceType.CUDA for e in prof.events()):
+        pytest.skip("the profiler records no kernels here")
     assert len(names) == bench.launches_per_step(n, stride, page_size, in_place, osk_impl, block_q), names
