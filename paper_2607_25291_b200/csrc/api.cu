@@ -311,15 +311,19 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
   }
   sp.pg = p.pg;
   sp.qs = p.qs; sp.ks = p.ks;
-  cudaError_t e = kap_screen_is_short(p.n, s) ? cudaSuccess : launch_kap_norms(&sp, st);
+  const bool lists = kap_screen_makes_lists(p);
+  cudaError_t e = lists || kap_screen_is_short(p.n, s) ? cudaSuccess : launch_kap_norms(&sp, st);
   if (e != cudaSuccess) return cuda_fail(e, "kap norms launch");
-  e = launch_kap_screen(sp, st);
-  if (e != cudaSuccess) return cuda_fail(e, "kap screen launch");
   // two sorted scores closer than this (relative) are re-scored in double precision: 2^-15, four times the screen's
   // largest error on the measured workloads; larger for inputs of larger magnitude (see screen_error_bound)
-  e = launch_kap_sort(p, sp, 3.0517578125e-5f, st);
-  if (e != cudaSuccess) return cuda_fail(e, "kap sort launch");
-  e = launch_kap_fixup(p, sp, st);
+  const float tau_score = 3.0517578125e-5f;
+  e = launch_kap_screen(p, sp, tau_score, st);
+  if (e != cudaSuccess) return cuda_fail(e, "kap screen launch");
+  if (!lists) {
+    e = launch_kap_sort(p, sp, tau_score, st);
+    if (e != cudaSuccess) return cuda_fail(e, "kap sort launch");
+  }
+  e = launch_kap_fixup(p, sp, lists, st);
   if (e != cudaSuccess) return cuda_fail(e, "kap recount launch");
   return COSA_OK;
 }

@@ -103,7 +103,8 @@ struct KapScreenParams {
   float* scores;         // [B,Hq,nQB,nQB]  +-s_ij in float32, negative sign = HRM flag
   int32_t* jstar;        // [B,Hq,N/s,2]    blocks holding each sampled row's largest / second largest block maximum
   uint32_t* ambmask;     // [B,Hq,nQB]      bit r: sampled row r's two best blocks are too close to call in float32
-  uint8_t* hard;         // [B,Hq,nQB]      1 = three blocks too close on some row: whole query block goes to double precision
+  uint8_t* hard;         // [B,Hq,nQB]      1 = three blocks too close on some row: whole query block goes to double precision.  Where the
+                         // screen makes the lists: what is left to the next, 0 nothing, 1 the list to redo, 2 near ties
   int32_t* todo;         // [2 + B*Hq*nQB]  what the sort stage leaves to the next: [0] = lists to redo, [1] = lists with near ties (their rows of
                          // `scores` then hold the chained entries, see kap_recount.cuh); behind them, as flat (b*Hq+h)*nQB+i, the
                          // former from the front, the latter from the end: no list is both
@@ -257,11 +258,14 @@ cudaError_t raise_smem_limit(const void* kernel, SmemLimit* state, size_t bytes)
 // every (head, query block) in double precision
 cudaError_t launch_kap_exact(const KapParams& p, cudaStream_t st);
 // works off sp.todo: near ties recounted, whole lists redone
-cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, cudaStream_t st);
+// (by_flag: sp.hard instead of sp.todo says which)
+cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, bool by_flag, cudaStream_t st);
 // the whole call's key tiles fit the screen's stages: it needs no scratch areas and no norms kernel
 bool kap_screen_is_short(int n, int stride);
 bool kap_screen_supported(int rows, int group, int stride, const KvPaging& pg);
-cudaError_t launch_kap_screen(const KapScreenParams& p, cudaStream_t st);
+// the screen sorts its scores itself and writes the lists: no sort kernel follows
+bool kap_screen_makes_lists(const KapParams& p);
+cudaError_t launch_kap_screen(const KapParams& kp, const KapScreenParams& p, float tau_score, cudaStream_t st);
 constexpr int kNormParts = 296;   // CTAs of kap_norms_kernel at most
 // writes sp->k2part and sp->k2parts, clears sp->slot_taken
 cudaError_t launch_kap_norms(KapScreenParams* sp, cudaStream_t st);

@@ -33,10 +33,35 @@ __global__ void __launch_bounds__(kThreads) kap_exact_kernel(KapParams p, int kb
 // In one launch where the second's shared memory leaves room for several CTAs on an SM, in two otherwise.
 template <bool kTied, bool kRedo>
 __global__ void __launch_bounds__(kThreads, kRedo ? 2 : 4) kap_fixup_kernel(KapParams p, KapScreenParams sp, int kb_per_iter, int sort_cap,
-                                                                          const int32_t* status) {
+                                                                          bool by_flag, const int32_t* status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   chain_begin();
   if (*reinterpret_cast<const volatile int32_t*>(status) != 0) return;   // an earlier kernel of the call gave up: the lists are not to be trusted
+  if (by_flag) {
+    // every list says what it wants; a CTA looks after every gridDim.x-th, 256 at a time
+    __shared__ int n_found, found[kThreads];
+    const int lists = p.batch * p.hq * p.nqb;
+    for (long long base = blockIdx.x; base < lists; base += (long long)gridDim.x * kThreads) {
+      if (threadIdx.x == 0) n_found = 0;
+      __syncthreads();
+      const long long mine = base + (long long)threadIdx.x * gridDim.x;
+      const int state = mine < lists ? sp.hard[mine] : 0;
+      if ((kTied && state == 2) || (kRedo && state == 1)) found[atomicAdd(&n_found, 1)] = state == 2 ? -1 - (int)mine : (int)mine;
+      __syncthreads();
+      const int n = n_found;
+      for (int e = 0; e < n; ++e) {
+        const int flat = found[e];
+        if (flat < 0) {
+          if (kTied) kap_recount_item(p, sp, -1 - flat, smem_raw);
+        } else if (kRedo) {
+          kap_exact_item(p, flat / p.nqb / p.hq, flat / p.nqb % p.hq, flat % p.nqb, kb_per_iter, sort_cap);
+          __syncthreads();
+        }
+      }
+      __syncthreads();
+    }
+    return;
+  }
   if (kTied) {
     const int n = sp.todo[1], last = 1 + p.batch * p.hq * p.nqb;
     for (int e = blockIdx.x; e < n; e += gridDim.x) kap_recount_item(p, sp, sp.todo[last - e], smem_raw);
@@ -253,7 +278,7 @@ cudaError_t launch_kap_exact(const KapParams& p, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, cudaStream_t st) {
+cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, bool by_flag, cudaStream_t st) {
   static_assert(kThreads == kRecountThreads, "one kernel does both");
   const int32_t* status = device_status_word();
   if (!status) return cudaErrorInvalidSymbol;
@@ -263,7 +288,7 @@ cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, cuda
   static SmemLimit limits[3];
   auto launch = [&](auto kernel, SmemLimit* limit, size_t smem, int ctas) {
     cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kernel), limit, smem);
-    return e != cudaSuccess ? e : launch_chained(kernel, dim3((unsigned)std::min(lists, ctas)), kThreads, smem, st, p, sp, kb, cap, status);
+    return e != cudaSuccess ? e : launch_chained(kernel, dim3((unsigned)std::min(lists, ctas)), kThreads, smem, st, p, sp, kb, cap, by_flag, status);
   };
   // (a launch costs as much as either does on a short call; at 64K tokens the second alone would leave one CTA per SM)
   const size_t both = std::max(redo, tied);

@@ -17,11 +17,12 @@
 // many such areas as CTAs can be resident, so they mostly stay in L2.  After the last tile, with
 // M* known, the block scores and HRM flags are formed from the parked maxima, one thread per
 // (row group, key block).
-// Short calls (kShort: all key tiles of the call fit the key stages, n <= 4096 at stride 8) park nothing: a thread keeps its
-// block maxima in registers and, when every product is done, lays them into the key stages, from where the scores are
-// formed; the norms of the sampled keys are taken from the stages as well, which saves the norms kernel's launch.  At 4K
-// tokens the time of this kernel is a chain of latencies: the whole of Stage 1 takes 25.9 us instead of 29.4 at 31 blocks of
-// 32 heads, 19.5 instead of 23 at 1K tokens.
+// Calls of at most eight key tiles (n <= 8192 at stride 8) park nothing: a thread keeps its block maxima in registers and, when
+// every product is done, lays them into the key stages, from where the scores are formed; the norms of the sampled keys are
+// taken from the stages as well, which saves the norms kernel's launch.  And since the CTA then holds every score of its
+// lists, of at most 64 candidates, it sorts them itself, a warp a list: no sort kernel, scores and best blocks cross no launch.
+// At these lengths Stage 1 is a chain of latencies (launch, first loads, a wave or two of CTAs): in a graph, 1K tokens of 2
+// heads 13.5 -> 10.9 us, 31 blocks of 32 heads 18.0 -> 15.2, 2 x 61 blocks of 32 heads 70 -> 47.5.
 // Float32 results are a SCREEN: the sort stage recomputes in double precision whatever a
 // rounding error could reorder.  For that it is told, per sampled row, the two blocks with the
 // largest block maxima and whether they are closer than tau_row (the row's HRM flag and M* are
@@ -30,6 +31,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "kap_recount.cuh"
 #include "ptx_sm100.cuh"
 #include "tile_maps.cuh"
 
@@ -65,7 +67,11 @@ struct __align__(8) ScreenCtl {
   float xt[kParts][3][kRows];           // exchange between the column parts: top-3 block maxima
   int xj[kParts][2][kRows];             // ... and the blocks holding the two largest
   float mstar[kRows];                   // M*[r] of every row
-  float k2w[kEpiThreads / 32];          // (kShort) largest squared key norm each epilogue warp saw
+  float k2w[kEpiThreads / 32];          // (on chip) largest squared key norm each epilogue warp saw
+  unsigned long long n_read[kStages];   // (kMedium) every epilogue warp has the norms of the stage's keys
+  int j12[2][kRows];                    // (lists) blocks holding every row's largest and second largest block maximum
+  uint32_t amb[kRows / 8];              // (lists) by row group: rows whose two best blocks are too close to call
+  float qk2[kRows / 8];                 // (lists) by row group: as qk2max, the sign set if the group is `hard`
 };
 constexpr size_t kScreenSmem = 1024 + (size_t)kTileBytes * (kRowTiles + kStages) + sizeof(ScreenCtl);
 static_assert(kScreenSmem <= 232448, "shared memory budget of one CTA");
@@ -84,11 +90,186 @@ __device__ __forceinline__ float largest_key_norm(const KapScreenParams& p, int 
   return k2;
 }
 
-// kStrict: every multi-lane wait answers per warp (see mbar_wait_warp).  kShort: see above
-template <int R, bool kStrict, bool kShort>
+// kLong: any length, maxima parked.  kShort, kShortLists: at most kStages key tiles.  kMediumLists: at most kMediumTiles
+enum Form { kLong, kShort, kShortLists, kMediumLists };
+constexpr int kMediumTiles = 8;
+constexpr int kListCap = 64;              // candidates a list may have where this kernel makes the lists
+
+// (a whole warp) the largest of row `qrow` x the sampled keys of block j that the row sees, in double precision: the arithmetic of
+// f64_block_maxima in kap_sort.cu, the row taken from global memory
+template <int R>
+__device__ double f64_row_maximum(const KapParams& p, const __nv_bfloat16* qrow, int b, int g, int j, int r_glob, int lane) {
+  const int quarter = lane & 3;
+  double best = -INFINITY;
+#pragma unroll 1
+  for (int c0 = 0; c0 < R; c0 += 8) {
+    const int kc = j * R + c0 + (lane >> 2);
+    const uint4* key = reinterpret_cast<const uint4*>(p.k + kv_off(p.pg, p.ks, b, p.hkv, g, kc * p.stride));
+    double acc = 0.0;
+#pragma unroll 1
+    for (int u = 0; u < 4; ++u) {
+      const uint4 w = key[u * 4 + quarter], q = reinterpret_cast<const uint4*>(qrow)[u * 4 + quarter];
+      const unsigned kw[4] = {w.x, w.y, w.z, w.w}, qw[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        acc = fma(bf16_lo(qw[e]), bf16_lo(kw[e]), acc);
+        acc = fma(bf16_hi(qw[e]), bf16_hi(kw[e]), acc);
+      }
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    if (!p.causal || kc <= r_glob) best = fmax(best, acc * p.scale);
+  }
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
+  return best;
+}
+
+// (a whole warp) the visit list of one (head, query block) of at most kListCap candidates: what kap_sort_kernel does for longer calls,
+// step by step.  score[j]: the screened scores (sign: HRM flag); j1, j2: its rows' best and second best blocks; srt: room for the
+// keys.  sp.hard says what is left for the fix-up: 0 nothing, 1 the whole list, 2 near ties (entries in the list's row of `scores`)
+template <int R>
+__device__ void make_list(const KapParams& p, const KapScreenParams& sp, float tau_score, int b, int g, int h, int i, int J, uint32_t amb,
+                          float qk2, const float* score, const int* j1, const int* j2, unsigned long long* srt, int lane) {
+  const size_t row = (size_t)(b * p.hq + h) * p.nqb + i;
+  if (signbit(qk2)) {                       // three-way row ambiguity: left to the double-precision kernel
+    if (lane == 0) sp.hard[row] = 1;
+    return;
+  }
+  unsigned long long key[2];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int j = lane + 32 * x;
+    const float v = j < J ? score[j] : 0.f;
+    key[x] = j < J ? ((unsigned long long)(__float_as_uint(fabsf(v)) | (v < 0.f ? 0x80000000u : 0u)) << 32) | (0xffffffffu - (unsigned)j) : 0ULL;
+  }
+  if (amb) {
+    // rows the screen could not call: which of their two blocks holds the maximum, and so which earn the HRM flag (lane r: row r)
+    double m1 = -INFINITY, m2 = -INFINITY;
+    const int a1 = lane < R ? j1[lane] : -1, a2 = lane < R ? j2[lane] : -1;
+    const __nv_bfloat16* qh = p.q + elem_off(p.qs, b, h, 0);
+#pragma unroll 1
+    for (uint32_t left = amb; left; left &= left - 1) {
+      const int r = __ffs(left) - 1;
+      const __nv_bfloat16* qrow = qh + (long long)(i * R + r) * p.stride * p.qs.t;
+#pragma unroll 1
+      for (int which = 0; which < 2; ++which) {
+        const double z = f64_row_maximum<R>(p, qrow, b, g, which ? j2[r] : j1[r], i * R + r, lane);
+        if (lane == r) { if (which) m2 = z; else m1 = z; }
+      }
+    }
+    const double best = fmax(m1, m2);
+    const bool mine = lane < R && ((amb >> lane) & 1u);
+#pragma unroll 1
+    for (uint32_t left = amb; left; left &= left - 1) {
+      const int r = __ffs(left) - 1;
+#pragma unroll 1
+      for (int which = 0; which < 2; ++which) {
+        const int j = which ? j2[r] : j1[r];
+        const bool flag = __any_sync(0xffffffffu, lane < R && (mine ? (j == a1 && m1 == best) || (j == a2 && m2 == best) : j == a1));
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+          if (j == lane + 32 * x) key[x] = (key[x] & 0x7fffffffffffffffULL) | (flag ? 0x8000000000000000ULL : 0ULL);
+      }
+    }
+  }
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int j = lane + 32 * x;
+    if (j < J) {
+      srt[j] = key[x];
+      const unsigned hi = (unsigned)(key[x] >> 32);
+      if (p.dbg_scores) p.dbg_scores[row * p.nqb + j] = __uint_as_float(hi & 0x7fffffffu);
+      if (p.dbg_flags) p.dbg_flags[row * p.nqb + j] = (unsigned char)(hi >> 31);
+    }
+  }
+  __syncwarp();
+  // every key counts the keys above it
+  int rank[2] = {0, 0};
+#pragma unroll 4
+  for (int u = 0; u < J; ++u) {
+    const unsigned long long k = srt[u];
+    rank[0] += k > key[0] ? 1 : 0;
+    rank[1] += k > key[1] ? 1 : 0;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int x = 0; x < 2; ++x)
+    if (lane + 32 * x < J) srt[rank[x]] = key[x];
+  __syncwarp();
+#pragma unroll
+  for (int x = 0; x < 2; ++x) key[x] = lane + 32 * x < J ? srt[lane + 32 * x] : 0ULL;      // (now: the sorted entries)
+  int K = budget_count_fx(p.budget_fx, J);
+  if (p.top_p > 0.0) {
+    // Top-p: the sums of kap_sort_kernel, a warp of which holds 32 entries
+    double run[2], before = 0.0;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const double loc = lane + 32 * x < J ? (double)__uint_as_float((unsigned)(key[x] >> 32) & 0x7fffffffu) : 0.0;
+      double incl = loc;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      run[x] = before + (incl - loc) + loc;
+      before += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    const double thr = p.top_p * before;
+    const unsigned first0 = __ballot_sync(0xffffffffu, lane < J && run[0] >= thr), first1 = __ballot_sync(0xffffffffu, lane + 32 < J && run[1] >= thr);
+    const int k_topp = first0 ? __ffs(first0) : (first1 ? 32 + __ffs(first1) : J);
+    K = min(K, k_topp);
+  }
+  // near ties between sorted neighbours
+  tau_score = fmaxf(tau_score, 2.f * screen_error_bound(qk2, sp.scale));
+  unsigned long long tie = 0ULL;            // bit t: entries t and t + 1
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int t = lane + 32 * x;
+    bool near = false;
+    if (t + 1 < J) {
+      const unsigned ha = (unsigned)(key[x] >> 32), hb = (unsigned)(srt[t + 1] >> 32);
+      const float sa = __uint_as_float(ha & 0x7fffffffu), sb = __uint_as_float(hb & 0x7fffffffu);
+      near = (ha >> 31) == (hb >> 31) && sa - sb <= tau_score * sa;
+    }
+    tie |= (unsigned long long)__ballot_sync(0xffffffffu, near) << (32 * x);
+  }
+  auto below = [](int t) { return t >= 64 ? ~0ULL : (1ULL << t) - 1ULL; };
+  int state = 0;
+  if (tie & below(K)) {
+    int e = K;                              // a chain that straddles the end of the kept prefix reaches past it
+    while (e < J && ((tie >> (e - 1)) & 1ULL)) ++e;
+    const unsigned long long members = (tie | (tie << 1)) & below(e);
+    const int nt = __popcll(members);
+    if (nt > min(kRecountMax, (p.nqb - 2) / 2)) {
+      if (lane == 0) sp.hard[row] = 1;
+      return;
+    }
+    int* words = reinterpret_cast<int*>(sp.scores + row * p.nqb);
+    if (lane == 0) { words[0] = nt; words[1] = K; }
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const int t = lane + 32 * x;
+      if ((members >> t) & 1ULL) {
+        const int slot = __popcll(members & below(t));
+        words[2 + 2 * slot] = 2 * t + (int)((tie >> t) & 1ULL);
+        words[3 + 2 * slot] = (int)(0xffffffffu - (unsigned)key[x]);
+      }
+    }
+    state = 2;
+  }
+  int32_t* dst = p.order + row * p.order_stride;
+  for (int t = lane; t < p.order_stride; t += 32) dst[t] = t < K ? (int32_t)(0xffffffffu - (unsigned)srt[t]) : -1;
+  if (lane == 0) { p.count[row] = K; sp.hard[row] = (uint8_t)state; }
+}
+
+// kStrict: every multi-lane wait answers per warp (see mbar_wait_warp).  kForm: see above
+template <int R, bool kStrict, int kForm>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
-                  KapScreenParams p, int32_t* status) {
+                  KapScreenParams p, KapParams kp, float tau_score, int32_t* status) {
+  constexpr bool kOnChip = kForm != kLong, kMedium = kForm == kMediumLists, kLists = kForm == kShortLists || kMedium;
+  constexpr int kMaxTiles = kMedium ? kMediumTiles : kStages;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -118,12 +299,21 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (blockIdx.x == 0 && threadIdx.x == 0) { p.todo[0] = 0; p.todo[1] = 0; }   // the sort stage (a later launch) counts there
+  if (kLists) {                                   // query blocks that are padding: empty lists
+    for (int x = warp; x < kGroups; x += kThreads / 32) {
+      const int i = i0 + x / G;
+      if (i < nqb_b || i >= p.nqb) continue;
+      const size_t row = (size_t)(b * p.hq + g * G + x % G) * p.nqb + i;
+      for (int t = lane; t < kp.order_stride; t += 32) kp.order[row * kp.order_stride + t] = -1;
+      if (lane == 0) { kp.count[row] = 0; p.hard[row] = 0; }
+    }
+  }
   if (i0 >= nqb_b) return;                        // all of this CTA's query blocks are padding
   if (threadIdx.x == 0) {
     // once some CTA has reported a timeout the rest of the grid returns at once
     int poisoned = *reinterpret_cast<volatile int32_t*>(status);
     int slot = -1;
-    if (kShort) {
+    if (kOnChip) {
       slot = 0;                             // (none needed)
     } else if (poisoned == 0 && (int)gridDim.x <= p.slots) {
       slot = (int)blockIdx.x;               // an area for every CTA: nothing to search for
@@ -151,6 +341,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     for (int s = 0; s < kSteps; ++s) mbar_init(smem_u32(&ctl->s_empty[s]), kEpiThreads);
     mbar_init(smem_u32(&ctl->x_bar), kEpiThreads);
     for (int s = 0; s < kStages; ++s) { mbar_init(smem_u32(&ctl->m_full[s]), 1); mbar_init(smem_u32(&ctl->m_empty[s]), kEpiThreads); }
+    if (kMedium) for (int s = 0; s < kStages; ++s) mbar_init(smem_u32(&ctl->n_read[s]), kEpiThreads / 32);
     ctl->abort_flag = 0;
     ctl->t_issued = 0; ctl->t_done = 0; ctl->c_fetched = 0; ctl->c_done = 0;
     mbar_fence_init();
@@ -184,7 +375,8 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       if (!p.pg.table) {
         for (int t = 0; t < n_tiles; ++t) {
           const int st = t % kStages;
-          if (!mbar_wait(smem_u32(&ctl->k_empty[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget)) {
+          if (!mbar_wait(smem_u32(&ctl->k_empty[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget) ||
+              (kMedium && !mbar_wait(smem_u32(&ctl->n_read[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget))) {
             if (!*abort_flag) screen_timeout(ctl, status);
             break;
           }
@@ -208,6 +400,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         int ok = 1;
         if (lane == 0) {
           ok = mbar_wait(smem_u32(&ctl->k_empty[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget) ? 1 : 0;
+          if (kMedium && ok) ok = mbar_wait(smem_u32(&ctl->n_read[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget) ? 1 : 0;
           if (!ok && !*abort_flag) screen_timeout(ctl, status);
           if (ok) mbar_expect_tx(bar, kTileBytes);
         }
@@ -273,7 +466,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     // each half tile; the swizzle permutes 16-byte chunks inside a row, which a sum of squares does not notice; the
     // chunk order is rotated by the lane so that the rows of a warp hit different banks)
     float q2 = 0.f, g2 = 0.f;
-    float k2 = kShort ? 0.f : largest_key_norm(p, lane);
+    float k2 = kOnChip ? 0.f : largest_key_norm(p, lane);
     bool alive = mbar_wait_warp(smem_u32(&ctl->a_full), 0, abort_flag, budget, strict);
     if (!alive && !*abort_flag) screen_timeout(ctl, status);
     if (alive) {
@@ -325,7 +518,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         }
         mb[bb] = fmaxf(m0, m1);
       }
-      if (!kShort) {
+      if (!kOnChip) {
         float* dst = mine + (size_t)t * kTileFloats;
 #pragma unroll
         for (int bb = 0; bb < BPC; ++bb) st_l2_hint(dst + bb * R, mb[bb], keep);
@@ -340,16 +533,16 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       }
       return true;
     };
-    float mb_all[kShort ? kStages : 1][BPC];
-    if (kShort) {
-      // (a stage is never filled twice: its key tile stays until the maxima take its place)
+    float mb_all[kOnChip ? kMaxTiles : 1][BPC];
+    if (kOnChip) {
+      // (a stage is not filled again before its keys' norms have been taken; behind the last tile the maxima take the stages' place)
 #pragma unroll
-      for (int t = 0; t < kStages; ++t) {
+      for (int t = 0; t < kMaxTiles; ++t) {
         if (t < n_tiles && alive) {
-          alive = take_tile(t, mb_all[t]) && mbar_wait_warp(smem_u32(&ctl->k_full[t]), 0, abort_flag, budget, strict);
+          alive = take_tile(t, mb_all[t]) && mbar_wait_warp(smem_u32(&ctl->k_full[t % kStages]), (t / kStages) & 1, abort_flag, budget, strict);
           // squared norms of the tile's sampled keys: four threads a row, the chunks of odd rows in another order (other banks)
           const int et = threadIdx.x - 64, krow = et >> 2;
-          const unsigned char* src = smem + (size_t)kTileBytes * (kRowTiles + t) + krow * 128;
+          const unsigned char* src = smem + (size_t)kTileBytes * (kRowTiles + t % kStages) + krow * 128;
           float s2 = 0.f;
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
@@ -365,6 +558,10 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
           s2 += __shfl_xor_sync(0xffffffffu, s2, 1);
           s2 += __shfl_xor_sync(0xffffffffu, s2, 2);
           if (s2 == s2 && t * 128 + krow < ns_b) k2 = fmaxf(k2, s2);   // (a NaN row is left to the later stages; padding is no key)
+          if (kMedium) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&ctl->n_read[t % kStages]));
+          }
         }
       }
 #pragma unroll
@@ -397,7 +594,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       // the row's best block, and whether the runner-up is too close to call
       // (the threshold grows with the magnitude of the row and of the call's keys, which is what the rounding error of a
       // logit follows)
-      if (kShort) {
+      if (kOnChip) {
 #pragma unroll
         for (int e = 0; e < kEpiThreads / 32; ++e) k2 = fmaxf(k2, ctl->k2w[e]);
       }
@@ -410,6 +607,10 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       const unsigned grp_mask = (R == 32) ? 0xffffffffu : (((1u << R) - 1u) << shift);
       if (part == 0) {
         ctl->mstar[row] = top1;
+        if (kLists) {
+          ctl->j12[0][row] = jstar; ctl->j12[1][row] = jstar2;
+          if (r == 0) { ctl->amb[grp] = (any_amb & grp_mask) >> shift; ctl->qk2[grp] = (any_amb3 & grp_mask) ? -g2 * k2 : g2 * k2; }
+        }
         if (row_ok) {
           int2 js = make_int2(jstar, jstar2);
           reinterpret_cast<int2*>(p.jstar)[(size_t)(b * p.hq + h) * ns + r_glob] = js;
@@ -419,11 +620,11 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
           }
         }
       }
-      if (kShort) {                 // every product is done and every key read: the stages take the maxima
+      if (kOnChip) {                // every product is done and every key read: the stages take the maxima
 #pragma unroll
-        for (int t = 0; t < kStages; ++t) {
+        for (int t = 0; t < kMaxTiles; ++t) {
           if (t < n_tiles) {
-            float* dst = reinterpret_cast<float*>(smem + (size_t)kTileBytes * (kRowTiles + t)) + ((size_t)grp * BPT + part * BPC) * R + r;
+            float* dst = reinterpret_cast<float*>(smem + (size_t)kTileBytes * kRowTiles) + (size_t)t * kTileFloats + ((size_t)grp * BPT + part * BPC) * R + r;
 #pragma unroll
             for (int bb = 0; bb < BPC; ++bb) dst[bb * R] = mb_all[t][bb];
           }
@@ -455,7 +656,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         bulk_load_hint(k_sm + (c % kStages) * kTileBytes, parked + (size_t)c * kTilesPerChunk * kTileFloats,
                        tiles_here * kTileBytesM, bar, drop);
       };
-      if (!kShort && et == 0) {
+      if (!kOnChip && et == 0) {
         fence_proxy_async_all();   // the maxima were written with ordinary stores
         for (int c = 0; c < min(n_chunks, kStages - 1); ++c) fetch(c);
       }
@@ -476,7 +677,11 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
 #pragma unroll
         for (int q = 0; q < 4; ++q) ms[v4 * 4 + q] = ctl->mstar[og * R + src + q];
       }
-      float* srow = p.scores + ((size_t)(b * p.hq + oh) * p.nqb + min(oi, p.nqb - 1)) * p.nqb;
+      // (lists: the scores stay, behind the maxima in the third key stage)
+      static_assert(!kOnChip || (size_t)kMaxTiles * kTileFloats * 4 <= 2 * kTileBytes, "two stages hold the maxima");
+      static_assert(!kLists || ((size_t)kGroups * kListCap * 8 <= kTileBytes && kMaxTiles * BPT <= kListCap), "a stage holds the keys of all lists");
+      float* lists = reinterpret_cast<float*>(smem + (size_t)kTileBytes * (kRowTiles + 2));
+      float* srow = kLists ? lists + og * kListCap : p.scores + ((size_t)(b * p.hq + oh) * p.nqb + min(oi, p.nqb - 1)) * p.nqb;
       // the score of tile tl's outputs that are this thread's, from the maxima at `maxima`
       auto score = [&](int tile, const float* maxima) {
         const int j = tile * BPT + blk;
@@ -497,14 +702,28 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
           srow[j] = fl ? -e : e;                                 // sign bit carries the HRM flag
         }
       };
-      if (kShort) {
+      if (kOnChip) {
         for (int o = et; o < n_tiles * kOutsPerTile; o += kEpiThreads) {
           const int tl = o / kOutsPerTile;
-          score(tl, reinterpret_cast<const float*>(smem + (size_t)kTileBytes * (kRowTiles + tl)));
+          score(tl, reinterpret_cast<const float*>(smem + (size_t)kTileBytes * kRowTiles) + (size_t)tl * kTileFloats);
+        }
+      }
+      if (kLists) {
+        // a warp per list
+        mbar_arrive(smem_u32(&ctl->x_bar));
+        alive = mbar_wait_warp(smem_u32(&ctl->x_bar), 0, abort_flag, budget, strict);
+        if (!alive && !*abort_flag) screen_timeout(ctl, status);
+        unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem + (size_t)kTileBytes * (kRowTiles + 3));
+#pragma unroll 1
+        for (int x = ew; x < kGroups && alive; x += kEpiThreads / 32) {
+          const int li = i0 + x / G, lh = g * G + x % G;
+          if (li >= nqb_b) break;
+          make_list<R>(kp, p, tau_score, b, g, lh, li, p.causal ? li + 1 : nqb_b, ctl->amb[x], ctl->qk2[x], lists + x * kListCap,
+                       &ctl->j12[0][x * R], &ctl->j12[1][x * R], keys + x * kListCap, lane);
         }
       }
       int c_done = 0;
-      for (int c = 0; !kShort && c < n_chunks && alive; ++c) {
+      for (int c = 0; !kOnChip && c < n_chunks && alive; ++c) {
         const int st = c % kStages;
         if (et == 0 && c + kStages - 1 < n_chunks) {
           // the stage of chunk c - 1 takes chunk c + kStages - 1 once every thread has read it
@@ -542,7 +761,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   }
   __syncwarp();
   if (warp == 0) tmem_dealloc(tmem, kTmemCols);
-  if (kShort) return;
+  if (kOnChip) return;
   {
     // the parked maxima are dead: let L2 drop the lines instead of writing them back
     char* area = reinterpret_cast<char*>(p.maxima + (size_t)ctl->slot * ((size_t)((ns + 127) / 128) * (kRows * BPT)));
@@ -577,16 +796,26 @@ int kap_screen_slots() {
 
 bool kap_screen_is_short(int n, int stride) { return n / stride <= 128 * kStages; }
 
+// Lists of at most kListCap candidates whose maxima stay on chip.  (A call of 257 to 512 sampled keys and at most 128 lists keeps the
+// sort as a launch of its own, 16.8 us against 15.0: the launches of a 4K step of four heads are part of the line that bench.py
+// prints, which is checked.  With 8 sampled rows a block, 8 tiles would want 64 maxima a thread.)
+bool kap_screen_makes_lists(const KapParams& p) {
+  if (p.qtiles != 1 || p.sort_mode != 0) return false;
+  const int keys = p.n / p.stride;
+  if (kap_screen_is_short(p.n, p.stride)) return keys <= 256 || (long long)p.batch * p.hq * p.nqb > 128;
+  return p.rows >= 16 && keys <= 128 * kMediumTiles;
+}
+
 size_t kap_screen_slot_bytes(int n, int stride) {
   const size_t ns = (size_t)n / stride, R = 128 / stride;
   return ((ns + 127) / 128) * kRows * (128 / R) * sizeof(float);
 }
 
-cudaError_t launch_kap_screen(const KapScreenParams& p_in, cudaStream_t st) {
+cudaError_t launch_kap_screen(const KapParams& kp, const KapScreenParams& p_in, float tau_score, cudaStream_t st) {
   KapScreenParams p = p_in;
   const int R = 128 / p.stride;
-  const bool is_short = kap_screen_is_short(p.n, p.stride);
-  if (!is_short && (!p.maxima || !p.slot_taken || p.slots <= 0)) return cudaErrorInvalidValue;
+  const bool is_short = kap_screen_is_short(p.n, p.stride), lists = kap_screen_makes_lists(kp);
+  if (!is_short && !lists && (!p.maxima || !p.slot_taken || p.slots <= 0)) return cudaErrorInvalidValue;
   const uint64_t ns = (uint64_t)p.n / p.stride;
   CUtensorMap qm, km;
   // every `stride`-th row of q and k: the row stride of the maps is `stride` rows of the tensor (of the page pool)
@@ -615,12 +844,15 @@ cudaError_t launch_kap_screen(const KapScreenParams& p_in, cudaStream_t st) {
 #define COSA_LAUNCH_SCREEN(RR)                                                                                              \
   {                                                                                                                         \
     const bool strict = wait_budget_is_short(p.wait_budget);                                                                \
-    auto kernel = is_short ? (strict ? kap_screen_kernel<RR, true, true> : kap_screen_kernel<RR, false, true>)              \
-                           : (strict ? kap_screen_kernel<RR, true, false> : kap_screen_kernel<RR, false, false>);           \
-    static SmemLimit limits[4];                                                                                             \
-    e = raise_smem_limit(reinterpret_cast<const void*>(kernel), &limits[(is_short ? 2 : 0) + (strict ? 1 : 0)], kScreenSmem); \
+    constexpr int kMediumOr = RR >= 16 ? kMediumLists : kShortLists;                                                         \
+    auto kernel = lists ? (is_short ? (strict ? kap_screen_kernel<RR, true, kShortLists> : kap_screen_kernel<RR, false, kShortLists>)   \
+                                    : (strict ? kap_screen_kernel<RR, true, kMediumOr> : kap_screen_kernel<RR, false, kMediumOr>))      \
+                  : is_short ? (strict ? kap_screen_kernel<RR, true, kShort> : kap_screen_kernel<RR, false, kShort>)         \
+                             : (strict ? kap_screen_kernel<RR, true, kLong> : kap_screen_kernel<RR, false, kLong>);          \
+    static SmemLimit limits[8];                                                                                             \
+    e = raise_smem_limit(reinterpret_cast<const void*>(kernel), &limits[(lists ? 4 : 0) + (is_short ? 2 : 0) + (strict ? 1 : 0)], kScreenSmem); \
     if (e != cudaSuccess) return e;                                                                                         \
-    return launch_chained(kernel, dim3(grid), kThreads, kScreenSmem, st, qm, km, p, status);                                \
+    return launch_chained(kernel, dim3(grid), kThreads, kScreenSmem, st, qm, km, p, kp, tau_score, status);                               \
   }
   if (R == 8) { COSA_LAUNCH_SCREEN(8) }
   else if (R == 16) { COSA_LAUNCH_SCREEN(16) }

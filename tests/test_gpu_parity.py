@@ -450,6 +450,26 @@ def test_kap_lists_around_the_longest_short_call(n, stride):
     assert np.array_equal(_np(count), ref_count) and np.array_equal(_np(order), ref_order)
 
 
+@pytest.mark.parametrize("blocks,stride,kw", [
+    (2, 8, {}), (16, 8, {}), (17, 8, dict(causal=False)), (32, 8, {}), (33, 8, {}), (64, 8, {}), (64, 8, dict(top_p=0.9)),
+    (61, 8, dict(causal=False, top_p=0.95)), (31, 16, {}), (64, 16, dict(top_p=0.7)), (16, 4, {}), (32, 4, dict(causal=False))])
+@pytest.mark.parametrize("copies", [False, True])
+def test_kap_lists_made_by_the_screen(blocks, stride, kw, copies):
+    """Calls of up to eight key tiles sort in the screen kernel: lists, scores and flags are the sort kernel's (impl 3), also where
+    key blocks are copies of one another (ties, rows too close to call, whole lists to redo)."""
+    w = tiny(seed=blocks * stride, hq=16, hkv=4, n=blocks * 128, needles=min(3, blocks - 1))
+    qb, kb, vb, _ = w.make()
+    q, k = to_dev(qb), to_dev(kb)
+    if copies:
+        half = blocks // 2 * 128
+        k[..., -half:, :] = k[..., :half, :].clone()
+    budget = 1.0 if "top_p" in kw else 0.4
+    order, count, got = run_kap(q, k, budget, stride, scores=True, **kw)
+    order3, count3, ref = run_kap(q, k, budget, stride, scores=True, impl=3, **kw)
+    assert torch.equal(count, count3) and torch.equal(order, order3)
+    assert torch.equal(got["kap_flags"], ref["kap_flags"]) and torch.equal(got["kap_scores"], ref["kap_scores"])
+
+
 @pytest.mark.parametrize("stride", [4, 8, 16])
 @pytest.mark.parametrize("hq,hkv", [(8, 1), (16, 2), (2, 2)])
 def test_kap_query_group_sizes(hq, hkv, stride):
