@@ -5,9 +5,10 @@
 // -- and two independent walks fill each other's gaps.  An SM's resources are therefore halved: 256 columns of tensor memory,
 // 113 KB of shared memory and 32 K registers per CTA, eight warps:
 //   warps 0..3   one thread per query row: S row to registers, row maximum, vote, exponentials, P, epilogue
-//   warp 4       work items; Q, K and V tiles ("physical jumping": only listed blocks are ever fetched)
+//   warp 4       K and V tiles ("physical jumping": only listed blocks are ever fetched)
 //   warp 5       issues the products
-//   warps 6, 7   idle (they give their registers to the first four)
+//   warp 6       work items: takes them over, looks up their lists, fetches Q
+//   warp 7       idle (warps 4 to 7 give registers to the first four)
 // The running row maxima live in the threads' registers, the tile vote of Eq. (5) is one barrier with an OR over the 128
 // rows, and every thread counts the computed blocks for itself: no exchange between warps beyond that barrier.
 //
@@ -21,12 +22,17 @@
 // goes to Y, and the slots change roles.  Computed: V(k) goes to Y, each 64-key half as soon as the product on the half before
 // it has released it, and K(k+2) to X when Q K^T of k+1 is done.
 // Work items: the grid has one CTA per item, but a CTA that nears the end of its walk takes over one that has not been started
-// (clusterlaunchcontrol): the next walk's list, Q and K tiles are fetched during the last product, and its first S is there when
-// the rows have written the output.  With a CTA an item, start and end of a walk kept a CTA 11,000 cycles busy (barriers, tensor
-// memory, list, first tiles, output, next CTA), three computed blocks' worth.  Asked too early, the last items are dealt out badly:
-// at a walk's start, all blocks of 16K (walks of 1 to 128 blocks) take 3 % longer than when four positions are left.  What
-// runs once an item is cold in the instruction cache and costs by its size: code is shared rather than unrolled or inlined
-// twice wherever a walk passes once (a form of 88 KB instead of 61: 236 us instead of 209 on walks of 3.4 blocks).
+// (clusterlaunchcontrol).  A warp of its own decodes it and looks up its list while the walk before goes on (in the load warp that
+// took 4,900 cycles between the last V tile and the next K tile); Q and K tiles follow when the last Q K^T has released theirs,
+// and the next walk's first S is there when the rows have written the output.  With a CTA an item, start and end of a walk kept a
+// CTA 11,000 cycles busy (barriers, tensor memory, list, first tiles, output, next CTA), three computed blocks' worth.  Asked too
+// early, the last items are dealt out badly: at a walk's start, all blocks of 16K (walks of 1 to 128 blocks) take 3 % longer than
+// when four positions are left.
+// What runs once an item is cold in the instruction cache and costs by its size, and the loop of a computed block (some 22 KB over
+// all roles) loses lines to it: 255 requests an item go to the next cache on walks of 3.4 blocks, 20 a block on long ones.  Code is
+// therefore shared rather than unrolled or inlined twice where walks are short (a form of 88 KB instead of 61: 236 us instead of
+// 209 on walks of 3.4 blocks; one place that fetches K and V tiles instead of two: 175 -> 169, 662 -> 642 on four prompts in
+// 16-token pages); long ones have it written out (kLongWalks).
 // What bounds it: tensor pipe and exponentials both want about 1,024 cycles (0.52 us) of an SM per computed block, 512 per skipped
 // one.  Fitted to single launches at the full clock, an SM takes 1.03 us a computed block with Stage 2 off, 1.19 with it on (the
 // vote keeps the four row warps together), 0.43 a skipped one and 2.2 a work item; the tensor pipe is busy half of the time, and
@@ -59,23 +65,29 @@ constexpr int kHalfKeys = kBlock / 2;
 constexpr int kThreads = 256;
 constexpr int kCtasPerSm = 2;
 constexpr int kTmemCols = 256;
-constexpr int kLoadWarp = 4, kMmaWarp = 5;
+constexpr int kLoadWarp = 4, kMmaWarp = 5, kItemWarp = 6;
 constexpr int kAskAhead = 4;                       // positions (or two computed blocks) before a walk's end at which more work is asked for
+constexpr int kShortWalk = 64, kShortWalkAll = 32;  // list pitch up to which walks count as short, with and without Stage 2
 constexpr uint32_t kDecComputed = 1, kDecEnd = 2;
 constexpr int kTimedOut = 1, kPoisoned = 2;
 
-struct Item {                      // a work item as the load warp hands it to the others
-  int b, h, i;                     // batch item (< 0: there are no more), query head, query block
+struct __align__(16) Item {        // a work item as the item warp hands it to the others
+  int row;                         // (batch item * query heads + query head) * query blocks + query block; < 0: there are no more
   int cnt, cap;                    // listed blocks, computed blocks at which Stage 2 ends the walk
+  float theta2;                    // ln(Delta / N) in base 2, -inf where the test is off
+  int j0, j1;                      // the first two listed blocks
+  long long out_at;                // element offset of the item's first output row
+  int b, g, i;                     // batch item, KV head, query block
   int q;                           // which Q tile it is
-  float theta2;                    // ln(Delta / N) in base 2
 };
+static_assert(sizeof(Item) == 48, "three 16-byte reads");
 
 struct __align__(16) Control {
   unsigned long long grant[2];     // the grid's answer to a request for another work item (16 bytes)
   unsigned long long grant_bar;    // it has come
   unsigned long long item_bar[2];  // the t-th work item (by parity of t) is in item[]
-  unsigned long long empty_done;   // rows and issuing thread are done with an item that has no blocks
+  unsigned long long item_read[2]; // ... and has been read by every role
+  unsigned long long q_free;       // every Q K^T of a walk has finished
   unsigned long long q_full;       // the item's Q tile has landed
   unsigned long long k_full[2];    // K(k) has landed (by parity of k)
   unsigned long long v_full[2];    // by half: the n-th V tile's half has landed
@@ -92,7 +104,7 @@ struct __align__(16) Control {
   volatile int req[6];             // requested by the time the load warp left: K tiles by parity, V tiles by half, Q tiles, work items
   volatile int diag[2];            // K(k) (by parity of k) is the diagonal block
   volatile uint32_t dec[2];
-  volatile Item item[2];
+  Item item[2];
 };
 
 constexpr size_t kSmemBytes = (size_t)kTileBytes * 3 + kHalfBytes + sizeof(Control);
@@ -113,7 +125,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 //          of the load warp issue side by side, each after its own table look-up.  Boxes land on 1024-byte boundaries of
 //          the tile (pages of at least 8 tokens), where the 128-byte swizzle, a function of the shared-memory address,
 //          gives the layout of the one-piece tile.
-template <bool kMask, bool kStage2, bool kSmallPages>
+// kLongWalks: copies of the code that runs once a position or once an item are written out (see above); else they are shared
+template <bool kMask, bool kStage2, bool kSmallPages, bool kLongWalks>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
               const __grid_constant__ CUtensorMap v_map, OskParams p, int32_t* status) {
@@ -133,9 +146,32 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
   const int G = p.hq / p.hkv;
   chain_wait();
 
-  // work items: KV head major, then query blocks from the longest list down, the group's query heads innermost, so that CTAs
-  // resident together read the same K/V pages
-  int b = 0, g = 0, h = 0, i = 0;          // (load warp) the item
+  // (whole warp) rows [first, first + rows) of key block j of K or V to dst, box after box: `box` bytes from one 64-column half
+  // of d to the other.  Lane 0 arms the barrier; with small pages every lane then fetches one page's part
+  int b = 0, g = 0, i = 0;                 // (load warp, item warp) batch item, KV head, query block
+  // (whole warp) part 0 or 1: that half of V's key block j to tile slot `slot`; part 2: K's key block j as tile K(k), box after box
+  auto fetch = [&](int part, int j, int slot, int k) {
+    const bool is_k = part == 2;
+    const CUtensorMap* map = is_k ? &k_map : &v_map;
+    const uint32_t bar = smem_u32(is_k ? &ctl->k_full[k & 1] : &ctl->v_full[part]);
+    const uint32_t dst = x_sm + slot * kTileBytes + (part == 1 ? kHalfBytes : 0), box = is_k ? kHalfBytes : kQuarterBytes;
+    const int row0 = j * kBlock + (part == 1 ? kHalfKeys : 0);
+    if (lane == 0) {
+      if (is_k) ctl->diag[k & 1] = p.causal && j == i;
+      mbar_expect_tx(bar, 2 * box);
+    }
+    if (kSmallPages) __syncwarp();
+    const int rows = is_k ? kBlock : kHalfKeys, ps = kSmallPages ? min(p.pg.page_size, rows) : rows, at = lane * ps;
+    if (at < rows) {                      // (a page holds whole key blocks: lane 0 alone)
+      const KvCoord c = kv_coord(p.pg, b, g, row0 + at);
+#pragma unroll
+      for (int x = 0; x < 2; ++x)
+        tma_load_tile(dst + x * box + at * 128, map, x * 64, c.row, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
+    }
+  };
+  // (item warp) work items: KV head major, then query blocks from the longest list down, the group's query heads innermost, so
+  // that CTAs resident together read the same K/V pages
+  int h = 0;
   auto decode = [&](int w) {
     const int per_kv = G * p.nqb, bg = w / per_kv, wk = w - bg * per_kv, back = wk / G;
     b = bg / p.hkv;
@@ -152,51 +188,20 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
     else if (!kMask && lane < 3 && lane <= p.order_stride) v = p.order[row * p.order_stride + lane - 1];
     return v;
   };
-  int head = 0;
-  if (warp == kLoadWarp) { decode(blockIdx.x); head = look_up(); }
-
-  // (whole load warp) rows [first, first + rows) of key block j of K or V to dst, box after box: `box` bytes from one 64-column half
-  // of d to the other.  Lane 0 arms the barrier; with small pages every lane then fetches one page's part
-  auto fetch = [&](const CUtensorMap* map, unsigned long long* bar_ptr, int j, int first, int rows, uint32_t dst, uint32_t box) {
-    const uint32_t bar = smem_u32(bar_ptr);
-    if (lane == 0) {
-      mbar_expect_tx(bar, 2 * box);
-      if (!kSmallPages) {                 // a page holds whole key blocks
-        const KvCoord c = kv_coord(p.pg, b, g, j * kBlock + first);
-        tma_load_tile(dst, map, 0, c.row, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
-        tma_load_tile(dst + box, map, 64, c.row, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
-      }
-    }
-    if (kSmallPages) {
-      __syncwarp();
-      const int ps = min(p.pg.page_size, rows), part = lane * ps;
-      if (part < rows) {
-        const KvCoord c = kv_coord(p.pg, b, g, j * kBlock + first + part);
-        tma_load_tile(dst + part * 128, map, 0, c.row, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
-        tma_load_tile(dst + box + part * 128, map, 64, c.row, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
-      }
-    }
-  };
-  auto fetch_k = [&](int k, int j, int slot) {
-    if (lane == 0) ctl->diag[k & 1] = p.causal && j == i;
-    fetch(&k_map, &ctl->k_full[k & 1], j, 0, kBlock, x_sm + slot * kTileBytes, kHalfBytes);
-  };
-  auto fetch_v = [&](int half, int j, int slot) {
-    fetch(&v_map, &ctl->v_full[half], j, half * kHalfKeys, kHalfKeys, x_sm + slot * kTileBytes + half * kHalfBytes, kQuarterBytes);
-  };
   auto fetch_q = [&]() {                  // (one lane)
     mbar_expect_tx(smem_u32(&ctl->q_full), kTileBytes);
     tma_load_tile(q_sm, &q_map, 0, i * kBlock, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->q_full));
     tma_load_tile(q_sm + kHalfBytes, &q_map, 64, i * kBlock, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->q_full));
   };
+  int head = 0;
+  if (warp == kItemWarp) { decode(blockIdx.x); head = look_up(); }
   auto clamp_id = [&](int j) { return min(max(j, 0), p.nqb - 1); };
 
-  if (warp == kLoadWarp) {
+  if (warp == kItemWarp) {
     if (lane == 0) {
-      mbar_init(smem_u32(&ctl->grant_bar), 1); mbar_init(smem_u32(&ctl->empty_done), 2);
-      mbar_init(smem_u32(&ctl->q_full), 1);
+      mbar_init(smem_u32(&ctl->grant_bar), 1); mbar_init(smem_u32(&ctl->q_full), 1); mbar_init(smem_u32(&ctl->q_free), 1);
       for (int s = 0; s < 2; ++s) {
-        mbar_init(smem_u32(&ctl->item_bar[s]), 1);
+        mbar_init(smem_u32(&ctl->item_bar[s]), 1); mbar_init(smem_u32(&ctl->item_read[s]), kBlock + 2);
         mbar_init(smem_u32(&ctl->k_full[s]), 1); mbar_init(smem_u32(&ctl->v_full[s]), 1);
         mbar_init(smem_u32(&ctl->dec_bar[s]), 1); mbar_init(smem_u32(&ctl->p_full[s]), kBlock);
         mbar_init(smem_u32(&ctl->pv_done[s]), 1);
@@ -226,58 +231,106 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
 
   if (warp >= kLoadWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-    if (warp == kLoadWarp) {
-      // ---------------------------------------------------------------- work items, tiles
-      // Counters run on from walk to walk, as the barriers' phases do: tiles K(k), positions decided, blocks computed before
-      // this walk.  All roles count alike.
-      // (one answer per warp: all lanes fetch together)
-      auto wait = [&](unsigned long long* bar, int phase) { return mbar_wait_warp(smem_u32(bar), phase & 1, abort_flag, budget, true); };
-      // Further items come from the grid itself, in launch order, as long as CTAs of it are waiting for an SM.  (A grid that fits
-      // on the chip asks for none: a CTA might take what an SM is about to start)
-      const bool ask = (int)gridDim.x > p.wave;
-      BlockWalk walk;                          // (kMask only)
-      int n_q = 1, n_k = 0, n_v = 0, n_grant = 0;   // requested (Q: the first above)
-      int n_walk = 0, n_empty = 0;             // items with and without blocks
-      int y = 0;                               // slot that takes the next V tile (or K tile after a skipped block)
-      bool v_in_y = false;                     // slot y holds, or held last, the V tile of the last computed block
-      int k_base = 0, pos_base = 0, n_base = 0;
+    // (one answer per warp: all lanes fetch together)
+    auto wait = [&](unsigned long long* bar, int phase) { return mbar_wait_warp(smem_u32(bar), phase & 1, abort_flag, budget, true); };
+    // Further items come from the grid itself, in launch order, as long as CTAs of it are waiting for an SM.  (A grid that fits
+    // on the chip asks for none: a CTA might take what an SM is about to start)
+    const bool ask = (int)gridDim.x > p.wave;
+    if (warp == kItemWarp) {
+      // ---------------------------------------------------------------- work items, Q tiles
+      // These waits last as long as a walk does, however short the steps of the others are: the caller's budget is theirs, and this
+      // warp leaves when one of them has run out
+      auto wait = [&](unsigned long long* bar, int phase) {
+        return mbar_wait_warp(smem_u32(bar), phase & 1, abort_flag, max(budget, 1LL << 31), true);
+      };
+      int n_q = 1, n_walk = 0;                 // Q tiles requested (the first above), items with blocks
       int b_known = -1, nqb_b = 0;             // batch item of the lengths below
-      float theta2 = 0.f;
+      float theta2 = -INFINITY;
       bool alive = true, more = true;
-      for (int t = 0; alive; ++t) {
+      for (int t = 0;; ++t) {
         const int raw_cnt = __shfl_sync(0xffffffffu, head, 0);
-        // key blocks of positions k, k + 1 and k + 2 (the last one requested a turn ahead), k starting at -2
-        int j0 = 0, j1 = 0, j2 = __shfl_sync(0xffffffffu, head, 1), j3 = __shfl_sync(0xffffffffu, head, 2);
+        int j0 = __shfl_sync(0xffffffffu, head, 1), j1 = __shfl_sync(0xffffffffu, head, 2);
         if (__shfl_sync(0xffffffffu, head, 3) != 0) {
           more = false;
           if (t == 0) *abort_flag = kPoisoned; // (Q has been requested for nothing)
         }
-        int cnt = 0, cap = 0, n_pos = 0;
+        int cnt = 0, cap = 0;
         if (more) {
           if (b != b_known) {
             b_known = b;
             nqb_b = item_blocks(p.pg, b, p.nqb);   // the item's own length in blocks; query blocks past it are padding
-            theta2 = (p.use_threshold ? item_theta(p.pg, b, p.theta, p.skip_scale, nqb_b) : 0.f) * 1.4426950408889634f;
+            // a batch item no longer than Delta would have ln(Delta/N) >= 0 and lose even its first block: the test is off for it
+            const float th = p.use_threshold ? item_theta(p.pg, b, p.theta, p.skip_scale, nqb_b) : 0.f;
+            theta2 = th < 0.f ? th * 1.4426950408889634f : -INFINITY;
           }
           const int J = p.causal ? i + 1 : max(nqb_b, 1);
-          if (kMask) walk.init(p, (size_t)(b * p.hq + h) * p.nqb + i, J);
-          cnt = i >= nqb_b ? 0 : (kMask ? min(walk.kept(), p.order_stride) : max(0, min(raw_cnt, p.order_stride)));
-          cap = p.stage2 ? min(cnt, budget_count_fx(p.cap_fx, J)) : cnt;
-          n_pos = cap > 1 ? cnt : min(cnt, 1);  // positions the walk can reach (the first block is always computed: with a cap of 1 the walk ends there)
-          if (kMask && cnt > 0) { j2 = walk.at(0); j3 = cnt > 1 ? walk.at(1) : 0; }
-          if (n_pos > 0 && t > 0) {             // Q's tile and slot y are free when the last Q K^T of the walk before has finished
-            if (k_base > 0) alive = wait(&ctl->s_full, k_base - 1);
-            if (!alive) break;
-            if (lane == 0) fetch_q();
-            ++n_q;
+          if (kMask) {
+            BlockWalk walk;
+            walk.init(p, (size_t)(b * p.hq + h) * p.nqb + i, J);
+            cnt = i >= nqb_b ? 0 : min(walk.kept(), p.order_stride);
+          } else {
+            cnt = i >= nqb_b ? 0 : max(0, min(raw_cnt, p.order_stride));
           }
+          cap = p.stage2 ? min(cnt, budget_count_fx(p.cap_fx, J)) : cnt;
         }
+        if (t >= 2) alive = wait(&ctl->item_read[t & 1], (t >> 1) - 1);   // the item before the last has been read
+        if (!alive) break;
+        const bool next_q = cnt > 0 && t > 0;
         if (lane == 0) {
-          volatile Item* it = &ctl->item[t & 1];
-          it->b = more ? b : -1; it->h = h; it->i = i; it->cnt = cnt; it->cap = cap; it->q = n_q - 1; it->theta2 = theta2;
+          Item* it = &ctl->item[t & 1];
+          it->row = more ? (b * p.hq + h) * p.nqb + i : -1;
+          it->cnt = cnt; it->cap = cap; it->theta2 = theta2; it->j0 = j0; it->j1 = j1;
+          it->out_at = more ? elem_off(p.os, b, h, i * kBlock) : 0;
+          it->b = b; it->g = g; it->i = i; it->q = next_q ? n_q : n_q - 1;
           mbar_arrive(smem_u32(&ctl->item_bar[t & 1]));
         }
         if (!more) break;
+        if (next_q) {                           // its tile is free when the last Q K^T of the walk before has finished
+          if (n_walk > 0) alive = wait(&ctl->q_free, n_walk - 1);
+          if (!alive) break;
+          if (lane == 0) fetch_q();
+          ++n_q;
+        } else if (t == 0 && cnt == 0) {
+          alive = wait(&ctl->q_full, 0);        // (requested before the count was known)
+          if (!alive) break;
+        }
+        if (cnt > 0) ++n_walk;
+        more = false;
+        if (ask) {
+          alive = wait(&ctl->grant_bar, t);
+          if (!alive) break;
+          const int w2 = granted_work(smem_u32(ctl->grant));
+          more = w2 >= 0;
+          head = 0;
+          if (more) { decode(w2); head = look_up(); }
+        }
+      }
+      if (lane == 0) {
+        if (!alive && !*abort_flag) *abort_flag = kTimedOut;
+        ctl->req[4] = n_q;
+      }
+    } else if (warp == kLoadWarp) {
+      // ---------------------------------------------------------------- tiles
+      // Counters run on from walk to walk, as the barriers' phases do: tiles K(k), positions decided, blocks computed before
+      // this walk.  All roles count alike.
+      BlockWalk walk;                          // (kMask only)
+      int n_k = 0, n_v = 0, n_grant = 0;       // requested
+      int n_walk = 0;                          // items with blocks
+      int y = 0;                               // slot that takes the next V tile (or K tile after a skipped block)
+      bool v_in_y = false;                     // slot y holds, or held last, the V tile of the last computed block
+      int k_base = 0, pos_base = 0, n_base = 0;
+      bool alive = true;
+      for (int t = 0; alive; ++t) {
+        alive = wait(&ctl->item_bar[t & 1], t >> 1);
+        if (!alive) break;
+        const uint32_t at = smem_u32(&ctl->item[t & 1]);
+        const uint4 f0 = ld_shared_128(at), f1 = ld_shared_128(at + 16), f2 = ld_shared_128(at + 32);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&ctl->item_read[t & 1]));
+        const int row = (int)f0.x, cnt = (int)f0.y, cap = (int)f0.z;
+        if (row < 0) break;
+        b = (int)f2.x; g = (int)f2.y; i = (int)f2.z;
+        const int n_pos = cap > 1 ? cnt : min(cnt, 1);   // positions the walk can reach (the first block is always computed: with a cap of 1 the walk ends there)
         bool asked = !ask;
         auto request = [&]() {
           asked = true;
@@ -288,42 +341,52 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
             request_work(smem_u32(ctl->grant), smem_u32(&ctl->grant_bar));
           }
         };
-        if (n_pos == 0) {
-          if (t == 0) alive = wait(&ctl->q_full, 0);          // (requested before the count was known)
-          if (alive) alive = wait(&ctl->empty_done, n_empty++);
-        } else {
-          const int32_t* list = p.order + ((size_t)(b * p.hq + h) * p.nqb + i) * p.order_stride;   // unused when kMask
+        if (n_pos > 0) {
+          // key blocks of positions k, k + 1 and k + 2 (the last one requested a turn ahead), k starting at -2
+          int j0 = 0, j1 = 0, j2 = (int)f1.x, j3 = (int)f1.y;
+          if (kMask) {
+            walk.init(p, (size_t)row, p.causal ? i + 1 : max(item_blocks(p.pg, b, p.nqb), 1));
+            j2 = walk.at(0);
+            j3 = cnt > 1 ? walk.at(1) : 0;
+          }
+          // slot y is free when the last Q K^T of the walk before has finished
+          if (k_base > 0) alive = wait(&ctl->s_full, k_base - 1);
+          const int32_t* list = p.order + (size_t)row * p.order_stride;   // unused when kMask
           // Turn k fetches V(k) and K(k + 2); turns -2 and -1: the first two K tiles, K(1) to the slot of the last V tile of the walk
           // before
           int k = -2, n = 0;                    // n: computed blocks before position k
           const bool v_before = v_in_y;
           v_in_y = false;
-          while (true) {
+          while (alive) {
             uint32_t d = 0;
             if (k >= 0) {
               d = kDecComputed | (k == cnt - 1 ? kDecEnd : 0u);
               if (k == 0 && t == 0) {
                 // (polled: a budget of a few cycles must run out here, see cosa_options.wait_cycles, and the wait is long)
                 alive = mbar_poll_warp(smem_u32(kStage2 ? &ctl->dec_bar[0] : &ctl->s_first), 0, abort_flag, budget);
-              } else if (kStage2) {
-                alive = wait(&ctl->dec_bar[(pos_base + k) & 1], (pos_base + k) >> 1);
-              } else if (k == 0) {
-                alive = wait(&ctl->s_first, n_walk);
+              } else if (kStage2 || k == 0) {
+                alive = wait(kStage2 ? &ctl->dec_bar[(pos_base + k) & 1] : &ctl->s_first, kStage2 ? (pos_base + k) >> 1 : n_walk);
               }
               if (kStage2) d = ctl->dec[(pos_base + k) & 1];
-              if (d & kDecComputed) {
-#pragma unroll 1
-                for (int half = 0; half < 2 && alive; ++half) {
-                  if (v_in_y) alive = wait(&ctl->pv_done[half], n_base + n - 1);
-                  if (alive) { fetch_v(half, clamp_id(j0), y); ++n_v; }
-                }
-              }
             }
             const bool computed = (d & kDecComputed) != 0;
-            if (alive && !(d & kDecEnd) && k + 2 < n_pos) {
-              if (computed) alive = wait(&ctl->s_full, k_base + k + 1);
-              else if (k == -1 ? v_before : v_in_y) alive = wait(&ctl->pv_done[1], n_base + n - 1);
-              if (alive) { fetch_k(k_base + k + 2, clamp_id(j2), computed || k == -1 ? y ^ 1 : y); ++n_k; }
+            // parts 0 and 1: the halves of V(k), each into a place that the product before has released; part 2: K(k + 2), into that of
+            // K(k + 1) or of the last V tile
+            const bool want_k = !(d & kDecEnd) && k + 2 < n_pos;
+            auto do_part = [&](int part) {
+              const bool is_k = part == 2, after_qk = is_k && computed;
+              if (after_qk || (is_k && k == -1 ? v_before : v_in_y))
+                alive = wait(after_qk ? &ctl->s_full : &ctl->pv_done[is_k ? 1 : part], after_qk ? k_base + k + 1 : n_base + n - 1);
+              if (!alive) return;
+              if (is_k) ++n_k; else ++n_v;
+              fetch(part, clamp_id(is_k ? j2 : j0), is_k && (computed || k == -1) ? y ^ 1 : y, k_base + k + 2);
+            };
+            if (!kLongWalks) {
+#pragma unroll 1
+              for (int part = computed ? 0 : 2; alive && part < (want_k ? 3 : 2); ++part) do_part(part);
+            } else {
+              if (computed) { do_part(0); if (alive) do_part(1); }
+              if (alive && want_k) do_part(2);
             }
             if (!alive) break;
             if (!asked && (k + kAskAhead >= n_pos || n + 2 >= cap)) request();
@@ -338,21 +401,11 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
           ++n_walk;
           y ^= 1;                               // (v_in_y: of the slot that is y ^ 1 from here on)
         }
-        if (alive) {
-          more = false;
-          if (ask) {
-            if (!asked) request();
-            alive = wait(&ctl->grant_bar, n_grant - 1);
-            const int w2 = granted_work(smem_u32(ctl->grant));
-            more = alive && w2 >= 0;
-            head = 0;
-            if (more) { decode(w2); head = look_up(); }
-          }
-        }
+        if (alive && !asked) request();
       }
       if (lane == 0) {
         if (!alive && !*abort_flag) *abort_flag = kTimedOut;
-        ctl->req[0] = (n_k + 1) / 2; ctl->req[1] = n_k / 2; ctl->req[2] = (n_v + 1) / 2; ctl->req[3] = n_v / 2; ctl->req[4] = n_q; ctl->req[5] = n_grant;
+        ctl->req[0] = (n_k + 1) / 2; ctl->req[1] = n_k / 2; ctl->req[2] = (n_v + 1) / 2; ctl->req[3] = n_v / 2; ctl->req[5] = n_grant;
       }
     } else if (warp == kMmaWarp && lane == 0) {
       // ---------------------------------------------------------------- products
@@ -374,11 +427,14 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       for (int t = 0;; ++t) {
         alive = wait(&ctl->item_bar[t & 1], t >> 1);
         if (!alive) break;
-        volatile Item* it = &ctl->item[t & 1];
-        const int cnt = it->cnt, n_pos = it->cap > 1 ? cnt : min(cnt, 1);
-        if (it->b < 0) break;
-        if (n_pos == 0) { mbar_arrive(smem_u32(&ctl->empty_done)); continue; }
-        alive = wait(&ctl->q_full, it->q);
+        const uint32_t at = smem_u32(&ctl->item[t & 1]);
+        const uint4 f0 = ld_shared_128(at);
+        const int q = (int)ld_shared_128(at + 32).w;
+        mbar_arrive(smem_u32(&ctl->item_read[t & 1]));
+        const int cnt = (int)f0.y, n_pos = (int)f0.z > 1 ? cnt : min(cnt, 1);
+        if ((int)f0.x < 0) break;
+        if (n_pos == 0) continue;
+        alive = wait(&ctl->q_full, q);
         int k = -1, n = 0;
         while (alive) {
           if (k >= 0) alive = wait(&ctl->s_read, pos_base + k);
@@ -394,6 +450,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
             d = ctl->dec[(pos_base + k) & 1];
           }
           if (!alive) break;
+          if (d & kDecEnd) mma_commit(smem_u32(&ctl->q_free));   // (Q K^T of a position that is not reached included)
           if (d & kDecComputed) {
 #pragma unroll 1
             for (int half = 0; half < 2 && alive; ++half) {
@@ -437,28 +494,28 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
     for (int t = 0;; ++t) {
       wait(&ctl->item_bar[t & 1], t >> 1);
       if (bar_red_or(1, kBlock, bad || *abort_flag)) break;
-      volatile Item* it = &ctl->item[t & 1];
-      const int b = it->b, h = it->h, i = it->i, cnt = it->cnt, cap = it->cap;
-      const float theta2 = it->theta2;
-      if (b < 0) break;
-      const size_t row = (size_t)(b * p.hq + h) * p.nqb + i;
-      const size_t lse_at = (size_t)(b * p.hq + h) * p.n + i * kBlock + r;
+      const uint32_t at = smem_u32(&ctl->item[t & 1]);
+      const uint4 f0 = ld_shared_128(at), f1 = ld_shared_128(at + 16);
+      mbar_arrive(smem_u32(&ctl->item_read[t & 1]));
+      const int cnt = (int)f0.y, cap = (int)f0.z;
+      const float theta2 = __uint_as_float(f0.w);
+      if ((int)f0.x < 0) break;
+      const size_t row = f0.x;
+      const size_t lse_at = row * kBlock + r;
+      __nv_bfloat16* const out_tile = p.out + (long long)(((unsigned long long)f1.w << 32) | f1.z);
       if (cnt == 0) {
         // an empty list (not produced by KAP except for padding): zero output, nothing visited
         uint4 z = make_uint4(0, 0, 0, 0);
-        uint4* dst = reinterpret_cast<uint4*>(p.out + elem_off(p.os, b, h, i * kBlock + r));
+        uint4* dst = reinterpret_cast<uint4*>(out_tile + r * p.os.t);
 #pragma unroll 1
         for (int c = 0; c < kHeadDim / 8; ++c) dst[c] = z;
         if (p.lse) p.lse[lse_at] = -INFINITY;
         if (r == 0) {
           if (p.visited) p.visited[row] = 0;
           if (p.scored) p.scored[row] = 0;
-          mbar_arrive(smem_u32(&ctl->empty_done));
         }
         continue;
       }
-      // a batch item no longer than Delta would have ln(Delta/N) >= 0 and lose even its first block: the test is off for it
-      const bool thr_on = p.use_threshold && theta2 < 0.f;
       float m = -INFINITY;                      // running row maximum (base 2)
       float l = 0.f;                            // row sum
       int n = 0, kk = 0;                        // computed blocks, list position
@@ -491,7 +548,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         if (kStage2) {
           // Eq. (5): skip iff max over the 128 rows of (m_loc - m) < ln(Delta/N), m including this block.  (Rows of a walk that was given
           // up vote on as long as their list lasts: nothing holds them any more)
-          const bool compute = bar_red_or(1, kBlock, !(thr_on && (m_loc - m_new) < theta2));
+          const bool compute = bar_red_or(1, kBlock, !((m_loc - m_new) < theta2));
           last = last || n + (compute ? 1 : 0) == cap;
           if (r == 0) {
             ctl->dec[(pos_base + kk) & 1] = (compute ? kDecComputed : 0u) | (last ? kDecEnd : 0u);
@@ -569,16 +626,19 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       // of a warp go out through the warp's own rows of P, 64 columns at a time, so that a store covers whole 128-byte lines
       // and no warp waits for another
       n_base += n;
+      const float lse = (m + log2f(l)) * 0.6931471805599453f;
       wait(&ctl->pv_done[1], n_base - 1);
       const int n_pos = cap > 1 ? cnt : 1, n_issued = min(kk + 2, n_pos);   // (Q K^T of a position that was not reached: done, too)
       k_base += n_issued; pos_base += kk + 1;
-      if (bar_red_or(1, kBlock, bad || *abort_flag)) break;
+      // (a warp that sees the walk given up writes nothing; all leave at the next barrier)
+      if (__any_sync(0xffffffffu, bad || *abort_flag)) continue;
       tc_fence_after();
-      const float inv = l > 0.f ? 1.f / l : 0.f;
+      const float inv = l > 0.f ? __frcp_rn(l) : 0.f;
+      const unsigned long long inv2 = pack_f32x2(inv, inv);
       unsigned char* stage = smem + 3 * kTileBytes + warp * 4096;
-      __nv_bfloat16* out = p.out + elem_off(p.os, b, h, i * kBlock + warp * 32 + (lane >> 3)) + (lane & 7) * 8;
-      const long long out_step = elem_off(p.os, b, h, 4) - elem_off(p.os, b, h, 0);
-#pragma unroll 1
+      __nv_bfloat16* out = out_tile + (warp * 32 + (lane >> 3)) * p.os.t + (lane & 7) * 8;
+      const long long out_step = 4 * p.os.t;
+#pragma unroll (kLongWalks ? 2 : 1)
       for (int half = 0; half < 2; ++half) {
         uint32_t o[64];
         tmem_ld32(tmem_o + lane_addr + half * 64, *reinterpret_cast<uint32_t(*)[32]>(&o[0]));
@@ -586,26 +646,29 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         tmem_wait_ld();
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-          const uint32_t* e = &o[c * 8];
-          uint4 pk;
-          pk.x = pack_bf16(__uint_as_float(e[0]) * inv, __uint_as_float(e[1]) * inv);
-          pk.y = pack_bf16(__uint_as_float(e[2]) * inv, __uint_as_float(e[3]) * inv);
-          pk.z = pack_bf16(__uint_as_float(e[4]) * inv, __uint_as_float(e[5]) * inv);
-          pk.w = pack_bf16(__uint_as_float(e[6]) * inv, __uint_as_float(e[7]) * inv);
-          *reinterpret_cast<uint4*>(stage + lane * 128 + ((c ^ (lane & 7)) << 4)) = pk;
+          uint32_t pk[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float lo, hi;
+            unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(o[c * 8 + 2 * e]), __uint_as_float(o[c * 8 + 2 * e + 1])), inv2), lo, hi);
+            pk[e] = pack_bf16(lo, hi);
+          }
+          *reinterpret_cast<uint4*>(stage + lane * 128 + ((c ^ (lane & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         }
         __syncwarp();
-#pragma unroll 4
+        uint4 piece[8];
+#pragma unroll
         for (int c = 0; c < 8; ++c) {         // four rows, eight lanes a row
           const int rr = c * 4 + (lane >> 3);
-          *reinterpret_cast<uint4*>(out + c * out_step + half * 64) =
-              *reinterpret_cast<const uint4*>(stage + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
+          piece[c] = *reinterpret_cast<const uint4*>(stage + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
         }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(out + c * out_step + half * 64) = piece[c];
         __syncwarp();
       }
       tc_fence_before();
       __syncwarp();
-      if (p.lse) p.lse[lse_at] = (m + log2f(l)) * 0.6931471805599453f;
+      if (p.lse) p.lse[lse_at] = lse;
       if (r == 32) {
         if (p.visited) p.visited[row] = n;
         if (p.scored) p.scored[row] = kk + 1;
@@ -649,14 +712,18 @@ cudaError_t launch_osk_tc(const OskParams& p_in, cudaStream_t st) {
       !make_kv_map(&vm, &vo, p.v, p.pg, p.ks, p.batch, p.hkv, p.n, v_box))
     return cudaErrorInvalidValue;
   const bool small_pages = p.pg.table && p.pg.page_size < kBlock;
-  auto pick = [&](auto mask_c) {
-    constexpr bool M = decltype(mask_c)::value;
-    return p.stage2 ? (small_pages ? osk_tc_kernel<M, true, true> : osk_tc_kernel<M, true, false>)
-                    : (small_pages ? osk_tc_kernel<M, false, true> : osk_tc_kernel<M, false, false>);
+  // Where the line lies, shared against written out (us a pass): Stage 2 on, lists of up to 16 blocks 241 / 247, of 52 the same, of
+  // 104 9,811 / 9,615, of 256 11,122 / 10,883; Stage 2 off, of 5 blocks 148 / 150, of 64 4,912 / 4,858
+  const bool long_walks = p.mask || p.order_stride > (p.stage2 ? kShortWalk : kShortWalkAll);
+  auto pick = [&](auto mask_c, auto long_c) {
+    constexpr bool M = decltype(mask_c)::value, L = decltype(long_c)::value;
+    return p.stage2 ? (small_pages ? osk_tc_kernel<M, true, true, L> : osk_tc_kernel<M, true, false, L>)
+                    : (small_pages ? osk_tc_kernel<M, false, true, L> : osk_tc_kernel<M, false, false, L>);
   };
-  auto kernel = p.mask ? pick(std::true_type{}) : pick(std::false_type{});
-  static SmemLimit limits[8];
-  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kernel), &limits[(p.mask ? 4 : 0) + (p.stage2 ? 2 : 0) + (small_pages ? 1 : 0)], kSmemBytes);
+  auto kernel = p.mask ? pick(std::true_type{}, std::true_type{}) : (long_walks ? pick(std::false_type{}, std::true_type{}) : pick(std::false_type{}, std::false_type{}));
+  static SmemLimit limits[16];
+  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kernel),
+                                   &limits[(p.mask ? 8 : 0) + (p.stage2 ? 4 : 0) + (small_pages ? 2 : 0) + (long_walks ? 1 : 0)], kSmemBytes);
   if (e != cudaSuccess) return e;
   if (p.decisions) {
     size_t words = (size_t)p.batch * p.hq * p.nqb * ((p.order_stride + 31) / 32);

@@ -93,6 +93,12 @@ __device__ __forceinline__ bool mbar_poll_warp(uint32_t bar, uint32_t parity, vo
   while (!(ok = mbar_test_wait(bar, parity)) && !*abort_flag && clock64() - t0 <= budget) __nanosleep(32);
   return __all_sync(0xffffffffu, ok) != 0;
 }
+// 16 bytes of shared memory another thread has written (ordered by the barrier waited for before)
+__device__ __forceinline__ uint4 ld_shared_128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
 // named barrier among `nthreads` threads of the CTA (ids 1..15; 0 is __syncthreads)
 __device__ __forceinline__ void bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -252,6 +258,11 @@ __device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, un
 __device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b) {
   unsigned long long r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long mul_f32x2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
 __device__ __forceinline__ float max3(float a, float b, float c) {

@@ -534,6 +534,31 @@ def test_osk_4k_workload(cfg1, impl):
     print("4k", stats)
 
 
+@pytest.mark.parametrize("tb,skip_scale", [(1.0, -1.0), (0.999, 500.0), (0.13, 500.0)])
+def test_osk_many_work_items_with_and_without_blocks(tb, skip_scale):
+    """More work items than the chip holds CTAs, of no, one, two and more blocks in any order, the first ones empty: what
+    the CTA of an earlier walk takes over, against the CUDA-core kernel.  Output and lse of an empty list are 0 and -inf."""
+    g = torch.Generator(device="cuda").manual_seed(17)
+    hq, hkv, nqb = 64, 8, 16
+    q, k, v = (torch.randn(1, h, nqb * 128, 128, device="cuda", generator=g).to(torch.bfloat16) for h in (hq, hkv, hkv))
+    count = torch.randint(0, 5, (1, hq, nqb), device="cuda", generator=g, dtype=torch.int32)
+    count[0, :8, -6:] = 0
+    count = torch.minimum(count, torch.arange(1, nqb + 1, device="cuda", dtype=torch.int32))
+    order = torch.full((1, hq, nqb, 8), -1, dtype=torch.int32, device="cuda")
+    for i in range(nqb):
+        ids = torch.rand(hq, i + 1, device="cuda", generator=g).argsort(-1)[:, :8].to(torch.int32)
+        order[0, :, i, :ids.shape[1]] = ids
+    order = torch.where(torch.arange(8, device="cuda") < count[..., None], order, -1)
+    got, ref = (run_osk(q, k, v, order, count, tb, skip_scale, impl) for impl in (0, 1))
+    assert torch.equal(got["visited"], ref["visited"]) and torch.equal(got["scored"], ref["scored"])
+    err = (got["out"].float() - ref["out"].float()).abs()
+    assert err.max() < OUT_MAX and err.mean() < OUT_MEAN
+    seen = torch.isfinite(ref["lse"])
+    assert torch.equal(torch.isfinite(got["lse"]), seen) and (got["lse"] - ref["lse"])[seen].abs().max() < LSE_TOL
+    empty = (count[0] == 0).repeat_interleave(128, 1)
+    assert bool((got["out"][0][empty] == 0).all()) and bool((got["lse"][0][empty] == -math.inf).all())
+
+
 @pytest.mark.parametrize("length", [1, 2, 3, 4, 7])
 @pytest.mark.parametrize("tb,skip_scale", [(1.0, -1.0), (0.999, 100.0), (0.999, 900.0), (0.13, 500.0), (0.3, -1.0)])
 def test_osk_short_walks_with_growing_maxima(small, length, tb, skip_scale):
