@@ -23,6 +23,10 @@
 // lists, of at most 64 candidates, it sorts them itself, a warp a list: no sort kernel, scores and best blocks cross no launch.
 // At these lengths Stage 1 is a chain of latencies (launch, first loads, a wave or two of CTAs): in a graph, 1K tokens of 2
 // heads 13.5 -> 10.9 us, 31 blocks of 32 heads 18.0 -> 15.2, 2 x 61 blocks of 32 heads 70 -> 47.5.
+// What bounds the tiles of long calls: 1,518 cycles of an SM a key tile, where the products want 1,024, for the comparisons of 64
+// logits a thread, which take two cycles an instruction and scheduler (no gain from three-input maxima, from asking for
+// barriers earlier in the issuing thread 0.6 %).  CTAs that stay for further items and fetch their tiles ahead save 6,000 cycles an
+// item but took 1,750 a tile (128K: 1,319 -> 1,417 us).
 // Float32 results are a SCREEN: the sort stage recomputes in double precision whatever a
 // rounding error could reorder.  For that it is told, per sampled row, the two blocks with the
 // largest block maxima and whether they are closer than tau_row (the row's HRM flag and M* are
@@ -274,11 +278,25 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - raw);
-  if (threadIdx.x == 0) { prefetch_tensormap(&q_map); prefetch_tensormap(&k_map); }
-  chain_wait();
   const uint32_t a_sm = base;
   const uint32_t k_sm = base + kRowTiles * kTileBytes;
   ScreenCtl* ctl = reinterpret_cast<ScreenCtl*>(smem + (size_t)kTileBytes * (kRowTiles + kStages));
+  // what needs nothing of the kernel before
+  if (threadIdx.x == 0) {
+    prefetch_tensormap(&q_map); prefetch_tensormap(&k_map);
+    mbar_init(smem_u32(&ctl->a_full), 1);
+    for (int s = 0; s < kStages; ++s) { mbar_init(smem_u32(&ctl->k_full[s]), 1); mbar_init(smem_u32(&ctl->k_empty[s]), 1); }
+    for (int s = 0; s < kSteps; ++s) mbar_init(smem_u32(&ctl->s_empty[s]), kEpiThreads);
+    mbar_init(smem_u32(&ctl->x_bar), kEpiThreads);
+    if (!kOnChip) for (int s = 0; s < kStages; ++s) { mbar_init(smem_u32(&ctl->m_full[s]), 1); mbar_init(smem_u32(&ctl->m_empty[s]), kEpiThreads); }
+    if (kMedium) for (int s = 0; s < kStages; ++s) mbar_init(smem_u32(&ctl->n_read[s]), kEpiThreads / 32);
+    ctl->abort_flag = 0;
+    ctl->t_issued = 0; ctl->t_done = 0; ctl->c_fetched = 0; ctl->c_done = 0;
+    mbar_fence_init();
+    fence_proxy_async_smem();
+  }
+  __syncwarp();
+  chain_wait();
 
   constexpr int BPT = 128 / R;                  // key blocks per key tile
   constexpr int kGroups = kRows / R;            // row groups (one query head of one query block each) per CTA
@@ -309,7 +327,53 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     }
   }
   if (i0 >= nqb_b) return;                        // all of this CTA's query blocks are padding
-  if (threadIdx.x == 0) {
+  // key tile t to its stage (lane 0; paged keys: the 128 sampled keys of a tile come from 128 / spp pages (spp sampled rows each) or
+  // from one page; one lane per page looks its page up and issues its two boxes.  Sampled keys past the sequence are masked
+  // later: any valid page will do for them)
+  auto fetch_k = [&](int t) {
+    const int st = t % kStages;
+    const uint32_t dst = k_sm + st * kTileBytes, bar = smem_u32(&ctl->k_full[st]);
+    if (lane == 0) mbar_expect_tx(bar, kTileBytes);
+    if (!p.pg.table) {
+      if (lane == 0) {
+        tma_load_tile(dst, &k_map, 0, t * 128, g, b, p.ko.row, p.ko.head, p.ko.outer, bar);
+        tma_load_tile(dst + kHalfBytes, &k_map, 64, t * 128, g, b, p.ko.row, p.ko.head, p.ko.outer, bar);
+      }
+    } else {
+      __syncwarp();
+      const int spp = min(128, p.pg.page_size / p.stride);
+      if (lane < 128 / spp) {
+        int tok = (t * 128 + lane * spp) * p.stride;
+        if (tok >= nqb_b * kBlock) tok = 0;
+        const KvCoord c = kv_coord(p.pg, b, g, tok);        // (a page's first sampled row is a multiple of the stride)
+        tma_load_tile(dst + lane * spp * 128, &k_map, 0, c.row / p.stride, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
+        tma_load_tile(dst + kHalfBytes + lane * spp * 128, &k_map, 64, c.row / p.stride, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
+      }
+      __syncwarp();
+    }
+  };
+  const int n_first = min(n_tiles, 1);            // (a tile takes its thread some 500 cycles)
+  if (warp == 0) {
+    // The first tiles at once; tensor memory, the status word and a scratch area come meanwhile (one after the other a CTA spent
+    // 4,300 cycles before its first request: Stage 1 at 32K 169 -> 167 us, of 4K tokens of 4 heads 17.4 -> 16.6).
+    // A tiles: strided boxes of R sampled rows of q_box_heads query heads of the group (all of them, if the layout has rows
+    // inside heads) per query block, a box pair per lane (one lane issuing 32 boxes in turn: 2 us)
+    if (lane == 0) mbar_expect_tx(smem_u32(&ctl->a_full), kRowTiles * kTileBytes);
+    __syncwarp();
+    static_assert(kGroups <= 32, "a lane per box pair");
+    const int a_grp = lane * p.q_box_heads;
+    if (a_grp < kGroups) {
+      const int i = i0 + a_grp / G, h = g * G + a_grp % G;
+      const uint32_t dst = a_sm + (a_grp * R / 128) * kTileBytes + (a_grp * R % 128) * 128;   // (rows past the head's last are zero-filled)
+      tma_load_tile(dst, &q_map, 0, i * R, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->a_full));
+      tma_load_tile(dst + kHalfBytes, &q_map, 64, i * R, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->a_full));
+    }
+    __syncwarp();
+    if (n_first > 0) fetch_k(0);
+  } else if (warp == 1) {
+    tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols);
+    tmem_relinquish();
+  } else if (threadIdx.x == 64) {
     // once some CTA has reported a timeout the rest of the grid returns at once
     int poisoned = *reinterpret_cast<volatile int32_t*>(status);
     int slot = -1;
@@ -332,22 +396,6 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     ctl->slot = slot;
     ctl->poisoned = poisoned;
   }
-  __syncthreads();
-  if (ctl->poisoned != 0) return;
-
-  if (threadIdx.x == 0) {
-    mbar_init(smem_u32(&ctl->a_full), 1);
-    for (int s = 0; s < kStages; ++s) { mbar_init(smem_u32(&ctl->k_full[s]), 1); mbar_init(smem_u32(&ctl->k_empty[s]), 1); }
-    for (int s = 0; s < kSteps; ++s) mbar_init(smem_u32(&ctl->s_empty[s]), kEpiThreads);
-    mbar_init(smem_u32(&ctl->x_bar), kEpiThreads);
-    for (int s = 0; s < kStages; ++s) { mbar_init(smem_u32(&ctl->m_full[s]), 1); mbar_init(smem_u32(&ctl->m_empty[s]), kEpiThreads); }
-    if (kMedium) for (int s = 0; s < kStages; ++s) mbar_init(smem_u32(&ctl->n_read[s]), kEpiThreads / 32);
-    ctl->abort_flag = 0;
-    ctl->t_issued = 0; ctl->t_done = 0; ctl->c_fetched = 0; ctl->c_done = 0;
-    mbar_fence_init();
-    fence_proxy_async_smem();
-  }
-  if (warp == 0) { tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -356,64 +404,37 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   volatile int* abort_flag = &ctl->abort_flag;
   const long long budget = p.wait_budget;
   constexpr bool strict = kStrict;
+  const bool poisoned = ctl->poisoned != 0;
 
-  if (warp == 0) {
-    int t_issued = 0;   // (lane 0) key tiles requested so far
-    // A tiles: strided boxes of R sampled rows of q_box_heads query heads of the group (all of them, if the layout has rows
-    // inside heads) per query block, a box pair per lane (one lane issuing 32 boxes in turn: 2 us)
-    if (lane == 0) mbar_expect_tx(smem_u32(&ctl->a_full), kRowTiles * kTileBytes);
-    __syncwarp();
-    static_assert(kGroups <= 32, "a lane per box pair");
-    const int a_grp = lane * p.q_box_heads;
-    if (a_grp < kGroups) {
-      const int i = i0 + a_grp / G, h = g * G + a_grp % G;
-      const uint32_t dst = a_sm + (a_grp * R / 128) * kTileBytes + (a_grp * R % 128) * 128;   // (rows past the head's last are zero-filled)
-      tma_load_tile(dst, &q_map, 0, i * R, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->a_full));
-      tma_load_tile(dst + kHalfBytes, &q_map, 64, i * R, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->a_full));
-    }
-    if (lane == 0) {
-      if (!p.pg.table) {
-        for (int t = 0; t < n_tiles; ++t) {
+  if (poisoned) {
+    if (threadIdx.x == 0) ctl->t_issued = n_first;
+  } else if (warp == 0) {
+    int t_issued = n_first;
+    if (!p.pg.table) {
+      if (lane == 0) {
+        for (int t = n_first; t < n_tiles; ++t) {
           const int st = t % kStages;
           if (!mbar_wait(smem_u32(&ctl->k_empty[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget) ||
               (kMedium && !mbar_wait(smem_u32(&ctl->n_read[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget))) {
             if (!*abort_flag) screen_timeout(ctl, status);
             break;
           }
-          const uint32_t dst = k_sm + st * kTileBytes, bar = smem_u32(&ctl->k_full[st]);
-          mbar_expect_tx(bar, kTileBytes);
-          tma_load_tile(dst, &k_map, 0, t * 128, g, b, p.ko.row, p.ko.head, p.ko.outer, bar);
-          tma_load_tile(dst + kHalfBytes, &k_map, 64, t * 128, g, b, p.ko.row, p.ko.head, p.ko.outer, bar);
+          fetch_k(t);
           t_issued = t + 1;
         }
       }
-    }
-    if (p.pg.table) {
-      // paged keys: the 128 sampled keys of a tile come from 128 / spp pages (spp sampled rows each) or from one page;
-      // one lane per page looks its page up and issues its two boxes.  Sampled keys past the sequence are masked
-      // later: any valid page will do for them.
-      const int spp = min(128, p.pg.page_size / p.stride);
-      const int parts = 128 / spp;
-      for (int t = 0; t < n_tiles; ++t) {
+    } else {
+      for (int t = n_first; t < n_tiles; ++t) {
         const int st = t % kStages;
-        const uint32_t dst = k_sm + st * kTileBytes, bar = smem_u32(&ctl->k_full[st]);
         int ok = 1;
         if (lane == 0) {
           ok = mbar_wait(smem_u32(&ctl->k_empty[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget) ? 1 : 0;
           if (kMedium && ok) ok = mbar_wait(smem_u32(&ctl->n_read[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget) ? 1 : 0;
           if (!ok && !*abort_flag) screen_timeout(ctl, status);
-          if (ok) mbar_expect_tx(bar, kTileBytes);
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) break;
-        if (lane < parts) {
-          int tok = (t * 128 + lane * spp) * p.stride;
-          if (tok >= nqb_b * kBlock) tok = 0;      // past the item's length: masked later, any valid page will do
-          const KvCoord c = kv_coord(p.pg, b, g, tok);        // (a page's first sampled row is a multiple of the stride)
-          tma_load_tile(dst + lane * spp * 128, &k_map, 0, c.row / p.stride, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
-          tma_load_tile(dst + kHalfBytes + lane * spp * 128, &k_map, 64, c.row / p.stride, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
-        }
-        __syncwarp();
+        fetch_k(t);
         t_issued = t + 1;
       }
     }
@@ -424,17 +445,25 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       bool alive = mbar_wait(smem_u32(&ctl->a_full), 0, abort_flag, budget);
       if (!alive && !*abort_flag) screen_timeout(ctl, status);
       int t_done = 0;
+      // (the barriers of the next tile are looked at between the products on this one's row tiles: asked behind them, the tensor
+      // pipe would idle for as long as two waits take)
+      bool k_here = false, s_here = false;
       for (int t = 0; t < n_tiles && alive; ++t) {
-        const int st = t % kStages, sb = t % kSteps;
-        alive = mbar_wait(smem_u32(&ctl->k_full[st]), (t / kStages) & 1, abort_flag, budget) &&
-                mbar_wait(smem_u32(&ctl->s_empty[sb]), ((t / kSteps) & 1) ^ 1, abort_flag, budget);
+        const int st = t % kStages, sb = t % kSteps, st1 = (t + 1) % kStages, sb1 = (t + 1) % kSteps;
+        alive = (k_here || mbar_wait(smem_u32(&ctl->k_full[st]), (t / kStages) & 1, abort_flag, budget)) &&
+                (s_here || mbar_wait(smem_u32(&ctl->s_empty[sb]), ((t / kSteps) & 1) ^ 1, abort_flag, budget));
         if (!alive) { if (!*abort_flag) screen_timeout(ctl, status); break; }
         tc_fence_after();
         const uint64_t kdesc = smem_desc_sw128(k_sm + st * kTileBytes, 16, 1024);
 #pragma unroll
-        for (int rt = 0; rt < kRowTiles; ++rt)
+        for (int rt = 0; rt < kRowTiles; ++rt) {
           mma_ss_x8<2, 4, 6, kHalfBytes / 16, kHalfBytes / 16 + 2, kHalfBytes / 16 + 4, kHalfBytes / 16 + 6>(
               tmem + (sb * kRowTiles + rt) * 128, smem_desc_sw128(a_sm + rt * kTileBytes, 16, 1024), kdesc, idesc);
+          if (rt == 0) {
+            k_here = mbar_test_wait(smem_u32(&ctl->k_full[st1]), ((t + 1) / kStages) & 1);
+            s_here = mbar_test_wait(smem_u32(&ctl->s_empty[sb1]), (((t + 1) / kSteps) & 1) ^ 1);
+          }
+        }
         mma_commit(smem_u32(&ctl->k_empty[st]));
         t_done = t + 1;
       }
@@ -527,9 +556,14 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       for (int bb = 0; bb < BPC; ++bb) {
         const float m = mb[bb];
         const int jb = t * BPT + part * BPC + bb;
-        if (m > top1) { top3 = top2; top2 = top1; jstar2 = jstar; top1 = m; jstar = jb; }
-        else if (m > top2) { top3 = top2; top2 = m; jstar2 = jb; }
-        else if (m > top3) top3 = m;
+        // (selects, not branches: some lane of the warp inserts nearly always.  Stage 1 of 61 blocks 47.9 -> 45.5 us, of four prompts in
+        // 16-token pages 164.8 -> 162, at 32K 167.5 -> 166.8; at 128K, where late tiles seldom hold a new maximum, 1,302 -> 1,308)
+        const bool first = m > top1, second = m > top2;
+        top3 = fmaxf(top3, fminf(m, top2));
+        jstar2 = first ? jstar : (second ? jb : jstar2);
+        top2 = fmaxf(top2, fminf(m, top1));
+        jstar = first ? jb : jstar;
+        top1 = fmaxf(top1, m);
       }
       return true;
     };
@@ -749,7 +783,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && *abort_flag) {
+  if (threadIdx.x == 0 && (poisoned || *abort_flag)) {
     // the kernel gave up somewhere: copies and products still in flight finish on their own and must have done so
     // before the CTA's shared and tensor memory go to the next one
     (void)mbar_wait_noabort(smem_u32(&ctl->a_full), 0);
@@ -759,10 +793,11 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     const int cf = ctl->c_fetched;
     for (int cc = max(ctl->c_done, cf - kStages); cc < cf; ++cc) (void)mbar_wait_noabort(smem_u32(&ctl->m_full[cc % kStages]), (cc / kStages) & 1);
   }
-  __syncwarp();
-  if (warp == 0) tmem_dealloc(tmem, kTmemCols);
+  __syncthreads();
+  if (warp == 1) tmem_dealloc(tmem, kTmemCols);
   if (kOnChip) return;
   {
+    if (ctl->slot < 0) return;            // (poisoned: the CTA has no area)
     // the parked maxima are dead: let L2 drop the lines instead of writing them back
     char* area = reinterpret_cast<char*>(p.maxima + (size_t)ctl->slot * ((size_t)((ns + 127) / 128) * (kRows * BPT)));
     const size_t bytes = (size_t)n_tiles * (kRows * BPT) * sizeof(float);
