@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(kThreads) kap_exact_kernel(KapParams p, int kb
 // 1-d grid: the CTAs share out what the sort stage left.  kTied: lists with near ties to recount; kRedo: lists to do over (normally none).
 // In one launch where the second's shared memory leaves room for several CTAs on an SM, in two otherwise.
 template <bool kTied, bool kRedo>
-__global__ void __launch_bounds__(kThreads, kRedo ? 2 : 4) kap_fixup_kernel(KapParams p, KapScreenParams sp, int kb_per_iter, int sort_cap,
+__global__ void __launch_bounds__(kThreads, 2) kap_fixup_kernel(KapParams p, KapScreenParams sp, int kb_per_iter, int sort_cap,
                                                                           bool by_flag, const int32_t* status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   chain_begin();
@@ -293,7 +293,7 @@ cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, bool
   // (a launch costs as much as either does on a short call; at 64K tokens the second alone would leave one CTA per SM)
   const size_t both = std::max(redo, tied);
   if (both <= 56 * 1024) return launch(kap_fixup_kernel<true, true>, &limits[0], both, 2 * sms);
-  const cudaError_t e = launch(kap_fixup_kernel<true, false>, &limits[1], tied, 4 * sms);
+  const cudaError_t e = launch(kap_fixup_kernel<true, false>, &limits[1], tied, 2 * sms);
   // As many CTAs as fit the chip (227 KB of shared memory, 3 x 256 threads of registers on an SM): the launch overlaps the recount,
   // whose CTAs still hold SMs, and one CTA per SM was placed two and three to an SM, where they share the FP64 unit and the
   // others idle (200 blocks of 8 heads, all keys the same: 8,223 us with one per SM, 4,942 when the launch came later)

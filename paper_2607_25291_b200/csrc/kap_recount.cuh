@@ -4,8 +4,8 @@
 // 2 * position + (tied with the next position) and the block id.  One CTA of eight warps per list: M*[r] from every row's best
 // block (and the runner-up of the rows the screen could not call) and the entries' block maxima, then every entry's score
 // sum_r exp(M[r,j] - M*[r]); chains are re-sorted by it, ties by ascending id, and the lists patched.  A kernel of its own
-// because it wants more registers than the sort, whose lists want many CTAs.  (128 where it shares a launch with the lists to redo;
-// alone, in long calls, four CTAs an SM leave it 64, of which it spills some 400 bytes.)  The products run on the FP64 matrix
+// because it wants more registers than the sort, whose lists want many CTAs: 128, two CTAs an SM (with 64 and four CTAs it spilled some
+// 400 bytes: Stage 1 at 32K 166.3 us instead of 162.4, of 201 blocks with Top-p 142.4 instead of 137.8).  The products run on the FP64 matrix
 // unit, eight rows by eight keys at a time: it has the vector unit's rate, but a warp issues one instruction and one read of
 // the query rows per 256 products (one lane per key and eight rows: 1,024 FMAs and 512 16-byte shared-memory reads a
 // block and warp, 10 k cycles; inside the sort kernel, at 40 registers, 15 to 20 k).
