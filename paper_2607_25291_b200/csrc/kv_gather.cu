@@ -9,36 +9,54 @@
 namespace cosa {
 namespace {
 
-// one 16-byte chunk per thread and turn; a row of d = 128 bf16 has 16 chunks.  every: copy only the rows whose token
-// index is a multiple of it (KAP reads nothing but its sampled rows; the other rows of the staging tensor stay unwritten)
-__global__ void __launch_bounds__(256) gather_pages_kernel(const uint4* __restrict__ pool, uint4* __restrict__ dense, KvPaging pg,
-                                                           int batch, int hkv, int n, int every) {
+// Sixteen lanes take a row (16 bytes each), a warp eight rows at a time: four table look-ups, then four loads in flight a lane.
+// grid (row blocks, (batch item, KV head), pools): K and V in one launch.  every: copy only the rows whose token index is a
+// multiple of it (KAP reads nothing but its sampled rows; the other rows of the staging tensor stay unwritten).  Bound by memory, or
+// by the launch where little is copied.  One chunk a thread and turn, each with its own divisions and look-up, K after V, outside the
+// chain of launches: 811 us a
+// pass instead of 802 on four prompts of up to 16K tokens in 16-token pages.
+constexpr int kThreads = 256, kRowsPerWarp = 8;
+struct Pools { const uint4* pool[2]; uint4* dense[2]; };
+__global__ void __launch_bounds__(kThreads) gather_pages_kernel(Pools t, KvPaging pg, int batch_heads, int hkv, int n, int every) {
   constexpr int kChunks = kHeadDim * 2 / 16;
-  const int rows = n / every;
-  const long long total = (long long)batch * hkv * rows * kChunks;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(idx % kChunks);
-    const long long row = idx / kChunks;            // ((b * hkv) + g) * rows + token / every
-    const int token = (int)(row % rows) * every;
-    const int bg = (int)(row / rows);
-    const int b = bg / hkv, g = bg % hkv;
-    if (pg.seq_lens && token >= pg.seq_lens[b]) continue;   // padding: never read as keys
-    const long long src = kv_off(pg, Strides{0, 0, 0}, b, hkv, g, token) / 8;   // (pools only: 16-byte chunks)
-    dense[((long long)bg * n + token) * kChunks + c] = pool[src + c];
+  chain_begin();
+  const int lane = threadIdx.x & 31, c = lane & 15;
+  const uint4* __restrict__ pool = t.pool[blockIdx.z];
+  uint4* __restrict__ dense = t.dense[blockIdx.z];
+  for (int bg = blockIdx.y; bg < batch_heads; bg += gridDim.y) {
+    const int b = bg / hkv, g = bg - b * hkv;
+    const int len = pg.seq_lens ? min(n, pg.seq_lens[b]) : n;      // (padding is never read as keys)
+    const int rows = (max(len, 0) + every - 1) / every;
+    const int32_t* table = pg.table + (long long)b * pg.pages_per_seq;
+    for (int r0 = (blockIdx.x * (kThreads / 32) + (int)(threadIdx.x >> 5)) * kRowsPerWarp; r0 < rows;
+         r0 += (int)gridDim.x * (kThreads / 32) * kRowsPerWarp) {
+      uint4 w[kRowsPerWarp / 2];
+#pragma unroll
+      for (int u = 0; u < kRowsPerWarp / 2; ++u) {
+        const int r = r0 + 2 * u + (lane >> 4), token = r * every;
+        if (r < rows)
+          w[u] = pool[(((long long)table[token >> pg.page_shift] * hkv + g) * pg.page_size + (token & (pg.page_size - 1))) * kChunks + c];
+      }
+#pragma unroll
+      for (int u = 0; u < kRowsPerWarp / 2; ++u) {
+        const int r = r0 + 2 * u + (lane >> 4);
+        if (r < rows) dense[((long long)bg * n + (long long)r * every) * kChunks + c] = w[u];
+      }
+    }
   }
 }
 
 }  // namespace
 
-cudaError_t launch_gather_pages(const __nv_bfloat16* pool, __nv_bfloat16* dense, const KvPaging& pg, int batch, int hkv, int n,
-                                int every, cudaStream_t st) {
+cudaError_t launch_gather_pages(const __nv_bfloat16* k_pool, __nv_bfloat16* k_dense, const __nv_bfloat16* v_pool, __nv_bfloat16* v_dense,
+                                const KvPaging& pg, int batch, int hkv, int n, int every, cudaStream_t st) {
   if (every < 1 || n % every != 0) return cudaErrorInvalidValue;
-  const long long total = (long long)batch * hkv * (n / every) * (kHeadDim * 2 / 16);
-  long long blocks = (total + 255) / 256;
-  if (blocks > 148LL * 32) blocks = 148LL * 32;
-  gather_pages_kernel<<<(unsigned)blocks, 256, 0, st>>>(reinterpret_cast<const uint4*>(pool), reinterpret_cast<uint4*>(dense), pg,
-                                                       batch, hkv, n, every);
-  return cudaGetLastError();
+  Pools t{};
+  t.pool[0] = reinterpret_cast<const uint4*>(k_pool); t.dense[0] = reinterpret_cast<uint4*>(k_dense);
+  t.pool[1] = reinterpret_cast<const uint4*>(v_pool); t.dense[1] = reinterpret_cast<uint4*>(v_dense);
+  const int per_cta = kThreads / 32 * kRowsPerWarp, heads = batch * hkv;
+  const dim3 grid((unsigned)((n / every + per_cta - 1) / per_cta), (unsigned)(heads < 65535 ? heads : 65535), v_pool ? 2 : 1);
+  return launch_chained(gather_pages_kernel, grid, kThreads, 0, st, t, pg, heads, hkv, n, every);
 }
 
 }  // namespace cosa
