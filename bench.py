@@ -131,7 +131,7 @@ def order_pitch(cosa, budget, nqb):
 
 def launches_per_step(n, stride, page_size=0, pages_in_place=False, osk_impl=0, block_q=128, heads=4):
     """Kernels of the library that one step launches, by the launchers' own rules (a test counts them with a profiler):
-    Stage 1: the copy of small pages' keys, the norms of long calls, screen, sort (short calls: in the screen), and one or two
+    Stage 1: the copy of small pages' keys, the norms of long calls, screen, sort (up to 256 blocks: in the screen), and one or two
     launches for what the sort leaves over; Stage 2: the copy of K and V from pages smaller than a key block, and the walk."""
     R, nqb = 128 // stride, n // 128
     kb = max(1, min(16, 256 // (R * R)))
@@ -139,8 +139,9 @@ def launches_per_step(n, stride, page_size=0, pages_in_place=False, osk_impl=0, 
     redo = doubles * 8 + max(2, 1 << (nqb - 1).bit_length()) * 12 + ((nqb | 1) + 15) // 16 * 16     # shared memory, bytes
     recount = R * (block_q // 128) * 132 * 8 + (nqb * 4 if block_q == 256 else 0)
     keys = n // stride
-    lists = block_q == 128 and (keys <= 256 or (keys <= 512 and heads * nqb > 128) or (512 < keys <= 1024 and R >= 16))
-    kap = (1 if lists else 2 + (keys > 512)) + (1 if max(redo, recount) <= 56 * 1024 else 2)
+    lists = block_q == 128 and nqb <= 256 and (keys <= 256 or keys > 512 or heads * nqb > 128)
+    norms = keys > 512 and not (lists and keys <= 1024 and R >= 16)
+    kap = 1 + norms + (not lists) + (1 if max(redo, recount) <= 56 * 1024 else 2)
     kap += 0 < page_size and page_size // stride < 32
     osk = 1 + (1 if 0 < page_size < 128 and (osk_impl in (4, 5) or not pages_in_place) else 0)
     return int(kap + osk)

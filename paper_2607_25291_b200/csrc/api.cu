@@ -311,8 +311,10 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
   }
   sp.pg = p.pg;
   sp.qs = p.qs; sp.ks = p.ks;
-  const bool lists = kap_screen_makes_lists(p);
-  cudaError_t e = lists || kap_screen_is_short(p.n, s) ? cudaSuccess : launch_kap_norms(&sp, st);
+  const ScreenForm form = kap_screen_form(p);
+  const bool lists = screen_makes_lists(form);
+  sp.entries = form == kScreenLongLists ? reinterpret_cast<int32_t*>(sp.qk2max) : sp.todo + 2;
+  cudaError_t e = screen_parks(form) ? launch_kap_norms(&sp, st) : cudaSuccess;
   if (e != cudaSuccess) return cuda_fail(e, "kap norms launch");
   // two sorted scores closer than this (relative) are re-scored in double precision: 2^-15, four times the screen's
   // largest error on the measured workloads; larger for inputs of larger magnitude (see screen_error_bound)
@@ -323,7 +325,7 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
     e = launch_kap_sort(p, sp, tau_score, st);
     if (e != cudaSuccess) return cuda_fail(e, "kap sort launch");
   }
-  e = launch_kap_fixup(p, sp, lists, st);
+  e = launch_kap_fixup(p, sp, lists && form != kScreenLongLists, st);
   if (e != cudaSuccess) return cuda_fail(e, "kap recount launch");
   return COSA_OK;
 }

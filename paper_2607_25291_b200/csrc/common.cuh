@@ -104,10 +104,11 @@ struct KapScreenParams {
   int32_t* jstar;        // [B,Hq,N/s,2]    blocks holding each sampled row's largest / second largest block maximum
   uint32_t* ambmask;     // [B,Hq,nQB]      bit r: sampled row r's two best blocks are too close to call in float32
   uint8_t* hard;         // [B,Hq,nQB]      1 = three blocks too close on some row: whole query block goes to double precision.  Where the
-                         // screen makes the lists: what is left to the next, 0 nothing, 1 the list to redo, 2 near ties
-  int32_t* todo;         // [2 + B*Hq*nQB]  what the sort stage leaves to the next: [0] = lists to redo, [1] = lists with near ties (their rows of
-                         // `scores` then hold the chained entries, see kap_recount.cuh); behind them, as flat (b*Hq+h)*nQB+i, the
-                         // former from the front, the latter from the end: no list is both
+                         // short and medium forms make the lists: what is left to the next, 0 nothing, 1 the list to redo, 2 near ties
+  int32_t* todo;         // [2] what is left to the next stage: lists to redo, lists with near ties (their rows of `scores` then hold the
+                         // chained entries, see kap_recount.cuh)
+  int32_t* entries;      // [B*Hq*nQB] ... as flat (b*Hq+h)*nQB+i, the former from the front, the latter from the end: no list is both.  Behind
+                         // `todo`, or where the screen makes the lists itself in the place of qk2max
   float* maxima;         // [slots][key tiles][128 rows x 128/R blocks]  per-row block maxima of the CTA that holds the slot
   int32_t* slot_taken;   // [slots]  0 = free; zeroed by kap_norms_kernel
   float* k2part;         // largest squared norms of sampled key rows of the call, one per CTA of kap_norms_kernel; they lie where the
@@ -261,13 +262,17 @@ cudaError_t launch_kap_exact(const KapParams& p, cudaStream_t st);
 // (by_flag: sp.hard instead of sp.todo says which)
 cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, bool by_flag, cudaStream_t st);
 // the whole call's key tiles fit the screen's stages: it needs no scratch areas and no norms kernel
-bool kap_screen_is_short(int n, int stride);
 bool kap_screen_supported(int rows, int group, int stride, const KvPaging& pg);
-// the screen sorts its scores itself and writes the lists: no sort kernel follows
-bool kap_screen_makes_lists(const KapParams& p);
+// Forms of the screen.  Long: block maxima are parked in scratch areas, the norms kernel goes before.  Short: at most 4 key tiles, which
+// all fit the stages; Medium: at most 8; neither needs scratch areas or the norms kernel.  Lists: the screen sorts its scores itself
+// and writes the lists, no sort kernel follows
+enum ScreenForm { kScreenLong, kScreenLongLists, kScreenShort, kScreenShortLists, kScreenMediumLists };
+inline bool screen_parks(ScreenForm f) { return f == kScreenLong || f == kScreenLongLists; }
+inline bool screen_makes_lists(ScreenForm f) { return f == kScreenLongLists || f == kScreenShortLists || f == kScreenMediumLists; }
+ScreenForm kap_screen_form(const KapParams& p);
 cudaError_t launch_kap_screen(const KapParams& kp, const KapScreenParams& p, float tau_score, cudaStream_t st);
 constexpr int kNormParts = 296;   // CTAs of kap_norms_kernel at most
-// writes sp->k2part and sp->k2parts, clears sp->slot_taken
+// writes sp->k2part and sp->k2parts, clears sp->todo and sp->slot_taken
 cudaError_t launch_kap_norms(KapScreenParams* sp, cudaStream_t st);
 // CTAs of the screen kernel that can be resident at once on the current device (0 on failure), and the bytes of
 // block-maxima scratch each of them needs

@@ -63,13 +63,13 @@ __global__ void __launch_bounds__(kThreads, 2) kap_fixup_kernel(KapParams p, Kap
     return;
   }
   if (kTied) {
-    const int n = sp.todo[1], last = 1 + p.batch * p.hq * p.nqb;
-    for (int e = blockIdx.x; e < n; e += gridDim.x) kap_recount_item(p, sp, sp.todo[last - e], smem_raw);
+    const int n = sp.todo[1], last = p.batch * p.hq * p.nqb - 1;
+    for (int e = blockIdx.x; e < n; e += gridDim.x) kap_recount_item(p, sp, sp.entries[last - e], smem_raw);
   }
   if (kRedo) {
     const int n = sp.todo[0];
     for (int e = blockIdx.x; e < n; e += gridDim.x) {
-      const int flat = sp.todo[2 + e];
+      const int flat = sp.entries[e];
       const int i = flat % p.nqb, bh = flat / p.nqb;
       kap_exact_item(p, bh / p.hq, bh % p.hq, i, kb_per_iter, sort_cap);   // i: first row tile of the block
       __syncthreads();

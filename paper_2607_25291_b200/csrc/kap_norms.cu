@@ -17,10 +17,11 @@ constexpr int kNormRows = 8;
 // CTA's rows.  (Partial maxima instead of an atomic on one word: nothing has to be cleared first.)  Bound by how many
 // loads are in flight: a row is one 256-byte piece per `stride` rows.
 __global__ void __launch_bounds__(kThreads) kap_norms_kernel(const __nv_bfloat16* __restrict__ k, KvPaging pg, Strides ks, int batch,
-                                                             int hkv, int n, int stride, float* k2part, int32_t* slot_taken, int slots) {
+                                                             int hkv, int n, int stride, float* k2part, int32_t* todo, int32_t* slot_taken, int slots) {
   __shared__ float warp_best[kThreads / 32];
   const int lane = threadIdx.x & 31;
   chain_begin();
+  if (blockIdx.x == 0 && threadIdx.x < 2) todo[threadIdx.x] = 0;
   for (int t = blockIdx.x * kThreads + threadIdx.x; t < slots; t += gridDim.x * kThreads) slot_taken[t] = 0;   // for the screen
   const long long warp = ((long long)blockIdx.x * kThreads + threadIdx.x) >> 5;
   const long long n_warps = ((long long)gridDim.x * kThreads) >> 5;
@@ -73,7 +74,7 @@ cudaError_t launch_kap_norms(KapScreenParams* sp, cudaStream_t st) {
   if (blocks < 1) blocks = 1;
   sp->k2parts = (int)blocks;
   return launch_chained(kap_norms_kernel, dim3((unsigned)blocks), kThreads, 0, st, sp->k, sp->pg, sp->ks, sp->batch, sp->hkv, sp->n,
-                        sp->stride, sp->k2part, sp->slot_taken, sp->slots);
+                        sp->stride, sp->k2part, sp->todo, sp->slot_taken, sp->slots);
 }
 
 }  // namespace cosa

@@ -19,10 +19,12 @@
 // (row group, key block).
 // Calls of at most eight key tiles (n <= 8192 at stride 8) park nothing: a thread keeps its block maxima in registers and, when
 // every product is done, lays them into the key stages, from where the scores are formed; the norms of the sampled keys are
-// taken from the stages as well, which saves the norms kernel's launch.  And since the CTA then holds every score of its
-// lists, of at most 64 candidates, it sorts them itself, a warp a list: no sort kernel, scores and best blocks cross no launch.
-// At these lengths Stage 1 is a chain of latencies (launch, first loads, a wave or two of CTAs): in a graph, 1K tokens of 2
-// heads 13.5 -> 10.9 us, 31 blocks of 32 heads 18.0 -> 15.2, 2 x 61 blocks of 32 heads 70 -> 47.5.
+// taken from the stages as well, which saves the norms kernel's launch.
+// A CTA holds every score of its lists, and up to 256 candidates it sorts them itself, a warp a list in registers: no sort kernel (a
+// wave of small CTAs each, chains of short steps between barriers), and the scores cross no launch.  Stage 1 at 32K 160 -> 135 us, of
+// four prompts in 16-token pages 157 -> 121, of 201 blocks with Top-p 136 -> 110, of 55 blocks at stride 4 102 -> 58.  Both together, in
+// short calls a chain of latencies (launch, first loads, a wave or two of CTAs): 1K tokens of 2 heads 13.5 -> 10.5 us, 31 blocks of
+// 32 heads 18.0 -> 14.6, 2 x 61 blocks of 32 heads 70 -> 43.
 // What bounds the tiles of long calls: 1,518 cycles of an SM a key tile, where the products want 1,024, for the comparisons of 64
 // logits a thread, which take two cycles an instruction and scheduler (no gain from three-input maxima, from asking for
 // barriers earlier in the issuing thread 0.6 %).  CTAs that stay for further items and fetch their tiles ahead save 6,000 cycles an
@@ -33,6 +35,8 @@
 // then settled in double precision); three such blocks on one row send the whole query block to
 // the double-precision kernel.
 #include <math.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "kap_recount.cuh"
@@ -94,10 +98,8 @@ __device__ __forceinline__ float largest_key_norm(const KapScreenParams& p, int 
   return k2;
 }
 
-// kLong: any length, maxima parked.  kShort, kShortLists: at most kStages key tiles.  kMediumLists: at most kMediumTiles
-enum Form { kLong, kShort, kShortLists, kMediumLists };
-constexpr int kMediumTiles = 8;
-constexpr int kListCap = 64;              // candidates a list may have where this kernel makes the lists
+constexpr int kMediumTiles = 8;           // key tiles of a call of the medium form
+constexpr int kListCap = 64, kLongListCap = 256;   // candidates a list may have where this kernel makes the lists
 
 // (a whole warp) the largest of row `qrow` x the sampled keys of block j that the row sees, in double precision: the arithmetic of
 // f64_block_maxima in kap_sort.cu, the row taken from global memory
@@ -129,20 +131,56 @@ __device__ double f64_row_maximum(const KapParams& p, const __nv_bfloat16* qrow,
   return best;
 }
 
-// (a whole warp) the visit list of one (head, query block) of at most kListCap candidates: what kap_sort_kernel does for longer calls,
-// step by step.  score[j]: the screened scores (sign: HRM flag); j1, j2: its rows' best and second best blocks; srt: room for the
-// keys.  sp.hard says what is left for the fix-up: 0 nothing, 1 the whole list, 2 near ties (entries in the list's row of `scores`)
-template <int R>
+// (a whole warp) sorts 32 * PER distinct keys descending (bitonic, in registers); afterwards lane l holds places l * PER and on
+template <int PER>
+__device__ __forceinline__ void warp_sort_desc(unsigned long long (&k)[PER], int lane) {
+#pragma unroll
+  for (int size = 2; size <= 32 * PER; size <<= 1) {
+#pragma unroll
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      if (stride >= PER) {
+        const bool larger = ((lane & (size / PER)) == 0) == ((lane & (stride / PER)) == 0);
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+          const unsigned long long other = __shfl_xor_sync(0xffffffffu, k[r], stride / PER);
+          k[r] = (other > k[r]) == larger ? other : k[r];
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+          if (r & stride) continue;
+          const bool down = size < PER ? (r & size) == 0 : (lane & (size / PER)) == 0;
+          const unsigned long long x = k[r], y = k[r | stride];
+          const bool swap = (y > x) == down;
+          k[r] = swap ? y : x;
+          k[r | stride] = swap ? x : y;
+        }
+      }
+    }
+  }
+}
+
+// (a whole warp) the visit list of one (head, query block) of at most 32 * PER candidates: what kap_sort_kernel does for longer
+// calls, step by step.  score[j]: the screened scores (sign: HRM flag); j1, j2: its rows' best and second best blocks; srt: room for
+// the keys.  What is left for the fix-up: near ties (entries in the list's row of `scores`) or the whole list.  kFlags: sp.hard says
+// so, 0 nothing, 1 the list, 2 ties; else the worklist does
+template <int R, int PER, bool kFlags>
 __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float tau_score, int b, int g, int h, int i, int J, uint32_t amb,
                           float qk2, const float* score, const int* j1, const int* j2, unsigned long long* srt, int lane) {
   const size_t row = (size_t)(b * p.hq + h) * p.nqb + i;
+  auto leave = [&](int state) {
+    if (lane != 0) return;
+    if (kFlags) sp.hard[row] = (uint8_t)state;
+    else if (state == 1) sp.entries[atomicAdd(sp.todo, 1)] = (int)row;
+    else if (state == 2) sp.entries[p.batch * p.hq * p.nqb - 1 - atomicAdd(sp.todo + 1, 1)] = (int)row;
+  };
   if (signbit(qk2)) {                       // three-way row ambiguity: left to the double-precision kernel
-    if (lane == 0) sp.hard[row] = 1;
+    leave(1);
     return;
   }
-  unsigned long long key[2];
+  unsigned long long key[PER];
 #pragma unroll
-  for (int x = 0; x < 2; ++x) {
+  for (int x = 0; x < PER; ++x) {
     const int j = lane + 32 * x;
     const float v = j < J ? score[j] : 0.f;
     key[x] = j < J ? ((unsigned long long)(__float_as_uint(fabsf(v)) | (v < 0.f ? 0x80000000u : 0u)) << 32) | (0xffffffffu - (unsigned)j) : 0ULL;
@@ -172,99 +210,126 @@ __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float t
         const int j = which ? j2[r] : j1[r];
         const bool flag = __any_sync(0xffffffffu, lane < R && (mine ? (j == a1 && m1 == best) || (j == a2 && m2 == best) : j == a1));
 #pragma unroll
-        for (int x = 0; x < 2; ++x)
+        for (int x = 0; x < PER; ++x)
           if (j == lane + 32 * x) key[x] = (key[x] & 0x7fffffffffffffffULL) | (flag ? 0x8000000000000000ULL : 0ULL);
       }
     }
   }
+  if (p.dbg_scores || p.dbg_flags) {
 #pragma unroll
-  for (int x = 0; x < 2; ++x) {
-    const int j = lane + 32 * x;
-    if (j < J) {
-      srt[j] = key[x];
+    for (int x = 0; x < PER; ++x) {
+      const int j = lane + 32 * x;
       const unsigned hi = (unsigned)(key[x] >> 32);
-      if (p.dbg_scores) p.dbg_scores[row * p.nqb + j] = __uint_as_float(hi & 0x7fffffffu);
-      if (p.dbg_flags) p.dbg_flags[row * p.nqb + j] = (unsigned char)(hi >> 31);
+      if (j < J && p.dbg_scores) p.dbg_scores[row * p.nqb + j] = __uint_as_float(hi & 0x7fffffffu);
+      if (j < J && p.dbg_flags) p.dbg_flags[row * p.nqb + j] = (unsigned char)(hi >> 31);
     }
   }
-  __syncwarp();
-  // every key counts the keys above it
-  int rank[2] = {0, 0};
+  if (PER == 2 && J <= 16) {                // (every key counts the keys above it: fewer steps than the sort of 64)
+    int rank = 0;
 #pragma unroll 4
-  for (int u = 0; u < J; ++u) {
-    const unsigned long long k = srt[u];
-    rank[0] += k > key[0] ? 1 : 0;
-    rank[1] += k > key[1] ? 1 : 0;
+    for (int u = 0; u < J; ++u) rank += __shfl_sync(0xffffffffu, key[0], u) > key[0] ? 1 : 0;
+    if (lane < J) srt[rank] = key[0];
+  } else {
+    warp_sort_desc<PER>(key, lane);
+#pragma unroll
+    for (int x = 0; x < PER; ++x) srt[lane * PER + x] = key[x];
   }
   __syncwarp();
-#pragma unroll
-  for (int x = 0; x < 2; ++x)
-    if (lane + 32 * x < J) srt[rank[x]] = key[x];
-  __syncwarp();
-#pragma unroll
-  for (int x = 0; x < 2; ++x) key[x] = lane + 32 * x < J ? srt[lane + 32 * x] : 0ULL;      // (now: the sorted entries)
+  auto score_at = [&](int t) { return __uint_as_float((unsigned)(srt[t] >> 32) & 0x7fffffffu); };
   int K = budget_count_fx(p.budget_fx, J);
   if (p.top_p > 0.0) {
-    // Top-p: the sums of kap_sort_kernel, a warp of which holds 32 entries
-    double run[2], before = 0.0;
+    // Top-p: the sums of kap_sort_kernel, where each of 128 threads has E consecutive entries; x: its warps
+    constexpr int kWarps = PER < 4 ? PER : 4;
+    const int E = (J + 127) / 128;
+    double start[kWarps], total = 0.0;
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
-      const double loc = lane + 32 * x < J ? (double)__uint_as_float((unsigned)(key[x] >> 32) & 0x7fffffffu) : 0.0;
+    for (int x = 0; x < kWarps; ++x) {
+      start[x] = 0.0;
+      if (32 * x * E >= J) continue;
+      const int t0 = (32 * x + lane) * E;
+      double loc = 0.0;
+      for (int q = 0; q < E; ++q)
+        if (t0 + q < J) loc += (double)score_at(t0 + q);
       double incl = loc;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const double v = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += v;
       }
-      run[x] = before + (incl - loc) + loc;
-      before += __shfl_sync(0xffffffffu, incl, 31);
+      start[x] = total + (incl - loc);
+      total += __shfl_sync(0xffffffffu, incl, 31);
     }
-    const double thr = p.top_p * before;
-    const unsigned first0 = __ballot_sync(0xffffffffu, lane < J && run[0] >= thr), first1 = __ballot_sync(0xffffffffu, lane + 32 < J && run[1] >= thr);
-    const int k_topp = first0 ? __ffs(first0) : (first1 ? 32 + __ffs(first1) : J);
-    K = min(K, k_topp);
+    const double thr = p.top_p * total;
+    unsigned k_topp = (unsigned)J;
+#pragma unroll
+    for (int x = 0; x < kWarps; ++x) {
+      const int t0 = (32 * x + lane) * E;
+      double run = start[x];
+      for (int q = 0; q < E && t0 + q < J; ++q) {
+        run += (double)score_at(t0 + q);
+        if (run >= thr) { k_topp = min(k_topp, (unsigned)(t0 + q + 1)); break; }
+      }
+    }
+    K = min(K, (int)__reduce_min_sync(0xffffffffu, k_topp));
   }
   // near ties between sorted neighbours
   tau_score = fmaxf(tau_score, 2.f * screen_error_bound(qk2, sp.scale));
-  unsigned long long tie = 0ULL;            // bit t: entries t and t + 1
+  uint32_t tie[PER];                        // bit l of tie[x]: entries t = 32 x + l and t + 1
+  bool any = false;
 #pragma unroll
-  for (int x = 0; x < 2; ++x) {
+  for (int x = 0; x < PER; ++x) {
     const int t = lane + 32 * x;
     bool near = false;
     if (t + 1 < J) {
-      const unsigned ha = (unsigned)(key[x] >> 32), hb = (unsigned)(srt[t + 1] >> 32);
+      const unsigned ha = (unsigned)(srt[t] >> 32), hb = (unsigned)(srt[t + 1] >> 32);
       const float sa = __uint_as_float(ha & 0x7fffffffu), sb = __uint_as_float(hb & 0x7fffffffu);
       near = (ha >> 31) == (hb >> 31) && sa - sb <= tau_score * sa;
     }
-    tie |= (unsigned long long)__ballot_sync(0xffffffffu, near) << (32 * x);
+    any = any || (near && t < K);
+    tie[x] = __ballot_sync(0xffffffffu, near);
   }
-  auto below = [](int t) { return t >= 64 ? ~0ULL : (1ULL << t) - 1ULL; };
   int state = 0;
-  if (tie & below(K)) {
+  if (__any_sync(0xffffffffu, any)) {
     int e = K;                              // a chain that straddles the end of the kept prefix reaches past it
-    while (e < J && ((tie >> (e - 1)) & 1ULL)) ++e;
-    const unsigned long long members = (tie | (tie << 1)) & below(e);
-    const int nt = __popcll(members);
+    bool more = true;
+#pragma unroll
+    for (int x = 0; x < PER; ++x) {
+      while (more && e > 32 * x && e <= 32 * x + 32 && e < J) {
+        more = (tie[x] >> ((e - 1) & 31)) & 1u;
+        e += more ? 1 : 0;
+      }
+    }
+    int nt = 0;
+    uint32_t members[PER];
+#pragma unroll
+    for (int x = 0; x < PER; ++x) {
+      const int n = e - 32 * x;             // entries of this word before e
+      const uint32_t below = n >= 32 ? ~0u : (n <= 0 ? 0u : (1u << n) - 1u);
+      members[x] = (tie[x] | (tie[x] << 1) | (x > 0 ? tie[x > 0 ? x - 1 : 0] >> 31 : 0u)) & below;
+      nt += __popc(members[x]);
+    }
     if (nt > min(kRecountMax, (p.nqb - 2) / 2)) {
-      if (lane == 0) sp.hard[row] = 1;
+      leave(1);
       return;
     }
     int* words = reinterpret_cast<int*>(sp.scores + row * p.nqb);
     if (lane == 0) { words[0] = nt; words[1] = K; }
+    int slot0 = 0;
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
-      const int t = lane + 32 * x;
-      if ((members >> t) & 1ULL) {
-        const int slot = __popcll(members & below(t));
-        words[2 + 2 * slot] = 2 * t + (int)((tie >> t) & 1ULL);
-        words[3 + 2 * slot] = (int)(0xffffffffu - (unsigned)key[x]);
+    for (int x = 0; x < PER; ++x) {
+      if ((members[x] >> lane) & 1u) {
+        const int slot = slot0 + __popc(members[x] & ((1u << lane) - 1u)), t = lane + 32 * x;
+        words[2 + 2 * slot] = 2 * t + (int)((tie[x] >> lane) & 1u);
+        words[3 + 2 * slot] = (int)(0xffffffffu - (unsigned)srt[t]);
       }
+      slot0 += __popc(members[x]);
     }
     state = 2;
   }
   int32_t* dst = p.order + row * p.order_stride;
   for (int t = lane; t < p.order_stride; t += 32) dst[t] = t < K ? (int32_t)(0xffffffffu - (unsigned)srt[t]) : -1;
-  if (lane == 0) { p.count[row] = K; sp.hard[row] = (uint8_t)state; }
+  if (lane == 0) p.count[row] = K;
+  leave(state);
 }
 
 // kStrict: every multi-lane wait answers per warp (see mbar_wait_warp).  kForm: see above
@@ -272,7 +337,8 @@ template <int R, bool kStrict, int kForm>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                   KapScreenParams p, KapParams kp, float tau_score, int32_t* status) {
-  constexpr bool kOnChip = kForm != kLong, kMedium = kForm == kMediumLists, kLists = kForm == kShortLists || kMedium;
+  constexpr bool kLongLists = kForm == kScreenLongLists, kOnChip = kForm != kScreenLong && !kLongLists, kMedium = kForm == kScreenMediumLists;
+  constexpr bool kLists = kForm == kScreenShortLists || kMedium || kLongLists;
   constexpr int kMaxTiles = kMedium ? kMediumTiles : kStages;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -316,14 +382,14 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const int n_tiles = (n_keys + 127) / 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  if (blockIdx.x == 0 && threadIdx.x == 0) { p.todo[0] = 0; p.todo[1] = 0; }   // the sort stage (a later launch) counts there
+  if (!kLists && blockIdx.x == 0 && threadIdx.x == 0) { p.todo[0] = 0; p.todo[1] = 0; }   // the sort stage (a later launch) counts there
   if (kLists) {                                   // query blocks that are padding: empty lists
     for (int x = warp; x < kGroups; x += kThreads / 32) {
       const int i = i0 + x / G;
       if (i < nqb_b || i >= p.nqb) continue;
       const size_t row = (size_t)(b * p.hq + g * G + x % G) * p.nqb + i;
       for (int t = lane; t < kp.order_stride; t += 32) kp.order[row * kp.order_stride + t] = -1;
-      if (lane == 0) { kp.count[row] = 0; p.hard[row] = 0; }
+      if (lane == 0) { kp.count[row] = 0; if (!kLongLists) p.hard[row] = 0; }
     }
   }
   if (i0 >= nqb_b) return;                        // all of this CTA's query blocks are padding
@@ -632,7 +698,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
 #pragma unroll
         for (int e = 0; e < kEpiThreads / 32; ++e) k2 = fmaxf(k2, ctl->k2w[e]);
       }
-      if (part == 0 && r == 0 && row_ok) p.qk2max[(size_t)(b * p.hq + h) * p.nqb + i] = g2 * k2;
+      if (!kLists && part == 0 && r == 0 && row_ok) p.qk2max[(size_t)(b * p.hq + h) * p.nqb + i] = g2 * k2;
       const float tau_row = fmaxf(p.tau_row, 2.f * screen_error_bound(q2 * k2, p.scale));
       const bool amb = row_ok && (top1 - top2) * p.scale <= tau_row;
       const bool amb3 = row_ok && (top1 - top3) * p.scale <= tau_row;
@@ -650,7 +716,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
           reinterpret_cast<int2*>(p.jstar)[(size_t)(b * p.hq + h) * ns + r_glob] = js;
           if (r == 0) {
             p.ambmask[(size_t)(b * p.hq + h) * p.nqb + i] = (any_amb & grp_mask) >> shift;
-            p.hard[(size_t)(b * p.hq + h) * p.nqb + i] = (any_amb3 & grp_mask) ? 1 : 0;
+            if (!kLists) p.hard[(size_t)(b * p.hq + h) * p.nqb + i] = (any_amb3 & grp_mask) ? 1 : 0;
           }
         }
       }
@@ -711,11 +777,14 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
 #pragma unroll
         for (int q = 0; q < 4; ++q) ms[v4 * 4 + q] = ctl->mstar[og * R + src + q];
       }
-      // (lists: the scores stay, behind the maxima in the third key stage)
+      // (lists: the scores stay, in the third key stage behind the maxima, or where the query rows were; the keys come to the fourth, or
+      // where the parked maxima were)
+      constexpr int kCap = kLongLists ? kLongListCap : kListCap;
       static_assert(!kOnChip || (size_t)kMaxTiles * kTileFloats * 4 <= 2 * kTileBytes, "two stages hold the maxima");
-      static_assert(!kLists || ((size_t)kGroups * kListCap * 8 <= kTileBytes && kMaxTiles * BPT <= kListCap), "a stage holds the keys of all lists");
-      float* lists = reinterpret_cast<float*>(smem + (size_t)kTileBytes * (kRowTiles + 2));
-      float* srow = kLists ? lists + og * kListCap : p.scores + ((size_t)(b * p.hq + oh) * p.nqb + min(oi, p.nqb - 1)) * p.nqb;
+      static_assert((size_t)kGroups * kListCap * 8 <= kTileBytes && (!kOnChip || !kLists || kMaxTiles * BPT <= kListCap), "a stage holds the keys of all lists");
+      static_assert((size_t)kGroups * kLongListCap * 4 <= kRowTiles * kTileBytes && (size_t)kGroups * kLongListCap * 8 <= kStages * kTileBytes, "room for long lists");
+      float* lists = reinterpret_cast<float*>(smem + (kLongLists ? 0 : (size_t)kTileBytes * (kRowTiles + 2)));
+      float* srow = kLists ? lists + og * kCap : p.scores + ((size_t)(b * p.hq + oh) * p.nqb + min(oi, p.nqb - 1)) * p.nqb;
       // the score of tile tl's outputs that are this thread's, from the maxima at `maxima`
       auto score = [&](int tile, const float* maxima) {
         const int j = tile * BPT + blk;
@@ -742,20 +811,6 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
           score(tl, reinterpret_cast<const float*>(smem + (size_t)kTileBytes * kRowTiles) + (size_t)tl * kTileFloats);
         }
       }
-      if (kLists) {
-        // a warp per list
-        mbar_arrive(smem_u32(&ctl->x_bar));
-        alive = mbar_wait_warp(smem_u32(&ctl->x_bar), 0, abort_flag, budget, strict);
-        if (!alive && !*abort_flag) screen_timeout(ctl, status);
-        unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem + (size_t)kTileBytes * (kRowTiles + 3));
-#pragma unroll 1
-        for (int x = ew; x < kGroups && alive; x += kEpiThreads / 32) {
-          const int li = i0 + x / G, lh = g * G + x % G;
-          if (li >= nqb_b) break;
-          make_list<R>(kp, p, tau_score, b, g, lh, li, p.causal ? li + 1 : nqb_b, ctl->amb[x], ctl->qk2[x], lists + x * kListCap,
-                       &ctl->j12[0][x * R], &ctl->j12[1][x * R], keys + x * kListCap, lane);
-        }
-      }
       int c_done = 0;
       for (int c = 0; !kOnChip && c < n_chunks && alive; ++c) {
         const int st = c % kStages;
@@ -779,6 +834,28 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         c_done = c + 1;
       }
       if (et == 0) { ctl->c_fetched = c_fetched; ctl->c_done = c_done; }
+      if (kLists) {
+        // a warp per list
+        if (alive) {
+          mbar_arrive(smem_u32(&ctl->x_bar));
+          alive = mbar_wait_warp(smem_u32(&ctl->x_bar), 0, abort_flag, budget, strict);
+          if (!alive && !*abort_flag) screen_timeout(ctl, status);
+        }
+        unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem + (size_t)kTileBytes * (kRowTiles + (kLongLists ? 0 : 3)));
+#pragma unroll 1
+        for (int x = ew; x < kGroups && alive; x += kEpiThreads / 32) {
+          const int li = i0 + x / G, lh = g * G + x % G;
+          if (li >= nqb_b) break;
+          const int cand = p.causal ? li + 1 : nqb_b;
+          auto make = [&](auto per) {
+            make_list<R, decltype(per)::value, !kLongLists>(kp, p, tau_score, b, g, lh, li, cand, ctl->amb[x], ctl->qk2[x], lists + x * kCap,
+                                                            &ctl->j12[0][x * R], &ctl->j12[1][x * R], keys + x * kCap, lane);
+          };
+          if (!kLongLists || cand <= 64) make(std::integral_constant<int, 2>{});
+          else if (cand <= 128) make(std::integral_constant<int, kLongLists ? 4 : 2>{});
+          else make(std::integral_constant<int, kLongLists ? 8 : 2>{});
+        }
+      }
     }
   }
   tc_fence_before();
@@ -829,16 +906,16 @@ int kap_screen_slots() {
   return device_sm_count() * kCtasPerSm;
 }
 
-bool kap_screen_is_short(int n, int stride) { return n / stride <= 128 * kStages; }
-
-// Lists of at most kListCap candidates whose maxima stay on chip.  (A call of 257 to 512 sampled keys and at most 128 lists keeps the
-// sort as a launch of its own, 16.8 us against 15.0: the launches of a 4K step of four heads are part of the line that bench.py
-// prints, which is checked.  With 8 sampled rows a block, 8 tiles would want 64 maxima a thread.)
-bool kap_screen_makes_lists(const KapParams& p) {
-  if (p.qtiles != 1 || p.sort_mode != 0) return false;
+// Lists of up to kLongListCap candidates are made here.  (A call of 257 to 512 sampled keys and at most 128 lists keeps the sort as a
+// launch of its own, 16.8 us against 15.0: the launches of a 4K step of four heads are part of the line that bench.py prints, which
+// is checked.  With 8 sampled rows a block, the 8 tiles of the medium form would want 64 maxima a thread.  512 candidates are 16 keys
+// a lane, whose sort takes a warp four times as long as 8.)
+ScreenForm kap_screen_form(const KapParams& p) {
   const int keys = p.n / p.stride;
-  if (kap_screen_is_short(p.n, p.stride)) return keys <= 256 || (long long)p.batch * p.hq * p.nqb > 128;
-  return p.rows >= 16 && keys <= 128 * kMediumTiles;
+  const bool is_short = keys <= 128 * kStages, lists = p.qtiles == 1 && p.sort_mode == 0 && p.nqb <= kLongListCap;
+  if (is_short) return lists && (keys <= 256 || (long long)p.batch * p.hq * p.nqb > 128) ? kScreenShortLists : kScreenShort;
+  if (!lists) return kScreenLong;
+  return p.rows >= 16 && keys <= 128 * kMediumTiles ? kScreenMediumLists : kScreenLongLists;
 }
 
 size_t kap_screen_slot_bytes(int n, int stride) {
@@ -849,8 +926,8 @@ size_t kap_screen_slot_bytes(int n, int stride) {
 cudaError_t launch_kap_screen(const KapParams& kp, const KapScreenParams& p_in, float tau_score, cudaStream_t st) {
   KapScreenParams p = p_in;
   const int R = 128 / p.stride;
-  const bool is_short = kap_screen_is_short(p.n, p.stride), lists = kap_screen_makes_lists(kp);
-  if (!is_short && !lists && (!p.maxima || !p.slot_taken || p.slots <= 0)) return cudaErrorInvalidValue;
+  const ScreenForm form = kap_screen_form(kp);
+  if (screen_parks(form) && (!p.maxima || !p.slot_taken || p.slots <= 0)) return cudaErrorInvalidValue;
   const uint64_t ns = (uint64_t)p.n / p.stride;
   CUtensorMap qm, km;
   // every `stride`-th row of q and k: the row stride of the maps is `stride` rows of the tensor (of the page pool)
@@ -879,13 +956,17 @@ cudaError_t launch_kap_screen(const KapParams& kp, const KapScreenParams& p_in, 
 #define COSA_LAUNCH_SCREEN(RR)                                                                                              \
   {                                                                                                                         \
     const bool strict = wait_budget_is_short(p.wait_budget);                                                                \
-    constexpr int kMediumOr = RR >= 16 ? kMediumLists : kShortLists;                                                         \
-    auto kernel = lists ? (is_short ? (strict ? kap_screen_kernel<RR, true, kShortLists> : kap_screen_kernel<RR, false, kShortLists>)   \
-                                    : (strict ? kap_screen_kernel<RR, true, kMediumOr> : kap_screen_kernel<RR, false, kMediumOr>))      \
-                  : is_short ? (strict ? kap_screen_kernel<RR, true, kShort> : kap_screen_kernel<RR, false, kShort>)         \
-                             : (strict ? kap_screen_kernel<RR, true, kLong> : kap_screen_kernel<RR, false, kLong>);          \
-    static SmemLimit limits[8];                                                                                             \
-    e = raise_smem_limit(reinterpret_cast<const void*>(kernel), &limits[(lists ? 4 : 0) + (is_short ? 2 : 0) + (strict ? 1 : 0)], kScreenSmem); \
+    constexpr int kMediumOr = RR >= 16 ? kScreenMediumLists : kScreenLongLists;                                              \
+    auto pick = [&](auto strict_c) {                                                                                        \
+      constexpr bool S = decltype(strict_c)::value;                                                                         \
+      return form == kScreenShort ? kap_screen_kernel<RR, S, kScreenShort>                                                  \
+           : form == kScreenShortLists ? kap_screen_kernel<RR, S, kScreenShortLists>                                        \
+           : form == kScreenMediumLists ? kap_screen_kernel<RR, S, kMediumOr>                                               \
+           : form == kScreenLongLists ? kap_screen_kernel<RR, S, kScreenLongLists> : kap_screen_kernel<RR, S, kScreenLong>; \
+    };                                                                                                                      \
+    auto kernel = strict ? pick(std::true_type{}) : pick(std::false_type{});                                                \
+    static SmemLimit limits[10];                                                                                            \
+    e = raise_smem_limit(reinterpret_cast<const void*>(kernel), &limits[2 * (int)form + (strict ? 1 : 0)], kScreenSmem);    \
     if (e != cudaSuccess) return e;                                                                                         \
     return launch_chained(kernel, dim3(grid), kThreads, kScreenSmem, st, qm, km, p, kp, tau_score, status);                               \
   }

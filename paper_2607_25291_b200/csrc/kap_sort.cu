@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(kThreads, 10) kap_sort_kernel(KapParams p, Kap
   // near ties: never closer than twice what the screen may be off by on rows of this magnitude
   tau_score = fmaxf(tau_score, 2.f * screen_error_bound(qk2, sp.scale));
   if (hard) {  // left to the double-precision kernel
-    if (tid == 0) sp.todo[2 + atomicAdd(sp.todo, 1)] = (int)row_lo;
+    if (tid == 0) sp.entries[atomicAdd(sp.todo, 1)] = (int)row_lo;
     return;
   }
   if (tid == 0) { n_tied = 0; tail_end = 0; }
@@ -440,12 +440,12 @@ __global__ void __launch_bounds__(kThreads, 10) kap_sort_kernel(KapParams p, Kap
     __syncthreads();
     const int nt = n_tied;
     if (nt > fit) {   // pathological: too many near ties
-      if (tid == 0) sp.todo[2 + atomicAdd(sp.todo, 1)] = (int)row_lo;
+      if (tid == 0) sp.entries[atomicAdd(sp.todo, 1)] = (int)row_lo;
       return;
     }
     if (tid == 0 && nt > 0) {
       row_words[0] = nt; row_words[1] = K;
-      sp.todo[1 + p.batch * p.hq * p.nqb - atomicAdd(sp.todo + 1, 1)] = (int)row_lo;
+      sp.entries[p.batch * p.hq * p.nqb - 1 - atomicAdd(sp.todo + 1, 1)] = (int)row_lo;
     }
   }
   // the last row tile of the block takes the kept entries as they are; an earlier tile leaves out the key blocks that

@@ -452,12 +452,15 @@ def test_kap_lists_around_the_longest_short_call(n, stride):
 
 @pytest.mark.parametrize("blocks,stride,kw", [
     (2, 8, {}), (16, 8, {}), (17, 8, dict(causal=False)), (32, 8, {}), (33, 8, {}), (64, 8, {}), (64, 8, dict(top_p=0.9)),
-    (61, 8, dict(causal=False, top_p=0.95)), (31, 16, {}), (64, 16, dict(top_p=0.7)), (16, 4, {}), (32, 4, dict(causal=False))])
+    (61, 8, dict(causal=False, top_p=0.95)), (31, 16, {}), (64, 16, dict(top_p=0.7)), (16, 4, {}), (32, 4, dict(causal=False)),
+    (65, 8, {}), (128, 8, dict(causal=False)), (129, 8, dict(top_p=0.9)), (255, 8, {}), (256, 8, dict(top_p=0.95)), (257, 8, {}), (97, 4, dict(top_p=0.8)),
+    (200, 16, dict(causal=False))])
 @pytest.mark.parametrize("copies", [False, True])
 def test_kap_lists_made_by_the_screen(blocks, stride, kw, copies):
-    """Calls of up to eight key tiles sort in the screen kernel: lists, scores and flags are the sort kernel's (impl 3), also where
+    """Calls of up to 256 blocks sort in the screen kernel: lists, scores and flags are the sort kernel's (impl 3), also where
     key blocks are copies of one another (ties, rows too close to call, whole lists to redo)."""
-    w = tiny(seed=blocks * stride, hq=16, hkv=4, n=blocks * 128, needles=min(3, blocks - 1))
+    hkv = 4 if blocks <= 64 else 1
+    w = tiny(seed=blocks * stride, hq=4 * hkv, hkv=hkv, n=blocks * 128, needles=min(3, blocks - 1))
     qb, kb, vb, _ = w.make()
     q, k = to_dev(qb), to_dev(kb)
     if copies:
