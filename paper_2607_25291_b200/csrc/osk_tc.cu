@@ -29,20 +29,21 @@
 // early, the last items are dealt out badly: at a walk's start, all blocks of 16K (walks of 1 to 128 blocks) take 3 % longer than
 // when four positions are left.
 // What runs once an item is cold in the instruction cache and costs by its size, and the loop of a computed block (some 22 KB over
-// all roles) loses lines to it: 255 requests an item go to the next cache on walks of 3.4 blocks, 20 a block on long ones.  Code is
+// all roles) loses lines to it: 225 requests an item go to the next cache on walks of 3.4 blocks, 20 a block on long ones.  Code is
 // therefore shared rather than unrolled or inlined twice where walks are short (a form of 88 KB instead of 61: 236 us instead of
 // 209 on walks of 3.4 blocks; one place that fetches K and V tiles instead of two: 175 -> 169, 662 -> 642 on four prompts in
 // 16-token pages); long ones have it written out (kLongWalks).
 // What bounds it: tensor pipe and exponentials both want about 1,024 cycles (0.52 us) of an SM per computed block, 512 per skipped
 // one.  Fitted to single launches at the full clock, an SM takes 1.03 us a computed block with Stage 2 off, 1.19 with it on (the
-// vote keeps the four row warps together), 0.43 a skipped one and 2.2 a work item; the tensor pipe is busy half of the time, and
-// the reads of its operands keep shared memory as busy.  Single launches, a CTA an item -> now: 128K tokens and 4 % computed
-// 7.51 -> 7.39 ms, 32K and 8 % 1.08 -> 1.02, all blocks of 16K 1.92 -> 1.89, walks of 3.4 blocks (2 x 7,808 tokens) 0.246 -> 0.214,
-// 16,384 items of 5.2 blocks 1.23 -> 1.11 (32 query heads everywhere; one CTA of twelve warps per SM with two softmax groups and a
-// controller warp, the arrangement before both: 8.1, 1.25 and 2.00 on the first three; it is still the better one, by up to 6 %,
-// where Stage 2 is on and skips next to nothing of long lists).  Measured and not used (when the first three took 7.15, 1.02
-// and 1.85): P over S in tensor memory (7.9 / 1.11 / 2.26), two threads per row (8.2 / 1.15 / 2.12), tiles prefetched into L2 (+2 to
-// 5 %), V(k) requested before the decision on k after a computed block (128K +4 to 5 %, 32K +6 to 8, walks of 3.4 blocks +9).
+// vote keeps the four row warps together), 0.43 a skipped one and 1.7 a work item; the tensor pipe is busy half of the time, and
+// the reads of its operands keep shared memory as busy.  Single launches, a CTA an item -> several, items decoded in the load
+// warp -> now: 128K tokens and 4 % computed 7.51 -> 7.39 -> 7.30 ms, 32K and 8 % 1.08 -> 1.02 -> 0.95, all blocks of 16K 1.92 ->
+// 1.89 -> 1.81, walks of 3.4 blocks (2 x 7,808 tokens) 0.246 -> 0.214 -> 0.167 (32 query heads everywhere; one CTA of twelve
+// warps per SM with two softmax groups and a controller warp, the arrangement before both: 8.1, 1.25 and 2.00 on the first
+// three; it is still the better one, by up to 6 %, where Stage 2 is on and skips next to nothing of long lists).  Measured and
+// not used (when the first three took 7.15, 1.02 and 1.85): P over S in tensor memory (7.9 / 1.11 / 2.26), two threads per row
+// (8.2 / 1.15 / 2.12), tiles prefetched into L2 (+2 to 5 %), V(k) requested before the decision on k after a computed block
+// (128K +4 to 5 %, 32K +6 to 8, walks of 3.4 blocks +9).
 // Every wait is bounded; a wait that runs out sets the device status word and the CTA winds down without writing
 // results: load and issue warps leave, the row threads, whom no wait holds any more, run to the end of their list.
 #include <math.h>
