@@ -81,7 +81,8 @@ typedef struct {
   int32_t* out_scored;     /* optional [B,Hq,nQB]: blocks whose logits OSK formed                */
   uint32_t* out_decisions; /* optional [B,Hq,nQB,ceil(order_stride/32)]: bit kk set = the block
                               at list position kk was computed                                   */
-  float*  kap_scores;      /* optional [B,Hq,nQB,nQB]: KAP block scores s_ij (Eq. 11), j <= i    */
+  float*  kap_scores;      /* optional [B,Hq,nQB,nQB]: KAP block scores s_ij (Eq. 11), j <= i (of a call whose
+                              wait_cycles ran out: any of them may have been written; so kap_flags)        */
   uint8_t* kap_flags;      /* optional [B,Hq,nQB,nQB]: HRM flags h_ij (Eq. 12)                   */
   void*   workspace;       /* device scratch; NULL -> the library's own per-device scratch,
                               which is allocated (cudaMalloc) on first use or growth and shared
@@ -157,7 +158,7 @@ typedef struct {
   int64_t out_strides[3];
   int64_t wait_cycles;     /* Clock cycles a wait inside a kernel may take before the kernel gives up, sets the
                               device status word (see cosa_device_status) and returns without writing further
-                              results.  0: the default, 2^31 (about a second).  A few cycles make every
+                              results: cosa_kap_select then leaves out_order and out_count as they were.  0: the default, 2^31 (about a second).  A few cycles make every
                               wait that is not already satisfied run out: that is how the tests reach this path
                               without ever leaving a kernel waiting                                       */
 } cosa_options;

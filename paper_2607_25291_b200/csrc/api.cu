@@ -325,7 +325,7 @@ int cosa_kap_select_ex(const void* q, const void* k, const cosa_shape* shape, fl
     e = launch_kap_sort(p, sp, tau_score, st);
     if (e != cudaSuccess) return cuda_fail(e, "kap sort launch");
   }
-  e = launch_kap_fixup(p, sp, lists && form != kScreenLongLists, st);
+  e = launch_kap_fixup(p, sp, form, st);
   if (e != cudaSuccess) return cuda_fail(e, "kap recount launch");
   return COSA_OK;
 }

@@ -104,11 +104,11 @@ struct KapScreenParams {
   int32_t* jstar;        // [B,Hq,N/s,2]    blocks holding each sampled row's largest / second largest block maximum
   uint32_t* ambmask;     // [B,Hq,nQB]      bit r: sampled row r's two best blocks are too close to call in float32
   uint8_t* hard;         // [B,Hq,nQB]      1 = three blocks too close on some row: whole query block goes to double precision.  Where the
-                         // short and medium forms make the lists: what is left to the next, 0 nothing, 1 the list to redo, 2 near ties
+                         // screen makes the lists: a ListState
   int32_t* todo;         // [2] what is left to the next stage: lists to redo, lists with near ties (their rows of `scores` then hold the
                          // chained entries, see kap_recount.cuh)
   int32_t* entries;      // [B*Hq*nQB] ... as flat (b*Hq+h)*nQB+i, the former from the front, the latter from the end: no list is both.  Behind
-                         // `todo`, or where the screen makes the lists itself in the place of qk2max
+                         // `todo`, or where the screen makes the lists itself in the place of qk2max (long calls; short ones have none)
   float* maxima;         // [slots][key tiles][128 rows x 128/R blocks]  per-row block maxima of the CTA that holds the slot
   int32_t* slot_taken;   // [slots]  0 = free; zeroed by kap_norms_kernel
   float* k2part;         // largest squared norms of sampled key rows of the call, one per CTA of kap_norms_kernel; they lie where the
@@ -258,9 +258,6 @@ cudaError_t raise_smem_limit(const void* kernel, SmemLimit* state, size_t bytes)
 
 // every (head, query block) in double precision
 cudaError_t launch_kap_exact(const KapParams& p, cudaStream_t st);
-// works off sp.todo: near ties recounted, whole lists redone
-// (by_flag: sp.hard instead of sp.todo says which)
-cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, bool by_flag, cudaStream_t st);
 // the whole call's key tiles fit the screen's stages: it needs no scratch areas and no norms kernel
 bool kap_screen_supported(int rows, int group, int stride, const KvPaging& pg);
 // Forms of the screen.  Long: block maxima are parked in scratch areas, the norms kernel goes before.  Short: at most 4 key tiles, which
@@ -268,6 +265,14 @@ bool kap_screen_supported(int rows, int group, int stride, const KvPaging& pg);
 // and writes the lists, no sort kernel follows
 enum ScreenForm { kScreenLong, kScreenLongLists, kScreenShort, kScreenShortLists, kScreenMediumLists };
 inline bool screen_parks(ScreenForm f) { return f == kScreenLong || f == kScreenLongLists; }
+// What the screen says of a list it makes: as it stands, all of it to redo, near ties to recount, padding (an empty list)
+enum ListState { kListMade, kListRedo, kListTies, kListPadding };
+// The lists wait in their rows of `scores` until every CTA of the screen has finished, because one of them may yet give up, and a
+// call that gives up leaves the caller's lists as they were; the fix-up hands them over.  Ids are below 256: a byte each, in the row's
+// last words, behind them K - 1; the chained entries of near ties begin the row.  (Against the screen writing to the caller's
+// arrays: Stage 1 of 256 blocks of 32 heads 171.8 -> 172.9 us, of 8 blocks of 2 heads the same.)
+__host__ __device__ constexpr int list_words(int nqb) { return nqb / 4 + 1; }
+__host__ __device__ constexpr int max_chained(int nqb, int most) { return (nqb - 2) / 2 < most ? (nqb - 2) / 2 : most; }
 inline bool screen_makes_lists(ScreenForm f) { return f == kScreenLongLists || f == kScreenShortLists || f == kScreenMediumLists; }
 ScreenForm kap_screen_form(const KapParams& p);
 cudaError_t launch_kap_screen(const KapParams& kp, const KapScreenParams& p, float tau_score, cudaStream_t st);
@@ -281,6 +286,9 @@ int kap_screen_grid(int batch, int hq, int hkv, int nqb, int stride);   // CTAs 
 size_t kap_screen_slot_bytes(int n, int stride);
 // sorts the screened scores, recomputes near-ties in double precision, writes the lists
 cudaError_t launch_kap_sort(const KapParams& p, const KapScreenParams& sp, float tau_score, cudaStream_t st);
+// works off sp.todo (in short and medium calls whose lists the screen made: sp.hard): near ties recounted, whole lists redone; hands
+// over the lists that the screen made
+cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, ScreenForm form, cudaStream_t st);
 size_t kap_exact_smem_bytes(int rows, int nqb, int qtiles);
 // copies the pages of the call's sequences into dense [B, Hkv, N, d] tensors (pools with pages smaller than a key block): K's, and
 // V's if there is a v_pool; every > 1: only the rows whose token index is a multiple of it (pools are contiguous; the staging

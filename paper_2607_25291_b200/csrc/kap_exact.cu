@@ -29,52 +29,96 @@ __global__ void __launch_bounds__(kThreads) kap_exact_kernel(KapParams p, int kb
   kap_exact_item(p, blockIdx.z, blockIdx.y, (p.nqb / p.qtiles - 1 - (int)blockIdx.x) * p.qtiles, kb_per_iter, sort_cap);
 }
 
+// A list of up to 256 blocks that the screen made: its state, its length - 1 and its ids, lane l those at l, l + 32, ...
+struct MadeList { int state, last, id[8]; };
+__device__ __forceinline__ MadeList load_list(const KapParams& p, const KapScreenParams& sp, long long row, int lane) {
+  const uint8_t* kept = reinterpret_cast<const uint8_t*>(sp.scores + (row + 1) * p.nqb - list_words(p.nqb));
+  MadeList m;
+  m.state = sp.hard[row];
+  m.last = kept[p.nqb];
+#pragma unroll
+  for (int x = 0; x < 8; ++x) m.id[x] = lane + 32 * x < p.nqb ? kept[lane + 32 * x] : 0;
+  return m;
+}
+__device__ __forceinline__ void hand_over(const KapParams& p, const MadeList& m, long long row, int lane) {
+  const int K = m.state == kListPadding ? 0 : m.last + 1;
+  int32_t* dst = p.order + row * p.order_stride;
+#pragma unroll
+  for (int x = 0; x < 8; ++x) {
+    const int t = lane + 32 * x;
+    if (t < p.order_stride) dst[t] = t < K ? m.id[x] : -1;
+  }
+  for (int t = lane + 256; t < p.order_stride; t += 32) dst[t] = -1;
+  if (lane == 0) p.count[row] = K;
+}
+
 // 1-d grid: the CTAs share out what the sort stage left.  kTied: lists with near ties to recount; kRedo: lists to do over (normally none).
 // In one launch where the second's shared memory leaves room for several CTAs on an SM, in two otherwise.
+// made: the screen made the lists, and they are handed over first; by_flag: sp.hard, not sp.todo, says what is left of them
 template <bool kTied, bool kRedo>
 __global__ void __launch_bounds__(kThreads, 2) kap_fixup_kernel(KapParams p, KapScreenParams sp, int kb_per_iter, int sort_cap,
-                                                                          bool by_flag, const int32_t* status) {
+                                                                          bool made, bool by_flag, const int32_t* status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int n_found, found[kThreads];
+  const int lists = p.batch * p.hq * p.nqb, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // a list a warp and turn; of lists with flags a thread looks after every gridDim.x-th, 256 a turn
+  long long row = blockIdx.x + (long long)warp * gridDim.x, base = blockIdx.x;
+  const long long row_step = (long long)gridDim.x * (kThreads / 32), mine_at = (long long)threadIdx.x * gridDim.x;
+  if (threadIdx.x == 0) n_found = 0;
   chain_begin();
-  if (*reinterpret_cast<const volatile int32_t*>(status) != 0) return;   // an earlier kernel of the call gave up: the lists are not to be trusted
+  // (all that the first turn reads is requested at once: on a short call this kernel is a chain of round trips)
+  const int poisoned = *reinterpret_cast<const volatile int32_t*>(status);
+  const bool hands_over = kTied && made;
+  MadeList m{};
+  if (hands_over && row < lists) m = load_list(p, sp, row, lane);
+  int state = by_flag && base + mine_at < lists ? sp.hard[base + mine_at] : kListMade;
+  const int n_tied = by_flag ? 0 : sp.todo[1], n_redo = by_flag ? 0 : sp.todo[0];
+  if (poisoned != 0) return;   // an earlier kernel of the call gave up: the lists are not to be trusted
+  while (hands_over && row < lists) {
+    const MadeList now = m;
+    const long long at = row;
+    row += row_step;
+    if (row < lists) m = load_list(p, sp, row, lane);
+    if (now.state == kListMade || now.state == kListPadding) hand_over(p, now, at, lane);
+  }
+  // (a list with near ties is handed over by the CTA that then patches it)
+  auto recount = [&](int r) {
+    if (made && warp == 0) hand_over(p, load_list(p, sp, r, lane), r, lane);
+    kap_recount_item(p, sp, r, smem_raw);
+  };
+  auto redo = [&](int r) {
+    const int i = r % p.nqb, bh = r / p.nqb;
+    kap_exact_item(p, bh / p.hq, bh % p.hq, i, kb_per_iter, sort_cap);   // i: first row tile of the block
+    __syncthreads();
+  };
   if (by_flag) {
-    // every list says what it wants; a CTA looks after every gridDim.x-th, 256 at a time
-    __shared__ int n_found, found[kThreads];
-    const int lists = p.batch * p.hq * p.nqb;
-    for (long long base = blockIdx.x; base < lists; base += (long long)gridDim.x * kThreads) {
-      if (threadIdx.x == 0) n_found = 0;
+    while (true) {
       __syncthreads();
-      const long long mine = base + (long long)threadIdx.x * gridDim.x;
-      const int state = mine < lists ? sp.hard[mine] : 0;
-      if ((kTied && state == 2) || (kRedo && state == 1)) found[atomicAdd(&n_found, 1)] = state == 2 ? -1 - (int)mine : (int)mine;
+      if ((kTied && state == kListTies) || (kRedo && state == kListRedo)) {
+        const int mine = (int)(base + mine_at);
+        found[atomicAdd(&n_found, 1)] = state == kListTies ? -1 - mine : mine;
+      }
       __syncthreads();
       const int n = n_found;
       for (int e = 0; e < n; ++e) {
         const int flat = found[e];
         if (flat < 0) {
-          if (kTied) kap_recount_item(p, sp, -1 - flat, smem_raw);
+          if (kTied) recount(-1 - flat);
         } else if (kRedo) {
-          kap_exact_item(p, flat / p.nqb / p.hq, flat / p.nqb % p.hq, flat % p.nqb, kb_per_iter, sort_cap);
-          __syncthreads();
+          redo(flat);
         }
       }
+      base += (long long)gridDim.x * kThreads;
+      if (base >= lists) return;
+      state = base + mine_at < lists ? sp.hard[base + mine_at] : kListMade;
       __syncthreads();
-    }
-    return;
-  }
-  if (kTied) {
-    const int n = sp.todo[1], last = p.batch * p.hq * p.nqb - 1;
-    for (int e = blockIdx.x; e < n; e += gridDim.x) kap_recount_item(p, sp, sp.entries[last - e], smem_raw);
-  }
-  if (kRedo) {
-    const int n = sp.todo[0];
-    for (int e = blockIdx.x; e < n; e += gridDim.x) {
-      const int flat = sp.entries[e];
-      const int i = flat % p.nqb, bh = flat / p.nqb;
-      kap_exact_item(p, bh / p.hq, bh % p.hq, i, kb_per_iter, sort_cap);   // i: first row tile of the block
-      __syncthreads();
+      if (threadIdx.x == 0) n_found = 0;
     }
   }
+  if (kTied)
+    for (int e = blockIdx.x; e < n_tied; e += gridDim.x) recount(sp.entries[lists - 1 - e]);
+  if (kRedo)
+    for (int e = blockIdx.x; e < n_redo; e += gridDim.x) redo(sp.entries[e]);
 }
 
 __device__ void kap_exact_item(const KapParams& p, const int b, const int h, const int i_lo, int kb_per_iter, int sort_cap) {
@@ -278,17 +322,18 @@ cudaError_t launch_kap_exact(const KapParams& p, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, bool by_flag, cudaStream_t st) {
+cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, ScreenForm form, cudaStream_t st) {
   static_assert(kThreads == kRecountThreads, "one kernel does both");
   const int32_t* status = device_status_word();
   if (!status) return cudaErrorInvalidSymbol;
   const int lists = p.batch * p.hq * (p.nqb / p.qtiles), sms = std::max(1, device_sm_count());
   const int kb = kb_per_iter_for(p.rows), cap = next_pow2(p.nqb);
   const size_t redo = kap_exact_smem_bytes(p.rows, p.nqb, p.qtiles), tied = kap_recount_smem_bytes(p.rows, p.qtiles, p.nqb);
+  const bool made = screen_makes_lists(form), by_flag = made && form != kScreenLongLists;
   static SmemLimit limits[3];
   auto launch = [&](auto kernel, SmemLimit* limit, size_t smem, int ctas) {
     cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kernel), limit, smem);
-    return e != cudaSuccess ? e : launch_chained(kernel, dim3((unsigned)std::min(lists, ctas)), kThreads, smem, st, p, sp, kb, cap, by_flag, status);
+    return e != cudaSuccess ? e : launch_chained(kernel, dim3((unsigned)std::min(lists, ctas)), kThreads, smem, st, p, sp, kb, cap, made, by_flag, status);
   };
   // (a launch costs as much as either does on a short call; at 64K tokens the second alone would leave one CTA per SM)
   const size_t both = std::max(redo, tied);

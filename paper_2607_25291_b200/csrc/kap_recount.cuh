@@ -1,7 +1,7 @@
 // Double-precision recount of a list's near ties (step 3 of the sort stage).
 //
 // The sort kernel leaves, in the list's row of screened scores, [0] = chained entries, [1] = kept count, then per entry
-// 2 * position + (tied with the next position) and the block id.  One CTA of eight warps per list: M*[r] from every row's best
+// chained_entry().  One CTA of eight warps per list: M*[r] from every row's best
 // block (and the runner-up of the rows the screen could not call) and the entries' block maxima, then every entry's score
 // sum_r exp(M[r,j] - M*[r]); chains are re-sorted by it, ties by ascending id, and the lists patched.  A kernel of its own
 // because it wants more registers than the sort, whose lists want many CTAs: 128, two CTAs an SM (with 64 and four CTAs it spilled some
@@ -23,6 +23,9 @@ constexpr int kRecountRows = 64;     // sampled rows of one (possibly two-tile) 
 constexpr int kRecountQuarter = kHeadDim / 4 + 1;      // pitch of a quarter row in doubles (the quarters lie in different banks)
 constexpr int kRecountPad = 4 * kRecountQuarter;       // row pitch
 constexpr int kRecountChunk = 16;    // entries whose maxima are held at a time
+
+// position in the order, tied with the next position, block id (blocks of a call: below 4096, else kap_exact.cu has no room)
+__device__ __forceinline__ int chained_entry(int pos, int link, int id) { return id << 16 | 2 * pos | link; }
 
 __device__ __forceinline__ double bf16_lo(unsigned w) { return (double)__uint_as_float(w << 16); }
 __device__ __forceinline__ double bf16_hi(unsigned w) { return (double)__uint_as_float(w & 0xffff0000u); }
@@ -88,8 +91,8 @@ __device__ __forceinline__ void kap_recount_item(const KapParams& p, const KapSc
   const int* words = reinterpret_cast<const int*>(sp.scores + row_lo * p.nqb);
   const int nt = words[0], K = words[1];
   if (tid < nt) {
-    const int w = words[2 + 2 * tid];
-    tied[tid].pos = w >> 1; tied[tid].link = w & 1; tied[tid].id = (unsigned)words[3 + 2 * tid];
+    const int w = words[2 + tid];
+    tied[tid].pos = (w & 0xffff) >> 1; tied[tid].link = w & 1; tied[tid].id = (unsigned)(w >> 16);
   }
   unsigned long long amb = 0ULL;
   for (int t = 0; t < T; ++t) amb |= (unsigned long long)sp.ambmask[row_lo + t] << (t * R);

@@ -21,8 +21,8 @@
 // every product is done, lays them into the key stages, from where the scores are formed; the norms of the sampled keys are
 // taken from the stages as well, which saves the norms kernel's launch.
 // A CTA holds every score of its lists, and up to 256 candidates it sorts them itself, a warp a list in registers: no sort kernel (a
-// wave of small CTAs each, chains of short steps between barriers), and the scores cross no launch.  Stage 1 at 32K 160 -> 135 us, of
-// four prompts in 16-token pages 157 -> 121, of 201 blocks with Top-p 136 -> 110, of 55 blocks at stride 4 102 -> 58.  Both together, in
+// wave of small CTAs each, chains of short steps between barriers), and no scores cross a launch, only the lists (a byte an entry).
+// Stage 1 at 32K 160 -> 135 us, of four prompts in 16-token pages 157 -> 121, of 201 blocks with Top-p 136 -> 110, of 55 blocks at stride 4 102 -> 58.  Both together, in
 // short calls a chain of latencies (launch, first loads, a wave or two of CTAs): 1K tokens of 2 heads 13.5 -> 10.5 us, 31 blocks of
 // 32 heads 18.0 -> 14.6, 2 x 61 blocks of 32 heads 70 -> 43.
 // What bounds the tiles of long calls: 1,518 cycles of an SM a key tile, where the products want 1,024, for the comparisons of 64
@@ -100,6 +100,14 @@ __device__ __forceinline__ float largest_key_norm(const KapScreenParams& p, int 
 
 constexpr int kMediumTiles = 8;           // key tiles of a call of the medium form
 constexpr int kListCap = 64, kLongListCap = 256;   // candidates a list may have where this kernel makes the lists
+constexpr bool rows_hold_lists() {
+  for (int nqb = 1; nqb <= kLongListCap; ++nqb) {
+    const int chained = max_chained(nqb, kRecountMax);
+    if (list_words(nqb) > nqb || (chained >= 2 && 2 + chained + list_words(nqb) > nqb)) return false;   // (a chain has two entries at least)
+  }
+  return true;
+}
+static_assert(rows_hold_lists(), "a row of scores holds a list and the entries of its near ties");
 
 // (a whole warp) the largest of row `qrow` x the sampled keys of block j that the row sees, in double precision: the arithmetic of
 // f64_block_maxima in kap_sort.cu, the row taken from global memory
@@ -162,20 +170,21 @@ __device__ __forceinline__ void warp_sort_desc(unsigned long long (&k)[PER], int
 
 // (a whole warp) the visit list of one (head, query block) of at most 32 * PER candidates: what kap_sort_kernel does for longer
 // calls, step by step.  score[j]: the screened scores (sign: HRM flag); j1, j2: its rows' best and second best blocks; srt: room for
-// the keys.  What is left for the fix-up: near ties (entries in the list's row of `scores`) or the whole list.  kFlags: sp.hard says
-// so, 0 nothing, 1 the list, 2 ties; else the worklist does
+// the keys.  The list waits in its row of `scores`; what is left for the fix-up: near ties (entries in the same row) or the whole list.
+// sp.hard says so, and without kFlags the worklist, too
 template <int R, int PER, bool kFlags>
 __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float tau_score, int b, int g, int h, int i, int J, uint32_t amb,
                           float qk2, const float* score, const int* j1, const int* j2, unsigned long long* srt, int lane) {
   const size_t row = (size_t)(b * p.hq + h) * p.nqb + i;
-  auto leave = [&](int state) {
+  auto leave = [&](ListState state) {
     if (lane != 0) return;
-    if (kFlags) sp.hard[row] = (uint8_t)state;
-    else if (state == 1) sp.entries[atomicAdd(sp.todo, 1)] = (int)row;
-    else if (state == 2) sp.entries[p.batch * p.hq * p.nqb - 1 - atomicAdd(sp.todo + 1, 1)] = (int)row;
+    sp.hard[row] = (uint8_t)state;
+    if (kFlags) return;
+    if (state == kListRedo) sp.entries[atomicAdd(sp.todo, 1)] = (int)row;
+    else if (state == kListTies) sp.entries[p.batch * p.hq * p.nqb - 1 - atomicAdd(sp.todo + 1, 1)] = (int)row;
   };
   if (signbit(qk2)) {                       // three-way row ambiguity: left to the double-precision kernel
-    leave(1);
+    leave(kListRedo);
     return;
   }
   unsigned long long key[PER];
@@ -288,7 +297,7 @@ __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float t
     any = any || (near && t < K);
     tie[x] = __ballot_sync(0xffffffffu, near);
   }
-  int state = 0;
+  ListState state = kListMade;
   if (__any_sync(0xffffffffu, any)) {
     int e = K;                              // a chain that straddles the end of the kept prefix reaches past it
     bool more = true;
@@ -308,8 +317,8 @@ __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float t
       members[x] = (tie[x] | (tie[x] << 1) | (x > 0 ? tie[x > 0 ? x - 1 : 0] >> 31 : 0u)) & below;
       nt += __popc(members[x]);
     }
-    if (nt > min(kRecountMax, (p.nqb - 2) / 2)) {
-      leave(1);
+    if (nt > max_chained(p.nqb, kRecountMax)) {
+      leave(kListRedo);
       return;
     }
     int* words = reinterpret_cast<int*>(sp.scores + row * p.nqb);
@@ -319,16 +328,23 @@ __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float t
     for (int x = 0; x < PER; ++x) {
       if ((members[x] >> lane) & 1u) {
         const int slot = slot0 + __popc(members[x] & ((1u << lane) - 1u)), t = lane + 32 * x;
-        words[2 + 2 * slot] = 2 * t + (int)((tie[x] >> lane) & 1u);
-        words[3 + 2 * slot] = (int)(0xffffffffu - (unsigned)srt[t]);
+        words[2 + slot] = chained_entry(t, (int)((tie[x] >> lane) & 1u), (int)(0xffffffffu - (unsigned)srt[t]));
       }
       slot0 += __popc(members[x]);
     }
-    state = 2;
+    state = kListTies;
   }
-  int32_t* dst = p.order + row * p.order_stride;
-  for (int t = lane; t < p.order_stride; t += 32) dst[t] = t < K ? (int32_t)(0xffffffffu - (unsigned)srt[t]) : -1;
-  if (lane == 0) p.count[row] = K;
+  const int n_words = list_words(p.nqb);
+  uint32_t* kept = reinterpret_cast<uint32_t*>(sp.scores + (row + 1) * p.nqb - n_words);
+  for (int w = lane; w < n_words; w += 32) {
+    uint32_t bytes = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int t = 4 * w + e;
+      bytes |= (t < K ? 0xffu - ((unsigned)srt[t] & 0xffu) : (t == p.nqb ? (unsigned)K - 1u : 0u)) << (8 * e);
+    }
+    kept[w] = bytes;
+  }
   leave(state);
 }
 
@@ -383,14 +399,9 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (!kLists && blockIdx.x == 0 && threadIdx.x == 0) { p.todo[0] = 0; p.todo[1] = 0; }   // the sort stage (a later launch) counts there
-  if (kLists) {                                   // query blocks that are padding: empty lists
-    for (int x = warp; x < kGroups; x += kThreads / 32) {
-      const int i = i0 + x / G;
-      if (i < nqb_b || i >= p.nqb) continue;
-      const size_t row = (size_t)(b * p.hq + g * G + x % G) * p.nqb + i;
-      for (int t = lane; t < kp.order_stride; t += 32) kp.order[row * kp.order_stride + t] = -1;
-      if (lane == 0) { kp.count[row] = 0; if (!kLongLists) p.hard[row] = 0; }
-    }
+  if (kLists && threadIdx.x < kGroups) {          // query blocks that are padding: empty lists
+    const int x = threadIdx.x, i = i0 + x / G;
+    if (i >= nqb_b && i < p.nqb) p.hard[(size_t)(b * p.hq + g * G + x % G) * p.nqb + i] = kListPadding;
   }
   if (i0 >= nqb_b) return;                        // all of this CTA's query blocks are padding
   // key tile t to its stage (lane 0; paged keys: the 128 sampled keys of a tile come from 128 / spp pages (spp sampled rows each) or

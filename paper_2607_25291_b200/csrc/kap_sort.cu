@@ -240,15 +240,16 @@ __global__ void __launch_bounds__(kThreads, 10) kap_sort_kernel(KapParams p, Kap
   const int tid = threadIdx.x;
   const size_t row_lo = (size_t)(b * p.hq + h) * p.nqb + i_lo;
   const size_t row = row_lo + (T - 1);
+  // a screen kernel that gave up has left the scratch half written: nothing of it may be used for addressing
+  const int poisoned = *reinterpret_cast<const volatile int32_t*>(status);   // (tested together with `hard` below)
   if (i >= nqb_b) {                           // padding past the item's length: empty lists
+    if (poisoned != 0) return;
     for (int tile = 0; tile < T; ++tile) {
       for (int t = tid; t < p.order_stride; t += kThreads) p.order[(row_lo + tile) * p.order_stride + t] = -1;
       if (tid == 0) p.count[row_lo + tile] = 0;
     }
     return;
   }
-  // a screen kernel that gave up has left the scratch half written: nothing of it may be used for addressing
-  const int poisoned = *reinterpret_cast<const volatile int32_t*>(status);   // (tested together with `hard` below)
   unsigned hard = 0u;                         // (tested only after the scores have been requested: one round trip, not two)
   float qk2 = 0.f;                            // largest product of squared norms of the block's sampled query rows and of its keys
   unsigned long long amb = 0ULL;              // bit r: sampled row r of the block was too close to call
@@ -425,15 +426,14 @@ __global__ void __launch_bounds__(kThreads, 10) kap_sort_kernel(KapParams p, Kap
       if (!need_full) break;
       L = sort_head_desc(keys, J, J, head, tmp, tie, &sort_sh, p.sort_mode == 1, tid, &srt);
     }
-    // entries: position and "tied with the next", id
+    // entries: position, "tied with the next", id
     int* row_words = reinterpret_cast<int*>(sp.scores + row_lo * p.nqb);
-    const int fit = min(kRecountMax, (p.nqb * T - 2) / 2);
+    const int fit = max_chained(p.nqb * T, kRecountMax);
     for (int t = tid; t < tail_end; t += kThreads) {
       if ((t > 0 && tie[t - 1]) || tie[t]) {
         const int slot = atomicAdd(&n_tied, 1);
         if (slot < fit) {
-          row_words[2 + 2 * slot] = 2 * t + tie[t];
-          row_words[3 + 2 * slot] = (int)(0xffffffffu - (unsigned)(srt[t] & 0xffffffffu));
+          row_words[2 + slot] = chained_entry(t, tie[t], (int)(0xffffffffu - (unsigned)(srt[t] & 0xffffffffu)));
         }
       }
     }

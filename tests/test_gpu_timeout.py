@@ -119,3 +119,36 @@ def test_osk_writes_no_decisions_of_a_walk_that_was_given_up(cfg1):
         assert bool(((words == 0) | (words == want)).all()), cycles
         given_up += int((~done).sum())
     assert given_up > 0
+
+
+@pytest.mark.parametrize("blocks,hq,hkv,lens", [
+    (31, 32, 8, None), (61, 32, 8, None), (97, 32, 8, None), (257, 8, 2, None),      # a call of each form of the screen
+    (32, 16, 4, (5, 32)), (64, 16, 4, (7, 50)), (100, 16, 4, (100, 9)), (260, 4, 1, (30, 260))])
+def test_kap_call_that_gave_up_leaves_the_lists_as_they_were(blocks, hq, hkv, lens):
+    """Budgets at which the waits of some CTAs run out and those of others do not: a call that reports a timeout has written no
+    list and no count, those of query blocks that are padding included."""
+    batch = 1 if lens is None else len(lens)
+    g = torch.Generator(device="cuda").manual_seed(blocks)
+    q, k = (torch.randn(batch, heads, blocks * 128, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv))
+    extra = {} if lens is None else dict(seq_lens=torch.tensor([x * 128 for x in lens], dtype=torch.int32, device="cuda"))
+
+    def lists(**kw):
+        order = torch.full((batch, hq, blocks, blocks + 1), -7, dtype=torch.int32, device="cuda")
+        count = torch.full((batch, hq, blocks), -7, dtype=torch.int32, device="cuda")
+        cosa.cosa_kap_select(q, k, 0.3, order, count, opt=cosa.default_options(**extra, **kw))
+        return order, count, cosa.cosa_device_status()
+
+    want_order, want_count, status = lists()
+    assert status == 0 and int(want_count.min()) >= (0 if lens else 1)
+    given_up = 0
+    for cycles in [1, 50, *range(200, 8200, 160), 20000, 50000]:
+        order, count, status = lists(wait_cycles=cycles)
+        if status == 0:
+            assert torch.equal(order, want_order) and torch.equal(count, want_count), cycles
+        else:
+            assert status == TIMEOUT and bool((order == -7).all()) and bool((count == -7).all()), cycles
+            given_up += 1
+    assert given_up > 0
+    cosa.cosa_debug_set_device_status(TIMEOUT)
+    order, count, status = lists()
+    assert status == TIMEOUT and bool((order == -7).all()) and bool((count == -7).all())
