@@ -158,7 +158,9 @@ typedef struct {
   int64_t out_strides[3];
   int64_t wait_cycles;     /* Clock cycles a wait inside a kernel may take before the kernel gives up, sets the
                               device status word (see cosa_device_status) and returns without writing further
-                              results: cosa_kap_select then leaves out_order and out_count as they were.  0: the default, 2^31 (about a second).  A few cycles make every
+                              results: cosa_kap_select then leaves out_order and out_count as they were,
+                              cosa_osk_attention writes out, lse, visited and scored of a (head, query block)
+                              all or none of them.  0: the default, 2^31 (about a second).  A few cycles make every
                               wait that is not already satisfied run out: that is how the tests reach this path
                               without ever leaving a kernel waiting                                       */
 } cosa_options;

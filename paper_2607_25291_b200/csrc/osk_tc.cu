@@ -640,14 +640,13 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       }
       // ---- epilogue: the last product, then O / l as bf16.  The next walk's Q and K tiles are on their way meanwhile; the rows
       // of a warp go out through the warp's own rows of P, 64 columns at a time, so that a store covers whole 128-byte lines
-      // and no warp waits for another
       n_base += n;
       const float lse = (m + log2f(l)) * 0.6931471805599453f;
       wait(&ctl->pv_done[1], n_base - 1);
       const int n_pos = cap > 1 ? cnt : 1, n_issued = min(kk + 2, n_pos);   // (Q K^T of a position that was not reached: done, too)
       k_base += n_issued; pos_base += kk + 1;
-      // (a warp that sees the walk given up writes nothing; all leave at the next barrier)
-      if (__any_sync(0xffffffffu, bad || *abort_flag)) continue;
+      // (all rows agree whether the walk was given up: a work item is written whole or not at all)
+      if (bar_red_or(1, kBlock, bad || *abort_flag)) break;
       tc_fence_after();
       const float inv = l > 0.f ? __frcp_rn(l) : 0.f;
       const unsigned long long inv2 = pack_f32x2(inv, inv);

@@ -152,3 +152,37 @@ def test_kap_call_that_gave_up_leaves_the_lists_as_they_were(blocks, hq, hkv, le
     cosa.cosa_debug_set_device_status(TIMEOUT)
     order, count, status = lists()
     assert status == TIMEOUT and bool((order == -7).all()) and bool((count == -7).all())
+
+
+@pytest.mark.parametrize("tb", [1.0, 0.999])
+def test_osk_writes_a_work_item_whole_or_not_at_all(tb):
+    """Budgets at which waits run out at every stage of a walk, and, as one CTA does many short walks, in the load and issue warps
+    while the rows write: out, lse, visited and scored of a work item are those of an undisturbed call, or all as they were."""
+    hq, hkv, nqb = 32, 8, 31
+    g = torch.Generator(device="cuda").manual_seed(3)
+    q, k, v = (torch.randn(1, heads, nqb * 128, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv, hkv))
+    order = torch.arange(nqb, dtype=torch.int32, device="cuda").expand(1, hq, nqb, nqb).contiguous()
+    count = (torch.arange(nqb, dtype=torch.int32, device="cuda") % 6).expand(1, hq, nqb).contiguous()     # (and some empty ones)
+
+    def call(**kw):
+        bufs = alloc_outputs(q, nqb)
+        bufs["out"].fill_(77.0)
+        bufs["lse"].fill_(77.0)
+        bufs["visited"].fill_(-7)
+        bufs["scored"].fill_(-7)
+        cosa.cosa_osk_attention(q, k, v, order, count, tb, bufs["out"], bufs["lse"], bufs["visited"], causal=False,
+                                opt=cosa.default_options(skip_scale=500.0, out_scored=bufs["scored"], **kw))
+        status = cosa.cosa_device_status()
+        return [bufs["out"].view(-1, 128 * 128), bufs["lse"].view(-1, 128), bufs["visited"].view(-1, 1), bufs["scored"].view(-1, 1)], status
+
+    want, status = call()
+    assert status == 0
+    in_part = 0
+    for cycles in [*range(1000, 6000, 10)]:
+        got, status = call(wait_cycles=cycles)
+        assert status in (0, TIMEOUT)
+        done = got[2][:, 0] != -7
+        for a, b, blank in zip(got, want, (77.0, 77.0, -7, -7)):
+            assert bool(torch.where(done[:, None], a == b, a == blank).all()), cycles
+        in_part += int(bool(done.any()) and not bool(done.all()))
+    assert in_part > 0
