@@ -79,7 +79,8 @@ struct __align__(8) ScreenCtl {
   unsigned long long n_read[kStages];   // (kMedium) every epilogue warp has the norms of the stage's keys
   int j12[2][kRows];                    // (lists) blocks holding every row's largest and second largest block maximum
   uint32_t amb[kRows / 8];              // (lists) by row group: rows whose two best blocks are too close to call
-  float qk2[kRows / 8];                 // (lists) by row group: as qk2max, the sign set if the group is `hard`
+  float qk2[kRows / 8];                 // (lists) by row group: as qk2max
+  bool hard[kRows / 8];                 // (lists) by row group: as `hard`
 };
 constexpr size_t kScreenSmem = 1024 + (size_t)kTileBytes * (kRowTiles + kStages) + sizeof(ScreenCtl);
 static_assert(kScreenSmem <= 232448, "shared memory budget of one CTA");
@@ -174,7 +175,7 @@ __device__ __forceinline__ void warp_sort_desc(unsigned long long (&k)[PER], int
 // sp.hard says so, and without kFlags the worklist, too
 template <int R, int PER, bool kFlags>
 __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float tau_score, int b, int g, int h, int i, int J, uint32_t amb,
-                          float qk2, const float* score, const int* j1, const int* j2, unsigned long long* srt, int lane) {
+                          bool hard, float qk2, const float* score, const int* j1, const int* j2, unsigned long long* srt, int lane) {
   const size_t row = (size_t)(b * p.hq + h) * p.nqb + i;
   auto leave = [&](ListState state) {
     if (lane != 0) return;
@@ -183,7 +184,7 @@ __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float t
     if (state == kListRedo) sp.entries[atomicAdd(sp.todo, 1)] = (int)row;
     else if (state == kListTies) sp.entries[p.batch * p.hq * p.nqb - 1 - atomicAdd(sp.todo + 1, 1)] = (int)row;
   };
-  if (signbit(qk2)) {                       // three-way row ambiguity: left to the double-precision kernel
+  if (hard) {                               // three-way row ambiguity: left to the double-precision kernel
     leave(kListRedo);
     return;
   }
@@ -720,7 +721,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         ctl->mstar[row] = top1;
         if (kLists) {
           ctl->j12[0][row] = jstar; ctl->j12[1][row] = jstar2;
-          if (r == 0) { ctl->amb[grp] = (any_amb & grp_mask) >> shift; ctl->qk2[grp] = (any_amb3 & grp_mask) ? -g2 * k2 : g2 * k2; }
+          if (r == 0) { ctl->amb[grp] = (any_amb & grp_mask) >> shift; ctl->qk2[grp] = g2 * k2; ctl->hard[grp] = (any_amb3 & grp_mask) != 0; }
         }
         if (row_ok) {
           int2 js = make_int2(jstar, jstar2);
@@ -859,7 +860,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
           if (li >= nqb_b) break;
           const int cand = p.causal ? li + 1 : nqb_b;
           auto make = [&](auto per) {
-            make_list<R, decltype(per)::value, !kLongLists>(kp, p, tau_score, b, g, lh, li, cand, ctl->amb[x], ctl->qk2[x], lists + x * kCap,
+            make_list<R, decltype(per)::value, !kLongLists>(kp, p, tau_score, b, g, lh, li, cand, ctl->amb[x], ctl->hard[x], ctl->qk2[x], lists + x * kCap,
                                                             &ctl->j12[0][x * R], &ctl->j12[1][x * R], keys + x * kCap, lane);
           };
           if (!kLongLists || cand <= 64) make(std::integral_constant<int, 2>{});

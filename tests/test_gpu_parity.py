@@ -1351,3 +1351,24 @@ def test_host_call_on_both_sides_of_the_split(n, hq, hkv):
     cosa.cosa_prefill_host(qh, kh, vh, shape, 0.2, 0.1, out_h, lse_h, vis_h, ws, opt=opt)
     assert cosa.cosa_device_status() == 0
     assert torch.equal(vis_h, vis.cpu()) and torch.equal(out_h, out.cpu()) and torch.equal(lse_h, lse.cpu())
+
+
+@pytest.mark.parametrize("blocks,stride", [(8, 8), (48, 8), (100, 8), (33, 16), (260, 8)])
+@pytest.mark.parametrize("infinite", [False, True])
+@pytest.mark.parametrize("huge,zero", [("q", "k"), ("k", "q")])
+def test_kap_rows_that_cannot_be_called_beside_norms_past_float32(blocks, stride, huge, zero, infinite):
+    """Inputs whose squared norms overflow float32, or one element of which is infinite, against zeros: the thresholds' product of
+    norms is infinity times zero and tells nothing.  Every block ties on the rows that are finite, and from three blocks on the
+    verdicts are the double-precision kernel's: every block flagged, ascending ids.  (Of one or two blocks the screen's own scores
+    stand, where a row with an infinity gives NaN and no flag.)"""
+    n = blocks * 128
+    t = {huge: torch.full((1, 2, n, 128), 3e19, dtype=torch.bfloat16, device="cuda"),
+         zero: torch.zeros(1, 2, n, 128, dtype=torch.bfloat16, device="cuda")}
+    if infinite:
+        t[huge][:, :, 2 * stride::128, 5] = math.inf
+    order, count, got = run_kap(t["q"], t["k"], 0.4, stride, scores=True)
+    order1, count1, ref = run_kap(t["q"], t["k"], 0.4, stride, scores=True, impl=1)
+    assert int(ref["kap_flags"].sum()) == 2 * blocks * (blocks + 1) // 2
+    assert torch.equal(got["kap_flags"][:, :, 2:], ref["kap_flags"][:, :, 2:])
+    assert torch.equal(got["kap_scores"].nan_to_num(nan=-1.0), ref["kap_scores"].nan_to_num(nan=-1.0))
+    assert torch.equal(count, count1) and torch.equal(order, order1)
