@@ -110,34 +110,64 @@ constexpr bool rows_hold_lists() {
 }
 static_assert(rows_hold_lists(), "a row of scores holds a list and the entries of its near ties");
 
-// (a whole warp) the largest of row `qrow` x the sampled keys of block j that the row sees, in double precision: the arithmetic of
-// f64_block_maxima in kap_sort.cu, the row taken from global memory
-template <int R>
-__device__ double f64_row_maximum(const KapParams& p, const __nv_bfloat16* qrow, int b, int g, int j, int r_glob, int lane) {
+// (a whole warp) the largest of row `qrow` x the sampled keys that the row sees of block j[0] and of block j[1], in double precision:
+// the arithmetic of f64_block_maxima in kap_sort.cu, the row taken from global memory.  Bound by round
+// trips to L2, with few warps to hide them, and by the conversions: the loads of both blocks and of 16 keys of each go out together, of
+// kAhead quarters of their 256 bytes (one block, 8 keys and a quarter at a time, with every block the copy of another: Stage 1 of 31
+// blocks of 32 heads 187 us instead of 138, of 200 blocks 2,097 instead of 1,940, of 8 blocks of 2 heads, whose rows all lie in one
+// CTA, 108 instead of 67; there the sort kernel, impl = 3, takes 56)
+template <int R, int kAhead>
+__device__ __forceinline__ void f64_row_maxima(const KapParams& p, const __nv_bfloat16* qrow, int b, int g, const int (&j)[2], int r_glob,
+                                               int lane, double (&best)[2]) {
+  constexpr int kKeys = R < 16 ? 1 : 2;
   const int quarter = lane & 3;
-  double best = -INFINITY;
+  best[0] = best[1] = -INFINITY;
 #pragma unroll 1
-  for (int c0 = 0; c0 < R; c0 += 8) {
-    const int kc = j * R + c0 + (lane >> 2);
-    const uint4* key = reinterpret_cast<const uint4*>(p.k + kv_off(p.pg, p.ks, b, p.hkv, g, kc * p.stride));
-    double acc = 0.0;
-#pragma unroll 1
-    for (int u = 0; u < 4; ++u) {
-      const uint4 w = key[u * 4 + quarter], q = reinterpret_cast<const uint4*>(qrow)[u * 4 + quarter];
-      const unsigned kw[4] = {w.x, w.y, w.z, w.w}, qw[4] = {q.x, q.y, q.z, q.w};
+  for (int c0 = 0; c0 < R; c0 += 8 * kKeys) {
+    const uint4* key[2][kKeys];
+    double acc[2][kKeys];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        acc = fma(bf16_lo(qw[e]), bf16_lo(kw[e]), acc);
-        acc = fma(bf16_hi(qw[e]), bf16_hi(kw[e]), acc);
+    for (int x = 0; x < 2; ++x)
+#pragma unroll
+      for (int c = 0; c < kKeys; ++c) {
+        key[x][c] = reinterpret_cast<const uint4*>(p.k + kv_off(p.pg, p.ks, b, p.hkv, g, (j[x] * R + c0 + 8 * c + (lane >> 2)) * p.stride)) + quarter;
+        acc[x][c] = 0.0;
       }
+#pragma unroll kAhead
+    for (int u = 0; u < 4; ++u) {
+      const uint4 q = reinterpret_cast<const uint4*>(qrow)[u * 4 + quarter];
+      const unsigned qw[4] = {q.x, q.y, q.z, q.w};
+      uint4 w[2][kKeys];
+#pragma unroll
+      for (int x = 0; x < 2; ++x)
+#pragma unroll
+        for (int c = 0; c < kKeys; ++c) w[x][c] = key[x][c][u * 4];
+#pragma unroll
+      for (int x = 0; x < 2; ++x)
+#pragma unroll
+        for (int c = 0; c < kKeys; ++c) {
+          const unsigned kw[4] = {w[x][c].x, w[x][c].y, w[x][c].z, w[x][c].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            acc[x][c] = fma(bf16_lo(qw[e]), bf16_lo(kw[e]), acc[x][c]);
+            acc[x][c] = fma(bf16_hi(qw[e]), bf16_hi(kw[e]), acc[x][c]);
+          }
+        }
     }
-    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-    if (!p.causal || kc <= r_glob) best = fmax(best, acc * p.scale);
+#pragma unroll
+    for (int x = 0; x < 2; ++x)
+#pragma unroll
+      for (int c = 0; c < kKeys; ++c) {
+        double z = acc[x][c];
+        z += __shfl_xor_sync(0xffffffffu, z, 1);
+        z += __shfl_xor_sync(0xffffffffu, z, 2);
+        if (!p.causal || j[x] * R + c0 + 8 * c + (lane >> 2) <= r_glob) best[x] = fmax(best[x], z * p.scale);
+      }
   }
 #pragma unroll
-  for (int o = 4; o < 32; o <<= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
-  return best;
+  for (int x = 0; x < 2; ++x)
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) best[x] = fmax(best[x], __shfl_xor_sync(0xffffffffu, best[x], o));
 }
 
 // (a whole warp) sorts 32 * PER distinct keys descending (bitonic, in registers); afterwards lane l holds places l * PER and on
@@ -204,11 +234,10 @@ __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float t
     for (uint32_t left = amb; left; left &= left - 1) {
       const int r = __ffs(left) - 1;
       const __nv_bfloat16* qrow = qh + (long long)(i * R + r) * p.stride * p.qs.t;
-#pragma unroll 1
-      for (int which = 0; which < 2; ++which) {
-        const double z = f64_row_maximum<R>(p, qrow, b, g, which ? j2[r] : j1[r], i * R + r, lane);
-        if (lane == r) { if (which) m2 = z; else m1 = z; }
-      }
+      const int two[2] = {j1[r], j2[r]};
+      double z[2];
+      f64_row_maxima<R, kFlags ? 4 : 1>(p, qrow, b, g, two, i * R + r, lane, z);   // (the long form has no registers for more)
+      if (lane == r) { m1 = z[0]; m2 = z[1]; }
     }
     const double best = fmax(m1, m2);
     const bool mine = lane < R && ((amb >> lane) & 1u);
