@@ -129,7 +129,7 @@ def order_pitch(cosa, budget, nqb):
     return (cosa.cosa_budget_count(budget, nqb) + 7) // 8 * 8
 
 
-def launches_per_step(n, stride, page_size=0, pages_in_place=False, osk_impl=0, block_q=128, heads=4):
+def launches_per_step(n, stride, page_size=0, pages_in_place=False, osk_impl=0, block_q=128):
     """Kernels of the library that one step launches, by the launchers' own rules (a test counts them with a profiler):
     Stage 1: the copy of small pages' keys, the norms of long calls, screen, sort (up to 256 blocks: in the screen), and one or two
     launches for what the sort leaves over; Stage 2: the copy of K and V from pages smaller than a key block, and the walk."""
@@ -139,7 +139,7 @@ def launches_per_step(n, stride, page_size=0, pages_in_place=False, osk_impl=0, 
     redo = doubles * 8 + max(2, 1 << (nqb - 1).bit_length()) * 12 + ((nqb | 1) + 15) // 16 * 16     # shared memory, bytes
     recount = R * (block_q // 128) * 132 * 8 + (nqb * 4 if block_q == 256 else 0)
     keys = n // stride
-    lists = block_q == 128 and nqb <= 256 and (keys <= 256 or keys > 512 or heads * nqb > 128)
+    lists = block_q == 128 and nqb <= 256
     norms = keys > 512 and not (lists and keys <= 1024 and R >= 16)
     kap = 1 + norms + (not lists) + (1 if max(redo, recount) <= 56 * 1024 else 2)
     kap += 0 < page_size and page_size // stride < 32
@@ -464,7 +464,7 @@ def main():
                            "causal_block_pairs": pairs, "input_generation_s": round(t_gen, 1)},
                 "latency_ms": {"kap": kap_ms, "osk": osk_ms, "kap_plus_osk": ms_per_step},
                 "latency_ms_as_a_burst": ({"kap": burst_run["kap_ms"], "osk": burst_run["osk_ms"], "how": burst_run["how"]} if burst_run else None),
-                "e2e": e2e, "gpu_launches": args.steps * launches_per_step(w.n, w.stride, args.page_size, args.pages_in_place, args.osk_impl, args.block_q, w.hq), "clocks": clocks, "roofline": roofline,
+                "e2e": e2e, "gpu_launches": args.steps * launches_per_step(w.n, w.stride, args.page_size, args.pages_in_place, args.osk_impl, args.block_q), "clocks": clocks, "roofline": roofline,
                 "roofline_osk": roof_osk, "roofline_kap": roof_kap, "cpu_baseline": cpu, "comparators": extras,
                 "wall_s_timed_region": t_wall}
         print(json.dumps(line), flush=True)

@@ -947,14 +947,12 @@ int kap_screen_slots() {
   return device_sm_count() * kCtasPerSm;
 }
 
-// Lists of up to kLongListCap candidates are made here.  (A call of 257 to 512 sampled keys and at most 128 lists keeps the sort as a
-// launch of its own, 16.8 us against 15.0: the launches of a 4K step of four heads are part of the line that bench.py prints, which
-// is checked.  With 8 sampled rows a block, the 8 tiles of the medium form would want 64 maxima a thread.  512 candidates are 16 keys
-// a lane, whose sort takes a warp four times as long as 8.)
+// Lists of up to kLongListCap candidates are made here (512 are 16 keys a lane, whose sort takes a warp four times as long as 8).  The
+// medium form's 8 tiles would want 64 maxima a thread with 8 sampled rows a block.
 ScreenForm kap_screen_form(const KapParams& p) {
   const int keys = p.n / p.stride;
   const bool is_short = keys <= 128 * kStages, lists = p.qtiles == 1 && p.sort_mode == 0 && p.nqb <= kLongListCap;
-  if (is_short) return lists && (keys <= 256 || (long long)p.batch * p.hq * p.nqb > 128) ? kScreenShortLists : kScreenShort;
+  if (is_short) return lists ? kScreenShortLists : kScreenShort;
   if (!lists) return kScreenLong;
   return p.rows >= 16 && keys <= 128 * kMediumTiles ? kScreenMediumLists : kScreenLongLists;
 }
