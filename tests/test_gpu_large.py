@@ -116,8 +116,8 @@ def test_qwen3_32k_full_kap_and_sampled_osk():
 
 
 def test_qwen3_32k_sort_routes_agree():
-    """The sort stage has three ways to the same list: the buckets at the head of the order (taken here by nearly every list),
-    every key compared with every other, everything sorted.  All 8192 lists must come out identical on each (the first one is
+    """Three ways to the same list: the screen's own sort (up to 256 blocks, as here), and the sort kernel with every key compared
+    with every other and with the whole order sorted.  All 8192 lists must come out identical on each (the first one is
     checked against the oracle, list by list, by the test above)."""
     w = WORKLOADS["qwen3_32k"]
     qb, kb, _, _ = w.make()

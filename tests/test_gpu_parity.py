@@ -333,11 +333,11 @@ MID_BLOCKS = [0, 1, 63, 64, 71, 72, 89, 90, 100, 117, 126, 127]
 @pytest.mark.parametrize("impl", [0, 2, 3])
 @pytest.mark.parametrize("budget", [0.05, 0.1, 0.25, 0.6])
 def test_kap_16k_head_of_the_order(mid, budget, impl):
-    """At 128 key blocks and a small budget the fast path selects and sorts only the head of the order (kept prefix
-    plus a margin); larger budgets and short candidate lists sort everything.  Both must give the oracle's lists."""
+    """128 key blocks: impl = 0 sorts in the screen kernel, 2 and 3 in the sort kernel, every key compared with every other.  All
+    give the oracle's lists.  (The head of the order alone is sorted from 257 blocks on: test_kap_order_where_the_sort_changes_its_way.)"""
     q, k, _ = mid["dev"]
     qf, kf, _ = mid["f64"]
-    order, count = run_kap(q, k, budget, 8, impl=impl)   # 2, 3: the sort stage's fall-back routes, forced
+    order, count = run_kap(q, k, budget, 8, impl=impl)
     ref_order, ref_count = O.kap_select(qf, kf, s=8, budget=budget, order_stride=order.shape[-1], query_blocks=MID_BLOCKS)
     for i in MID_BLOCKS:
         assert np.array_equal(_np(count)[:, i], ref_count[:, i]), i
@@ -345,9 +345,9 @@ def test_kap_16k_head_of_the_order(mid, budget, impl):
 
 
 def test_kap_16k_tie_chain_longer_than_the_margin(mid):
-    """Forty identical key blocks score exactly alike: a chain of near ties far longer than the margin kept beyond the
-    prefix, which the head selection must hand over to the full sort, and whose members the double-precision
-    recount must put in ascending-id order."""
+    """Forty identical key blocks score exactly alike: a chain of near ties that reaches far beyond the kept prefix, whose members
+    the double-precision recount must put in ascending-id order, after the screen's sort as after the sort kernel's.  (For the
+    margin of the sort kernel's head see the next test.)"""
     q, k, _ = mid["dev"]
     qf, kf, _ = mid["f64"]
     k2, kf2 = k.clone(), kf.copy()
@@ -361,6 +361,32 @@ def test_kap_16k_tie_chain_longer_than_the_margin(mid):
         for i in blocks:
             assert np.array_equal(_np(count)[:, i], ref_count[:, i]), (budget, i)
             assert np.array_equal(_np(order)[:, i], ref_order[:, i]), (budget, i)
+
+
+def test_kap_tie_chain_longer_than_the_margin_of_a_long_call():
+    """300 blocks: the sort kernel orders the head alone, the kept prefix and a margin of 32 entries.  Ninety identical key blocks are
+    a chain that begins inside the prefix and ends beyond the margin: the rest is sorted, too, and the recount puts the chain in
+    ascending-id order."""
+    w = tiny(seed=300, hq=2, hkv=1, n=300 * 128, needles=8)
+    qb, kb, _, _ = w.make()
+    kb = kb.copy()
+    for dst in range(101, 190):
+        kb[:, dst * 128:(dst + 1) * 128] = kb[:, 100 * 128:101 * 128]
+    q, k = to_dev(qb), to_dev(kb)
+    qf, kf = widen(qb, kb)
+    blocks, chains = [200, 256, 299], 0
+    whole, _ = O.kap_select(qf, kf, s=16, budget=1.0, order_stride=300, query_blocks=blocks)
+    for budget in (0.2, 0.3):
+        order, count = run_kap(q, k, budget, 16)
+        for h in range(2):
+            for i in blocks:
+                K = O.budget_count(budget, i + 1)
+                assert int(_np(count)[h, i]) == K
+                assert np.array_equal(_np(order)[h, i, :K], whole[h, i, :K]) and (_np(order)[h, i, K:] == -1).all(), (budget, h, i)
+                at = np.flatnonzero((whole[h, i] >= 100) & (whole[h, i] < 190))
+                assert len(at) == 90 and at[-1] - at[0] == 89
+                chains += int(at[0] < K and at[-1] >= K + 32 + 16)     # (a bucket holds some eight keys)
+    assert chains >= 3
 
 
 def _scaled_bits(bits, factor, outliers=(), outlier_factor=1.0):
@@ -1094,6 +1120,46 @@ def test_batch_with_different_lengths(impl, causal, n, lens):
     paged = run(q2, kpool, vpool, 2, n, seq_lens=seq_lens, kv_page_table=table, kv_page_size=page_size,
                 kv_num_pages=kpool.shape[0])
     check(paged)
+
+
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("n,lens", [(4096, [32, 13]), (8192, [21, 64]), (8192, [64, 1]), (12288, [96, 37]), (12288, [70, 96]), (32768, [131, 256]),
+                                    (33280, [260, 9])])
+def test_kap_batch_with_different_lengths_on_every_form(n, lens, causal):
+    """Prompts of `lens` blocks padded to n tokens, in calls of up to four key tiles, of up to eight and of more, whose lists the screen
+    makes, and in one the sort kernel takes: whole CTAs of the screen and parts of one lie in the padding, and copied key blocks leave
+    lists to recount and lists to redo.  Dense and in pages of 256 tokens, read in place, every item is what a call on its
+    unpadded tensors gives with the sort kernel."""
+    nqb = n // 128
+    g = torch.Generator(device="cuda").manual_seed(nqb)
+    q, k = (torch.randn(2, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (4, 2))
+    kb = k.view(2, 2, nqb, 128, 128)
+    kb[:, 0, 5::7] = kb[:, 0, 5:6].clone()                     # many alike: lists to redo
+    kb[:, 1, 8] = kb[:, 1, 3]                                  # one pair: lists to recount
+
+    def lists(q, k, n_tok, **kw):
+        order = torch.full((q.shape[0], 4, n_tok // 128, nqb), -7, dtype=torch.int32, device="cuda")
+        count = torch.full((q.shape[0], 4, n_tok // 128), -7, dtype=torch.int32, device="cuda")
+        cosa.cosa_kap_select(q, k, 0.3, order, count, causal=causal, opt=cosa.default_options(**kw))
+        assert cosa.cosa_device_status() == 0
+        return order, count
+
+    seq_lens = torch.tensor([x * 128 for x in lens], dtype=torch.int32, device="cuda")
+    both = [lists(q, k, n, seq_lens=seq_lens)]
+    pages = n // 256
+    at = torch.randperm(2 * pages, generator=torch.Generator().manual_seed(5)).cuda()
+    pool = torch.empty(2 * pages, 2, 256, 128, dtype=torch.bfloat16, device="cuda")
+    pool[at] = k.view(2, 2, pages, 256, 128).transpose(1, 2).reshape(2 * pages, 2, 256, 128)
+    table = at.view(2, pages).to(torch.int32)
+    for b, blocks in enumerate(lens):
+        table[b, (blocks + 1) // 2:] = 0                       # past the length: some other page
+    both.append(lists(q, pool, n, seq_lens=seq_lens, kv_page_table=table, kv_page_size=256, kv_num_pages=2 * pages))
+    for b, blocks in enumerate(lens):
+        cut = lambda t: t[b:b + 1, :, :blocks * 128].contiguous()
+        order1, count1 = lists(cut(q), cut(k), blocks * 128, impl=3)
+        for order, count in both:
+            assert torch.equal(count[b:b + 1, :, :blocks], count1) and torch.equal(order[b:b + 1, :, :blocks], order1), b
+            assert bool((count[b, :, blocks:] == 0).all()) and bool((order[b, :, blocks:] == -1).all()), b
 
 
 @pytest.mark.parametrize("impl", OSK_IMPLS)

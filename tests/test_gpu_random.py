@@ -27,7 +27,8 @@ def _draw_heads(rng):
 
 
 def test_random_kap_routes_agree():
-    """Screen + buckets at the head, all keys in one bucket, full sort and the fp64 kernel write the same lists (bit-exact)."""
+    """The screen's own sort (up to 256 blocks), the sort kernel with all keys in one bucket and with a full sort, and the fp64
+    kernel write the same lists (bit-exact)."""
     rng = np.random.default_rng(20260725)
     for _ in range(24):
         hq, hkv = _draw_heads(rng)
@@ -50,6 +51,33 @@ def test_random_kap_routes_agree():
         for impl, (order, count) in enumerate(results[1:], start=1):
             assert torch.equal(count, results[0][1]), (impl, what)
             assert torch.equal(order, results[0][0]), (impl, what)
+
+
+def test_random_kap_routes_agree_on_long_calls():
+    """The same from 257 blocks on, where the sort kernel's buckets at the head of the order are the default."""
+    rng = np.random.default_rng(20260728)
+    for _ in range(10):
+        hq, hkv = _draw_heads(rng)
+        nqb = int(rng.integers(257, 420))
+        stride = int(rng.choice([8, 16]))
+        budget = float(rng.choice([0.03, 0.1, 0.2, 0.5, 1.0]))
+        causal = bool(rng.random() < 0.8)
+        g = torch.Generator(device="cuda").manual_seed(int(rng.integers(1, 10**6)))
+        q, k = (torch.randn(1, heads, nqb * 128, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv))
+        kb = k.view(1, hkv, nqb, 128, 128)
+        src, dst = (torch.from_numpy(rng.permutation(nqb)[:int(rng.integers(0, 12))].astype(np.int64)).cuda() for _ in range(2))
+        m = min(len(src), len(dst))
+        kb[:, :, dst[:m]] = kb[:, :, src[:m]]                # a few copies: near ties
+        results = []
+        for impl in (0, 1, 2, 3):
+            order = torch.full((1, hq, nqb, nqb), -5, dtype=torch.int32, device="cuda")
+            count = torch.full((1, hq, nqb), -5, dtype=torch.int32, device="cuda")
+            cosa.cosa_kap_select(q, k, budget, order, count, causal=causal, opt=cosa.default_options(stride=stride, impl=impl))
+            assert cosa.cosa_device_status() == 0
+            results.append((order, count))
+        what = dict(hq=hq, hkv=hkv, nqb=nqb, stride=stride, budget=budget, causal=causal)
+        for impl, (order, count) in enumerate(results[1:], start=1):
+            assert torch.equal(count, results[0][1]) and torch.equal(order, results[0][0]), (impl, what)
 
 
 def test_random_osk_kernels_agree():
