@@ -378,7 +378,7 @@ __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float t
   leave(state);
 }
 
-// kStrict: every multi-lane wait answers per warp (see mbar_wait_warp).  kForm: see above
+// kStrict: the call's budget for waits is short; waits are polled and answer per warp (see mbar_poll).  kForm: see above
 template <int R, bool kStrict, int kForm>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
@@ -510,7 +510,12 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const uint32_t tmem = ctl->tmem_base;
   volatile int* abort_flag = &ctl->abort_flag;
   const long long budget = p.wait_budget;
-  constexpr bool strict = kStrict;
+  auto wait = [&](uint32_t bar, uint32_t parity) {
+    return kStrict ? mbar_poll(bar, parity, abort_flag, budget) : mbar_wait(bar, parity, abort_flag, budget);
+  };
+  auto wait_warp = [&](uint32_t bar, uint32_t parity) {
+    return kStrict ? mbar_poll_warp(bar, parity, abort_flag, budget) : mbar_wait(bar, parity, abort_flag, budget);
+  };
   const bool poisoned = ctl->poisoned != 0;
 
   if (poisoned) {
@@ -521,8 +526,8 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       if (lane == 0) {
         for (int t = n_first; t < n_tiles; ++t) {
           const int st = t % kStages;
-          if (!mbar_wait(smem_u32(&ctl->k_empty[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget) ||
-              (kMedium && !mbar_wait(smem_u32(&ctl->n_read[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget))) {
+          if (!wait(smem_u32(&ctl->k_empty[st]), ((t / kStages) & 1) ^ 1) ||
+              (kMedium && !wait(smem_u32(&ctl->n_read[st]), ((t / kStages) & 1) ^ 1))) {
             if (!*abort_flag) screen_timeout(ctl, status);
             break;
           }
@@ -535,8 +540,8 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         const int st = t % kStages;
         int ok = 1;
         if (lane == 0) {
-          ok = mbar_wait(smem_u32(&ctl->k_empty[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget) ? 1 : 0;
-          if (kMedium && ok) ok = mbar_wait(smem_u32(&ctl->n_read[st]), ((t / kStages) & 1) ^ 1, abort_flag, budget) ? 1 : 0;
+          ok = wait(smem_u32(&ctl->k_empty[st]), ((t / kStages) & 1) ^ 1) ? 1 : 0;
+          if (kMedium && ok) ok = wait(smem_u32(&ctl->n_read[st]), ((t / kStages) & 1) ^ 1) ? 1 : 0;
           if (!ok && !*abort_flag) screen_timeout(ctl, status);
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -549,7 +554,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16(128, 128, 0, 0);
-      bool alive = mbar_wait(smem_u32(&ctl->a_full), 0, abort_flag, budget);
+      bool alive = wait(smem_u32(&ctl->a_full), 0);
       if (!alive && !*abort_flag) screen_timeout(ctl, status);
       int t_done = 0;
       // (the barriers of the next tile are looked at between the products on this one's row tiles: asked behind them, the tensor
@@ -557,8 +562,8 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       bool k_here = false, s_here = false;
       for (int t = 0; t < n_tiles && alive; ++t) {
         const int st = t % kStages, sb = t % kSteps, st1 = (t + 1) % kStages, sb1 = (t + 1) % kSteps;
-        alive = (k_here || mbar_wait(smem_u32(&ctl->k_full[st]), (t / kStages) & 1, abort_flag, budget)) &&
-                (s_here || mbar_wait(smem_u32(&ctl->s_empty[sb]), ((t / kSteps) & 1) ^ 1, abort_flag, budget));
+        alive = (k_here || wait(smem_u32(&ctl->k_full[st]), (t / kStages) & 1)) &&
+                (s_here || wait(smem_u32(&ctl->s_empty[sb]), ((t / kSteps) & 1) ^ 1));
         if (!alive) { if (!*abort_flag) screen_timeout(ctl, status); break; }
         tc_fence_after();
         const uint64_t kdesc = smem_desc_sw128(k_sm + st * kTileBytes, 16, 1024);
@@ -603,7 +608,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     // chunk order is rotated by the lane so that the rows of a warp hit different banks)
     float q2 = 0.f, g2 = 0.f;
     float k2 = kOnChip ? 0.f : largest_key_norm(p, lane);
-    bool alive = mbar_wait_warp(smem_u32(&ctl->a_full), 0, abort_flag, budget, strict);
+    bool alive = wait_warp(smem_u32(&ctl->a_full), 0);
     if (!alive && !*abort_flag) screen_timeout(ctl, status);
     if (alive) {
       const unsigned char* arow = smem + (size_t)rt * kTileBytes + (size_t)(row % 128) * 128;
@@ -624,7 +629,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     // one key tile: this row's block maxima, and the three largest so far
     auto take_tile = [&](int t, float (&mb)[BPC]) {
       const int sb = t % kSteps, st = t % kStages;
-      if (!mbar_wait_warp(smem_u32(&ctl->k_empty[st]), (t / kStages) & 1, abort_flag, budget, strict)) {   // this tile's MMAs finished
+      if (!wait_warp(smem_u32(&ctl->k_empty[st]), (t / kStages) & 1)) {   // this tile's MMAs finished
         if (!*abort_flag) screen_timeout(ctl, status);
         return false;
       }
@@ -680,7 +685,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
 #pragma unroll
       for (int t = 0; t < kMaxTiles; ++t) {
         if (t < n_tiles && alive) {
-          alive = take_tile(t, mb_all[t]) && mbar_wait_warp(smem_u32(&ctl->k_full[t % kStages]), (t / kStages) & 1, abort_flag, budget, strict);
+          alive = take_tile(t, mb_all[t]) && wait_warp(smem_u32(&ctl->k_full[t % kStages]), (t / kStages) & 1);
           // squared norms of the tile's sampled keys: four threads a row, the chunks of odd rows in another order (other banks)
           const int et = threadIdx.x - 64, krow = et >> 2;
           const unsigned char* src = smem + (size_t)kTileBytes * (kRowTiles + t % kStages) + krow * 128;
@@ -716,7 +721,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       ctl->xt[part][0][row] = top1; ctl->xt[part][1][row] = top2; ctl->xt[part][2][row] = top3;
       ctl->xj[part][0][row] = jstar; ctl->xj[part][1][row] = jstar2;
       mbar_arrive(smem_u32(&ctl->x_bar));
-      alive = mbar_wait_warp(smem_u32(&ctl->x_bar), 0, abort_flag, budget, strict);
+      alive = wait_warp(smem_u32(&ctl->x_bar), 0);
       if (!alive && !*abort_flag) screen_timeout(ctl, status);
     }
     if (alive) {
@@ -774,7 +779,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       // every row's M* in shared memory and every parked maximum visible to the whole CTA
       __threadfence_block();
       mbar_arrive(smem_u32(&ctl->x_bar));
-      alive = mbar_wait_warp(smem_u32(&ctl->x_bar), 1, abort_flag, budget, strict);
+      alive = wait_warp(smem_u32(&ctl->x_bar), 1);
       if (!alive && !*abort_flag) screen_timeout(ctl, status);
     }
     if (alive) {
@@ -857,13 +862,13 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         const int st = c % kStages;
         if (et == 0 && c + kStages - 1 < n_chunks) {
           // the stage of chunk c - 1 takes chunk c + kStages - 1 once every thread has read it
-          if (c > 0 && !mbar_wait(smem_u32(&ctl->m_empty[(c - 1) % kStages]), ((c - 1) / kStages) & 1, abort_flag, budget)) {
+          if (c > 0 && !wait(smem_u32(&ctl->m_empty[(c - 1) % kStages]), ((c - 1) / kStages) & 1)) {
             if (!*abort_flag) screen_timeout(ctl, status);
           } else {
             fetch(c + kStages - 1);
           }
         }
-        alive = mbar_wait_warp(smem_u32(&ctl->m_full[st]), (c / kStages) & 1, abort_flag, budget, strict);
+        alive = wait_warp(smem_u32(&ctl->m_full[st]), (c / kStages) & 1);
         if (!alive) { if (!*abort_flag) screen_timeout(ctl, status); break; }
         const int tiles_here = min(kTilesPerChunk, n_tiles - c * kTilesPerChunk);
         const float* stage = reinterpret_cast<const float*>(smem + (size_t)kTileBytes * (kRowTiles + st));
@@ -879,7 +884,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         // a warp per list
         if (alive) {
           mbar_arrive(smem_u32(&ctl->x_bar));
-          alive = mbar_wait_warp(smem_u32(&ctl->x_bar), 0, abort_flag, budget, strict);
+          alive = wait_warp(smem_u32(&ctl->x_bar), 0);
           if (!alive && !*abort_flag) screen_timeout(ctl, status);
         }
         unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem + (size_t)kTileBytes * (kRowTiles + (kLongLists ? 0 : 3)));

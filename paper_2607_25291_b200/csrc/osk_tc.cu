@@ -252,7 +252,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
   if (warp >= kLoadWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     // (one answer per warp: all lanes fetch together)
-    auto wait = [&](unsigned long long* bar, int phase) { return mbar_wait_warp(smem_u32(bar), phase & 1, abort_flag, budget, true); };
+    auto wait = [&](unsigned long long* bar, int phase) { return mbar_wait_warp(smem_u32(bar), phase & 1, abort_flag, budget); };
     // Further items come from the grid itself, in launch order, as long as CTAs of it are waiting for an SM.  (A grid that fits
     // on the chip asks for none: a CTA might take what an SM is about to start)
     const bool ask = (int)gridDim.x > p.wave;
@@ -261,7 +261,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       // These waits last as long as a walk does, however short the steps of the others are: the caller's budget is theirs, and this
       // warp leaves when one of them has run out
       auto wait = [&](unsigned long long* bar, int phase) {
-        return mbar_wait_warp(smem_u32(bar), phase & 1, abort_flag, max(budget, 1LL << 31), true);
+        return mbar_wait_warp(smem_u32(bar), phase & 1, abort_flag, max(budget, 1LL << 31));
       };
       int n_q = 1, n_walk = 0;                 // Q tiles requested (the first above), items with blocks
       int b_known = -1, nqb_b = 0;             // batch item of the lengths below

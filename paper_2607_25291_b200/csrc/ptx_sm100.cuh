@@ -72,26 +72,26 @@ __device__ __forceinline__ bool mbar_wait_noabort(uint32_t bar, uint32_t parity,
     if (clock64() - t0 > budget) return false;
   return true;
 }
-// For code all 32 lanes of a warp run together: the same bounded wait, with one answer for the whole warp when
-// `unanimous` is set.  Lanes poll on their own (the cheapest way to wait), so they can see the budget run out at
-// different moments, and what follows -- tcgen05.ld/st, __syncwarp -- must be executed by all lanes or by none.  With
-// the regular budget (about a second) the lanes of a warp, which start their waits within a few cycles of each other,
-// cannot disagree unless the barrier completes in the very cycles in which a second of waiting ends.  The OSK's load warp always
-// votes; the screen, in which sixteen warps wait for every tile, has an instantiation with the votes, launched when the
-// caller has set a short budget (wait_budget_is_short), where lanes disagreeing is the expected case.
+// For code all 32 lanes of a warp run together: the same bounded wait, with one answer for the whole warp.  Lanes poll on their own
+// (the cheapest way to wait), so they can see the budget run out at different moments, and what follows -- tcgen05.ld/st,
+// __syncwarp -- must be executed by all lanes or by none.  With the regular budget (about a second) the lanes of a warp, which
+// start their waits within a few cycles of each other, cannot disagree unless the barrier completes in the very cycles in
+// which a second of waiting ends.  The OSK's load warp always votes; the screen, in which sixteen warps wait for every tile, has
+// an instantiation with votes, launched when the caller has set a short budget, where lanes disagreeing is the expected case.
 __host__ __device__ inline bool wait_budget_is_short(long long budget) { return budget < (1LL << 24); }
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget,
-                                               bool unanimous) {
-  const bool ok = mbar_wait(bar, parity, abort_flag, budget);
-  return unanimous ? (__all_sync(0xffffffffu, ok) != 0) : ok;
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, budget)) != 0;
 }
-// A bounded wait (all lanes, one answer) that never suspends beyond its budget: mbarrier.try_wait may be suspended until the phase
-// completes and then report success, however short the budget is.
-__device__ __forceinline__ bool mbar_poll_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget) {
+// Waits that never suspend beyond their budget (mbarrier.try_wait may be suspended until the phase completes and then report
+// success, however short the budget is): of one thread, and of a warp with one answer
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget) {
   const long long t0 = clock64();
   bool ok;
   while (!(ok = mbar_test_wait(bar, parity)) && !*abort_flag && clock64() - t0 <= budget) __nanosleep(32);
-  return __all_sync(0xffffffffu, ok) != 0;
+  return ok;
+}
+__device__ __forceinline__ bool mbar_poll_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget) {
+  return __all_sync(0xffffffffu, mbar_poll(bar, parity, abort_flag, budget)) != 0;
 }
 // 16 bytes of shared memory another thread has written (ordered by the barrier waited for before)
 __device__ __forceinline__ uint4 ld_shared_128(uint32_t addr) {

@@ -149,6 +149,8 @@ def test_kap_call_that_gave_up_leaves_the_lists_as_they_were(blocks, hq, hkv, le
             assert status == TIMEOUT and bool((order == -7).all()) and bool((count == -7).all()), cycles
             given_up += 1
     assert given_up > 0
+    for _ in range(20):          # a wait that is not satisfied on the spot is not slept through, either
+        assert lists(wait_cycles=1)[2] == TIMEOUT
     cosa.cosa_debug_set_device_status(TIMEOUT)
     order, count, status = lists()
     assert status == TIMEOUT and bool((order == -7).all()) and bool((count == -7).all())
