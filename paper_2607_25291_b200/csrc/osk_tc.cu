@@ -68,7 +68,7 @@ constexpr int kCtasPerSm = 2;
 constexpr int kTmemCols = 256;
 constexpr int kLoadWarp = 4, kMmaWarp = 5, kItemWarp = 6;
 constexpr int kAskAhead = 4;                       // positions (or two computed blocks) before a walk's end at which more work is asked for
-constexpr int kShortWalk = 64, kShortWalkAll = 32;  // list pitch up to which walks count as short, with and without Stage 2
+constexpr int kShortWalk = 64, kShortWalkAll = 16;  // list pitch up to which walks count as short, with and without Stage 2
 constexpr uint32_t kDecComputed = 1, kDecEnd = 2;
 constexpr int kTimedOut = 1, kPoisoned = 2;
 
@@ -727,8 +727,13 @@ cudaError_t launch_osk_tc(const OskParams& p_in, cudaStream_t st) {
       !make_kv_map(&vm, &vo, p.v, p.pg, p.ks, p.batch, p.hkv, p.n, v_box))
     return cudaErrorInvalidValue;
   const bool small_pages = p.pg.table && p.pg.page_size < kBlock;
-  // Where the line lies, shared against written out (us a pass): Stage 2 on, lists of up to 16 blocks 241 / 247, of 52 the same, of
-  // 104 9,811 / 9,615, of 256 11,122 / 10,883; Stage 2 off, of 5 blocks 148 / 150, of 64 4,912 / 4,858
+  // Where the line lies, by the pitch, since the host knows no lengths.  Shared / written out, us a launch, 16K tokens of 32 heads,
+  // lists of at most
+  //                          4        8       16       24       32         48         64         96        128 blocks
+  // Stage 2 off        157/161  270/271  493/488  737/699  935/898  1338/1282  1615/1546  2023/1967  2147/2089
+  // on                 166/175  262/275  436/447  559/571  669/676    881/871  1005/1026  1187/1177  1265/1258
+  // on, cap half of it  93/ 96  133/150  237/253  341/360  465/478    724/733    920/915  1167/1146  1227/1196
+  // (two runs of one side differ by up to 5 % from 8 to 48 blocks; of 256 blocks, 64K tokens, on: 11,122/10,883)
   const bool long_walks = p.mask || p.order_stride > (p.stage2 ? kShortWalk : kShortWalkAll);
   auto pick = [&](auto mask_c, auto long_c) {
     constexpr bool M = decltype(mask_c)::value, L = decltype(long_c)::value;
