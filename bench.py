@@ -129,6 +129,10 @@ def order_pitch(cosa, budget, nqb):
     return (cosa.cosa_budget_count(budget, nqb) + 7) // 8 * 8
 
 
+def screen_makes_lists(n, block_q=128):
+    return block_q == 128 and n // 128 <= 256
+
+
 def launches_per_step(n, stride, page_size=0, pages_in_place=False, osk_impl=0, block_q=128):
     """Kernels of the library that one step launches, by the launchers' own rules (a test counts them with a profiler):
     Stage 1: the copy of small pages' keys, the norms of long calls, screen, sort (up to 256 blocks: in the screen), and one or two
@@ -139,7 +143,7 @@ def launches_per_step(n, stride, page_size=0, pages_in_place=False, osk_impl=0, 
     redo = doubles * 8 + max(2, 1 << (nqb - 1).bit_length()) * 12 + ((nqb | 1) + 15) // 16 * 16     # shared memory, bytes
     recount = R * (block_q // 128) * 132 * 8 + (nqb * 4 if block_q == 256 else 0)
     keys = n // stride
-    lists = block_q == 128 and nqb <= 256
+    lists = screen_makes_lists(n, block_q)
     norms = keys > 512 and not (lists and keys <= 1024 and R >= 16)
     kap = 1 + norms + (not lists) + (1 if max(redo, recount) <= 56 * 1024 else 2)
     kap += 0 < page_size and page_size // stride < 32
@@ -410,13 +414,14 @@ def main():
         roof_osk["as_a_burst"] = {"ms": burst_run["osk_ms"], "achieved": b_tflops, "frac_of_burst": b_tflops / peaks["bf16_tflops"],
                                   "how": burst_run["how"]}
     # KAP: the screen kernel forms the sampled logits on the tensor cores (one pass over the key tiles; whole tiles,
-    # so somewhat more than the causal pairs), the sort kernel is ALU work; the algorithmic FLOPs (causal pairs only)
+    # so somewhat more than the causal pairs), the sort (of up to 256 blocks in the screen, else a kernel) is ALU work; the algorithmic FLOPs (causal pairs only)
     # are set against the tensor peak, and the algorithmic bytes (sampled rows read once, lists written once)
     # against the copy bandwidth
-    roof_kap = tensor_roof("kap_screen_kernel+kap_sort_kernel", kap_tflops,
+    kap_kernels = ["kap_screen_kernel"] + ([] if screen_makes_lists(w.n, args.block_q) else ["kap_sort_kernel"])
+    roof_kap = tensor_roof("+".join(kap_kernels), kap_tflops,
                            {"hbm_gbs_on_algorithmic_bytes": kap_bytes / (kap_ms * 1e-3) / 1e9,
                             "hbm_frac_of_measured": kap_bytes / (kap_ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
-                            "traffic": ((traffic or {}).get("kap_screen_kernel", 0) + (traffic or {}).get("kap_sort_kernel", 0)) or None})
+                            "traffic": sum((traffic or {}).get(name, 0) for name in kap_kernels) or None})
     roofline = roof_osk if osk_ms >= kap_ms else roof_kap
 
     extras = {}

@@ -160,7 +160,9 @@ typedef struct {
                               device status word (see cosa_device_status) and returns without writing further
                               results: cosa_kap_select then leaves out_order and out_count as they were,
                               cosa_osk_attention writes out, lse, visited and scored of a (head, query block)
-                              all or none of them.  0: the default, 2^31 (about a second).  A few cycles make every
+                              all or none of them.  (One warp of cosa_osk_attention, which hands out its work
+                              items, waits for whole walks of the others: never less than the default, and it
+                              leaves when one of them gives up.)  0: the default, 2^31 (about a second).  A few cycles make every
                               wait that is not already satisfied run out: that is how the tests reach this path
                               without ever leaving a kernel waiting                                       */
 } cosa_options;

@@ -258,11 +258,10 @@ cudaError_t raise_smem_limit(const void* kernel, SmemLimit* state, size_t bytes)
 
 // every (head, query block) in double precision
 cudaError_t launch_kap_exact(const KapParams& p, cudaStream_t st);
-// the whole call's key tiles fit the screen's stages: it needs no scratch areas and no norms kernel
 bool kap_screen_supported(int rows, int group, int stride, const KvPaging& pg);
 // Forms of the screen.  Long: block maxima are parked in scratch areas, the norms kernel goes before.  Short: at most 4 key tiles, which
-// all fit the stages; Medium: at most 8; neither needs scratch areas or the norms kernel.  Lists: the screen sorts its scores itself
-// and writes the lists, no sort kernel follows
+// all fit the stages; Medium: at most 8; neither needs scratch areas or the norms kernel.  Lists: the screen sorts its scores itself,
+// no sort kernel follows
 enum ScreenForm { kScreenLong, kScreenLongLists, kScreenShort, kScreenShortLists, kScreenMediumLists };
 inline bool screen_parks(ScreenForm f) { return f == kScreenLong || f == kScreenLongLists; }
 // What the screen says of a list it makes: as it stands, all of it to redo, near ties to recount, padding (an empty list)

@@ -339,7 +339,7 @@ cudaError_t launch_kap_fixup(const KapParams& p, const KapScreenParams& sp, Scre
   const size_t both = std::max(redo, tied);
   if (both <= 56 * 1024) return launch(kap_fixup_kernel<true, true>, &limits[0], both, 2 * sms);
   const cudaError_t e = launch(kap_fixup_kernel<true, false>, &limits[1], tied, 2 * sms);
-  // As many CTAs as fit the chip (227 KB of shared memory, 3 x 256 threads of registers on an SM): the launch overlaps the recount,
+  // As many CTAs as shared memory lets an SM hold, three at most (registers hold two; a third finds its lists later): the launch overlaps the recount,
   // whose CTAs still hold SMs, and one CTA per SM was placed two and three to an SM, where they share the FP64 unit and the
   // others idle (200 blocks of 8 heads, all keys the same: 8,223 us with one per SM, 4,942 when the launch came later)
   const int fit = (int)std::min<size_t>(3, 227 * 1024 / (redo + 1024));

@@ -17,13 +17,14 @@
 // many such areas as CTAs can be resident, so they mostly stay in L2.  After the last tile, with
 // M* known, the block scores and HRM flags are formed from the parked maxima, one thread per
 // (row group, key block).
-// Calls of at most eight key tiles (n <= 8192 at stride 8) park nothing: a thread keeps its block maxima in registers and, when
+// Calls of at most four key tiles (512 sampled keys) park nothing, nor do those of at most eight whose lists are made here and whose
+// blocks have 16 sampled rows or more: a thread keeps its block maxima in registers and, when
 // every product is done, lays them into the key stages, from where the scores are formed; the norms of the sampled keys are
 // taken from the stages as well, which saves the norms kernel's launch.
 // A CTA holds every score of its lists, and up to 256 candidates it sorts them itself, a warp a list in registers: no sort kernel (a
 // wave of small CTAs each, chains of short steps between barriers), and no scores cross a launch, only the lists (a byte an entry).
-// Stage 1 at 32K 160 -> 135 us, of four prompts in 16-token pages 157 -> 121, of 201 blocks with Top-p 136 -> 110, of 55 blocks at stride 4 102 -> 58.  Both together, in
-// short calls a chain of latencies (launch, first loads, a wave or two of CTAs): 1K tokens of 2 heads 13.5 -> 10.5 us, 31 blocks of
+// Stage 1 at 32K 160 -> 135 us, of four prompts of 8K to 16K tokens in 16-token pages 157 -> 121, of 201 blocks with Top-p 136 -> 110,
+// of 55 blocks at stride 4 102 -> 58.  Both together, in short calls a chain of latencies (launch, first loads, a wave or two of CTAs): 1K tokens of 2 heads 13.5 -> 10.5 us, 31 blocks of
 // 32 heads 18.0 -> 14.6, 2 x 61 blocks of 32 heads 70 -> 43.
 // What bounds the tiles of long calls: 1,518 cycles of an SM a key tile, where the products want 1,024, for the comparisons of 64
 // logits a thread, which take two cycles an instruction and scheduler (no gain from three-input maxima, from asking for
@@ -59,6 +60,8 @@ constexpr int kEpiThreads = 128 * kRowTiles * kParts;
 constexpr int kThreads = 64 + kEpiThreads;    // producer warp, MMA warp, epilogue warps
 constexpr int kSteps = 2;             // key tiles whose logits are in tensor memory at once
 constexpr int kTmemCols = 128 * kRowTiles * kSteps;
+// 18 warps: five on one of the four schedulers, so a thread has 96 registers.  The forms spill: long ones up to 16 bytes, those that make
+// lists up to 72, 88 of loads (32 sampled rows a block, long)
 constexpr int kCtasPerSm = 1;
 static_assert(kTmemCols == 512 && kPartCols == 64, "TMEM budget and two 32-column loads per thread and tile");
 

@@ -31,8 +31,8 @@
 // What runs once an item is cold in the instruction cache and costs by its size, and the loop of a computed block (some 22 KB over
 // all roles) loses lines to it: 225 requests an item go to the next cache on walks of 3.4 blocks, 20 a block on long ones.  Code is
 // therefore shared rather than unrolled or inlined twice where walks are short (a form of 88 KB instead of 61: 236 us instead of
-// 209 on walks of 3.4 blocks; one place that fetches K and V tiles instead of two: 175 -> 169, 662 -> 642 on four prompts in
-// 16-token pages); long ones have it written out (kLongWalks).
+// 209 on walks of 3.4 blocks; one place that fetches K and V tiles instead of two: 175 -> 169, and 3 % of the walks of four
+// prompts in 16-token pages); long ones have it written out (kLongWalks).
 // What bounds it: tensor pipe and exponentials both want about 1,024 cycles (0.52 us) of an SM per computed block, 512 per skipped
 // one.  Fitted to single launches at the full clock, an SM takes 1.03 us a computed block with Stage 2 off, 1.19 with it on (the
 // vote keeps the four row warps together), 0.43 a skipped one and 1.7 a work item; the tensor pipe is busy half of the time, and
@@ -45,7 +45,7 @@
 // (8.2 / 1.15 / 2.12), tiles prefetched into L2 (+2 to 5 %), V(k) requested before the decision on k after a computed block
 // (128K +4 to 5 %, 32K +6 to 8, walks of 3.4 blocks +9).
 // Every wait is bounded; a wait that runs out sets the device status word and the CTA winds down without writing
-// results: load and issue warps leave, the row threads, whom no wait holds any more, run to the end of their list.
+// further results (a work item's are written whole or not at all): load and issue warps leave, the row threads, whom no wait holds any more, run to the end of their list.
 #include <math.h>
 
 #include <type_traits>
@@ -166,10 +166,10 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
   const int G = p.hq / p.hkv;
   chain_wait();
 
-  // (whole warp) rows [first, first + rows) of key block j of K or V to dst, box after box: `box` bytes from one 64-column half
-  // of d to the other.  Lane 0 arms the barrier; with small pages every lane then fetches one page's part
   int b = 0, g = 0, i = 0;                 // (load warp, item warp) batch item, KV head, query block
-  // (whole warp) part 0 or 1: that half of V's key block j to tile slot `slot`; part 2: K's key block j as tile K(k), box after box
+  // (whole warp) part 0 or 1: that half of V's key block j to tile slot `slot`; part 2: K's key block j as tile K(k).  Box
+  // after box: `box` bytes from one 64-column half of d to the other.  Lane 0 arms the barrier; with small pages every lane then
+  // fetches one page's part
   auto fetch = [&](int part, int j, int slot, int k) {
     const bool is_k = part == 2;
     const CUtensorMap* map = is_k ? &k_map : &v_map;
