@@ -429,7 +429,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   const int ns_b = nqb_b * R;                   // ... that the item really has
   const int n_keys = p.causal ? (i_max + 1) * R : ns_b;
   const int n_tiles = (n_keys + 127) / 128;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (uniform, which the compiler cannot know)
 
   if (!kLists && blockIdx.x == 0 && threadIdx.x == 0) { p.todo[0] = 0; p.todo[1] = 0; }   // the sort stage (a later launch) counts there
   if (kLists && threadIdx.x < kGroups) {          // query blocks that are padding: empty lists
@@ -437,30 +437,30 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     if (i >= nqb_b && i < p.nqb) p.hard[(size_t)(b * p.hq + g * G + x % G) * p.nqb + i] = kListPadding;
   }
   if (i0 >= nqb_b) return;                        // all of this CTA's query blocks are padding
-  // key tile t to its stage (lane 0; paged keys: the 128 sampled keys of a tile come from 128 / spp pages (spp sampled rows each) or
-  // from one page; one lane per page looks its page up and issues its two boxes.  Sampled keys past the sequence are masked
-  // later: any valid page will do for them)
-  auto fetch_k = [&](int t) {
+  // key tile t to its stage: by one thread, or, with pages, by a whole warp (the 128 sampled keys of a tile come from 128 / spp pages,
+  // spp sampled rows each, or from one page; one lane per page looks its page up and issues its two boxes.  Sampled keys past the
+  // sequence are masked later: any valid page will do for them)
+  auto fetch_dense = [&](int t) {
     const int st = t % kStages;
     const uint32_t dst = k_sm + st * kTileBytes, bar = smem_u32(&ctl->k_full[st]);
-    if (lane == 0) mbar_expect_tx(bar, kTileBytes);
-    if (!p.pg.table) {
-      if (lane == 0) {
-        tma_load_tile(dst, &k_map, 0, t * 128, g, b, p.ko.row, p.ko.head, p.ko.outer, bar);
-        tma_load_tile(dst + kHalfBytes, &k_map, 64, t * 128, g, b, p.ko.row, p.ko.head, p.ko.outer, bar);
-      }
-    } else {
-      __syncwarp();
-      const int spp = min(128, p.pg.page_size / p.stride);
-      if (lane < 128 / spp) {
-        int tok = (t * 128 + lane * spp) * p.stride;
-        if (tok >= nqb_b * kBlock) tok = 0;
-        const KvCoord c = kv_coord(p.pg, b, g, tok);        // (a page's first sampled row is a multiple of the stride)
-        tma_load_tile(dst + lane * spp * 128, &k_map, 0, c.row / p.stride, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
-        tma_load_tile(dst + kHalfBytes + lane * spp * 128, &k_map, 64, c.row / p.stride, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
-      }
-      __syncwarp();
+    mbar_expect_tx(bar, kTileBytes);
+    tma_load_tile(dst, &k_map, 0, t * 128, g, b, p.ko.row, p.ko.head, p.ko.outer, bar);
+    tma_load_tile(dst + kHalfBytes, &k_map, 64, t * 128, g, b, p.ko.row, p.ko.head, p.ko.outer, bar);
+  };
+  auto fetch_pages = [&](int t) {
+    const int st = t % kStages;
+    const uint32_t dst = k_sm + st * kTileBytes, bar = smem_u32(&ctl->k_full[st]);
+    if (elect_one()) mbar_expect_tx(bar, kTileBytes);
+    __syncwarp();
+    const int spp = min(128, p.pg.page_size / p.stride);
+    if (lane < 128 / spp) {
+      int tok = (t * 128 + lane * spp) * p.stride;
+      if (tok >= nqb_b * kBlock) tok = 0;
+      const KvCoord c = kv_coord(p.pg, b, g, tok);        // (a page's first sampled row is a multiple of the stride)
+      tma_load_tile(dst + lane * spp * 128, &k_map, 0, c.row / p.stride, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
+      tma_load_tile(dst + kHalfBytes + lane * spp * 128, &k_map, 64, c.row / p.stride, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
     }
+    __syncwarp();
   };
   const int n_first = min(n_tiles, 1);            // (a tile takes its thread some 500 cycles)
   if (warp == 0) {
@@ -479,7 +479,10 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       tma_load_tile(dst + kHalfBytes, &q_map, 64, i * R, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->a_full));
     }
     __syncwarp();
-    if (n_first > 0) fetch_k(0);
+    if (n_first > 0) {
+      if (p.pg.table) fetch_pages(0);
+      else if (elect_one()) fetch_dense(0);
+    }
   } else if (warp == 1) {
     tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols);
     tmem_relinquish();
@@ -526,7 +529,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   } else if (warp == 0) {
     int t_issued = n_first;
     if (!p.pg.table) {
-      if (lane == 0) {
+      if (elect_one()) {
         for (int t = n_first; t < n_tiles; ++t) {
           const int st = t % kStages;
           if (!wait(smem_u32(&ctl->k_empty[st]), ((t / kStages) & 1) ^ 1) ||
@@ -534,9 +537,10 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
             if (!*abort_flag) screen_timeout(ctl, status);
             break;
           }
-          fetch_k(t);
+          fetch_dense(t);
           t_issued = t + 1;
         }
+        ctl->t_issued = t_issued;
       }
     } else {
       for (int t = n_first; t < n_tiles; ++t) {
@@ -549,13 +553,13 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) break;
-        fetch_k(t);
+        fetch_pages(t);
         t_issued = t + 1;
       }
+      if (lane == 0) ctl->t_issued = t_issued;
     }
-    if (lane == 0) ctl->t_issued = t_issued;
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = idesc_bf16(128, 128, 0, 0);
       bool alive = wait(smem_u32(&ctl->a_full), 0);
       if (!alive && !*abort_flag) screen_timeout(ctl, status);

@@ -162,13 +162,13 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
   const uint32_t p_sm = base + 3 * kTileBytes;      // 64 keys of P
   Control* ctl = reinterpret_cast<Control*>(smem + (size_t)kTileBytes * 3 + kHalfBytes);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (uniform, which the compiler cannot know)
   const int G = p.hq / p.hkv;
   chain_wait();
 
   int b = 0, g = 0, i = 0;                 // (load warp, item warp) batch item, KV head, query block
   // (whole warp) part 0 or 1: that half of V's key block j to tile slot `slot`; part 2: K's key block j as tile K(k).  Box
-  // after box: `box` bytes from one 64-column half of d to the other.  Lane 0 arms the barrier; with small pages every lane then
+  // after box: `box` bytes from one 64-column half of d to the other.  One lane arms the barrier; with small pages every lane then
   // fetches one page's part
   auto fetch = [&](int part, int j, int slot, int k) {
     const bool is_k = part == 2;
@@ -176,17 +176,21 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
     const uint32_t bar = smem_u32(is_k ? &ctl->k_full[k & 1] : &ctl->v_full[part]);
     const uint32_t dst = x_sm + slot * kTileBytes + (part == 1 ? kHalfBytes : 0), box = is_k ? kHalfBytes : kQuarterBytes;
     const int row0 = j * kBlock + (part == 1 ? kHalfKeys : 0);
-    if (lane == 0) {
-      if (is_k) ctl->diag[k & 1] = p.causal && j == i;
-      mbar_expect_tx(bar, 2 * box);
-    }
-    if (kSmallPages) __syncwarp();
-    const int rows = is_k ? kBlock : kHalfKeys, ps = kSmallPages ? min(p.pg.page_size, rows) : rows, at = lane * ps;
-    if (at < rows) {                      // (a page holds whole key blocks: lane 0 alone)
+    auto part_of = [&](int at) {
       const KvCoord c = kv_coord(p.pg, b, g, row0 + at);
 #pragma unroll
       for (int x = 0; x < 2; ++x)
         tma_load_tile(dst + x * box + at * 128, map, x * 64, c.row, c.head, c.outer, p.ko.row, p.ko.head, p.ko.outer, bar);
+    };
+    if (elect_one()) {
+      if (is_k) ctl->diag[k & 1] = p.causal && j == i;
+      mbar_expect_tx(bar, 2 * box);
+      if (!kSmallPages) part_of(0);       // (a page holds whole key blocks)
+    }
+    if (kSmallPages) {
+      __syncwarp();
+      const int rows = is_k ? kBlock : kHalfKeys, ps = min(p.pg.page_size, rows), at = lane * ps;
+      if (at < rows) part_of(at);
     }
   };
   // (item warp) work items: KV head major, then query blocks from the longest list down, the group's query heads innermost, so
@@ -308,7 +312,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         if (next_q) {                           // its tile is free when the last Q K^T of the walk before has finished
           if (n_walk > 0) alive = wait(&ctl->q_free, n_walk - 1);
           if (!alive) break;
-          if (lane == 0) fetch_q();
+          if (elect_one()) fetch_q();
           ++n_q;
         } else if (t == 0 && cnt == 0) {
           alive = wait(&ctl->q_full, 0);        // (requested before the count was known)
@@ -427,7 +431,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         if (!alive && !*abort_flag) *abort_flag = kTimedOut;
         ctl->req[0] = (n_k + 1) / 2; ctl->req[1] = n_k / 2; ctl->req[2] = (n_v + 1) / 2; ctl->req[3] = n_v / 2; ctl->req[5] = n_grant;
       }
-    } else if (warp == kMmaWarp && lane == 0) {
+    } else if (warp == kMmaWarp && elect_one()) {
       // ---------------------------------------------------------------- products
       auto wait = [&](unsigned long long* bar, int phase) { return mbar_wait(smem_u32(bar), phase & 1, abort_flag, budget); };
       const uint32_t idesc_qk = idesc_bf16(kBlock, kBlock, 0, 0);    // Q [M x K], K_j [N x K], both K-major
