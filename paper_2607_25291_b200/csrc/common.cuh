@@ -125,6 +125,8 @@ struct KapScreenParams {
   Strides qs, ks;        // strides of q and of k (dense k; pools are contiguous)
   TileOrder qo, ko;      // coordinate order of the tensor maps over the sampled rows of q and of k (set by the launcher)
   int q_box_heads;       // query heads one box of the map over q takes (set by the launcher)
+  int group_shift;       // log2 of the query heads per KV head (set by the launcher, as is all that a CTA would otherwise divide for)
+  int n_iq;              // CTAs per (batch item, KV head)
   long long wait_budget; // clock cycles a device-side wait may take before the kernel gives up
   KvPaging pg;
 };

@@ -57,10 +57,11 @@ constexpr int kRows = 128 * kRowTiles;
 constexpr int kParts = 2;             // column parts of a tile: one epilogue warp per row tile, part and sub-partition
 constexpr int kPartCols = 128 / kParts;
 constexpr int kEpiThreads = 128 * kRowTiles * kParts;
-constexpr int kThreads = 64 + kEpiThreads;    // producer warp, MMA warp, epilogue warps
+constexpr int kAuxThreads = 64;       // two warps for what a CTA needs once: scratch area, norms
+constexpr int kThreads = 64 + kEpiThreads + kAuxThreads;    // producer warp, MMA warp, epilogue warps, aux warps
 constexpr int kSteps = 2;             // key tiles whose logits are in tensor memory at once
 constexpr int kTmemCols = 128 * kRowTiles * kSteps;
-// 18 warps: five on one of the four schedulers, so a thread has 96 registers.  The forms spill: long ones up to 16 bytes, those that make
+// 20 warps, five a scheduler: a thread has 96 registers.  The forms spill: long ones up to 16 bytes, those that make
 // lists up to 72, 88 of loads (32 sampled rows a block, long)
 constexpr int kCtasPerSm = 1;
 static_assert(kTmemCols == 512 && kPartCols == 64, "TMEM budget and two 32-column loads per thread and tile");
@@ -68,18 +69,21 @@ static_assert(kTmemCols == 512 && kPartCols == 64, "TMEM budget and two 32-colum
 struct __align__(8) ScreenCtl {
   unsigned long long a_full, k_full[kStages];
   unsigned long long k_empty[kStages];  // the tile's MMAs finished: stage free and logits ready
-  unsigned long long s_empty[kSteps], x_bar;
+  unsigned long long s_empty[kSteps];
+  unsigned long long slot_bar;          // the CTA has its scratch area
+  unsigned long long norm_bar;          // norms are there
+  unsigned long long parked_bar;        // every maximum of the CTA is parked
   unsigned long long m_full[kStages], m_empty[kStages];   // parked maxima fetched back into a key stage / read by all
   uint32_t tmem_base;
   volatile int abort_flag;
   volatile int t_issued, t_done, c_fetched, c_done;   // key tiles requested / multiplied, chunks of parked maxima requested / read
-  int slot;                             // scratch area held by this CTA, -1 = none
-  int poisoned;
+  int slot;                             // scratch area held by this CTA, -1 = none: it does nothing
   float xt[kParts][3][kRows];           // exchange between the column parts: top-3 block maxima
   int xj[kParts][2][kRows];             // ... and the blocks holding the two largest
   float mstar[kRows];                   // M*[r] of every row
-  float k2w[kEpiThreads / 32];          // (on chip) largest squared key norm each epilogue warp saw
-  unsigned long long n_read[kStages];   // (kMedium) every epilogue warp has the norms of the stage's keys
+  float q2[kRows];                      // squared norm of every row
+  float k2w[kAuxThreads / 32];          // largest squared key norm each aux warp saw
+  unsigned long long n_read[kStages];   // (kMedium) both aux warps have the norms of the stage's keys
   int j12[2][kRows];                    // (lists) blocks holding every row's largest and second largest block maximum
   uint32_t amb[kRows / 8];              // (lists) by row group: rows whose two best blocks are too close to call
   float qk2[kRows / 8];                 // (lists) by row group: as qk2max
@@ -402,9 +406,10 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     mbar_init(smem_u32(&ctl->a_full), 1);
     for (int s = 0; s < kStages; ++s) { mbar_init(smem_u32(&ctl->k_full[s]), 1); mbar_init(smem_u32(&ctl->k_empty[s]), 1); }
     for (int s = 0; s < kSteps; ++s) mbar_init(smem_u32(&ctl->s_empty[s]), kEpiThreads);
-    mbar_init(smem_u32(&ctl->x_bar), kEpiThreads);
+    mbar_init(smem_u32(&ctl->norm_bar), kAuxThreads / 32);
+    mbar_init(smem_u32(&ctl->slot_bar), 1); mbar_init(smem_u32(&ctl->parked_bar), 1);
     if (!kOnChip) for (int s = 0; s < kStages; ++s) { mbar_init(smem_u32(&ctl->m_full[s]), 1); mbar_init(smem_u32(&ctl->m_empty[s]), kEpiThreads); }
-    if (kMedium) for (int s = 0; s < kStages; ++s) mbar_init(smem_u32(&ctl->n_read[s]), kEpiThreads / 32);
+    if (kMedium) for (int s = 0; s < kStages; ++s) mbar_init(smem_u32(&ctl->n_read[s]), kAuxThreads / 32);
     ctl->abort_flag = 0;
     ctl->t_issued = 0; ctl->t_done = 0; ctl->c_fetched = 0; ctl->c_done = 0;
     mbar_fence_init();
@@ -415,17 +420,17 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
 
   constexpr int BPT = 128 / R;                  // key blocks per key tile
   constexpr int kGroups = kRows / R;            // row groups (one query head of one query block each) per CTA
-  const int G = p.hq / p.hkv;
-  const int QB = kGroups / G;                   // query blocks per CTA
-  const int n_iq = (p.nqb + QB - 1) / QB;
-  const int w = blockIdx.x;
-  const int b = w / (p.hkv * n_iq);
-  const int g = (w / n_iq) % p.hkv;
-  const int iq = n_iq - 1 - (w % n_iq);         // longest first
+  const int lg = p.group_shift, G = 1 << lg;    // query heads of the group (a power of two: see kap_screen_supported)
+  const int QB = kGroups >> lg;                 // query blocks per CTA
+  const int n_iq = p.n_iq;
+  const int bg = (int)blockIdx.x / n_iq;
+  const int b = bg / p.hkv;
+  const int g = bg - b * p.hkv;
+  const int iq = n_iq - 1 - ((int)blockIdx.x - bg * n_iq);   // longest first
   const int i0 = iq * QB;
   const int nqb_b = item_blocks(p.pg, b, p.nqb);      // the item's own length in blocks
   const int i_max = min(i0 + QB, nqb_b) - 1;
-  const int ns = p.n / p.stride;                // sampled rows per head (tensor pitch)
+  const int ns = p.nqb * R;                     // sampled rows per head (tensor pitch)
   const int ns_b = nqb_b * R;                   // ... that the item really has
   const int n_keys = p.causal ? (i_max + 1) * R : ns_b;
   const int n_tiles = (n_keys + 127) / 128;
@@ -433,8 +438,8 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
 
   if (!kLists && blockIdx.x == 0 && threadIdx.x == 0) { p.todo[0] = 0; p.todo[1] = 0; }   // the sort stage (a later launch) counts there
   if (kLists && threadIdx.x < kGroups) {          // query blocks that are padding: empty lists
-    const int x = threadIdx.x, i = i0 + x / G;
-    if (i >= nqb_b && i < p.nqb) p.hard[(size_t)(b * p.hq + g * G + x % G) * p.nqb + i] = kListPadding;
+    const int x = threadIdx.x, i = i0 + (x >> lg);
+    if (i >= nqb_b && i < p.nqb) p.hard[(size_t)(b * p.hq + g * G + (x & (G - 1))) * p.nqb + i] = kListPadding;
   }
   if (i0 >= nqb_b) return;                        // all of this CTA's query blocks are padding
   // key tile t to its stage: by one thread, or, with pages, by a whole warp (the 128 sampled keys of a tile come from 128 / spp pages,
@@ -473,7 +478,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     static_assert(kGroups <= 32, "a lane per box pair");
     const int a_grp = lane * p.q_box_heads;
     if (a_grp < kGroups) {
-      const int i = i0 + a_grp / G, h = g * G + a_grp % G;
+      const int i = i0 + (a_grp >> lg), h = g * G + (a_grp & (G - 1));
       const uint32_t dst = a_sm + (a_grp * R / 128) * kTileBytes + (a_grp * R % 128) * 128;   // (rows past the head's last are zero-filled)
       tma_load_tile(dst, &q_map, 0, i * R, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->a_full));
       tma_load_tile(dst + kHalfBytes, &q_map, 64, i * R, h, b, p.qo.row, p.qo.head, p.qo.outer, smem_u32(&ctl->a_full));
@@ -486,28 +491,6 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   } else if (warp == 1) {
     tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols);
     tmem_relinquish();
-  } else if (threadIdx.x == 64) {
-    // once some CTA has reported a timeout the rest of the grid returns at once
-    int poisoned = *reinterpret_cast<volatile int32_t*>(status);
-    int slot = -1;
-    if (kOnChip) {
-      slot = 0;                             // (none needed)
-    } else if (poisoned == 0 && (int)gridDim.x <= p.slots) {
-      slot = (int)blockIdx.x;               // an area for every CTA: nothing to search for
-    } else if (poisoned == 0) {
-      // a scratch area no resident CTA holds: there are as many as CTAs can be resident, so one is free; the
-      // search starts at this SM's number and normally ends at once
-      unsigned smid;
-      asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-      for (int s = 0; s < 8 * p.slots && slot < 0; ++s) {
-        const int cand = (int)((smid * kCtasPerSm + s) % (unsigned)p.slots);
-        if (atomicCAS(&p.slot_taken[cand], 0, 1) == 0) slot = cand;
-      }
-      if (slot < 0) { atomicMin(status, (int32_t)COSA_ERR_DEVICE_TIMEOUT); poisoned = 1; }
-      __threadfence();
-    }
-    ctl->slot = slot;
-    ctl->poisoned = poisoned;
   }
   tc_fence_before();
   __syncthreads();
@@ -522,11 +505,8 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   auto wait_warp = [&](uint32_t bar, uint32_t parity) {
     return kStrict ? mbar_poll_warp(bar, parity, abort_flag, budget) : mbar_wait(bar, parity, abort_flag, budget);
   };
-  const bool poisoned = ctl->poisoned != 0;
 
-  if (poisoned) {
-    if (threadIdx.x == 0) ctl->t_issued = n_first;
-  } else if (warp == 0) {
+  if (warp == 0) {
     int t_issued = n_first;
     if (!p.pg.table) {
       if (elect_one()) {
@@ -558,6 +538,31 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       }
       if (lane == 0) ctl->t_issued = t_issued;
     }
+    __syncwarp();
+    if (!kOnChip && elect_one()) {
+      // the parked maxima come back through the key stages, a chunk of tiles each, when every one of them is parked
+      int c_fetched = 0;
+      bool alive = wait(smem_u32(&ctl->parked_bar), 0);
+      if (alive) {
+        const float* parked = p.maxima + (size_t)ctl->slot * ((size_t)((ns + 127) / 128) * (kRows * BPT));
+        const uint64_t drop = l2_policy_evict_first();
+        fence_proxy_async_all();   // the maxima were written with ordinary stores
+        constexpr int kTileFloats = kRows * BPT, kTilesPerChunk = kTileBytes / (kTileFloats * 4);
+        const int n_chunks = (n_tiles + kTilesPerChunk - 1) / kTilesPerChunk;
+        for (int c = 0; c < n_chunks; ++c) {
+          const int st = c % kStages;
+          if (c >= kStages) alive = wait(smem_u32(&ctl->m_empty[st]), ((c - kStages) / kStages) & 1);
+          if (!alive) break;
+          const int tiles_here = min(kTilesPerChunk, n_tiles - c * kTilesPerChunk);
+          const uint32_t bar = smem_u32(&ctl->m_full[st]);
+          mbar_expect_tx(bar, tiles_here * kTileFloats * 4);
+          bulk_load_hint(k_sm + st * kTileBytes, parked + (size_t)c * kTilesPerChunk * kTileFloats, tiles_here * kTileFloats * 4, bar, drop);
+          c_fetched = c + 1;
+        }
+      }
+      if (!alive && !*abort_flag) screen_timeout(ctl, status);
+      ctl->c_fetched = c_fetched;
+    }
   } else if (warp == 1) {
     if (elect_one()) {
       const uint32_t idesc = idesc_bf16(128, 128, 0, 0);
@@ -588,6 +593,82 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       }
       ctl->t_done = t_done;
     }
+  } else if (warp >= 2 + kEpiThreads / 32) {
+    // ---------------------------------------------------------------- scratch area, squared norms of the sampled rows
+    const int at = threadIdx.x - (64 + kEpiThreads);
+    if (at == 0) {
+      // once some CTA has reported a timeout the rest of the grid winds down at once
+      int poisoned = *reinterpret_cast<volatile int32_t*>(status);
+      int slot = -1;
+      if (poisoned == 0 && kOnChip) {
+        slot = 0;                             // (none needed)
+      } else if (poisoned == 0 && (int)gridDim.x <= p.slots) {
+        slot = (int)blockIdx.x;               // an area for every CTA: nothing to search for
+      } else if (poisoned == 0) {
+        // a scratch area no resident CTA holds: there are as many as CTAs can be resident, so one is free; the
+        // search starts at this SM's number and normally ends at once
+        unsigned smid;
+        asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+        for (int s = 0; s < 8 * p.slots && slot < 0; ++s) {
+          const int cand = (int)((smid * kCtasPerSm + s) % (unsigned)p.slots);
+          if (atomicCAS(&p.slot_taken[cand], 0, 1) == 0) slot = cand;
+        }
+        if (slot < 0) { atomicMin(status, (int32_t)COSA_ERR_DEVICE_TIMEOUT); poisoned = 1; }
+        __threadfence();
+      }
+      ctl->slot = slot;
+      if (poisoned) ctl->abort_flag = 1;
+      mbar_arrive(smem_u32(&ctl->slot_bar));
+    }
+    __syncwarp();
+    auto wait_all = [&](uint32_t bar, uint32_t parity) { return kStrict ? mbar_poll_warp(bar, parity, abort_flag, budget) : mbar_wait_warp(bar, parity, abort_flag, budget); };
+    // of the row at `row` and its other half a half tile further on (2 x 128 bytes; the swizzle permutes 16-byte chunks inside a row,
+    // which a sum of squares does not notice; the chunk order is rotated by the lane so that the rows of a warp hit different banks)
+    auto norm2 = [&](const unsigned char* row) {
+      unsigned long long s0 = pack_f32x2(0.f, 0.f), s1 = s0;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        const uint4 wv = *reinterpret_cast<const uint4*>(row + (c >> 3) * kHalfBytes + (((c + lane) & 7) << 4));
+        const unsigned ws4[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const unsigned long long two = pack_f32x2(__uint_as_float(ws4[u] << 16), __uint_as_float(ws4[u] & 0xffff0000u));
+          if (u & 1) s1 = fma_f32x2(two, two, s1); else s0 = fma_f32x2(two, two, s0);
+        }
+      }
+      float x, y;
+      unpack_f32x2(add_f32x2(s0, s1), x, y);
+      return x + y;
+    };
+    float k2 = kOnChip ? 0.f : largest_key_norm(p, lane);
+    bool alive = wait_all(smem_u32(&ctl->a_full), 0);
+    if (alive) {
+#pragma unroll 1
+      for (int row = at; row < kRows; row += kAuxThreads) ctl->q2[row] = norm2(smem + (size_t)(row / 128) * kTileBytes + (size_t)(row % 128) * 128);
+    }
+    if (kOnChip) {
+      // (a stage is not filled again before its keys' norms have been taken)
+#pragma unroll 1
+      for (int t = 0; t < n_tiles && alive; ++t) {
+        alive = wait_all(smem_u32(&ctl->k_full[t % kStages]), (t / kStages) & 1);
+        if (!alive) break;
+#pragma unroll 1
+        for (int row = at; row < 128; row += kAuxThreads) {
+          const float s2 = norm2(smem + (size_t)kTileBytes * (kRowTiles + t % kStages) + row * 128);
+          if (s2 == s2 && t * 128 + row < ns_b) k2 = fmaxf(k2, s2);   // (a NaN row is left to the later stages; padding is no key)
+        }
+        if (kMedium) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&ctl->n_read[t % kStages]));
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) k2 = fmaxf(k2, __shfl_xor_sync(0xffffffffu, k2, o));
+    }
+    if (!alive && !*abort_flag) screen_timeout(ctl, status);
+    if (lane == 0) ctl->k2w[at >> 5] = k2;
+    __syncwarp();
+    if (alive && lane == 0) mbar_arrive(smem_u32(&ctl->norm_bar));
   } else {
     // ---------------------------------------------------------------- kParts threads per sampled query row
     const int ew = warp - 2;
@@ -597,7 +678,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     const int row = rt * 128 + sub * 32 + lane;
     const uint32_t lane_addr = (uint32_t)(sub * 32) << 16;
     const int grp = row / R, r = row % R;
-    const int i = i0 + grp / G, h = g * G + grp % G;
+    const int i = i0 + (grp >> lg), h = g * G + (grp & (G - 1));
     const bool row_ok = i < nqb_b;
     const int r_glob = i * R + r;                        // index among the head's sampled rows
     const int c_limit = p.causal ? r_glob : ns_b - 1;    // last sampled key this row may see
@@ -607,32 +688,13 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     // the CTA's block maxima: [tile][row group][block of the tile][row of the group], so that the R maxima one
     // score needs are contiguous
     constexpr int kTileFloats = kRows * BPT;
-    float* parked = p.maxima + (size_t)ctl->slot * ((size_t)((ns + 127) / 128) * kTileFloats);
-    float* mine = parked + ((size_t)grp * BPT + part * BPC) * R + r;
-    const uint64_t keep = l2_policy_evict_last(), drop = l2_policy_evict_first();
-    // squared norm of this thread's sampled query row, from the A tile in shared memory (a row is 2 x 128 bytes, one in
-    // each half tile; the swizzle permutes 16-byte chunks inside a row, which a sum of squares does not notice; the
-    // chunk order is rotated by the lane so that the rows of a warp hit different banks)
-    float q2 = 0.f, g2 = 0.f;
-    float k2 = kOnChip ? 0.f : largest_key_norm(p, lane);
-    bool alive = wait_warp(smem_u32(&ctl->a_full), 0);
+    const uint64_t keep = l2_policy_evict_last();
+    // The epilogue warps meet at named barriers: every one of them comes, also after a wait that ran out, and all go on or none
+    auto agree = [&](bool ok) { return !bar_red_or(1, kEpiThreads, !ok); };
+    bool alive = wait_warp(smem_u32(&ctl->slot_bar), 0);
     if (!alive && !*abort_flag) screen_timeout(ctl, status);
-    if (alive) {
-      const unsigned char* arow = smem + (size_t)rt * kTileBytes + (size_t)(row % 128) * 128;
-#pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        const uint4 wv = *reinterpret_cast<const uint4*>(arow + (c >> 3) * kHalfBytes + (((c + lane) & 7) << 4));
-        const unsigned ws4[4] = {wv.x, wv.y, wv.z, wv.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float lo = __uint_as_float(ws4[u] << 16), hi = __uint_as_float(ws4[u] & 0xffff0000u);
-          q2 = fmaf(lo, lo, fmaf(hi, hi, q2));
-        }
-      }
-      g2 = q2;                                           // the group's rows are R consecutive lanes
-#pragma unroll
-      for (int o = 1; o < R; o <<= 1) g2 = fmaxf(g2, __shfl_xor_sync(0xffffffffu, g2, o));
-    }
+    alive = alive && ctl->slot >= 0;        // (a CTA without one sets the abort flag before it says so: no lane sees it alive)
+    float* mine = p.maxima + (size_t)max(ctl->slot, 0) * ((size_t)((ns + 127) / 128) * kTileFloats) + ((size_t)grp * BPT + part * BPC) * R + r;
     // one key tile: this row's block maxima, and the three largest so far
     auto take_tile = [&](int t, float (&mb)[BPC]) {
       const int sb = t % kSteps, st = t % kStages;
@@ -688,38 +750,10 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     };
     float mb_all[kOnChip ? kMaxTiles : 1][BPC];
     if (kOnChip) {
-      // (a stage is not filled again before its keys' norms have been taken; behind the last tile the maxima take the stages' place)
+      // (unrolled: the maxima are registers)
 #pragma unroll
-      for (int t = 0; t < kMaxTiles; ++t) {
-        if (t < n_tiles && alive) {
-          alive = take_tile(t, mb_all[t]) && wait_warp(smem_u32(&ctl->k_full[t % kStages]), (t / kStages) & 1);
-          // squared norms of the tile's sampled keys: four threads a row, the chunks of odd rows in another order (other banks)
-          const int et = threadIdx.x - 64, krow = et >> 2;
-          const unsigned char* src = smem + (size_t)kTileBytes * (kRowTiles + t % kStages) + krow * 128;
-          float s2 = 0.f;
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int c = ((et & 3) + 4 * u) ^ ((krow & 1) << 2);
-            const uint4 wv = *reinterpret_cast<const uint4*>(src + (c >> 3) * kHalfBytes + (c & 7) * 16);
-            const unsigned ws4[4] = {wv.x, wv.y, wv.z, wv.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float lo = __uint_as_float(ws4[e] << 16), hi = __uint_as_float(ws4[e] & 0xffff0000u);
-              s2 = fmaf(lo, lo, fmaf(hi, hi, s2));
-            }
-          }
-          s2 += __shfl_xor_sync(0xffffffffu, s2, 1);
-          s2 += __shfl_xor_sync(0xffffffffu, s2, 2);
-          if (s2 == s2 && t * 128 + krow < ns_b) k2 = fmaxf(k2, s2);   // (a NaN row is left to the later stages; padding is no key)
-          if (kMedium) {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&ctl->n_read[t % kStages]));
-          }
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) k2 = fmaxf(k2, __shfl_xor_sync(0xffffffffu, k2, o));
-      if (lane == 0) ctl->k2w[ew] = k2;
+      for (int t = 0; t < kMaxTiles; ++t)
+        if (t < n_tiles && alive) alive = take_tile(t, mb_all[t]);
     } else {
       for (int t = 0; t < n_tiles && alive; ++t) alive = take_tile(t, mb_all[0]);
     }
@@ -727,10 +761,10 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       // all tiles seen: merge the column parts' top-3 block maxima of every row
       ctl->xt[part][0][row] = top1; ctl->xt[part][1][row] = top2; ctl->xt[part][2][row] = top3;
       ctl->xj[part][0][row] = jstar; ctl->xj[part][1][row] = jstar2;
-      mbar_arrive(smem_u32(&ctl->x_bar));
-      alive = wait_warp(smem_u32(&ctl->x_bar), 0);
+      alive = wait_warp(smem_u32(&ctl->norm_bar), 0);
       if (!alive && !*abort_flag) screen_timeout(ctl, status);
     }
+    alive = agree(alive);
     if (alive) {
 #pragma unroll
       for (int other = 1; other < kParts; ++other) {
@@ -747,10 +781,11 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       // the row's best block, and whether the runner-up is too close to call
       // (the threshold grows with the magnitude of the row and of the call's keys, which is what the rounding error of a
       // logit follows)
-      if (kOnChip) {
+      const float k2 = fmaxf(ctl->k2w[0], ctl->k2w[1]), q2 = ctl->q2[row];
+      static_assert(kAuxThreads == 64, "two aux warps");
+      float g2 = q2;                                       // the group's rows are R consecutive lanes
 #pragma unroll
-        for (int e = 0; e < kEpiThreads / 32; ++e) k2 = fmaxf(k2, ctl->k2w[e]);
-      }
+      for (int o = 1; o < R; o <<= 1) g2 = fmaxf(g2, __shfl_xor_sync(0xffffffffu, g2, o));
       if (!kLists && part == 0 && r == 0 && row_ok) p.qk2max[(size_t)(b * p.hq + h) * p.nqb + i] = g2 * k2;
       const float tau_row = fmaxf(p.tau_row, 2.f * screen_error_bound(q2 * k2, p.scale));
       const bool amb = row_ok && (top1 - top2) * p.scale <= tau_row;
@@ -785,37 +820,23 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       }
       // every row's M* in shared memory and every parked maximum visible to the whole CTA
       __threadfence_block();
-      mbar_arrive(smem_u32(&ctl->x_bar));
-      alive = wait_warp(smem_u32(&ctl->x_bar), 1);
-      if (!alive && !*abort_flag) screen_timeout(ctl, status);
+      bar_sync(1, kEpiThreads);
+      if (!kOnChip && threadIdx.x == 64) mbar_arrive(smem_u32(&ctl->parked_bar));
     }
     if (alive) {
       // block scores s_ij = sum over the group's rows of exp(M[r,j] - M*[r]) and HRM flags.  The parked maxima
       // come back through the key stages, which are idle by now: bulk copies of a stage's worth of tiles, several
-      // in flight (the fetch is a matter of latency, and no thread could hold that many bytes in registers); one
-      // thread per (tile, row group, key block) then reads its R maxima from shared memory.
+      // in flight, by the producer (the fetch is a matter of latency, and no thread could hold that many bytes in registers);
+      // one thread per (tile, row group, key block) then reads its R maxima from shared memory.
       constexpr int kOutsPerTile = kGroups * BPT;
       constexpr int kTileBytesM = kTileFloats * 4;
       constexpr int kTilesPerChunk = kTileBytes / kTileBytesM;
       static_assert(kTilesPerChunk >= 1 && kTileBytes % kTileBytesM == 0, "a stage holds whole tiles of maxima");
       const int et = threadIdx.x - 64;
       const int n_chunks = (n_tiles + kTilesPerChunk - 1) / kTilesPerChunk;
-      int c_fetched = 0;          // (thread et == 0) chunks requested so far
-      auto fetch = [&](int c) {   // thread et == 0 only
-        c_fetched = c + 1;
-        const int tiles_here = min(kTilesPerChunk, n_tiles - c * kTilesPerChunk);
-        const uint32_t bar = smem_u32(&ctl->m_full[c % kStages]);
-        mbar_expect_tx(bar, tiles_here * kTileBytesM);
-        bulk_load_hint(k_sm + (c % kStages) * kTileBytes, parked + (size_t)c * kTilesPerChunk * kTileFloats,
-                       tiles_here * kTileBytesM, bar, drop);
-      };
-      if (!kOnChip && et == 0) {
-        fence_proxy_async_all();   // the maxima were written with ordinary stores
-        for (int c = 0; c < min(n_chunks, kStages - 1); ++c) fetch(c);
-      }
       const int oo = et % kOutsPerTile;
       const int blk = oo % BPT, og = oo / BPT;             // consecutive lanes: consecutive key blocks
-      const int oi = i0 + og / G, oh = g * G + og % G;
+      const int oi = i0 + (og >> lg), oh = g * G + (og & (G - 1));
       const int J = p.causal ? oi + 1 : nqb_b;
       const float kLog2e = 1.4426950408889634f;
       const float scale2 = p.scale * kLog2e;
@@ -823,13 +844,14 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       // lanes of a quarter warp hit different banks; M* is taken in the same rotated order
       constexpr int kVecs = R / 4;
       const int rot = (lane / (8 / kVecs > 0 ? 8 / kVecs : 1)) % kVecs;
-      float ms[R];
+      float nms[R];                                          // -M*
 #pragma unroll
       for (int v4 = 0; v4 < kVecs; ++v4) {
         const int src = ((v4 + rot) % kVecs) * 4;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) ms[v4 * 4 + q] = ctl->mstar[og * R + src + q];
+        for (int q = 0; q < 4; ++q) nms[v4 * 4 + q] = -ctl->mstar[og * R + src + q];
       }
+      const unsigned long long scale22 = pack_f32x2(scale2, scale2);
       // (lists: the scores stay, in the third key stage behind the maxima, or where the query rows were; the keys come to the fourth, or
       // where the parked maxima were)
       constexpr int kCap = kLongLists ? kLongListCap : kListCap;
@@ -843,17 +865,23 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         const int j = tile * BPT + blk;
         if (oi < nqb_b && j < J) {
           const float4* src = reinterpret_cast<const float4*>(maxima + ((size_t)og * BPT + blk) * R);
-          float e0 = 0.f, e1 = 0.f;
+          unsigned long long sum = pack_f32x2(0.f, 0.f);         // (two sums, over even and odd rows)
           bool fl = false;
+          // exp(M[r,j] - M*[r]) of two rows; 0 for invisible blocks
+          auto two = [&](float x, float y, int r) {
+            float u, v;
+            unpack_f32x2(mul_f32x2(add_f32x2(pack_f32x2(x, y), pack_f32x2(nms[r], nms[r + 1])), scale22), u, v);
+            sum = add_f32x2(sum, pack_f32x2(ex2_approx(u), ex2_approx(v)));
+            fl = fl || x == -nms[r] || y == -nms[r + 1];
+          };
 #pragma unroll
           for (int v4 = 0; v4 < kVecs; ++v4) {
             const float4 x = src[(v4 + rot) % kVecs];
-            e0 += ex2_approx((x.x - ms[v4 * 4]) * scale2);       // exp(M[r,j] - M*[r]); 0 for invisible blocks
-            e1 += ex2_approx((x.y - ms[v4 * 4 + 1]) * scale2);
-            e0 += ex2_approx((x.z - ms[v4 * 4 + 2]) * scale2);
-            e1 += ex2_approx((x.w - ms[v4 * 4 + 3]) * scale2);
-            fl = fl || x.x == ms[v4 * 4] || x.y == ms[v4 * 4 + 1] || x.z == ms[v4 * 4 + 2] || x.w == ms[v4 * 4 + 3];
+            two(x.x, x.y, v4 * 4);
+            two(x.z, x.w, v4 * 4 + 2);
           }
+          float e0, e1;
+          unpack_f32x2(sum, e0, e1);
           const float e = e0 + e1;
           srow[j] = fl ? -e : e;                                 // sign bit carries the HRM flag
         }
@@ -867,14 +895,6 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       int c_done = 0;
       for (int c = 0; !kOnChip && c < n_chunks && alive; ++c) {
         const int st = c % kStages;
-        if (et == 0 && c + kStages - 1 < n_chunks) {
-          // the stage of chunk c - 1 takes chunk c + kStages - 1 once every thread has read it
-          if (c > 0 && !wait(smem_u32(&ctl->m_empty[(c - 1) % kStages]), ((c - 1) / kStages) & 1)) {
-            if (!*abort_flag) screen_timeout(ctl, status);
-          } else {
-            fetch(c + kStages - 1);
-          }
-        }
         alive = wait_warp(smem_u32(&ctl->m_full[st]), (c / kStages) & 1);
         if (!alive) { if (!*abort_flag) screen_timeout(ctl, status); break; }
         const int tiles_here = min(kTilesPerChunk, n_tiles - c * kTilesPerChunk);
@@ -886,18 +906,14 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         mbar_arrive(smem_u32(&ctl->m_empty[st]));
         c_done = c + 1;
       }
-      if (et == 0) { ctl->c_fetched = c_fetched; ctl->c_done = c_done; }
+      if (et == 0) ctl->c_done = c_done;
       if (kLists) {
         // a warp per list
-        if (alive) {
-          mbar_arrive(smem_u32(&ctl->x_bar));
-          alive = wait_warp(smem_u32(&ctl->x_bar), 0);
-          if (!alive && !*abort_flag) screen_timeout(ctl, status);
-        }
+        alive = agree(alive);
         unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem + (size_t)kTileBytes * (kRowTiles + (kLongLists ? 0 : 3)));
 #pragma unroll 1
         for (int x = ew; x < kGroups && alive; x += kEpiThreads / 32) {
-          const int li = i0 + x / G, lh = g * G + x % G;
+          const int li = i0 + (x >> lg), lh = g * G + (x & (G - 1));
           if (li >= nqb_b) break;
           const int cand = p.causal ? li + 1 : nqb_b;
           auto make = [&](auto per) {
@@ -913,7 +929,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && (poisoned || *abort_flag)) {
+  if (threadIdx.x == 0 && *abort_flag) {
     // the kernel gave up somewhere: copies and products still in flight finish on their own and must have done so
     // before the CTA's shared and tensor memory go to the next one
     (void)mbar_wait_noabort(smem_u32(&ctl->a_full), 0);
@@ -1003,6 +1019,9 @@ cudaError_t launch_kap_screen(const KapParams& kp, const KapScreenParams& p_in, 
   int32_t* status = device_status_word();
   if (!status) return cudaErrorInvalidSymbol;
   const int grid = kap_screen_grid(p.batch, p.hq, p.hkv, p.nqb, p.stride);
+  p.n_iq = grid / (p.batch * p.hkv);
+  p.group_shift = 0;
+  while ((1 << p.group_shift) < group) ++p.group_shift;
   cudaError_t e;
 #define COSA_LAUNCH_SCREEN(RR)                                                                                              \
   {                                                                                                                         \
