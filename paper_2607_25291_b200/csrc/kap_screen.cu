@@ -77,11 +77,12 @@ struct __align__(8) ScreenCtl {
   uint32_t tmem_base;
   volatile int abort_flag;
   volatile int t_issued, t_done, c_fetched, c_done;   // key tiles requested / multiplied, chunks of parked maxima requested / read
-  int slot;                             // scratch area held by this CTA, -1 = none: it does nothing
+  int slot;                             // scratch area held by this CTA, -1 = none
+  bool poisoned;                        // some CTA has reported a timeout: this one does nothing
   float xt[kParts][3][kRows];           // exchange between the column parts: top-3 block maxima
   int xj[kParts][2][kRows];             // ... and the blocks holding the two largest
   float mstar[kRows];                   // M*[r] of every row
-  float q2[kRows];                      // squared norm of every row
+  float q2[kParts][kRows];              // squared norm of every row (by two threads, half a row each, or whole in the first)
   float k2w[kAuxThreads / 32];          // largest squared key norm each aux warp saw
   unsigned long long n_read[kStages];   // (kMedium) both aux warps have the norms of the stage's keys
   int j12[2][kRows];                    // (lists) blocks holding every row's largest and second largest block maximum
@@ -95,6 +96,13 @@ static_assert(kScreenSmem <= 232448, "shared memory budget of one CTA");
 __device__ __forceinline__ void screen_timeout(ScreenCtl* c, int32_t* status) {
   c->abort_flag = 1;
   atomicMin(status, (int32_t)COSA_ERR_DEVICE_TIMEOUT);
+}
+
+// Takes a scratch area if it is free; what its last holder did with it has happened then
+__device__ __forceinline__ bool take_area(int32_t* taken) {
+  int32_t was;
+  asm volatile("atom.acquire.gpu.global.cas.b32 %0, [%1], 0, 1;" : "=r"(was) : "l"(taken) : "memory");
+  return was == 0;
 }
 
 // (a whole warp) the largest squared norm of a sampled key row of the call
@@ -177,9 +185,9 @@ __device__ __forceinline__ void f64_row_maxima(const KapParams& p, const __nv_bf
     for (int o = 4; o < 32; o <<= 1) best[x] = fmax(best[x], __shfl_xor_sync(0xffffffffu, best[x], o));
 }
 
-// (a whole warp) sorts 32 * PER distinct keys descending (bitonic, in registers); afterwards lane l holds places l * PER and on
+// (a whole warp) sorts 32 * PER keys descending (bitonic, in registers); afterwards lane l holds places l * PER and on
 template <int PER>
-__device__ __forceinline__ void warp_sort_desc(unsigned long long (&k)[PER], int lane) {
+__device__ __forceinline__ void warp_sort_desc(uint32_t (&k)[PER], int lane) {
 #pragma unroll
   for (int size = 2; size <= 32 * PER; size <<= 1) {
 #pragma unroll
@@ -188,22 +196,45 @@ __device__ __forceinline__ void warp_sort_desc(unsigned long long (&k)[PER], int
         const bool larger = ((lane & (size / PER)) == 0) == ((lane & (stride / PER)) == 0);
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
-          const unsigned long long other = __shfl_xor_sync(0xffffffffu, k[r], stride / PER);
-          k[r] = (other > k[r]) == larger ? other : k[r];
+          const uint32_t other = __shfl_xor_sync(0xffffffffu, k[r], stride / PER);
+          k[r] = larger ? max(k[r], other) : min(k[r], other);
         }
       } else {
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
           if (r & stride) continue;
           const bool down = size < PER ? (r & size) == 0 : (lane & (size / PER)) == 0;
-          const unsigned long long x = k[r], y = k[r | stride];
-          const bool swap = (y > x) == down;
-          k[r] = swap ? y : x;
-          k[r | stride] = swap ? x : y;
+          const uint32_t x = max(k[r], k[r | stride]), y = min(k[r], k[r | stride]);
+          k[r] = down ? x : y;
+          k[r | stride] = down ? y : x;
         }
       }
     }
   }
+}
+// (a whole warp) puts 32 * PER distinct keys that are all but sorted, held as above, in descending order: neighbours change places
+// until none has to
+template <int PER>
+__device__ __forceinline__ void warp_settle_desc(unsigned long long (&k)[PER], int lane) {
+  bool swapped;
+  do {
+    swapped = false;
+    auto order = [&](unsigned long long& x, unsigned long long& y) {
+      const bool swap = y > x;
+      const unsigned long long t = x;
+      x = swap ? y : x;
+      y = swap ? t : y;
+      swapped = swapped || swap;
+    };
+#pragma unroll
+    for (int r = 0; r + 1 < PER; r += 2) order(k[r], k[r + 1]);
+#pragma unroll
+    for (int r = 1; r + 1 < PER; r += 2) order(k[r], k[r + 1]);
+    // the last key of a lane and the first of the next
+    const unsigned long long next = __shfl_down_sync(0xffffffffu, k[0], 1), before = __shfl_up_sync(0xffffffffu, k[PER - 1], 1);
+    if (lane < 31 && next > k[PER - 1]) { k[PER - 1] = next; swapped = true; }
+    if (lane > 0 && before < k[0]) { k[0] = before; swapped = true; }
+  } while (__any_sync(0xffffffffu, swapped));
 }
 
 // (a whole warp) the visit list of one (head, query block) of at most 32 * PER candidates: what kap_sort_kernel does for longer
@@ -276,7 +307,19 @@ __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float t
     for (int u = 0; u < J; ++u) rank += __shfl_sync(0xffffffffu, key[0], u) > key[0] ? 1 : 0;
     if (lane < J) srt[rank] = key[0];
   } else {
-    warp_sort_desc<PER>(key, lane);
+    // Sorted by words of a flag, the leading bits of the score and the id, which is a third of the work of sorting whole keys; what that
+    // leaves out of order is close together and settled after.  (Ids are below 256.  A word of 0 is no key, or the last of 256)
+    static_assert(32 * PER <= 256, "an id is a byte");
+    uint32_t word[PER];
+#pragma unroll
+    for (int x = 0; x < PER; ++x) word[x] = ((uint32_t)(key[x] >> 32) & 0xffffff00u) | (lane + 32 * x < J ? 0xffu - (uint32_t)(lane + 32 * x) : 0u);
+    warp_sort_desc<PER>(word, lane);
+#pragma unroll
+    for (int x = 0; x < PER; ++x) {
+      const uint32_t j = 0xffu - (word[x] & 0xffu);
+      key[x] = lane * PER + x < J ? ((unsigned long long)((word[x] & 0x80000000u) | __float_as_uint(fabsf(score[j]))) << 32) | (0xffffffffu - j) : 0ULL;
+    }
+    warp_settle_desc<PER>(key, lane);
 #pragma unroll
     for (int x = 0; x < PER; ++x) srt[lane * PER + x] = key[x];
   }
@@ -506,6 +549,26 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     return kStrict ? mbar_poll_warp(bar, parity, abort_flag, budget) : mbar_wait(bar, parity, abort_flag, budget);
   };
 
+  // squared norm of the row of a tile at `row`, 128 bytes of it or all 256, the other half a half tile further on (the swizzle permutes
+  // 16-byte chunks inside 128 bytes, which a sum of squares does not notice; the chunk order is rotated by the lane so that the rows
+  // of a warp hit different banks)
+  auto norm2 = [&](const unsigned char* row, auto chunks) {
+    unsigned long long s0 = pack_f32x2(0.f, 0.f), s1 = s0;
+#pragma unroll
+    for (int c = 0; c < decltype(chunks)::value; ++c) {
+      const uint4 wv = *reinterpret_cast<const uint4*>(row + (c >> 3) * kHalfBytes + (((c + lane) & 7) << 4));
+      const unsigned ws4[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const unsigned long long two = pack_f32x2(__uint_as_float(ws4[u] << 16), __uint_as_float(ws4[u] & 0xffff0000u));
+        if (u & 1) s1 = fma_f32x2(two, two, s1); else s0 = fma_f32x2(two, two, s0);
+      }
+    }
+    float x, y;
+    unpack_f32x2(add_f32x2(s0, s1), x, y);
+    return x + y;
+  };
+
   if (warp == 0) {
     int t_issued = n_first;
     if (!p.pg.table) {
@@ -600,51 +663,33 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       // once some CTA has reported a timeout the rest of the grid winds down at once
       int poisoned = *reinterpret_cast<volatile int32_t*>(status);
       int slot = -1;
-      if (poisoned == 0 && kOnChip) {
+      if (kOnChip) {
         slot = 0;                             // (none needed)
-      } else if (poisoned == 0 && (int)gridDim.x <= p.slots) {
+      } else if ((int)gridDim.x <= p.slots) {
         slot = (int)blockIdx.x;               // an area for every CTA: nothing to search for
-      } else if (poisoned == 0) {
+      } else {
         // a scratch area no resident CTA holds: there are as many as CTAs can be resident, so one is free; the
         // search starts at this SM's number and normally ends at once
         unsigned smid;
         asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
         for (int s = 0; s < 8 * p.slots && slot < 0; ++s) {
           const int cand = (int)((smid * kCtasPerSm + s) % (unsigned)p.slots);
-          if (atomicCAS(&p.slot_taken[cand], 0, 1) == 0) slot = cand;
+          if (take_area(&p.slot_taken[cand])) slot = cand;
         }
         if (slot < 0) { atomicMin(status, (int32_t)COSA_ERR_DEVICE_TIMEOUT); poisoned = 1; }
-        __threadfence();
       }
       ctl->slot = slot;
+      ctl->poisoned = poisoned != 0;
       if (poisoned) ctl->abort_flag = 1;
       mbar_arrive(smem_u32(&ctl->slot_bar));
     }
     __syncwarp();
     auto wait_all = [&](uint32_t bar, uint32_t parity) { return kStrict ? mbar_poll_warp(bar, parity, abort_flag, budget) : mbar_wait_warp(bar, parity, abort_flag, budget); };
-    // of the row at `row` and its other half a half tile further on (2 x 128 bytes; the swizzle permutes 16-byte chunks inside a row,
-    // which a sum of squares does not notice; the chunk order is rotated by the lane so that the rows of a warp hit different banks)
-    auto norm2 = [&](const unsigned char* row) {
-      unsigned long long s0 = pack_f32x2(0.f, 0.f), s1 = s0;
-#pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        const uint4 wv = *reinterpret_cast<const uint4*>(row + (c >> 3) * kHalfBytes + (((c + lane) & 7) << 4));
-        const unsigned ws4[4] = {wv.x, wv.y, wv.z, wv.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const unsigned long long two = pack_f32x2(__uint_as_float(ws4[u] << 16), __uint_as_float(ws4[u] & 0xffff0000u));
-          if (u & 1) s1 = fma_f32x2(two, two, s1); else s0 = fma_f32x2(two, two, s0);
-        }
-      }
-      float x, y;
-      unpack_f32x2(add_f32x2(s0, s1), x, y);
-      return x + y;
-    };
     float k2 = kOnChip ? 0.f : largest_key_norm(p, lane);
     bool alive = wait_all(smem_u32(&ctl->a_full), 0);
-    if (alive) {
+    if (alive && !kOnChip) {
 #pragma unroll 1
-      for (int row = at; row < kRows; row += kAuxThreads) ctl->q2[row] = norm2(smem + (size_t)(row / 128) * kTileBytes + (size_t)(row % 128) * 128);
+      for (int row = at; row < kRows; row += kAuxThreads) ctl->q2[0][row] = norm2(smem + (size_t)(row / 128) * kTileBytes + (size_t)(row % 128) * 128, std::integral_constant<int, 16>{});
     }
     if (kOnChip) {
       // (a stage is not filled again before its keys' norms have been taken)
@@ -654,7 +699,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
         if (!alive) break;
 #pragma unroll 1
         for (int row = at; row < 128; row += kAuxThreads) {
-          const float s2 = norm2(smem + (size_t)kTileBytes * (kRowTiles + t % kStages) + row * 128);
+          const float s2 = norm2(smem + (size_t)kTileBytes * (kRowTiles + t % kStages) + row * 128, std::integral_constant<int, 16>{});
           if (s2 == s2 && t * 128 + row < ns_b) k2 = fmaxf(k2, s2);   // (a NaN row is left to the later stages; padding is no key)
         }
         if (kMedium) {
@@ -693,7 +738,12 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
     auto agree = [&](bool ok) { return !bar_red_or(1, kEpiThreads, !ok); };
     bool alive = wait_warp(smem_u32(&ctl->slot_bar), 0);
     if (!alive && !*abort_flag) screen_timeout(ctl, status);
-    alive = alive && ctl->slot >= 0;        // (a CTA without one sets the abort flag before it says so: no lane sees it alive)
+    alive = alive && !ctl->poisoned;        // (set before the barrier completes: no lane sees it otherwise)
+    if (kOnChip && alive) {                 // (nothing else to do until the first product is there)
+      alive = wait_warp(smem_u32(&ctl->a_full), 0);
+      if (!alive && !*abort_flag) screen_timeout(ctl, status);
+      ctl->q2[part][row] = norm2(smem + (size_t)rt * kTileBytes + (size_t)(row % 128) * 128 + part * kHalfBytes, std::integral_constant<int, 8>{});
+    }
     float* mine = p.maxima + (size_t)max(ctl->slot, 0) * ((size_t)((ns + 127) / 128) * kTileFloats) + ((size_t)grp * BPT + part * BPC) * R + r;
     // one key tile: this row's block maxima, and the three largest so far
     auto take_tile = [&](int t, float (&mb)[BPC]) {
@@ -781,8 +831,8 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
       // the row's best block, and whether the runner-up is too close to call
       // (the threshold grows with the magnitude of the row and of the call's keys, which is what the rounding error of a
       // logit follows)
-      const float k2 = fmaxf(ctl->k2w[0], ctl->k2w[1]), q2 = ctl->q2[row];
-      static_assert(kAuxThreads == 64, "two aux warps");
+      const float k2 = fmaxf(ctl->k2w[0], ctl->k2w[1]), q2 = kOnChip ? ctl->q2[0][row] + ctl->q2[1][row] : ctl->q2[0][row];
+      static_assert(kAuxThreads == 64 && kParts == 2, "two aux warps, two halves");
       float g2 = q2;                                       // the group's rows are R consecutive lanes
 #pragma unroll
       for (int o = 1; o < R; o <<= 1) g2 = fmaxf(g2, __shfl_xor_sync(0xffffffffu, g2, o));
@@ -943,7 +993,7 @@ kap_screen_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_consta
   if (warp == 1) tmem_dealloc(tmem, kTmemCols);
   if (kOnChip) return;
   {
-    if (ctl->slot < 0) return;            // (poisoned: the CTA has no area)
+    if (ctl->slot < 0) return;            // (the CTA has no area)
     // the parked maxima are dead: let L2 drop the lines instead of writing them back
     char* area = reinterpret_cast<char*>(p.maxima + (size_t)ctl->slot * ((size_t)((ns + 127) / 128) * (kRows * BPT)));
     const size_t bytes = (size_t)n_tiles * (kRows * BPT) * sizeof(float);
