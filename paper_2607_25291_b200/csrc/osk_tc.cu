@@ -9,8 +9,8 @@
 //   warp 5       issues the products
 //   warp 6       work items: takes them over, looks up their lists, fetches Q
 //   warp 7       idle (warps 4 to 7 give registers to the first four)
-// The running row maxima live in the threads' registers, the tile vote of Eq. (5) is one barrier with an OR over the 128
-// rows, and every thread counts the computed blocks for itself: no exchange between warps beyond that barrier.
+// The running row maxima live in the threads' registers, the tile vote of Eq. (5) is one barrier, which only warps that would skip
+// wait at, and every thread counts the computed blocks for itself: no exchange between warps beyond that barrier.
 //
 // Tensor memory has room for one S (128 columns) beside O (128); the second S buffer is the row threads' registers: they copy S
 // out at once, and Q K^T of the next position runs while they work on this one, before it is known whether the block will be
@@ -105,6 +105,7 @@ struct __align__(16) Control {
   volatile int req[6];             // requested by the time the load warp left: K tiles by parity, V tiles by half, Q tiles, work items
   volatile int diag[2];            // K(k) (by parity of k) is the diagonal block
   volatile uint32_t dec[2];
+  volatile int yes[3];             // the last position (by threes) that some row votes to compute
   Item item[2];
 };
 
@@ -227,13 +228,14 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       for (int s = 0; s < 2; ++s) {
         mbar_init(smem_u32(&ctl->item_bar[s]), 1); mbar_init(smem_u32(&ctl->item_read[s]), kBlock + 2);
         mbar_init(smem_u32(&ctl->k_full[s]), 1); mbar_init(smem_u32(&ctl->v_full[s]), 1);
-        mbar_init(smem_u32(&ctl->dec_bar[s]), 1); mbar_init(smem_u32(&ctl->p_full[s]), kBlock);
+        mbar_init(smem_u32(&ctl->dec_bar[s]), 4); mbar_init(smem_u32(&ctl->p_full[s]), kBlock);
         mbar_init(smem_u32(&ctl->pv_done[s]), 1);
       }
       mbar_init(smem_u32(&ctl->s_full), 1); mbar_init(smem_u32(&ctl->s_first), 1); mbar_init(smem_u32(&ctl->s_read), kBlock);
       mbar_init(smem_u32(&ctl->fin), 1);
       ctl->abort_flag = 0;
       for (int q = 0; q < 6; ++q) ctl->req[q] = 0;
+      for (int q = 0; q < 3; ++q) ctl->yes[q] = -1;
       mbar_fence_init();
       fence_proxy_async_smem();
       // the first Q at once: its address needs nothing from global memory, while the list entries, the count and the status
@@ -515,6 +517,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       }
     };
     int k_base = 0, pos_base = 0, n_base = 0; // as in the load warp
+    int turn = 0;                             // of the vote's barriers
     for (int t = 0;; ++t) {
       wait(&ctl->item_bar[t & 1], t >> 1);
       if (bar_red_or(1, kBlock, bad || *abort_flag)) break;
@@ -568,11 +571,27 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         if (kStage2) {
           // Eq. (5): skip iff max over the 128 rows of (m_loc - m) < ln(Delta/N), m including this block.  (Rows of a walk that was given
           // up vote on as long as their list lasts: nothing holds them any more)
-          const bool compute = bar_red_or(1, kBlock, !((m_loc - m_new) < theta2));
+          // A warp that votes to compute knows the outcome and goes on to its exponentials; the others wait for it.  Three barriers take
+          // turns: Q K^T of the next position waits until every row has read S, so no warp votes twice ahead of another, and a warp whose
+          // wait has run out goes on with the others only.  (All four at one barrier, an OR over its threads: 32K tokens 1,058 ->
+          // 1,045 us, 128K 8,029 -> 7,955, walks of 3.4 blocks 179 -> 176, of 2 blocks 33.3 -> 32.5, 4K of 4 heads 14.4 -> 13.7)
+          const int pos = pos_base + kk;
+          bool compute = __any_sync(0xffffffffu, !((m_loc - m_new) < theta2));
+          if (compute && lane == 0) ctl->yes[turn] = pos;
+          __syncwarp();
+          if (compute && !__any_sync(0xffffffffu, bad)) {
+            bar_arrive(2 + turn, kBlock);
+          } else {
+            bar_sync(2 + turn, kBlock);
+            compute = ctl->yes[turn] == pos;
+          }
+          turn = turn == 2 ? 0 : turn + 1;
           last = last || n + (compute ? 1 : 0) == cap;
+          if (lane == 0) {
+            ctl->dec[pos & 1] = (compute ? kDecComputed : 0u) | (last ? kDecEnd : 0u);
+            mbar_arrive(smem_u32(&ctl->dec_bar[pos & 1]));
+          }
           if (r == 0) {
-            ctl->dec[(pos_base + kk) & 1] = (compute ? kDecComputed : 0u) | (last ? kDecEnd : 0u);
-            mbar_arrive(smem_u32(&ctl->dec_bar[(pos_base + kk) & 1]));
             if (compute) dec_word |= 1u << (kk & 31);
             if (p.decisions && ((kk & 31) == 31 || last) && !*abort_flag) { p.decisions[row * dec_words + (kk >> 5)] = dec_word; dec_word = 0; }
           }

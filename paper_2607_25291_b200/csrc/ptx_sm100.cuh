@@ -111,7 +111,10 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
-
+// the same without waiting
+__device__ __forceinline__ void bar_arrive(int id, int nthreads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
 // the same barrier; true for every thread iff `pred` is true for any
 __device__ __forceinline__ bool bar_red_or(int id, int nthreads, bool pred) {
   uint32_t any;
