@@ -15,7 +15,11 @@
 // Tensor memory has room for one S (128 columns) beside O (128); the second S buffer is the row threads' registers: they copy S
 // out at once, and Q K^T of the next position runs while they work on this one, before it is known whether the block will be
 // computed or skipped.  P therefore cannot lie over S: it goes to shared memory, 64 keys at a time (16 KB, what Q and two tile
-// slots leave), so that the product of its first half runs while the exponentials of the second are formed.  (32 keys at a time
+// slots leave), so that the product of its first half runs while the exponentials of the second are formed.  With Stage 2 off the
+// first half goes to tensor memory, into the columns S has left, and Q K^T of the next position follows the product on it: it
+// has the second half's exponentials to run under, V's first half comes a position ahead, and neither half waits for the
+// other's place (all blocks of 16K 2,009 -> 1,965 us, 64K at 12.5 % 4,232 -> 4,199; both halves there, S behind the
+// whole block: 2,130 and 4,494).  With Stage 2 on S must not wait for a V tile that is asked for after the vote.  (32 keys at a time
 // through the same buffer: 2 to 6 % slower, each hand-over costs the rows a proxy fence.  Operands of Q K^T and P V both come
 // from shared memory: measured at the full 512 cycles per 128 x 128 x 128 product, also while tiles stream in.)
 // Tiles: two slots X and Y.  When block k is decided, X holds K(k+1) and Y is free or holds the last V tile.  Skipped: K(k+2)
@@ -94,9 +98,9 @@ struct __align__(16) Control {
   unsigned long long v_full[2];    // by half: the n-th V tile's half has landed
   unsigned long long s_full;       // Q K^T of the position has finished
   unsigned long long s_first;      // the same for the first position of a walk (a waiter may come when the second has finished, too)
-  unsigned long long s_read;       // every row has taken its S to registers
+  unsigned long long s_read;       // (Stage 2) every row has taken its S to registers
   unsigned long long dec_bar[2];   // the decision of a position (by parity) is in dec[]
-  unsigned long long p_full[2];    // by half: the n-th P's half is in shared memory
+  unsigned long long p_full[2];    // by half: the n-th P's half is in shared memory (the first with Stage 2 off: in tensor memory)
   unsigned long long pv_done[2];   // by half: the n-th product with that half has finished (one barrier each: a waiter may be
                                    // a whole block late, and one parity bit cannot tell two phases apart)
   unsigned long long fin;          // every product has finished
@@ -407,7 +411,21 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
               if (is_k) ++n_k; else ++n_v;
               fetch(part, clamp_id(is_k ? j2 : j0), is_k && (computed || k == -1) ? y ^ 1 : y, k_base + k + 2);
             };
-            if (!kLongWalks) {
+            if (!kStage2) {
+              // (V's first half a turn ahead: its place is free before Q K^T of the next position begins)
+              auto v_part = [&](int part, int at, int j) {
+                if (at > 0) alive = wait(&ctl->pv_done[part], n_base + at - 1);
+                if (!alive) return;
+                ++n_v;
+                fetch(part, clamp_id(j), y, 0);
+              };
+              if (k >= 0) {
+                if (k == 0) v_part(0, 0, j0);
+                if (alive) v_part(1, k, j0);
+                if (alive && !(d & kDecEnd)) v_part(0, k + 1, j1);
+              }
+              if (alive && want_k) do_part(2);
+            } else if (!kLongWalks) {
 #pragma unroll 1
               for (int part = computed ? 0 : 2; alive && part < (want_k ? 3 : 2); ++part) do_part(part);
             } else {
@@ -463,8 +481,9 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         alive = wait(&ctl->q_full, q);
         int k = -1, n = 0;
         while (alive) {
-          if (k >= 0) alive = wait(&ctl->s_read, pos_base + k);
-          if (alive && k + 1 < n_pos) alive = issue_qk(k_base + k + 1, k < 0 ? y : y ^ 1);
+          if (!kStage2 && k < 0 && n_base > 0) alive = wait(&ctl->pv_done[0], n_base - 1);   // (the walk before: P lay in S's place)
+          if (kStage2 && k >= 0) alive = wait(&ctl->s_read, pos_base + k);
+          if (alive && (kStage2 || k < 0) && k + 1 < n_pos) alive = issue_qk(k_base + k + 1, k < 0 ? y : y ^ 1);
           if (k < 0) {
             if (!kStage2 && alive) mma_commit(smem_u32(&ctl->s_first));
             ++k;
@@ -483,6 +502,12 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
               alive = wait(&ctl->v_full[half], n_base + n) && wait(&ctl->p_full[half], n_base + n);
               if (!alive) break;
               tc_fence_after();
+              if (!kStage2 && half == 0) {           // P's first half lies in S's place: the next S behind its product
+                mma_ts_x4<128, 256, 384>(tmem_o, tmem_s, vdesc0 + (uint64_t)(y * kTileBytes / 16), idesc_pv, n > 0);
+                mma_commit(smem_u32(&ctl->pv_done[0]));
+                if (k + 1 < n_pos) alive = wait(&ctl->pv_done[0], n_base + n) && issue_qk(k_base + k + 1, y ^ 1);
+                continue;
+              }
               // 16 keys per MMA: 32 bytes of a P row, 2 KiB (two 8-key groups) of the V half
               mma_ss_x4<2, 4, 6, 128, 256, 384>(tmem_o, pdesc, vdesc0 + (uint64_t)((y * kTileBytes + half * kHalfBytes) / 16), idesc_pv,
                                                 n + half > 0);
@@ -557,7 +582,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         for (int c = 0; c < 4; ++c) tmem_ld32(tmem_s + lane_addr + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
         tmem_wait_ld();
         tc_fence_before();
-        mbar_arrive(smem_u32(&ctl->s_read));
+        if (kStage2) mbar_arrive(smem_u32(&ctl->s_read));
         // (three-input maxima: half the instructions of the two-input form)
         float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
@@ -614,10 +639,10 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
           // the buffer's last reader: the second half of the block before, the first half of this one (asked now, needed
-          // after the exponentials)
-          const int last_n = n_base + n - 1 + half;
-          unsigned long long* last_reader = &ctl->pv_done[half ^ 1];
-          const bool is_free = n + half == 0 || mbar_test_wait(smem_u32(last_reader), last_n & 1);
+          // after the exponentials).  Without Stage 2 only second halves lie there, and O may be rescaled behind the last product
+          const int last_n = n_base + n - 1 + (kStage2 ? half : 0);
+          unsigned long long* last_reader = &ctl->pv_done[kStage2 ? half ^ 1 : 1];
+          const bool is_free = (kStage2 ? n + half == 0 : n == 0 || (half == 0 && !moved)) || mbar_test_wait(smem_u32(last_reader), last_n & 1);
 #pragma unroll
           for (int c = half * kHalfKeys; c < (half + 1) * kHalfKeys; c += 4) {
             float e0, e1, e2, e3;
@@ -643,12 +668,18 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
             }
             tmem_wait_st();
           }
+          if (!kStage2 && half == 0) {
+            __syncwarp();
+            tmem_st32(tmem_s + lane_addr, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+            tmem_wait_st();
+          } else {
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            const uint32_t* e = &s[half * 32 + c * 4];
-            *reinterpret_cast<uint4*>(prow + ((c ^ (r & 7)) << 4)) = make_uint4(e[0], e[1], e[2], e[3]);
+            for (int c = 0; c < 8; ++c) {
+              const uint32_t* e = &s[half * 32 + c * 4];
+              *reinterpret_cast<uint4*>(prow + ((c ^ (r & 7)) << 4)) = make_uint4(e[0], e[1], e[2], e[3]);
+            }
+            fence_proxy_async_smem();
           }
-          fence_proxy_async_smem();
           if (half == 0) tc_fence_before();         // (a rescaled O)
           mbar_arrive(smem_u32(&ctl->p_full[half]));
         }
