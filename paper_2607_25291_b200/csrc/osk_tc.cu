@@ -36,7 +36,7 @@
 // all roles) loses lines to it: 225 requests an item go to the next cache on walks of 3.4 blocks, 20 a block on long ones.  Code is
 // therefore shared rather than unrolled or inlined twice where walks are short (a form of 88 KB instead of 61: 236 us instead of
 // 209 on walks of 3.4 blocks; one place that fetches K and V tiles instead of two: 175 -> 169, and 3 % of the walks of four
-// prompts in 16-token pages); long ones have it written out (kLongWalks).
+// prompts in 16-token pages); with Stage 2 long ones have it written out (kLongWalks).
 // What bounds it: tensor pipe and exponentials both want about 1,024 cycles (0.52 us) of an SM per computed block, 512 per skipped
 // one.  Fitted to single launches at the full clock, an SM takes 1.03 us a computed block with Stage 2 off, 1.19 with it on (the
 // vote keeps the four row warps together), 0.43 a skipped one and 1.7 a work item; the tensor pipe is busy half of the time, and
@@ -72,7 +72,7 @@ constexpr int kCtasPerSm = 2;
 constexpr int kTmemCols = 256;
 constexpr int kLoadWarp = 4, kMmaWarp = 5, kItemWarp = 6;
 constexpr int kAskAhead = 4;                       // positions (or two computed blocks) before a walk's end at which more work is asked for
-constexpr int kShortWalk = 64, kShortWalkAll = 16;  // list pitch up to which walks count as short, with and without Stage 2
+constexpr int kShortWalk = 8;                      // list pitch up to which walks count as short, with Stage 2
 constexpr uint32_t kDecComputed = 1, kDecEnd = 2;
 constexpr int kTimedOut = 1, kPoisoned = 2;
 
@@ -150,7 +150,7 @@ __device__ __forceinline__ void mask_diagonal(uint32_t s, int warp, int lane) {
 //          of the load warp issue side by side, each after its own table look-up.  Boxes land on 1024-byte boundaries of
 //          the tile (pages of at least 8 tokens), where the 128-byte swizzle, a function of the shared-memory address,
 //          gives the layout of the one-piece tile.
-// kLongWalks: copies of the code that runs once a position or once an item are written out (see above); else they are shared
+// kLongWalks: (Stage 2) copies of the code that runs once a position or once an item are written out (see above); else they are shared
 template <bool kMask, bool kStage2, bool kSmallPages, bool kLongWalks>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
@@ -412,19 +412,20 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
               fetch(part, clamp_id(is_k ? j2 : j0), is_k && (computed || k == -1) ? y ^ 1 : y, k_base + k + 2);
             };
             if (!kStage2) {
-              // (V's first half a turn ahead: its place is free before Q K^T of the next position begins)
-              auto v_part = [&](int part, int at, int j) {
-                if (at > 0) alive = wait(&ctl->pv_done[part], n_base + at - 1);
-                if (!alive) return;
-                ++n_v;
-                fetch(part, clamp_id(j), y, 0);
-              };
-              if (k >= 0) {
-                if (k == 0) v_part(0, 0, j0);
-                if (alive) v_part(1, k, j0);
-                if (alive && !(d & kDecEnd)) v_part(0, k + 1, j1);
+              // V(0)'s first half, V(k)'s second, V(k + 1)'s first (a turn ahead: its place is free before Q K^T of the next position begins),
+              // K(k + 2)
+#pragma unroll 1
+              for (int step = k < 0 ? 3 : (k == 0 ? 0 : 1); step < 4; ++step) {
+                const bool is_k = step == 3;
+                if (is_k ? !want_k : step == 2 && (d & kDecEnd)) continue;
+                const int at = step == 0 ? 0 : k + step - 1;       // (V) whose tile it is
+                const bool after_qk = is_k && computed;
+                if (is_k ? after_qk || (k == -1 && v_before) : at > 0)
+                  alive = wait(after_qk ? &ctl->s_full : &ctl->pv_done[is_k || step == 1 ? 1 : 0], after_qk ? k_base + k + 1 : n_base + (is_k ? n : at) - 1);
+                if (!alive) break;
+                if (is_k) ++n_k; else ++n_v;
+                fetch(is_k ? 2 : step & 1, clamp_id(is_k ? j2 : (step == 2 ? j1 : j0)), is_k && (computed || k == -1) ? y ^ 1 : y, k_base + k + 2);
               }
-              if (alive && want_k) do_part(2);
             } else if (!kLongWalks) {
 #pragma unroll 1
               for (int part = computed ? 0 : 2; alive && part < (want_k ? 3 : 2); ++part) do_part(part);
@@ -784,17 +785,19 @@ cudaError_t launch_osk_tc(const OskParams& p_in, cudaStream_t st) {
   // Where the line lies, by the pitch, since the host knows no lengths.  Shared / written out, us a launch, 16K tokens of 32 heads,
   // lists of at most
   //                          4        8       16       24       32         48         64         96        128 blocks
-  // Stage 2 off        157/161  270/271  493/488  737/699  935/898  1338/1282  1615/1546  2023/1967  2147/2089
-  // on                 166/175  262/275  436/447  559/571  669/676    881/871  1005/1026  1187/1177  1265/1258
-  // on, cap half of it  93/ 96  133/150  237/253  341/360  465/478    724/733    920/915  1167/1146  1227/1196
-  // (two runs of one side differ by up to 5 % from 8 to 48 blocks; of 256 blocks, 64K tokens, on: 11,122/10,883)
-  const bool long_walks = p.mask || p.order_stride > (p.stage2 ? kShortWalk : kShortWalkAll);
-  auto pick = [&](auto mask_c, auto long_c) {
-    constexpr bool M = decltype(mask_c)::value, L = decltype(long_c)::value;
-    return p.stage2 ? (small_pages ? osk_tc_kernel<M, true, true, L> : osk_tc_kernel<M, true, false, L>)
-                    : (small_pages ? osk_tc_kernel<M, false, true, L> : osk_tc_kernel<M, false, false, L>);
+  // Stage 2 off        112/115  179/193  316/322  446/459  562/573    811/817  1040/1038  1529/1532  2008/2010 (in one place: 107, 182, 308, 435, ...)
+  // on                 111/113  167/179  277/265  362/354  425/413    554/540    693/678    917/901  1139/1116
+  // on, cap half of it   95/102  128/131  209/209  304/300  393/382    540/528    665/652    918/905  1128/1101
+  // (the 128K layer, Stage 2 on: 7,860/7,757).  With Stage 2 off the tiles' code is shared at every length
+  const bool long_walks = p.stage2 && (p.mask || p.order_stride > kShortWalk);
+  auto pick = [&](auto mask_c, auto stage2_c, auto long_c) {
+    constexpr bool M = decltype(mask_c)::value, S = decltype(stage2_c)::value, L = decltype(long_c)::value;
+    return small_pages ? osk_tc_kernel<M, S, true, L> : osk_tc_kernel<M, S, false, L>;
   };
-  auto kernel = p.mask ? pick(std::true_type{}, std::true_type{}) : (long_walks ? pick(std::false_type{}, std::true_type{}) : pick(std::false_type{}, std::false_type{}));
+  constexpr std::true_type yes{};
+  constexpr std::false_type no{};
+  auto kernel = !p.stage2 ? (p.mask ? pick(yes, no, no) : pick(no, no, no))
+                          : (p.mask ? pick(yes, yes, yes) : (long_walks ? pick(no, yes, yes) : pick(no, yes, no)));
   static SmemLimit limits[16];
   cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kernel),
                                    &limits[(p.mask ? 8 : 0) + (p.stage2 ? 4 : 0) + (small_pages ? 2 : 0) + (long_walks ? 1 : 0)], kSmemBytes);
