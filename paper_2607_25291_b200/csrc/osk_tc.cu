@@ -168,7 +168,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
   Control* ctl = reinterpret_cast<Control*>(smem + (size_t)kTileBytes * 3 + kHalfBytes);
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (uniform, which the compiler cannot know)
-  const int G = p.hq / p.hkv;
+  const int G = p.group;
   chain_wait();
 
   int b = 0, g = 0, i = 0;                 // (load warp, item warp) batch item, KV head, query block
@@ -202,8 +202,8 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
   // that CTAs resident together read the same K/V pages
   int h = 0;
   auto decode = [&](int w) {
-    const int per_kv = G * p.nqb, bg = w / per_kv, wk = w - bg * per_kv, back = wk / G;
-    b = bg / p.hkv;
+    const int bg = divided(w, p.by_kv), wk = w - bg * (G * p.nqb), back = divided(wk, p.by_group);
+    b = divided(bg, p.by_hkv);
     g = bg - b * p.hkv;
     i = p.nqb - 1 - back;
     h = g * G + wk - back * G;
@@ -809,6 +809,8 @@ cudaError_t launch_osk_tc(const OskParams& p_in, cudaStream_t st) {
   }
   int32_t* status = device_status_word();
   if (!status) return cudaErrorInvalidSymbol;
+  p.group = p.hq / p.hkv;
+  p.by_kv = fast_div(p.group * p.nqb); p.by_group = fast_div(p.group); p.by_hkv = fast_div(p.hkv);
   const int n_sm = device_sm_count();
   p.wave = n_sm > 0 ? kCtasPerSm * n_sm : 1 << 30;   // (a CTA an item if the SM count cannot be read)
   return launch_chained(kernel, dim3(p.batch * p.hq * p.nqb), kThreads, kSmemBytes, st, qm, km, vm, p, status);
