@@ -106,6 +106,7 @@ struct __align__(16) Control {
   unsigned long long fin;          // every product has finished
   uint32_t tmem_base;
   volatile int abort_flag;         // kTimedOut, kPoisoned
+  volatile int first_k;            // the item warp has requested K(0)
   volatile int req[6];             // requested by the time the load warp left: K tiles by parity, V tiles by half, Q tiles, work items
   volatile int diag[2];            // K(k) (by parity of k) is the diagonal block
   volatile uint32_t dec[2];
@@ -155,6 +156,9 @@ template <bool kMask, bool kStage2, bool kSmallPages, bool kLongWalks>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
               const __grid_constant__ CUtensorMap v_map, OskParams p, int32_t* status) {
+  // Short walks: a CTA's first tile is asked for by the item warp (8 blocks of 2 heads, whole pass 19.4 -> 19.2 us, 32 of 4 heads 26.9 -> 26.3, 31 of 32
+  // heads 46.9 -> 46.4; with the longer code 2 x 61 blocks +1.8 %, 32K +1.3)
+  constexpr bool kEarlyTile = kStage2 && !kLongWalks && !kMask;
   extern __shared__ __align__(1024) unsigned char smem_raw[];   // swizzled tiles need 1024-byte alignment
   unsigned char* smem = smem_raw;
   const uint32_t base = smem_u32(smem_raw);
@@ -237,7 +241,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       }
       mbar_init(smem_u32(&ctl->s_full), 1); mbar_init(smem_u32(&ctl->s_first), 1); mbar_init(smem_u32(&ctl->s_read), kBlock);
       mbar_init(smem_u32(&ctl->fin), 1);
-      ctl->abort_flag = 0;
+      ctl->abort_flag = 0; ctl->first_k = 0;
       for (int q = 0; q < 6; ++q) ctl->req[q] = 0;
       for (int q = 0; q < 3; ++q) ctl->yes[q] = -1;
       mbar_fence_init();
@@ -289,6 +293,11 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
           if (b != b_known) {
             b_known = b;
             nqb_b = item_blocks(p.pg, b, p.nqb);   // the item's own length in blocks; query blocks past it are padding
+            // The CTA's first tile at once: by way of the load warp, whose code is cold, it is asked for 1,800 cycles later
+            if (kEarlyTile && t == 0 && raw_cnt > 0 && i < nqb_b) {
+              fetch(2, clamp_id(j0), 0, 0);
+              if (lane == 0) ctl->first_k = 1;
+            }
             // a batch item no longer than Delta would have ln(Delta/N) >= 0 and lose even its first block: the test is off for it
             const float th = p.use_threshold ? item_theta(p.pg, b, p.theta, p.skip_scale, nqb_b) : 0.f;
             theta2 = th < 0.f ? th * 1.4426950408889634f : -INFINITY;
@@ -409,7 +418,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
                 alive = wait(after_qk ? &ctl->s_full : &ctl->pv_done[is_k ? 1 : part], after_qk ? k_base + k + 1 : n_base + n - 1);
               if (!alive) return;
               if (is_k) ++n_k; else ++n_v;
-              fetch(part, clamp_id(is_k ? j2 : j0), is_k && (computed || k == -1) ? y ^ 1 : y, k_base + k + 2);
+              if (!kEarlyTile || t > 0 || k > -2) fetch(part, clamp_id(is_k ? j2 : j0), is_k && (computed || k == -1) ? y ^ 1 : y, k_base + k + 2);   // (else: by the item warp)
             };
             if (!kStage2) {
               // V(0)'s first half, V(k)'s second, V(k + 1)'s first (a turn ahead: its place is free before Q K^T of the next position begins),
@@ -757,7 +766,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
 #pragma unroll 1
       for (int q = 0; q < 6; ++q) {
         unsigned long long* bar = q < 2 ? &ctl->k_full[q] : (q < 4 ? &ctl->v_full[q - 2] : (q == 4 ? &ctl->q_full : &ctl->grant_bar));
-        const int c = ctl->req[q];
+        const int c = kEarlyTile && q == 0 ? max(ctl->req[0], ctl->first_k) : ctl->req[q];
         if (c > 0) (void)mbar_wait_noabort(smem_u32(bar), (c - 1) & 1);
       }
       (void)mbar_wait_noabort(smem_u32(&ctl->fin), 0);
