@@ -499,6 +499,29 @@ def test_kap_lists_made_by_the_screen(blocks, stride, kw, copies):
     assert torch.equal(got["kap_flags"], ref["kap_flags"]) and torch.equal(got["kap_scores"], ref["kap_scores"])
 
 
+@pytest.mark.parametrize("blocks,stride,kw", [(16, 8, {}), (17, 8, {}), (33, 4, {}), (64, 8, dict(causal=False)), (65, 8, {}), (130, 16, {}),
+                                              (255, 8, {}), (256, 8, dict(top_p=0.9))])
+def test_kap_lists_whose_scores_differ_in_their_last_bits(blocks, stride, kw):
+    """Key blocks in groups of four that differ by an ulp or two of one element of a sampled key: scores 2^-16 or so apart, which share
+    a sort word of the screen's lists whatever their order.  Lists, scores and flags are the sort kernel's (impl 3), the kept
+    ids the double-precision kernel's."""
+    w = tiny(seed=blocks, hq=4, hkv=1, n=blocks * 128, needles=min(3, blocks - 1))
+    qb, kb, vb, _ = w.make()
+    q, k = to_dev(qb), to_dev(kb)
+    kk = k.view(torch.int16).view(1, 1, blocks, 128, 128)
+    for j in range(blocks):
+        kk[:, :, j] = kk[:, :, j // 4 * 4]
+        kk[:, :, j, j % (128 // stride) * stride, j * 13 % 128] += j % 4
+    budget = 1.0 if "top_p" in kw else 0.4
+    order, count, got = run_kap(q, k, budget, stride, scores=True, **kw)
+    order3, count3, ref = run_kap(q, k, budget, stride, scores=True, impl=3, **kw)
+    assert torch.equal(count, count3) and torch.equal(order, order3)
+    assert torch.equal(got["kap_flags"], ref["kap_flags"]) and torch.equal(got["kap_scores"], ref["kap_scores"])
+    exact, _ = run_kap(q, k, budget, stride, impl=1, **kw)
+    kept = torch.arange(order.shape[-1], device="cuda") < count[..., None]
+    assert torch.equal(torch.where(kept, order, -1), torch.where(kept, exact, -1))
+
+
 @pytest.mark.parametrize("stride", [4, 8, 16])
 @pytest.mark.parametrize("hq,hkv", [(8, 1), (16, 2), (2, 2)])
 def test_kap_query_group_sizes(hq, hkv, stride):
@@ -644,6 +667,32 @@ def test_osk_weight_of_a_rows_maximum_is_exact(sharpness, tb, impl):
     bound = 2.0 ** -8 * (np.abs(ref) + rest @ np.abs(vf)) + 2.0 ** -14 * (w @ np.abs(vf))
     over = np.abs(out - ref) > bound
     assert not over.any(), (int(over.sum()), float((np.abs(out - ref) / bound).max()))
+
+
+@pytest.mark.parametrize("tb,skip_scale", [(1.0, -1.0), (0.999, 300.0), (0.3, -1.0), (0.15, 500.0)])
+@pytest.mark.parametrize("batch", [1, 16])
+def test_osk_lists_of_one_length_at_two_pitches(batch, tb, skip_scale):
+    """The kernel for lists of up to 8 blocks and the one for longer lists: the same lists of 0 to 8 blocks at pitch 8 and at pitch 9
+    give the same bits, with a CTA a work item and with CTAs that take over further ones."""
+    hq, hkv, n = 8, 2, 1024
+    nqb = n // 128
+    g = torch.Generator(device="cuda").manual_seed(batch)
+    q, k, v = (torch.randn(batch, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv, hkv))
+    order = torch.argsort(torch.rand(batch, hq, nqb, nqb, device="cuda", generator=g), dim=-1).to(torch.int32)
+    count = torch.randint(0, nqb + 1, (batch, hq, nqb), device="cuda", generator=g, dtype=torch.int32)
+    got = []
+    for pitch in (8, 9):
+        lists = torch.full((batch, hq, nqb, pitch), -1, dtype=torch.int32, device="cuda")
+        lists[..., :8] = order
+        out = torch.full_like(q, 3.0)
+        lse = torch.full(q.shape[:3], 3.0, device="cuda")
+        vis = torch.full(count.shape, -7, dtype=torch.int32, device="cuda")
+        cosa.cosa_osk_attention(q, k, v, lists, count, tb, out, lse, vis, causal=False,
+                                opt=cosa.default_options(skip_scale=skip_scale, order_stride=pitch))
+        assert cosa.cosa_device_status() == 0
+        got.append((out, lse, vis))
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
 
 
 @pytest.mark.parametrize("walk", ["dense", "mask", "page16"])
