@@ -20,8 +20,7 @@
 // has the second half's exponentials to run under, V's first half comes a position ahead, and neither half waits for the
 // other's place (all blocks of 16K 2,009 -> 1,965 us, 64K at 12.5 % 4,232 -> 4,199; both halves there, S behind the
 // whole block: 2,130 and 4,494).  With Stage 2 on S must not wait for a V tile that is asked for after the vote.  (32 keys at a time
-// through the same buffer: 2 to 6 % slower, each hand-over costs the rows a proxy fence.  Operands of Q K^T and P V both come
-// from shared memory: measured at the full 512 cycles per 128 x 128 x 128 product, also while tiles stream in.)
+// through the same buffer: 2 to 6 % slower, each hand-over costs the rows a proxy fence.)
 // Tiles: two slots X and Y.  When block k is decided, X holds K(k+1) and Y is free or holds the last V tile.  Skipped: K(k+2)
 // goes to Y, and the slots change roles.  Computed: V(k) goes to Y, each 64-key half as soon as the product on the half before
 // it has released it, and K(k+2) to X when Q K^T of k+1 is done.
@@ -38,16 +37,18 @@
 // 209 on walks of 3.4 blocks; one place that fetches K and V tiles instead of two: 175 -> 169, and 3 % of the walks of four
 // prompts in 16-token pages); with Stage 2 long ones have it written out (kLongWalks).
 // What bounds it: tensor pipe and exponentials both want about 1,024 cycles (0.52 us) of an SM per computed block, 512 per skipped
-// one.  Fitted to single launches at the full clock, an SM takes 1.03 us a computed block with Stage 2 off, 1.19 with it on (the
-// vote keeps the four row warps together), 0.43 a skipped one and 1.7 a work item; the tensor pipe is busy half of the time, and
-// the reads of its operands keep shared memory as busy.  Single launches, a CTA an item -> several, items decoded in the load
-// warp -> now: 128K tokens and 4 % computed 7.51 -> 7.39 -> 7.30 ms, 32K and 8 % 1.08 -> 1.02 -> 0.95, all blocks of 16K 1.92 ->
-// 1.89 -> 1.81, walks of 3.4 blocks (2 x 7,808 tokens) 0.246 -> 0.214 -> 0.167 (32 query heads everywhere; one CTA of twelve
-// warps per SM with two softmax groups and a controller warp, the arrangement before both: 8.1, 1.25 and 2.00 on the first
-// three; it is still the better one, by up to 6 %, where Stage 2 is on and skips next to nothing of long lists).  Measured and
-// not used (when the first three took 7.15, 1.02 and 1.85): P over S in tensor memory (7.9 / 1.11 / 2.26), two threads per row
-// (8.2 / 1.15 / 2.12), tiles prefetched into L2 (+2 to 5 %), V(k) requested before the decision on k after a computed block
-// (128K +4 to 5 %, 32K +6 to 8, walks of 3.4 blocks +9).
+// one.  By clock stamps an SM takes 1,600 cycles a computed block with Stage 2 off, 2,100 with it on (the vote, and V only after it), 620 a
+// skipped one -- a product whose operands both come from shared memory takes the tensor pipe 570 to 600, not 512 -- and 2,600 a work
+// item.  At 32K tokens the pipe is busy 58 % of the time, shared memory's data pipe 82 % (operands 58, threads 24).  A walk alone on an
+// SM takes 3,900 cycles a computed block: two fill each other's waits, the row threads of both together want 2,500 for two blocks.
+// Single launches, a CTA an item -> several -> items decoded in a warp of their own -> now: 128K tokens and 4 % computed 7.51 -> 7.39 -> 7.30 ->
+// 6.8 ms, 32K and 8 % 1.08 -> 1.02 -> 0.95 -> 0.90, all blocks of 16K 1.92 -> 1.89 -> 1.81 -> 1.77, walks of 3.4 blocks (2 x 7,808 tokens) 0.246
+// -> 0.214 -> 0.167 -> 0.157 (32 query heads everywhere; one CTA of twelve warps per SM with two softmax groups and a controller
+// warp, the arrangement before all of these: 8.1, 1.25 and 2.00 on the first three).  Measured and not used: P over S in tensor memory with
+// the next S behind both halves (all blocks of 16K +6.5 %), two threads per row (8.2 / 1.15 / 2.12 ms when the first three took
+// 7.15, 1.02 and 1.85), tiles prefetched into L2 (+2 to 5 %), V(k) requested before the decision on k after a computed block (+4 to
+// 9 %; V(0), which is certain, gains nothing), a share of the exponentials by polynomial (+2 to 10 %: their issue slots are the other warps'),
+// Q K^T held back where the next computed block ends the walk (+0.3 to 3.5 %), the output by TMA or in 32-byte stores without staging (+0 to 11 %).
 // Every wait is bounded; a wait that runs out sets the device status word and the CTA winds down without writing
 // further results (a work item's are written whole or not at all): load and issue warps leave, the row threads, whom no wait holds any more, run to the end of their list.
 #include <math.h>
@@ -236,7 +237,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
       for (int s = 0; s < 2; ++s) {
         mbar_init(smem_u32(&ctl->item_bar[s]), 1); mbar_init(smem_u32(&ctl->item_read[s]), kBlock + 2);
         mbar_init(smem_u32(&ctl->k_full[s]), 1); mbar_init(smem_u32(&ctl->v_full[s]), 1);
-        mbar_init(smem_u32(&ctl->dec_bar[s]), 4); mbar_init(smem_u32(&ctl->p_full[s]), kBlock);
+        mbar_init(smem_u32(&ctl->dec_bar[s]), 4); mbar_init(smem_u32(&ctl->p_full[s]), kStage2 ? kBlock : 4);
         mbar_init(smem_u32(&ctl->pv_done[s]), 1);
       }
       mbar_init(smem_u32(&ctl->s_full), 1); mbar_init(smem_u32(&ctl->s_first), 1); mbar_init(smem_u32(&ctl->s_read), kBlock);
@@ -612,8 +613,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
           // 1,045 us, 128K 8,029 -> 7,955, walks of 3.4 blocks 179 -> 176, of 2 blocks 33.3 -> 32.5, 4K of 4 heads 14.4 -> 13.7)
           const int pos = pos_base + kk;
           bool compute = __any_sync(0xffffffffu, !((m_loc - m_new) < theta2));
-          if (compute && lane == 0) ctl->yes[turn] = pos;
-          __syncwarp();
+          if (compute) ctl->yes[turn] = pos;
           if (compute && !__any_sync(0xffffffffu, bad)) {
             bar_arrive(2 + turn, kBlock);
           } else {
@@ -622,13 +622,14 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
           }
           turn = turn == 2 ? 0 : turn + 1;
           last = last || n + (compute ? 1 : 0) == cap;
-          if (lane == 0) {
-            ctl->dec[pos & 1] = (compute ? kDecComputed : 0u) | (last ? kDecEnd : 0u);
-            mbar_arrive(smem_u32(&ctl->dec_bar[pos & 1]));
-          }
-          if (r == 0) {
+          ctl->dec[pos & 1] = (compute ? kDecComputed : 0u) | (last ? kDecEnd : 0u);
+          mbar_arrive_if(smem_u32(&ctl->dec_bar[pos & 1]), lane == 0);
+          if (p.decisions) {
             if (compute) dec_word |= 1u << (kk & 31);
-            if (p.decisions && ((kk & 31) == 31 || last) && !*abort_flag) { p.decisions[row * dec_words + (kk >> 5)] = dec_word; dec_word = 0; }
+            if ((kk & 31) == 31 || last) {
+              if (r == 0 && !*abort_flag) p.decisions[row * dec_words + (kk >> 5)] = dec_word;
+              dec_word = 0;
+            }
           }
           if (!compute) {                           // skipped: nothing is added to l or O, and no maximum has moved
             if (last) break;
@@ -691,7 +692,9 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
             fence_proxy_async_smem();
           }
           if (half == 0) tc_fence_before();         // (a rescaled O)
-          mbar_arrive(smem_u32(&ctl->p_full[half]));
+          // (one arrival a warp: all blocks of 16K 1,947 -> 1,924 us; with Stage 2 on equal, every thread arrives)
+          if (!kStage2) __syncwarp();
+          mbar_arrive_if(smem_u32(&ctl->p_full[half]), kStage2 || lane == 0);
         }
         {
           float r0, r1, r2, r3;
