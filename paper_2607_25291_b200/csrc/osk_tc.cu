@@ -42,8 +42,8 @@
 // item.  At 32K tokens the pipe is busy 58 % of the time, shared memory's data pipe 82 % (operands 58, threads 24).  A walk alone on an
 // SM takes 3,900 cycles a computed block: two fill each other's waits, the row threads of both together want 2,500 for two blocks.
 // Single launches, a CTA an item -> several -> items decoded in a warp of their own -> now: 128K tokens and 4 % computed 7.51 -> 7.39 -> 7.30 ->
-// 6.8 ms, 32K and 8 % 1.08 -> 1.02 -> 0.95 -> 0.90, all blocks of 16K 1.92 -> 1.89 -> 1.81 -> 1.77, walks of 3.4 blocks (2 x 7,808 tokens) 0.246
-// -> 0.214 -> 0.167 -> 0.157 (32 query heads everywhere; one CTA of twelve warps per SM with two softmax groups and a controller
+// 6.71 ms, 32K and 8 % 1.08 -> 1.02 -> 0.95 -> 0.90, all blocks of 16K 1.92 -> 1.89 -> 1.81 -> 1.74, walks of 3.4 blocks (2 x 7,808 tokens) 0.246
+// -> 0.214 -> 0.167 -> 0.158 (32 query heads everywhere; one CTA of twelve warps per SM with two softmax groups and a controller
 // warp, the arrangement before all of these: 8.1, 1.25 and 2.00 on the first three).  Measured and not used: P over S in tensor memory with
 // the next S behind both halves (all blocks of 16K +6.5 %), two threads per row (8.2 / 1.15 / 2.12 ms when the first three took
 // 7.15, 1.02 and 1.85), tiles prefetched into L2 (+2 to 5 %), V(k) requested before the decision on k after a computed block (+4 to
