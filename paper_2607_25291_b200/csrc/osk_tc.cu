@@ -19,7 +19,8 @@
 // first half goes to tensor memory, into the columns S has left, and Q K^T of the next position follows the product on it: it
 // has the second half's exponentials to run under, V's first half comes a position ahead, and neither half waits for the
 // other's place (all blocks of 16K 2,009 -> 1,965 us, 64K at 12.5 % 4,232 -> 4,199; both halves there, S behind the
-// whole block: 2,130 and 4,494).  With Stage 2 on S must not wait for a V tile that is asked for after the vote.  (32 keys at a time
+// whole block: 2,130 and 4,494).  Not with Stage 2 on, where S must not wait for a V tile that is asked for after the vote, and not
+// with pages smaller than a key block: a tile of theirs is many copies, and K(k + 2) would be asked for later.  (32 keys at a time
 // through the same buffer: 2 to 6 % slower, each hand-over costs the rows a proxy fence.)
 // Tiles: two slots X and Y.  When block k is decided, X holds K(k+1) and Y is free or holds the last V tile.  Skipped: K(k+2)
 // goes to Y, and the slots change roles.  Computed: V(k) goes to Y, each 64-key half as soon as the product on the half before
@@ -35,7 +36,7 @@
 // all roles) loses lines to it: 225 requests an item go to the next cache on walks of 3.4 blocks, 20 a block on long ones.  Code is
 // therefore shared rather than unrolled or inlined twice where walks are short (a form of 88 KB instead of 61: 236 us instead of
 // 209 on walks of 3.4 blocks; one place that fetches K and V tiles instead of two: 175 -> 169, and 3 % of the walks of four
-// prompts in 16-token pages); with Stage 2 long ones have it written out (kLongWalks).
+// prompts in 16-token pages); with Stage 2 and with small pages long ones have it written out (kLongWalks).
 // What bounds it: tensor pipe and exponentials both want about 1,024 cycles (0.52 us) of an SM per computed block, 512 per skipped
 // one.  By clock stamps an SM takes 1,600 cycles a computed block with Stage 2 off, 2,100 with it on (the vote, and V only after it), 620 a
 // skipped one -- a product whose operands both come from shared memory takes the tensor pipe 570 to 600, not 512 -- and 2,600 a work
@@ -73,7 +74,7 @@ constexpr int kCtasPerSm = 2;
 constexpr int kTmemCols = 256;
 constexpr int kLoadWarp = 4, kMmaWarp = 5, kItemWarp = 6;
 constexpr int kAskAhead = 4;                       // positions (or two computed blocks) before a walk's end at which more work is asked for
-constexpr int kShortWalk = 8;                      // list pitch up to which walks count as short, with Stage 2
+constexpr int kShortWalk = 8, kShortWalkPages = 4;  // list pitch up to which walks count as short, with Stage 2 and, without it, with small pages
 constexpr uint32_t kDecComputed = 1, kDecEnd = 2;
 constexpr int kTimedOut = 1, kPoisoned = 2;
 
@@ -99,9 +100,9 @@ struct __align__(16) Control {
   unsigned long long v_full[2];    // by half: the n-th V tile's half has landed
   unsigned long long s_full;       // Q K^T of the position has finished
   unsigned long long s_first;      // the same for the first position of a walk (a waiter may come when the second has finished, too)
-  unsigned long long s_read;       // (Stage 2) every row has taken its S to registers
+  unsigned long long s_read;       // (unless P goes over S) every row has taken its S to registers
   unsigned long long dec_bar[2];   // the decision of a position (by parity) is in dec[]
-  unsigned long long p_full[2];    // by half: the n-th P's half is in shared memory (the first with Stage 2 off: in tensor memory)
+  unsigned long long p_full[2];    // by half: the n-th P's half is in shared memory (the first may be in tensor memory)
   unsigned long long pv_done[2];   // by half: the n-th product with that half has finished (one barrier each: a waiter may be
                                    // a whole block late, and one parity bit cannot tell two phases apart)
   unsigned long long fin;          // every product has finished
@@ -152,11 +153,13 @@ __device__ __forceinline__ void mask_diagonal(uint32_t s, int warp, int lane) {
 //          of the load warp issue side by side, each after its own table look-up.  Boxes land on 1024-byte boundaries of
 //          the tile (pages of at least 8 tokens), where the 128-byte swizzle, a function of the shared-memory address,
 //          gives the layout of the one-piece tile.
-// kLongWalks: (Stage 2) copies of the code that runs once a position or once an item are written out (see above); else they are shared
+// kLongWalks: (Stage 2 or small pages) copies of the code that runs once a position or once an item are written out (see above); else they
+//          are shared
 template <bool kMask, bool kStage2, bool kSmallPages, bool kLongWalks>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
               const __grid_constant__ CUtensorMap v_map, OskParams p, int32_t* status) {
+  constexpr bool kPInTmem = !kStage2 && !kSmallPages;   // P's first half goes to tensor memory, over S
   // Short walks: a CTA's first tile is asked for by the item warp (8 blocks of 2 heads, whole pass 19.4 -> 19.2 us, 32 of 4 heads 26.9 -> 26.3, 31 of 32
   // heads 46.9 -> 46.4; with the longer code 2 x 61 blocks +1.8 %, 32K +1.3)
   constexpr bool kEarlyTile = kStage2 && !kLongWalks && !kMask;
@@ -421,7 +424,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
               if (is_k) ++n_k; else ++n_v;
               if (!kEarlyTile || t > 0 || k > -2) fetch(part, clamp_id(is_k ? j2 : j0), is_k && (computed || k == -1) ? y ^ 1 : y, k_base + k + 2);   // (else: by the item warp)
             };
-            if (!kStage2) {
+            if (kPInTmem) {
               // V(0)'s first half, V(k)'s second, V(k + 1)'s first (a turn ahead: its place is free before Q K^T of the next position begins),
               // K(k + 2)
 #pragma unroll 1
@@ -492,9 +495,9 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         alive = wait(&ctl->q_full, q);
         int k = -1, n = 0;
         while (alive) {
-          if (!kStage2 && k < 0 && n_base > 0) alive = wait(&ctl->pv_done[0], n_base - 1);   // (the walk before: P lay in S's place)
-          if (kStage2 && k >= 0) alive = wait(&ctl->s_read, pos_base + k);
-          if (alive && (kStage2 || k < 0) && k + 1 < n_pos) alive = issue_qk(k_base + k + 1, k < 0 ? y : y ^ 1);
+          if (kPInTmem && k < 0 && n_base > 0) alive = wait(&ctl->pv_done[0], n_base - 1);   // (the walk before: P lay in S's place)
+          if (!kPInTmem && k >= 0) alive = wait(&ctl->s_read, pos_base + k);
+          if (alive && (!kPInTmem || k < 0) && k + 1 < n_pos) alive = issue_qk(k_base + k + 1, k < 0 ? y : y ^ 1);
           if (k < 0) {
             if (!kStage2 && alive) mma_commit(smem_u32(&ctl->s_first));
             ++k;
@@ -513,7 +516,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
               alive = wait(&ctl->v_full[half], n_base + n) && wait(&ctl->p_full[half], n_base + n);
               if (!alive) break;
               tc_fence_after();
-              if (!kStage2 && half == 0) {           // P's first half lies in S's place: the next S behind its product
+              if (kPInTmem && half == 0) {           // P's first half lies in S's place: the next S behind its product
                 mma_ts_x4<128, 256, 384>(tmem_o, tmem_s, vdesc0 + (uint64_t)(y * kTileBytes / 16), idesc_pv, n > 0);
                 mma_commit(smem_u32(&ctl->pv_done[0]));
                 if (k + 1 < n_pos) alive = wait(&ctl->pv_done[0], n_base + n) && issue_qk(k_base + k + 1, y ^ 1);
@@ -593,7 +596,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
         for (int c = 0; c < 4; ++c) tmem_ld32(tmem_s + lane_addr + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
         tmem_wait_ld();
         tc_fence_before();
-        if (kStage2) mbar_arrive(smem_u32(&ctl->s_read));
+        if (!kPInTmem) mbar_arrive(smem_u32(&ctl->s_read));
         // (three-input maxima: half the instructions of the two-input form)
         float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
@@ -650,10 +653,11 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
           // the buffer's last reader: the second half of the block before, the first half of this one (asked now, needed
-          // after the exponentials).  Without Stage 2 only second halves lie there, and O may be rescaled behind the last product
-          const int last_n = n_base + n - 1 + (kStage2 ? half : 0);
-          unsigned long long* last_reader = &ctl->pv_done[kStage2 ? half ^ 1 : 1];
-          const bool is_free = (kStage2 ? n + half == 0 : n == 0 || (half == 0 && !moved)) || mbar_test_wait(smem_u32(last_reader), last_n & 1);
+          // after the exponentials).  With the first half in tensor memory only second halves lie there, and O may be rescaled behind the
+          // last product
+          const int last_n = n_base + n - 1 + (kPInTmem ? 0 : half);
+          unsigned long long* last_reader = &ctl->pv_done[kPInTmem ? 1 : half ^ 1];
+          const bool is_free = (kPInTmem ? n == 0 || (half == 0 && !moved) : n + half == 0) || mbar_test_wait(smem_u32(last_reader), last_n & 1);
 #pragma unroll
           for (int c = half * kHalfKeys; c < (half + 1) * kHalfKeys; c += 4) {
             float e0, e1, e2, e3;
@@ -679,7 +683,7 @@ osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__
             }
             tmem_wait_st();
           }
-          if (!kStage2 && half == 0) {
+          if (kPInTmem && half == 0) {
             __syncwarp();
             tmem_st32(tmem_s + lane_addr, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
             tmem_wait_st();
@@ -800,16 +804,26 @@ cudaError_t launch_osk_tc(const OskParams& p_in, cudaStream_t st) {
   // Stage 2 off        112/115  179/193  316/322  446/459  562/573    811/817  1040/1038  1529/1532  2008/2010 (in one place: 107, 182, 308, 435, ...)
   // on                 111/113  167/179  277/265  362/354  425/413    554/540    693/678    917/901  1139/1116
   // on, cap half of it   95/102  128/131  209/209  304/300  393/382    540/528    665/652    918/905  1128/1101
-  // (the 128K layer, Stage 2 on: 7,860/7,757).  With Stage 2 off the tiles' code is shared at every length
-  const bool long_walks = p.stage2 && (p.mask || p.order_stride > kShortWalk);
-  auto pick = [&](auto mask_c, auto stage2_c, auto long_c) {
-    constexpr bool M = decltype(mask_c)::value, S = decltype(stage2_c)::value, L = decltype(long_c)::value;
-    return small_pages ? osk_tc_kernel<M, S, true, L> : osk_tc_kernel<M, S, false, L>;
+  // (the 128K layer, Stage 2 on: 7,860/7,757).  With Stage 2 off the tiles' code is shared at every length, but for small pages.  Those,
+  // read in place, Stage 2 off (P's first half over S and shared code, at pitches from 8 up: 8 to 12 % more than the written-out form,
+  // pages of 64 2 to 4):
+  //                          2        4        8       16       32         64 blocks
+  // pages of 8         129/121  234/218  441/408  851/787  1663/1535  3267/3009
+  // of 16              105/101  182/169  335/307  646/624  1348/1231  2575/2430
+  // of 32              101/106  163/157  291/274  602/554  1173/1089  2320/2128
+  // of 64              107/114  166/177  286/274  552/542  1067/1072  2118/2130
+  const bool off_pages = !p.stage2 && small_pages;
+  const bool long_walks = off_pages ? p.mask || p.order_stride > kShortWalkPages : p.stage2 && (p.mask || p.order_stride > kShortWalk);
+  auto pick = [&](auto mask_c, auto stage2_c, auto pages_c, auto long_c) {
+    return osk_tc_kernel<decltype(mask_c)::value, decltype(stage2_c)::value, decltype(pages_c)::value, decltype(long_c)::value>;
   };
   constexpr std::true_type yes{};
   constexpr std::false_type no{};
-  auto kernel = !p.stage2 ? (p.mask ? pick(yes, no, no) : pick(no, no, no))
-                          : (p.mask ? pick(yes, yes, yes) : (long_walks ? pick(no, yes, yes) : pick(no, yes, no)));
+  auto kernel = off_pages ? (p.mask ? pick(yes, no, yes, yes) : (long_walks ? pick(no, no, yes, yes) : pick(no, no, yes, no)))
+              : !p.stage2 ? (p.mask ? pick(yes, no, no, no) : pick(no, no, no, no))
+              : p.mask    ? (small_pages ? pick(yes, yes, yes, yes) : pick(yes, yes, no, yes))
+              : long_walks ? (small_pages ? pick(no, yes, yes, yes) : pick(no, yes, no, yes))
+                           : (small_pages ? pick(no, yes, yes, no) : pick(no, yes, no, no));
   static SmemLimit limits[16];
   cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kernel),
                                    &limits[(p.mask ? 8 : 0) + (p.stage2 ? 4 : 0) + (small_pages ? 2 : 0) + (long_walks ? 1 : 0)], kSmemBytes);

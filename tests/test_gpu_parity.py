@@ -740,6 +740,70 @@ def test_osk_ctas_that_take_over_further_work_items(tb, skip_scale, walk):
             assert torch.equal(x[b:b + 1], y)
 
 
+def _scattered(x, table, page_size):
+    """The pool of `page_size`-token pages that holds x [B,H,N,d] as `table` [B,N/page_size] lays it out."""
+    b, h, n, d = x.shape
+    pool = torch.empty(table.numel(), h, page_size, d, dtype=x.dtype, device=x.device)
+    pool[table.view(-1).long()] = x.view(b, h, n // page_size, page_size, d).transpose(1, 2).reshape(-1, h, page_size, d)
+    return pool
+
+
+@pytest.mark.parametrize("pitch", [1, 4, 5, 33, "mask"])
+@pytest.mark.parametrize("page_size", [8, 16, 32, 64])
+def test_osk_small_pages_in_place_stage2_off(page_size, pitch):
+    """Each form that walks pages smaller than a key block with Stage 2 off: bit-equal to the dense tensors, lists of every length
+    and empty ones among them, CTAs that take over further work items."""
+    batch, hq, hkv, n = 2, 8, 2, 40 * 128
+    nqb = n // 128
+    g = torch.Generator(device="cuda").manual_seed(page_size)
+    q, k, v = (torch.randn(batch, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv, hkv))
+    length = nqb if pitch == "mask" else pitch
+    order = torch.argsort(torch.rand(batch, hq, nqb, nqb, device="cuda", generator=g), dim=-1)[..., :length].to(torch.int32).contiguous()
+    count = torch.randint(0, length + 1, (batch, hq, nqb), device="cuda", generator=g, dtype=torch.int32)
+    bits = torch.randint(-2**31, 2**31, (batch, hq, nqb, 2), device="cuda", generator=g, dtype=torch.int64).to(torch.int32)
+    kw = {"logical_mask": bits} if pitch == "mask" else {}
+    table = torch.randperm(batch * n // page_size, device="cuda", generator=g).to(torch.int32).view(batch, -1).contiguous()
+    paged = dict(kv_page_table=table, kv_page_size=page_size, kv_num_pages=table.numel(), kv_pages_in_place=1)
+    got = []
+    for kk, vv, extra in ((k, v, {}), (_scattered(k, table, page_size), _scattered(v, table, page_size), paged)):
+        out = torch.full_like(q, 3.0)
+        lse = torch.full(q.shape[:3], 3.0, device="cuda")
+        vis = torch.full(count.shape, -7, dtype=torch.int32, device="cuda")
+        cosa.cosa_osk_attention(q, kk, vv, order, count, 1.0, out, lse, vis, causal=pitch == "mask",
+                                opt=cosa.default_options(skip_scale=-1.0, order_stride=length, **kw, **extra))
+        assert cosa.cosa_device_status() == 0
+        got.append((out, lse, vis))
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
+
+
+def test_osk_small_pages_in_place_stage2_off_is_not_the_slower_way():
+    """Where every listed block is computed either way, walks without the vote take no longer than walks with it (8-token pages; 2 %
+    for the clock: the forms are 3 % apart on the right side, and were 8 % apart on the wrong one)."""
+    hq, hkv, n, ps, length = 32, 8, 8192, 8, 32
+    nqb = n // 128
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q, k, v = (torch.randn(1, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv, hkv))
+    table = torch.randperm(n // ps, device="cuda", generator=g).to(torch.int32).view(1, -1).contiguous()
+    k, v = _scattered(k, table, ps), _scattered(v, table, ps)
+    order = torch.argsort(torch.rand(1, hq, nqb, nqb, device="cuda", generator=g), dim=-1)[..., :length].to(torch.int32).contiguous()
+    count = torch.full((1, hq, nqb), length, dtype=torch.int32, device="cuda")
+    out, lse, vis = torch.empty_like(q), torch.empty(1, hq, n, device="cuda"), torch.empty_like(count)
+    opt = cosa.default_options(skip_scale=-1.0, order_stride=length, kv_page_table=table, kv_page_size=ps, kv_num_pages=n // ps,
+                               kv_pages_in_place=1)
+    best = {}
+    for _ in range(12):
+        for tb in (1.0, 0.999):
+            begin, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            begin.record()
+            cosa.cosa_osk_attention(q, k, v, order, count, tb, out, lse, vis, causal=False, opt=opt)
+            end.record()
+            torch.cuda.synchronize()
+            assert bool((vis == length).all())
+            best[tb] = min(best.get(tb, float("inf")), begin.elapsed_time(end))
+    assert best[1.0] <= 1.02 * best[0.999], best
+
+
 @pytest.mark.parametrize("impl", OSK_IMPLS)
 def test_osk_noncausal(small, impl):
     q, k, v = small["dev"]
