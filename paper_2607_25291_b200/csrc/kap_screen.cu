@@ -44,6 +44,7 @@
 
 #include "common.cuh"
 #include "kap_recount.cuh"
+#include "list_sort.cuh"
 #include "ptx_sm100.cuh"
 #include "tile_maps.cuh"
 
@@ -187,58 +188,6 @@ __device__ __forceinline__ void f64_row_maxima(const KapParams& p, const __nv_bf
     for (int o = 4; o < 32; o <<= 1) best[x] = fmax(best[x], __shfl_xor_sync(0xffffffffu, best[x], o));
 }
 
-// (a whole warp) sorts 32 * PER keys descending (bitonic, in registers); afterwards lane l holds places l * PER and on
-template <int PER>
-__device__ __forceinline__ void warp_sort_desc(uint32_t (&k)[PER], int lane) {
-#pragma unroll
-  for (int size = 2; size <= 32 * PER; size <<= 1) {
-#pragma unroll
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      if (stride >= PER) {
-        const bool larger = ((lane & (size / PER)) == 0) == ((lane & (stride / PER)) == 0);
-#pragma unroll
-        for (int r = 0; r < PER; ++r) {
-          const uint32_t other = __shfl_xor_sync(0xffffffffu, k[r], stride / PER);
-          k[r] = larger ? max(k[r], other) : min(k[r], other);
-        }
-      } else {
-#pragma unroll
-        for (int r = 0; r < PER; ++r) {
-          if (r & stride) continue;
-          const bool down = size < PER ? (r & size) == 0 : (lane & (size / PER)) == 0;
-          const uint32_t x = max(k[r], k[r | stride]), y = min(k[r], k[r | stride]);
-          k[r] = down ? x : y;
-          k[r | stride] = down ? y : x;
-        }
-      }
-    }
-  }
-}
-// (a whole warp) puts 32 * PER distinct keys that are all but sorted, held as above, in descending order: neighbours change places
-// until none has to
-template <int PER>
-__device__ __forceinline__ void warp_settle_desc(unsigned long long (&k)[PER], int lane) {
-  bool swapped;
-  do {
-    swapped = false;
-    auto order = [&](unsigned long long& x, unsigned long long& y) {
-      const bool swap = y > x;
-      const unsigned long long t = x;
-      x = swap ? y : x;
-      y = swap ? t : y;
-      swapped = swapped || swap;
-    };
-#pragma unroll
-    for (int r = 0; r + 1 < PER; r += 2) order(k[r], k[r + 1]);
-#pragma unroll
-    for (int r = 1; r + 1 < PER; r += 2) order(k[r], k[r + 1]);
-    // the last key of a lane and the first of the next
-    const unsigned long long next = __shfl_down_sync(0xffffffffu, k[0], 1), before = __shfl_up_sync(0xffffffffu, k[PER - 1], 1);
-    if (lane < 31 && next > k[PER - 1]) { k[PER - 1] = next; swapped = true; }
-    if (lane > 0 && before < k[0]) { k[0] = before; swapped = true; }
-  } while (__any_sync(0xffffffffu, swapped));
-}
-
 // (a whole warp) the visit list of one (head, query block) of at most 32 * PER candidates: what kap_sort_kernel does for longer
 // calls, step by step.  score[j]: the screened scores (sign: HRM flag); j1, j2: its rows' best and second best blocks; srt: room for
 // the keys.  The list waits in its row of `scores`; what is left for the fix-up: near ties (entries in the same row) or the whole list.
@@ -309,21 +258,7 @@ __device__ void make_list(const KapParams& p, const KapScreenParams& sp, float t
     for (int u = 0; u < J; ++u) rank += __shfl_sync(0xffffffffu, key[0], u) > key[0] ? 1 : 0;
     if (lane < J) srt[rank] = key[0];
   } else {
-    // Sorted by words of a flag, the leading bits of the score and the id, which is a third of the work of sorting whole keys; what that
-    // leaves out of order is close together and settled after.  (Ids are below 256.  A word of 0 is no key, or the last of 256)
-    static_assert(32 * PER <= 256, "an id is a byte");
-    uint32_t word[PER];
-#pragma unroll
-    for (int x = 0; x < PER; ++x) word[x] = ((uint32_t)(key[x] >> 32) & 0xffffff00u) | (lane + 32 * x < J ? 0xffu - (uint32_t)(lane + 32 * x) : 0u);
-    warp_sort_desc<PER>(word, lane);
-#pragma unroll
-    for (int x = 0; x < PER; ++x) {
-      const uint32_t j = 0xffu - (word[x] & 0xffu);
-      key[x] = lane * PER + x < J ? ((unsigned long long)((word[x] & 0x80000000u) | __float_as_uint(fabsf(score[j]))) << 32) | (0xffffffffu - j) : 0ULL;
-    }
-    warp_settle_desc<PER>(key, lane);
-#pragma unroll
-    for (int x = 0; x < PER; ++x) srt[lane * PER + x] = key[x];
+    sort_list<PER>(key, score, J, srt, lane);
   }
   __syncwarp();
   auto score_at = [&](int t) { return __uint_as_float((unsigned)(srt[t] >> 32) & 0x7fffffffu); };
