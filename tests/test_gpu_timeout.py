@@ -188,3 +188,74 @@ def test_osk_writes_a_work_item_whole_or_not_at_all(tb):
             assert bool(torch.where(done[:, None], a == b, a == blank).all()), cycles
         in_part += int(bool(done.any()) and not bool(done.all()))
     assert in_part > 0
+
+
+# the forms of the OSK kernel that the lists above (pitch 31 and 32) do not reach: (list pitch, Stage-2 cap, page size in place or 0)
+SHORT_FORMS = [(8, 0.999, 0), (8, 0.999, 16), (31, 0.999, 16), (4, 1.0, 16), (31, 1.0, 16), (8, 1.0, 0)]
+
+
+def _short_call(pitch, tb, page_size):
+    """hq 32, hkv 8, 31 query blocks, lists of 0 to min(pitch, 5) blocks; returns call(**options) -> ([out, lse, visited, scored] by work
+    item, status)."""
+    hq, hkv, nqb = 32, 8, 31
+    n = nqb * 128
+    g = torch.Generator(device="cuda").manual_seed(3)
+    q, k, v = (torch.randn(1, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv, hkv))
+    order = torch.arange(pitch, dtype=torch.int32, device="cuda").expand(1, hq, nqb, pitch).contiguous()
+    count = (torch.arange(nqb, dtype=torch.int32, device="cuda") % (min(pitch, 5) + 1)).expand(1, hq, nqb).contiguous()
+    paging = {}
+    if page_size:
+        table = torch.randperm(n // page_size, device="cuda", generator=g).to(torch.int32).view(1, -1).contiguous()
+        pools = []
+        for x in (k, v):
+            pool = torch.empty(n // page_size, hkv, page_size, 128, dtype=torch.bfloat16, device="cuda")
+            pool[table.view(-1).long()] = x.view(hkv, n // page_size, page_size, 128).transpose(0, 1)
+            pools.append(pool)
+        k, v = pools
+        paging = dict(kv_page_table=table, kv_page_size=page_size, kv_num_pages=n // page_size, kv_pages_in_place=1)
+
+    def call(**kw):
+        bufs = alloc_outputs(q, nqb)
+        bufs["out"].fill_(77.0)
+        bufs["lse"].fill_(77.0)
+        bufs["visited"].fill_(-7)
+        bufs["scored"].fill_(-7)
+        cosa.cosa_osk_attention(q, k, v, order, count, tb, bufs["out"], bufs["lse"], bufs["visited"], causal=False,
+                                opt=cosa.default_options(skip_scale=500.0 if tb < 1 else -1.0, out_scored=bufs["scored"], order_stride=pitch, **paging, **kw))
+        status = cosa.cosa_device_status()
+        return [bufs["out"].view(-1, 128 * 128), bufs["lse"].view(-1, 128), bufs["visited"].view(-1, 1), bufs["scored"].view(-1, 1)], status
+
+    return call
+
+
+@pytest.mark.parametrize("pitch,tb,page_size", SHORT_FORMS)
+def test_osk_writes_a_work_item_whole_or_not_at_all_on_every_form(pitch, tb, page_size):
+    """The same budgets, and some at which the load warp leaves before it has read a work item (its first tile is then on its way all
+    the same where the item warp asks for it)."""
+    call = _short_call(pitch, tb, page_size)
+    want, status = call()
+    assert status == 0
+    in_part = 0
+    for cycles in [1, 20, 100, *range(200, 1000, 50), *range(1000, 9000, 25)]:
+        got, status = call(wait_cycles=cycles)
+        assert status in (0, TIMEOUT)
+        done = got[2][:, 0] != -7
+        for a, b, blank in zip(got, want, (77.0, 77.0, -7, -7)):
+            assert bool(torch.where(done[:, None], a == b, a == blank).all()), cycles
+        in_part += int(bool(done.any()) and not bool(done.all()))
+    assert in_part > 0
+    got, status = call()
+    assert status == 0 and all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("pitch,tb,page_size", SHORT_FORMS)
+def test_osk_wait_budget_of_one_cycle_on_every_form(pitch, tb, page_size):
+    call = _short_call(pitch, tb, page_size)
+    want, status = call()
+    assert status == 0
+    for _ in range(20):
+        got, status = call(wait_cycles=1)
+        assert status == TIMEOUT and cosa.cosa_device_status() == 0
+        assert int((got[2] == -7).sum()) > 0
+    got, status = call()
+    assert status == 0 and all(torch.equal(a, b) for a, b in zip(got, want))
