@@ -695,6 +695,92 @@ def test_osk_lists_of_one_length_at_two_pitches(batch, tb, skip_scale):
         assert torch.equal(x, y)
 
 
+def _lists_that_begin_with_the_diagonal_block(batch, hq, nqb, pitch, g, least):
+    """Causal lists of `least` to all candidates in random order behind the query block itself -> order [.., pitch], count"""
+    blocks = torch.arange(nqb, device="cuda")
+    rank = torch.rand(batch, hq, nqb, nqb, device="cuda", generator=g)
+    rank = rank.masked_fill(blocks[None, :] > blocks[:, None], 2.0).masked_fill(blocks[None, :] == blocks[:, None], -1.0)
+    order = torch.full((batch, hq, nqb, pitch), -1, dtype=torch.int32, device="cuda")
+    order[..., :nqb] = torch.argsort(rank, dim=-1).to(torch.int32)
+    count = least + torch.rand(batch, hq, nqb, device="cuda", generator=g) * (blocks + 2 - least)
+    return order, torch.minimum(count.to(torch.int32), (blocks + 1).to(torch.int32)).contiguous()
+
+
+@pytest.mark.parametrize("tb,skip_scale", [(0.999, 300.0), (0.3, -1.0), (0.15, 500.0)])
+@pytest.mark.parametrize("batch", [1, 16])
+def test_osk_short_lists_that_begin_with_the_diagonal_block(batch, tb, skip_scale):
+    """The tile which the item warp asks for is the masked one: the kernel for lists of up to 8 blocks and the one for longer lists
+    give the same bits."""
+    hq, hkv, n = 8, 2, 1024
+    g = torch.Generator(device="cuda").manual_seed(20 + batch)
+    q, k, v = (torch.randn(batch, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv, hkv))
+    order, count = _lists_that_begin_with_the_diagonal_block(batch, hq, 8, 9, g, 1)
+    got = []
+    for pitch in (8, 9):
+        out = torch.full_like(q, 3.0)
+        lse = torch.full(q.shape[:3], 3.0, device="cuda")
+        vis = torch.full(count.shape, -7, dtype=torch.int32, device="cuda")
+        cosa.cosa_osk_attention(q, k, v, order[..., :pitch].contiguous(), count, tb, out, lse, vis,
+                                opt=cosa.default_options(skip_scale=skip_scale, order_stride=pitch))
+        assert cosa.cosa_device_status() == 0
+        got.append((out, lse, vis))
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("pitch", [8, 9])
+def test_osk_stage2_off_against_the_check_kernel(pitch):
+    """Lists of 0 to 8 blocks with Stage 2 off against the kernel without tensor cores (tolerances of the randomised comparison of the
+    two)."""
+    batch, hq, hkv, n = 4, 8, 2, 1024
+    g = torch.Generator(device="cuda").manual_seed(pitch)
+    q, k, v = (torch.randn(batch, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv, hkv))
+    order, count = _lists_that_begin_with_the_diagonal_block(batch, hq, 8, pitch, g, 0)
+    got = []
+    for impl in (0, 1):
+        out = torch.full_like(q, 3.0)
+        lse = torch.full(q.shape[:3], 3.0, device="cuda")
+        vis = torch.full(count.shape, -7, dtype=torch.int32, device="cuda")
+        cosa.cosa_osk_attention(q, k, v, order, count, 1.0, out, lse, vis, opt=cosa.default_options(skip_scale=-1.0, order_stride=pitch, impl=impl))
+        assert cosa.cosa_device_status() == 0
+        got.append((out.float(), lse, vis))
+    assert torch.equal(got[0][2], count) and torch.equal(got[1][2], count)
+    assert float((got[0][0] - got[1][0]).abs().max()) < 4e-2
+    rows = (count > 0).repeat_interleave(128, dim=-1)
+    assert float((got[0][1] - got[1][1])[rows].abs().max()) < 2e-3
+    assert bool(torch.isinf(got[0][1][~rows]).all()) and bool((got[0][0][~rows] == 0).all())
+
+
+@pytest.mark.parametrize("page_size", [16, 32])
+@pytest.mark.parametrize("n,hkv,lens", [(8192, 8, (64, 33)), (16384, 8, (70, 128)), (5120, 16, (1, 40, 23))])
+def test_osk_page_copies_of_prompts_of_different_lengths(n, hkv, lens, page_size):
+    """Copies in which a warp takes 4, 8 and 7 turns, of prompts that end anywhere in them and whose table rows name some other page
+    behind their end: the walks of the dense tensors."""
+    batch, hq, nqb = len(lens), 16, n // 128
+    g = torch.Generator(device="cuda").manual_seed(n + page_size)
+    q, k, v = (torch.randn(batch, heads, n, 128, device="cuda", generator=g).to(torch.bfloat16) for heads in (hq, hkv, hkv))
+    seq_lens = torch.tensor([x * 128 for x in lens], dtype=torch.int32, device="cuda")
+    inside = torch.arange(nqb, device="cuda") < torch.tensor(lens, device="cuda")[:, None]
+    rank = torch.rand(batch, hq, nqb, nqb, device="cuda", generator=g).masked_fill(~inside[:, None, None, :], 2.0)
+    order = torch.argsort(rank, dim=-1)[..., :12].to(torch.int32).contiguous()
+    count = torch.tensor([min(x, 12) for x in lens], dtype=torch.int32, device="cuda")[:, None, None].expand(batch, hq, nqb).contiguous()
+    table = torch.randperm(batch * n // page_size, device="cuda", generator=g).to(torch.int32).view(batch, -1).contiguous()
+    pools = _scattered(k, table, page_size), _scattered(v, table, page_size)
+    for b, blocks in enumerate(lens):
+        table[b, blocks * 128 // page_size:] = 0
+    got = []
+    for kk, vv, extra in ((k, v, {}), (*pools, dict(kv_page_table=table, kv_page_size=page_size, kv_num_pages=table.numel()))):
+        out = torch.full_like(q, 3.0)
+        lse = torch.full(q.shape[:3], 3.0, device="cuda")
+        vis = torch.full(count.shape, -7, dtype=torch.int32, device="cuda")
+        cosa.cosa_osk_attention(q, kk, vv, order, count, 0.999, out, lse, vis, causal=False,
+                                opt=cosa.default_options(skip_scale=100.0, order_stride=12, seq_lens=seq_lens, **extra))
+        assert cosa.cosa_device_status() == 0
+        got.append((out, lse, vis))
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
+
+
 @pytest.mark.parametrize("walk", ["dense", "mask", "page16"])
 @pytest.mark.parametrize("tb,skip_scale", [(1.0, -1.0), (0.999, 300.0), (0.3, -1.0), (0.15, 500.0)])
 def test_osk_ctas_that_take_over_further_work_items(tb, skip_scale, walk):
