@@ -71,7 +71,9 @@ cudaError_t launch_gather_pages(const __nv_bfloat16* k_pool, __nv_bfloat16* k_de
   t.pool[0] = reinterpret_cast<const uint4*>(k_pool); t.dense[0] = reinterpret_cast<uint4*>(k_dense);
   t.pool[1] = reinterpret_cast<const uint4*>(v_pool); t.dense[1] = reinterpret_cast<uint4*>(v_dense);
   const int per_cta = kThreads / 32 * kRowsPerWarp, heads = batch * hkv, parts = (n / every + per_cta - 1) / per_cta;
-  // (turns only where some thousand CTAs are left)
+  // Turns only where some thousand CTAs are left.  K and V in 16-token pages of 8 KV heads, cold, us with one turn / with the rule's: 4K
+  // tokens (one) 16.4, 8K (2 turns) 22.5 / 22.5, 12K (3) 28.7 / 28.7, 16K (4) 35.3 / 34.8, 24K (6) 49.2 / 45.1, 32K (8) 61.4 / 56.8, 128K (8)
+  // 221 / 186, four prompts of 10K to 16K (8) 98 / 82.  Twelve gain no more (55 to 184 and 84); two where the rule gives eight lose (225, 106)
   const int turns = v_pool ? (int)std::min<long long>(8, std::max<long long>(1, (long long)parts * heads * 2 / 1024)) : 1;
   const dim3 grid((unsigned)((parts + turns - 1) / turns), (unsigned)(heads < 65535 ? heads : 65535), v_pool ? 2 : 1);
   return launch_chained(turns > 1 ? gather_pages_kernel<true> : gather_pages_kernel<false>, grid, kThreads, 0, st, t, pg, heads, hkv, n, every);

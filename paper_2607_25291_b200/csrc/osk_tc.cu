@@ -804,7 +804,7 @@ cudaError_t launch_osk_tc(const OskParams& p_in, cudaStream_t st) {
   // Stage 2 off        112/115  179/193  316/322  446/459  562/573    811/817  1040/1038  1529/1532  2008/2010 (in one place: 107, 182, 308, 435, ...)
   // on                 111/113  167/179  277/265  362/354  425/413    554/540    693/678    917/901  1139/1116
   // on, cap half of it   95/102  128/131  209/209  304/300  393/382    540/528    665/652    918/905  1128/1101
-  // (the 128K layer, Stage 2 on: 7,860/7,757).  With Stage 2 off the tiles' code is shared at every length, but for small pages.  Those,
+  // (the 128K layer, Stage 2 on: 7,860/7,757; of 9 to 15 blocks 318/314, 359/350, 392/371, 420/418, 456/454, 510/500, 522/517).  With Stage 2 off the tiles' code is shared at every length, but for small pages.  Those,
   // read in place, Stage 2 off (P's first half over S and shared code, at pitches from 8 up: 8 to 12 % more than the written-out form,
   // pages of 64 2 to 4):
   //                          2        4        8       16       32         64 blocks
