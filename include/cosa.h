@@ -135,8 +135,8 @@ typedef struct {
                               is 0): every tile is assembled from the pages themselves, one pair of boxes per page,
                               issued side by side by the lanes of a warp after their table look-ups.  Same results;
                               slower with small pages on long lists, since the copy engine works box by box (128K tokens:
-                              7.6 ms staged; 9.1 in place at 16-token pages, 7.5 at 64; four prompts of 10K to 16K
-                              tokens in 16-token pages: 0.69 staged, 0.70 in place)                           */
+                              7.1 ms staged; 8.1 in place at 16-token pages, 7.1 at 64; four prompts of 9K to 16K
+                              tokens in 16-token pages: 0.54 to 0.79 staged, 2 to 5 % more in place)          */
   const int32_t* seq_lens; /* Non-NULL: device array [B]; batch item b holds seq_lens[b] tokens, a multiple
                               of 128 in [128, N] (a batch of prompts of different lengths, padded to N;
                               Sec. C.1 runs inside a paged serving engine, where this is the rule).  Rows

@@ -21,18 +21,16 @@
 // blocks have 16 sampled rows or more: a thread keeps its block maxima in registers and, when
 // every product is done, lays them into the key stages, from where the scores are formed; the norms of the sampled keys are
 // taken from the stages as well, which saves the norms kernel's launch.
-// A CTA holds every score of its lists, and up to 256 candidates it sorts them itself, a warp a list in registers: no sort kernel (a
-// wave of small CTAs each, chains of short steps between barriers), and no scores cross a launch, only the lists (a byte an entry).
-// Stage 1 at 32K 160 -> 135 us, of four prompts of 8K to 16K tokens in 16-token pages 157 -> 121, of 201 blocks with Top-p 136 -> 110,
-// of 55 blocks at stride 4 102 -> 58.  Both together, in short calls a chain of latencies (launch, first loads, a wave or two of CTAs): 1K tokens of 2 heads 13.5 -> 10.5 us, 31 blocks of
-// 32 heads 18.0 -> 14.6, 2 x 61 blocks of 32 heads 70 -> 43.
+// A CTA holds every score of its lists, and up to 256 candidates it sorts them itself, a warp a list in registers (list_sort.cuh): no sort
+// kernel (a wave of small CTAs each, chains of short steps between barriers), and no scores cross a launch, only the lists (a byte an
+// entry).  Against the sort kernel Stage 1 took 135 us instead of 160 at 32K, 58 instead of 102 for 55 blocks at stride 4, 43 instead of 70
+// for 2 x 61 blocks of 32 heads.
 // What bounds the tiles of long calls: the tensor pipe, which takes 1,139 cycles of an SM a key tile for two products; with both operands
-// in shared memory and 128 columns a product takes 570 or more, not 512.  (Issued under lane == 0, not elect.sync, a tile took 1,518:
-// Stage 1 at 128K 1,314 -> 1,213 us, at 32K 140 -> 129.)  A CTA at 32K (16.5 tiles): 41,400 cycles, of them 6,600 to the first logits,
-// 19,000 for tiles, 1,700 for M* and thresholds, 5,700 for scores, 7,500 for lists; at 128K (64.5 tiles) 97,000, scores 16,000.  What a CTA
-// needs once has two warps of its own, which work while products run (32K 129 -> 124 us, four paged prompts 120 -> 113, 31 blocks of 32
-// heads 14.1 -> 12.9).  CTAs that stay for further items, whose query rows and first tiles come under the lists, were not kept:
-// four paged prompts 108 -> 99 us, 32K 116 -> 113, 64K 356 -> 351, 128K the same, for a slower second phase and a page of code.
+// in shared memory and 128 columns a product takes 570 or more, not 512.  (Issued under lane == 0, not elect.sync, a tile took 1,518.)
+// A CTA at 32K (16.5 tiles): 41,400 cycles, of them 6,600 to the first logits, 19,000 for tiles, 1,700 for M* and thresholds, 5,700 for
+// scores, 7,500 for lists; at 128K (64.5 tiles) 97,000, scores 16,000.  Short calls are a chain of latencies: launch, first loads, a wave
+// or two of CTAs.  What a CTA needs once has two warps of its own, which work while products run (by the epilogue warps first: 129 us at
+// 32K instead of 124, 14.1 for 31 blocks of 32 heads instead of 12.9).
 // Float32 results are a SCREEN: the sort stage recomputes in double precision whatever a
 // rounding error could reorder.  For that it is told, per sampled row, the two blocks with the
 // largest block maxima and whether they are closer than tau_row (the row's HRM flag and M* are
@@ -65,7 +63,8 @@ constexpr int kAuxThreads = 64;       // two warps for what a CTA needs once: sc
 constexpr int kThreads = 64 + kEpiThreads + kAuxThreads;    // producer warp, MMA warp, epilogue warps, aux warps
 constexpr int kSteps = 2;             // key tiles whose logits are in tensor memory at once
 constexpr int kTmemCols = 128 * kRowTiles * kSteps;
-// 20 warps, five a scheduler: a thread has 96 registers.  The forms spill up to 24 bytes
+// 20 warps, five a scheduler: a thread has 96 registers.  The forms spill up to 24 bytes (loads: up to 32, of the long form with lists and 32
+// sampled rows a block 64)
 constexpr int kCtasPerSm = 1;
 static_assert(kTmemCols == 512 && kPartCols == 64, "TMEM budget and two 32-column loads per thread and tile");
 

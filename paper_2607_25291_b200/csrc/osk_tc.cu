@@ -37,19 +37,14 @@
 // therefore shared rather than unrolled or inlined twice where walks are short (a form of 88 KB instead of 61: 236 us instead of
 // 209 on walks of 3.4 blocks; one place that fetches K and V tiles instead of two: 175 -> 169, and 3 % of the walks of four
 // prompts in 16-token pages); with Stage 2 and with small pages long ones have it written out (kLongWalks).
-// What bounds it: tensor pipe and exponentials both want about 1,024 cycles (0.52 us) of an SM per computed block, 512 per skipped
-// one.  By clock stamps an SM takes 1,600 cycles a computed block with Stage 2 off, 2,100 with it on (the vote, and V only after it), 620 a
+// What bounds it: tensor pipe and exponentials both want about 1,024 cycles of an SM per computed block, 512 per skipped one.  By
+// clock stamps an SM takes 1,600 cycles a computed block with Stage 2 off, 2,100 with it on (the vote, and V only after it), 620 a
 // skipped one -- a product whose operands both come from shared memory takes the tensor pipe 570 to 600, not 512 -- and 2,600 a work
-// item.  At 32K tokens the pipe is busy 58 % of the time, shared memory's data pipe 82 % (operands 58, threads 24).  A walk alone on an
-// SM takes 3,900 cycles a computed block: two fill each other's waits, the row threads of both together want 2,500 for two blocks.
-// Single launches, a CTA an item -> several -> items decoded in a warp of their own -> now: 128K tokens and 4 % computed 7.51 -> 7.39 -> 7.30 ->
-// 6.71 ms, 32K and 8 % 1.08 -> 1.02 -> 0.95 -> 0.90, all blocks of 16K 1.92 -> 1.89 -> 1.81 -> 1.74, walks of 3.4 blocks (2 x 7,808 tokens) 0.246
-// -> 0.214 -> 0.167 -> 0.158 (32 query heads everywhere; one CTA of twelve warps per SM with two softmax groups and a controller
-// warp, the arrangement before all of these: 8.1, 1.25 and 2.00 on the first three).  Measured and not used: P over S in tensor memory with
-// the next S behind both halves (all blocks of 16K +6.5 %), two threads per row (8.2 / 1.15 / 2.12 ms when the first three took
-// 7.15, 1.02 and 1.85), tiles prefetched into L2 (+2 to 5 %), V(k) requested before the decision on k after a computed block (+4 to
-// 9 %; V(0), which is certain, gains nothing), a share of the exponentials by polynomial (+2 to 10 %: their issue slots are the other warps'),
-// Q K^T held back where the next computed block ends the walk (+0.3 to 3.5 %), the output by TMA or in 32-byte stores without staging (+0 to 11 %).
+// item.  (Cycles of the SM's own counter, which runs at 1.65 to 1.75 GHz under this kernel even where 1,965 MHz are reported.)  At 32K
+// tokens the pipe is busy 58 % of the time, shared memory's data pipe 82 % (operands 58, threads 24).  A walk alone on an SM takes
+// 3,900 cycles a computed block: two fill each other's waits, the row threads of both together want 2,500 for two blocks.
+// Single launches, 32 query heads: 128K tokens and 4 % computed 6.7 to 7.0 ms on four GPUs, 32K and 8 % 0.90, all blocks of 16K 1.74, walks of
+// 3.4 blocks (2 x 7,808 tokens) 0.158 (with a CTA an item 7.51, 1.08, 1.92 and 0.246).
 // Every wait is bounded; a wait that runs out sets the device status word and the CTA winds down without writing
 // further results (a work item's are written whole or not at all): load and issue warps leave, the row threads, whom no wait holds any more, run to the end of their list.
 #include <math.h>
@@ -160,8 +155,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 osk_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
               const __grid_constant__ CUtensorMap v_map, OskParams p, int32_t* status) {
   constexpr bool kPInTmem = !kStage2 && !kSmallPages;   // P's first half goes to tensor memory, over S
-  // Short walks: a CTA's first tile is asked for by the item warp (8 blocks of 2 heads, whole pass 19.4 -> 19.2 us, 32 of 4 heads 26.9 -> 26.3, 31 of 32
-  // heads 46.9 -> 46.4; with the longer code 2 x 61 blocks +1.8 %, 32K +1.3)
+  // Short walks: a CTA's first tile is asked for by the item warp (8 blocks of 2 heads 7.4 -> 6.9 us; whole passes enqueued ahead of the
+  // device, medians of 25 within 0.1 to 0.3: 8 blocks of 2 heads 18.9 -> 18.5, 32 of 4 heads 27.1 -> 26.4, 31 of 32 heads 47.3 -> 47.0; with the
+  // longer code 2 x 61 blocks +1.8 %, 32K +1.3)
   constexpr bool kEarlyTile = kStage2 && !kLongWalks && !kMask;
   extern __shared__ __align__(1024) unsigned char smem_raw[];   // swizzled tiles need 1024-byte alignment
   unsigned char* smem = smem_raw;

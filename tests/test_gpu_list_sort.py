@@ -82,7 +82,7 @@ def test_lists_are_sorted_whatever_their_scores(sort_lists, J, kind):
 @pytest.mark.parametrize("kind", ["equal", "rising", "one word"])
 def test_lists_of_scores_close_together_take_a_bounded_time(sort_lists, kind):
     """256 candidates, their scores in one sort word: at most six times the time of scores far apart.  (By instructions, words sorted and
-    settled in two turns come to some 1,050, the same with eight turns and a sort of whole keys to 4,350; 128 turns to 10,500.)"""
+    settled in two turns come to some 1,050, with six turns and a second sort of words to 2,300, 128 turns to 10,500.)"""
     rng = np.random.default_rng(1)
     far, close = (np.median([sort_lists(scores_of(k, 64, 256, rng))[1] for _ in range(3)]) for k in ("spread", kind))
     assert close <= 6 * far, (close, far)
